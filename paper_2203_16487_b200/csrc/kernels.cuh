@@ -855,79 +855,6 @@ __global__ void k_accept(const RowPart* __restrict__ part, int n_tiles, const fl
     if (fc.on) { __syncthreads(); commit_post(fc.s, fc.post); }
 }
 
-// The same rule on caller-provided logits [B, k+1, V]: one block per sequence walks the rows
-// in order and stops at the first rejected draft, so it needs no scratch memory.
-__global__ void k_accept_logits(const float* __restrict__ logits, const int* __restrict__ draft, int k, int V,
-                                int beta, float tau, int* __restrict__ accepted, int* __restrict__ bif) {
-    __shared__ RowPart wsm[32];
-    __shared__ int stop;
-    const int b = blockIdx.x;
-    for (int c = 0; c <= k; ++c) {
-        const float* l = logits + ((size_t)b * (k + 1) + c) * V;
-        const int tok = (c < k) ? draft[b * k + c] : -1;
-        const float ld = (c == k) ? CUDART_INF_F : ((tok >= 0 && tok < V) ? l[tok] : -CUDART_INF_F);
-        RowPart m; m.mx = -CUDART_INF_F; m.arg = 0x7fffffff; m.sum = 0.f; m.cnt = 0;
-        for (int v = threadIdx.x; v < V; v += blockDim.x) {
-            RowPart q; q.mx = l[v]; q.arg = v; q.sum = 1.f; q.cnt = (l[v] > ld) ? 1 : 0;
-            part_merge(m, q);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            RowPart q;
-            q.mx = __shfl_xor_sync(0xffffffffu, m.mx, o);
-            q.arg = __shfl_xor_sync(0xffffffffu, m.arg, o);
-            q.sum = __shfl_xor_sync(0xffffffffu, m.sum, o);
-            q.cnt = __shfl_xor_sync(0xffffffffu, m.cnt, o);
-            part_merge(m, q);
-        }
-        if ((threadIdx.x & 31) == 0) wsm[threadIdx.x >> 5] = m;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) part_merge(m, wsm[w]);
-            const bool ok = (c < k) && (m.cnt <= beta - 1) && ((m.mx - ld) <= tau);
-            stop = ok ? 0 : 1;
-            if (!ok) { accepted[b] = c; bif[b] = m.arg; }
-        }
-        __syncthreads();
-        if (stop) return;
-    }
-}
-
-// Per (row, tile of `tile` columns) statistics of caller-provided logits [rows, V]: the first stage of the
-// two-stage acceptance scan whose partials live in the library's static scratch array.
-__global__ void k_logit_tile_stats(const float* __restrict__ logits, const int* __restrict__ draft, int k, int V,
-                                   int tile, int n_tiles, RowPart* __restrict__ part, float* __restrict__ ld_out,
-                                   int* __restrict__ id_out) {
-    __shared__ RowPart wsm[32];
-    const int row = blockIdx.y, t = blockIdx.x, b = row / (k + 1), c = row % (k + 1);
-    const float* l = logits + (size_t)row * V;
-    const int tok = (c < k) ? draft[b * k + c] : -1;
-    const bool ok = tok >= 0 && tok < V;
-    const float ld = (c == k) ? CUDART_INF_F : (ok ? l[tok] : -CUDART_INF_F);
-    RowPart m; m.mx = -CUDART_INF_F; m.arg = 0x7fffffff; m.sum = 0.f; m.cnt = 0;
-    const int v1 = min(V, (t + 1) * tile);
-    for (int v = t * tile + threadIdx.x; v < v1; v += blockDim.x) {
-        RowPart q; q.mx = l[v]; q.arg = v; q.sum = 1.f; q.cnt = (l[v] > ld) ? 1 : 0;
-        part_merge(m, q);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        RowPart q;
-        q.mx = __shfl_xor_sync(0xffffffffu, m.mx, o);
-        q.arg = __shfl_xor_sync(0xffffffffu, m.arg, o);
-        q.sum = __shfl_xor_sync(0xffffffffu, m.sum, o);
-        q.cnt = __shfl_xor_sync(0xffffffffu, m.cnt, o);
-        part_merge(m, q);
-    }
-    if ((threadIdx.x & 31) == 0) wsm[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) part_merge(m, wsm[w]);
-        part[(size_t)row * n_tiles + t] = m;
-        if (t == 0) { ld_out[row] = ld; id_out[row] = (c == k) ? -1 : (ok ? tok : -2); }
-    }
-}
-
 // ------------------------------------------------------------------ drafter argmax
 // script (optional; benchmark / test hook): draft i of a sequence with j committed tokens is replaced by
 // script[b * stride + j + i] wherever that entry is >= 0 (len = the committed lengths, k = drafts per sequence).
