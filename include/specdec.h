@@ -264,12 +264,11 @@ int specdec_profile_read(specdec_handle* h, double* h_ms, long long* h_launches)
  *                does not.  Takes effect at the next specdec_encode.
  * "gemm"         0 SIMT reference GEMM / 1 tcgen05 tensor-core GEMM (bf16 handles; default 1)
  * "attn"         0 warp-per-row reference attention / 1 tensor-core tile attention (bf16, 64-wide heads; default 1)
- * "skinny"       0/1 weight-streaming GEMM with fused LayerNorm for passes of at most 32 rows (default 1)
- * "sk_cluster"   0 off / 1 (default): those GEMMs run in clusters of 8 CTAs that share the normalised input rows
- *                through distributed shared memory; 2 / 3 also the GEMMs without a LayerNorm (K <= 512 / all)
+ * "skinny"       0/1 weight-streaming GEMM for passes of at most 384 rows (default 1), up to 144 rows with the LayerNorm
+ *                in front fused
+ * "sk_cluster"   0/1 (default 1): that GEMM splits reductions of 1024 and more across a cluster of 2 or 4 CTAs
  * "pair"         0/1 two-SM tensor-core tiles (cta_group::2) for GEMMs with >= 1024 rows and columns (default 0)
- * "enc_skinny"   0 / 1 (default) / 2: the weight-streaming GEMM also serves neither / the drafter's / both encoders when a
- *                source has at most 32 positions
+ * "enc_skinny"   0 / 1 (default) / 2: the weight-streaming GEMM does not / does / does serve the encoders (up to 208 rows)
  * "ln_fuse"      0/1 the LayerNorm that reads the residual stream next runs inside the residual GEMM (default 0)
  * "splitk"       0/1 residual GEMMs with K >= 1024 over few row tiles split K across a cluster (default 1)
  * "attn_rs"      0 never / 1 by rule (default) / 2 whenever the keys allow: scores stay in the MMA accumulators

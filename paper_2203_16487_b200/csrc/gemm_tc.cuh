@@ -459,17 +459,16 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     constexpr int STAGES = Cfg::STAGES;
     constexpr int A_BYTES = AR * TC_BK * 2;          // activation part of a stage
     if (threadIdx.x == 0) tc_stamp(g.trace, 0);
-    // The kernel sets itself up (barriers, tensor memory) and lets its successors start before its predecessor has
-    // finished (programmatic dependent launch).  With a row count known on the host, or rows that fit one row tile
-    // whatever their count (one_m_tile), it also knows its first tile and starts streaming that tile's weights; a
-    // device-side count is read after the wait.  (Requesting the first tile's weights before the wait for those
-    // launches too -- tiles numbered column tile fastest, a drain path for CTAs left without a tile -- measured no gain.)
-    const bool early = g.rows_static >= 0 || g.one_m_tile;
-    int R = g.rows_static >= 0 ? g.rows_static : 0;
-    int m_tiles = g.one_m_tile ? 1 : (R + TC_BM - 1) / TC_BM;
+    // The kernel sets itself up (barriers, tensor memory), starts streaming its first tile's weights and lets its successors
+    // start before its predecessor has finished (programmatic dependent launch).  A row count on the device is written at the
+    // start of the step, before the first kernel of the chain can begin, so it may be read ahead of the wait.  A CTA
+    // without a tile leaves at once; with no rows at all one row tile still runs (on rows nobody reads, storing nothing), so
+    // that the grid never completes ahead of its predecessor.
+    const int R = g.rows_static >= 0 ? g.rows_static : *g.n_rows;
+    const int m_tiles = max((R + TC_BM - 1) / TC_BM, 1);
     const int n_tiles = (g.N + BN - 1) / BN;
-    int total = m_tiles * n_tiles;
-    if (g.rows_static >= 0 && (int)blockIdx.x >= total) return;   // (static count) whole CTA leaves before touching barriers or tensor memory
+    const int total = m_tiles * n_tiles;
+    if ((int)blockIdx.x >= total) return;              // whole CTA leaves before touching barriers or tensor memory
 
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[STAGES], bar_empty[STAGES], bar_acc_full[2], bar_acc_empty[2];
@@ -509,23 +508,16 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     volatile int* abort_flag = &abort_s;
     if (threadIdx.x == 0 && tmem_d != 0xffffffffu) tc_stamp(g.trace, 1);   // (the test pins the stamp behind the read)
     int pre = 0;                                       // stages whose weight half was requested before the wait
-    if (early) {
-        if (threadIdx.x == 0) {
-            const int n0 = (LNF ? (int)blockIdx.x % n_tiles : (int)blockIdx.x / m_tiles) * BN;
-            for (; pre < STAGES && pre < nkb; ++pre) {
-                const uint32_t bar = smem_u32(&bar_full[pre]);
-                mbar_expect_tx(bar, Cfg::STAGE_BYTES);
-                tma_load_2d(tiles + pre * Cfg::STAGE_BYTES + A_BYTES, &tmW, pre * TC_BK, n0, bar);
-            }
+    if (threadIdx.x == 0) {
+        const int n0 = (LNF ? (int)blockIdx.x % n_tiles : (int)blockIdx.x / m_tiles) * BN;
+        for (; pre < STAGES && pre < nkb; ++pre) {
+            const uint32_t bar = smem_u32(&bar_full[pre]);
+            mbar_expect_tx(bar, Cfg::STAGE_BYTES);
+            tma_load_2d(tiles + pre * Cfg::STAGE_BYTES + A_BYTES, &tmW, pre * TC_BK, n0, bar);
         }
     }
     pdl_launch_dependents();
     pdl_wait();                                        // activations, residual and outputs belong to the predecessors until here
-    if (g.rows_static < 0) {
-        R = *g.n_rows;
-        if (!g.one_m_tile) m_tiles = (R + TC_BM - 1) / TC_BM;
-        total = m_tiles * n_tiles;                     // a CTA without a tile walks through its empty loops to the common exit
-    }
 
     if (warp == 0) {
         if (lane == 0) {
@@ -776,7 +768,6 @@ inline int tc_launch_ln_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cud
 }
 inline int gemm_tc_launch_ln(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
     if (!enc.ready) return -1;
-    g.one_m_tile = 0;
     // 64-wide tiles (clusters of up to 8) while there are few row tiles, 128-wide otherwise and for wide models
     const bool narrow = rows_ub <= 2 * TC_BM && g.N <= 512;
     return narrow ? tc_launch_ln_one<64>(enc, g, rows_ub, st) : tc_launch_ln_one<128>(enc, g, rows_ub, st);
@@ -825,7 +816,6 @@ inline int gemm_tc_launch(TmaEncoder& enc, int epi, GemmArgs<bf16>& g, int rows_
         if (enc.force_bn == 128 || enc.force_bn == 256 || (enc.force_bn == 224 && rows_ub <= TC_BM)) bn = enc.force_bn;
         g.n_tiles = 2 * ((g.N + bn - 1) / bn);                   // two column halves per tile
         if (n_tiles_out) *n_tiles_out = g.n_tiles;
-        g.one_m_tile = (bn == 224);
         if (bn == 224)      // one tile per CTA: the ring is as deep as shared memory allows, most of it requested up front
             return rows_ub <= 32 ? tc_launch_one<EPI_STATS, 224, 32>(enc, g, rows_ub, st)
                  : rows_ub <= 64 ? tc_launch_one<EPI_STATS, 224, 64>(enc, g, rows_ub, st)
@@ -835,7 +825,6 @@ inline int gemm_tc_launch(TmaEncoder& enc, int epi, GemmArgs<bf16>& g, int rows_
     const int fb = enc.force_bn;
     const bool forced = (fb == 32 || fb == 64 || fb == 128 || fb == 192 || fb == 256) && fb <= g.N;
     const int bn = forced ? fb : tc_pick_bn(g.N, rows_ub, enc.n_sm);
-    g.one_m_tile = rows_ub <= TC_BM;        // one row tile whatever the device-side count says: set up and prefetch before the wait
     switch (epi) {
         case EPI_STORE: return tc_launch_bn<EPI_STORE>(enc, bn, g, rows_ub, st);
         case EPI_RELU: return tc_launch_bn<EPI_RELU>(enc, bn, g, rows_ub, st);

@@ -441,7 +441,6 @@ inline int vocab_pair_launch(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cu
 
 inline int gemm_tc_pair_launch(TmaEncoder& enc, int epi, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st, int* n_tiles_out) {
     if (!enc.ready) return -1;
-    g.one_m_tile = 0;
     switch (epi) {
         case EPI_QKV: return tc_pair_launch_one<EPI_QKV, 256>(enc, g, rows_ub, st);
         case EPI_RELU: return tc_pair_launch_one<EPI_RELU, 256>(enc, g, rows_ub, st);

@@ -61,7 +61,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // One link of a chain of dependent launches (diagnostics: what one kernel boundary costs inside a step): waits for its
 // predecessor, reads the word it wrote, and the first thread writes it back incremented.
-__global__ void k_link(int* word) {
+static __global__ void k_link(int* word) {
     pdl_launch_dependents();
     pdl_wait();
     const int v = *reinterpret_cast<volatile int*>(word);
@@ -76,13 +76,13 @@ struct Session {
     int* src_len;      // [B]
     int* out;          // [B, out_stride] committed ids
     int out_stride;
-    int* counters;     // [8]: 0 rows of the drafter's full pass, 1 rows of its mask-only pass,
-                       //      2 verify rows, 3 encoder rows, 4 unfinished sequences
+    int* counters;     // [16]: 0 rows of the drafter's full pass, 1 rows of its mask-only pass,
+                       //       2 verify rows, 3 encoder rows, 4 unfinished sequences, 8 longest committed length
     unsigned long long* stats;  // [4]: seq_iterations, drafted, accepted, emitted
     int* dlen;         // [B] prefix-causal drafter: positions of [BOS, committed...] whose K/V its cache already holds
     int* dticket;      // [1] block ticket of the drafter's row preparation
 };
-enum { CNT_DRAFT_ALL = 0, CNT_DRAFT_MASK = 1, CNT_VERIFY = 2, CNT_ENC = 3, CNT_ACTIVE = 4, CNT_TICKET = 5, CNT_SEQ = 6 };
+enum { CNT_DRAFT_ALL = 0, CNT_DRAFT_MASK = 1, CNT_VERIFY = 2, CNT_ENC = 3, CNT_ACTIVE = 4, CNT_TICKET = 5, CNT_SEQ = 6, CNT_MAXLEN = 8 };
 
 // Per-row metadata of the pass being run.
 struct Rows {
@@ -97,11 +97,12 @@ struct Rows {
     int* slot;      // mask-only pass: index into the [B,k] draft array
     int* q_off;     // [B] first row of the sequence in this pass
     int* q_cnt;     // [B] rows of the sequence in this pass (0: none)
+    int* slot_seq;  // [B] verify pass: the sequence whose block starts at row slot * (k + 1)
 };
 
 // ------------------------------------------------------------------ row preparation
 // Encoder: rows are the padded [B,S_max] grid.
-__global__ void k_enc_prep(const int* __restrict__ src, const int* __restrict__ src_len, int B, int S_max,
+static __global__ void k_enc_prep(const int* __restrict__ src, const int* __restrict__ src_len, int B, int S_max,
                            Rows r, int* counters) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) counters[CNT_ENC] = B * S_max;
@@ -115,46 +116,59 @@ __global__ void k_enc_prep(const int* __restrict__ src, const int* __restrict__ 
     r.nk_cross[i] = src_len[b];
 }
 
-// Verify block: row b*(k+1)+i holds [last committed token (BOS if none), drafts] at positions j..j+k.
-__global__ void k_verify_prep(Session s, const int* __restrict__ draft, int B, int k, int S_max, int bos,
-                              Rows r) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) s.counters[CNT_VERIFY] = B * (k + 1);
-    if (i < B) { r.kv_off_cross[i] = i * S_max; r.q_off[i] = i * (k + 1); r.q_cnt[i] = k + 1; }
-    if (i >= B * (k + 1)) return;
-    int b = i / (k + 1), c = i % (k + 1);
-    int j = s.len[b];
-    r.tok[i] = (c == 0) ? (j == 0 ? bos : s.out[(size_t)b * s.out_stride + j - 1]) : draft[b * k + c - 1];
-    r.pos[i] = j + c;
-    r.seq[i] = b;
-    r.nk_self[i] = j + c + 1;     // causal: positions 0..j+c
-    r.nk_cross[i] = s.src_len[b];
-}
-
-// The same, together with the embedding of the block's rows (x = sqrt(d) E[tok] + P[pos]): one block per row.  The row
-// metadata is complete before the block lets its successors start, because kernels further down the chain read it
-// ahead of their own dependency waits.
+// Verify block: row slot * (k+1) + c holds [last committed token (BOS if none), drafts] at positions j..j+k of the slot's
+// sequence, together with its embedding (x = sqrt(d) E[tok] + P[pos]); one block per row.  compact = 0: slot = sequence.
+// compact = 1 (the generation loop): the slots are the unfinished sequences only, in index order -- in a ragged batch
+// more than half of all blocks would belong to sequences that ended iterations ago.  The row metadata is complete before the
+// block lets its successors start, because kernels further down the chain read it ahead of their own dependency waits.
 template <typename T>
 __global__ void k_verify_prep_embed(Session s, const int* __restrict__ draft, int B, int k, int S_max, int bos, Rows r,
                                     const T* __restrict__ E, const float* __restrict__ P, float* __restrict__ x, int d,
-                                    float scale, int vocab, int max_pos) {
-    const int i = blockIdx.x;                      // row b * (k + 1) + c
+                                    float scale, int vocab, int max_pos, int compact) {
+    __shared__ int s_b, s_live;
+    const int i = blockIdx.x;                      // row slot * (k + 1) + c
     pdl_wait();                                    // session state comes from the previous step's commit
-    const int b = i / (k + 1), c = i % (k + 1);
-    const int j = s.len[b];
-    const int tok = (c == 0) ? (j == 0 ? bos : s.out[(size_t)b * s.out_stride + j - 1]) : draft[b * k + c - 1];
+    const int slot = i / (k + 1), c = i % (k + 1);
+    int b = slot;
+    if (compact) {
+        if (threadIdx.x < 32) {                    // the slot-th unfinished sequence, and how many there are
+            int seen = 0, found = -1;
+            for (int o = 0; o < B; o += 32) {
+                const int q = o + (int)threadIdx.x;
+                const bool fin = q >= B || s.finished[q] != 0;
+                const unsigned live = __ballot_sync(0xffffffffu, !fin);
+                if (!fin && seen + __popc(live & ((1u << threadIdx.x) - 1u)) == slot) found = q;
+                if (i == 0 && fin && q < B) r.q_cnt[q] = 0;
+                seen += __popc(live);
+            }
+            for (int o = 16; o > 0; o >>= 1) found = max(found, __shfl_xor_sync(0xffffffffu, found, o));
+            if (threadIdx.x == 0) { s_b = found; s_live = seen; }
+        }
+        __syncthreads();
+        b = s_b;
+    }
+    int j = 0, tok = 0;
+    if (b >= 0) {
+        j = s.len[b];
+        tok = (c == 0) ? (j == 0 ? bos : s.out[(size_t)b * s.out_stride + j - 1]) : draft[b * k + c - 1];
+    }
     if (threadIdx.x == 0) {
-        if (i == 0) s.counters[CNT_VERIFY] = B * (k + 1);
-        if (c == 0) { r.kv_off_cross[b] = b * S_max; r.q_off[b] = b * (k + 1); r.q_cnt[b] = k + 1; }
-        r.tok[i] = tok;
-        r.pos[i] = j + c;
-        r.seq[i] = b;
-        r.nk_self[i] = j + c + 1;     // causal: positions 0..j+c
-        r.nk_cross[i] = s.src_len[b];
+        if (i == 0) s.counters[CNT_VERIFY] = (compact ? s_live : B) * (k + 1);
+        if (b >= 0) {
+            if (c == 0) { r.kv_off_cross[b] = b * S_max; r.q_off[b] = slot * (k + 1); r.q_cnt[b] = k + 1; r.slot_seq[slot] = b; }
+            r.tok[i] = tok;
+            r.pos[i] = j + c;
+            r.seq[i] = b;
+            r.nk_self[i] = j + c + 1;     // causal: positions 0..j+c
+            r.nk_cross[i] = s.src_len[b];
+        } else if (c == 0) {
+            r.slot_seq[slot] = -1;
+        }
         __threadfence();
     }
     __syncthreads();
     pdl_launch_dependents();
+    if (b < 0) return;
     const int t = min(max(tok, 0), vocab - 1), p = min(max(j + c, 0), max_pos - 1);
     for (int e = threadIdx.x; e < d; e += blockDim.x)
         x[(size_t)i * d + e] = scale * to_f(E[(size_t)t * d + e]) + P[(size_t)p * d + e];
@@ -332,7 +346,7 @@ __global__ void k_embed(const int* __restrict__ tok, const int* __restrict__ pos
         x[(size_t)row * d + e] = scale * to_f(E[(size_t)t * d + e]) + P[(size_t)p * d + e];
 }
 
-__global__ void k_gather_rows(const float* __restrict__ x, const int* __restrict__ src_row,
+static __global__ void k_gather_rows(const float* __restrict__ x, const int* __restrict__ src_row,
                               const int* __restrict__ n_rows, float* __restrict__ out, int d) {
     int row = blockIdx.x;
     pdl_launch_dependents();
@@ -422,7 +436,8 @@ __global__ void k_layernorm(const float* __restrict__ x, const float* __restrict
 template <typename T, int NC>
 __global__ void k_layernorm_ld(const float* __restrict__ x, const float* __restrict__ g, const float* __restrict__ b,
                                T* __restrict__ y, int d, float eps, const T* __restrict__ E, const int* __restrict__ draft,
-                               int B, int k, int vocab, float* __restrict__ ld, int* __restrict__ ld_id) {
+                               const int* __restrict__ slot_seq, const int* __restrict__ n_rows, int k, int vocab,
+                               float* __restrict__ ld, int* __restrict__ ld_id) {
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     float4 gm[NC], bt[NC];
 #pragma unroll
@@ -431,9 +446,9 @@ __global__ void k_layernorm_ld(const float* __restrict__ x, const float* __restr
         gm[c] = __ldg(reinterpret_cast<const float4*>(g + e));
         bt[c] = __ldg(reinterpret_cast<const float4*>(b + e));
     }
-    const bool in_range = row < B * (k + 1);
-    const int bs = in_range ? row / (k + 1) : 0, c0 = in_range ? row % (k + 1) : k;
-    const int tok = (in_range && c0 < k) ? draft[bs * k + c0] : -1;       // drafts predate the step's kernel chain
+    const bool in_range = row < *n_rows;             // (row metadata and drafts predate the step's kernel chain)
+    const int c0 = in_range ? row % (k + 1) : k;
+    const int tok = c0 < k ? draft[slot_seq[row / (k + 1)] * k + c0] : -1;
     const bool ok = tok >= 0 && tok < vocab;
     pdl_launch_dependents();
     pdl_wait();
@@ -580,7 +595,6 @@ struct GemmArgs {
     int N, K;
     const int* n_rows;          // device row count
     int rows_static;            // >= 0: the row count is known on the host (saves a dependent load); else read n_rows
-    int one_m_tile;             // tensor-core path: the rows fit one 128-row tile whatever n_rows says
     T* out; int ldo;            // EPI_STORE / EPI_RELU
     int act;                    // EPI_RELU: 0 ReLU, 1 exact GELU
     // EPI_RESID on the tensor-core path, optional: also write LayerNorm(new residual rows) as bf16 [rows, N]
@@ -702,15 +716,16 @@ __global__ void __launch_bounds__(256) k_gemm_simt(GemmArgs<T> g) {
 // normalised hidden state with the draft's embedding row.  Row k (bonus) has no draft.
 template <typename T>
 __global__ void k_draft_logit(const T* __restrict__ y, const T* __restrict__ E, const int* __restrict__ draft,
-                              int B, int k, int d, int vocab, float* __restrict__ ld, int* __restrict__ ld_id) {
+                              const int* __restrict__ slot_seq, const int* __restrict__ n_rows, int k, int d, int vocab,
+                              float* __restrict__ ld, int* __restrict__ ld_id) {
     int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     int lane = threadIdx.x & 31;
     // The draft ids were written before this step's kernel chain began and the embedding table is a weight: with bf16
     // rows of at most 512 columns a lane fetches its 16 columns of the draft's embedding row before the dependency wait.
     const bool vec = std::is_same<T, bf16>::value && d % 16 == 0 && d <= 512;
-    const bool in_range = row < B * (k + 1);
-    const int b = in_range ? row / (k + 1) : 0, c = in_range ? row % (k + 1) : k;
-    const int tok = (in_range && c < k) ? draft[b * k + c] : -1;
+    const bool in_range = row < *n_rows;             // (row metadata and drafts predate the step's kernel chain)
+    const int c = in_range ? row % (k + 1) : k;
+    const int tok = c < k ? draft[slot_seq[row / (k + 1)] * k + c] : -1;
     const bool ok = tok >= 0 && tok < vocab;
     uint4 ev[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
     if (vec && ok && lane * 16 < d) {
@@ -761,22 +776,25 @@ __device__ __forceinline__ void commit_sequence(const Session& s, int b, const i
     }
     if (j >= mt) fin = true;
     s.len[b] = j;
+    atomicMax(&s.counters[CNT_MAXLEN], j);
     atomicAdd(&s.stats[0], 1ull);
     atomicAdd(&s.stats[1], (unsigned long long)k);
     atomicAdd(&s.stats[2], (unsigned long long)a);
     atomicAdd(&s.stats[3], (unsigned long long)(j - n0));
     if (fin) { s.finished[b] = 1; atomicSub(&s.counters[CNT_ACTIVE], 1); }
 }
-// The last block of the grid to get here posts (commits of this handle so far) << 32 | (sequences still decoding) to the
-// host-mapped word the generation loop polls: no copy, no event between the iterations.  Call after __syncthreads().
+// The last block of the grid to get here posts (commits of this handle so far) << 32 | (sequences still decoding) << 16 |
+// (longest committed length), the latter two saturated at 65535, to the host-mapped word the generation loop polls: no copy,
+// no event between the iterations.  Call after __syncthreads().
 __device__ __forceinline__ void commit_post(const Session& s, unsigned long long* post) {
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(&s.counters[CNT_TICKET], 1) == (int)gridDim.x - 1) {
             s.counters[CNT_TICKET] = 0;
             const int seq = ++s.counters[CNT_SEQ];
-            const int active = atomicAdd(&s.counters[CNT_ACTIVE], 0);
-            *reinterpret_cast<volatile unsigned long long*>(post) = ((unsigned long long)(unsigned)seq << 32) | (unsigned)active;
+            const int active = atomicAdd(&s.counters[CNT_ACTIVE], 0), longest = atomicAdd(&s.counters[CNT_MAXLEN], 0);
+            *reinterpret_cast<volatile unsigned long long*>(post) =
+                ((unsigned long long)(unsigned)seq << 32) | (unsigned)(min(active, 65535) << 16) | (unsigned)min(longest, 65535);
             __threadfence_system();
         }
     }
@@ -785,17 +803,19 @@ __device__ __forceinline__ void commit_post(const Session& s, unsigned long long
 struct FusedCommit { Session s; const int* draft; int eos; unsigned long long* post; int on; };
 
 // ------------------------------------------------------------------ acceptance scan (Eq. 7-9)
-// One block per sequence: warps merge the per-tile statistics of the k+1 rows, thread 0
+// One block per slot (verify block): warps merge the per-tile statistics of the k+1 rows, thread 0
 // finds the first rejected draft.  row_stats (optional) receives 6 floats per row.
-__global__ void k_accept(const RowPart* __restrict__ part, int n_tiles, const float* __restrict__ ld,
+static __global__ void k_accept(const RowPart* __restrict__ part, int n_tiles, const float* __restrict__ ld,
                          const int* __restrict__ ld_id, int k, int beta, float tau, int* __restrict__ accepted,
-                         int* __restrict__ bif, float* __restrict__ row_stats, int want_sum, FusedCommit fc) {
+                         int* __restrict__ bif, float* __restrict__ row_stats, int want_sum, const int* __restrict__ slot_seq, FusedCommit fc) {
     extern __shared__ unsigned char sm_acc[];
     RowPart* rs = reinterpret_cast<RowPart*>(sm_acc);       // [k+1]
     __shared__ unsigned char ok_s[256];                     // row c passes both tests (k <= 255 rows take this path)
     const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int sq = slot_seq[b];                             // the slot's sequence (metadata of the step: readable ahead of the wait); -1: none
     pdl_launch_dependents();
     pdl_wait();
+    if (sq >= 0) {
     for (int c = warp; c <= k; c += nw) {
         const RowPart* p = part + ((size_t)b * (k + 1) + c) * n_tiles;
         // the draft's logit of this row is requested with the first partials, not by the serial scan afterwards
@@ -842,9 +862,9 @@ __global__ void k_accept(const RowPart* __restrict__ part, int n_tiles, const fl
             if (!ok) break;
             ++a;
         }
-        accepted[b] = a;
-        bif[b] = rs[a].arg;
-        if (fc.on) commit_sequence(fc.s, b, fc.draft, a, rs[a].arg, k, fc.eos);
+        accepted[sq] = a;
+        bif[sq] = rs[a].arg;
+        if (fc.on) commit_sequence(fc.s, sq, fc.draft, a, rs[a].arg, k, fc.eos);
     }
     if (row_stats)
         for (int c = threadIdx.x; c <= k; c += blockDim.x) {
@@ -852,13 +872,14 @@ __global__ void k_accept(const RowPart* __restrict__ part, int n_tiles, const fl
             o[0] = rs[c].mx; o[1] = (float)rs[c].arg; o[2] = want_sum ? rs[c].mx + logf(rs[c].sum) : 0.f;
             o[3] = (float)rs[c].cnt; o[4] = ld[b * (k + 1) + c]; o[5] = (float)ld_id[b * (k + 1) + c];
         }
+    }
     if (fc.on) { __syncthreads(); commit_post(fc.s, fc.post); }
 }
 
 // ------------------------------------------------------------------ drafter argmax
 // script (optional; benchmark / test hook): draft i of a sequence with j committed tokens is replaced by
 // script[b * stride + j + i] wherever that entry is >= 0 (len = the committed lengths, k = drafts per sequence).
-__global__ void k_draft_argmax(const RowPart* __restrict__ part, int n_tiles, const int* __restrict__ n_rows,
+static __global__ void k_draft_argmax(const RowPart* __restrict__ part, int n_tiles, const int* __restrict__ n_rows,
                                const int* __restrict__ slot, int* __restrict__ draft, const int* __restrict__ script,
                                int stride, const int* __restrict__ len, int k) {
     int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -897,21 +918,8 @@ __global__ void k_draft_argmax(const RowPart* __restrict__ part, int n_tiles, co
     }
 }
 
-// Scripted drafts (benchmark / test hook): draft i of a sequence with j committed tokens is
-// replaced by script[b, j + i] where that entry is >= 0.  The drafter pass has already run.
-__global__ void k_apply_script(Session s, const int* __restrict__ script, int stride, int B, int k,
-                               int* __restrict__ draft) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    pdl_wait();
-    if (i >= B * k) return;
-    int b = i / k, c = i % k;
-    if (s.finished[b]) return;
-    int p = s.len[b] + c;
-    if (p < stride) { int t = script[(size_t)b * stride + p]; if (t >= 0) draft[i] = t; }
-}
-
 // Commit as a kernel of its own (specdec_commit; explicit keep / next).
-__global__ void k_commit(Session s, const int* __restrict__ draft, const int* __restrict__ keep,
+static __global__ void k_commit(Session s, const int* __restrict__ draft, const int* __restrict__ keep,
                          const int* __restrict__ next, int B, int k, int eos, unsigned long long* post) {
     int b = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();                                    // no early trigger: the lengths written here are read by later kernels BEFORE their waits
@@ -920,7 +928,7 @@ __global__ void k_commit(Session s, const int* __restrict__ draft, const int* __
     commit_post(s, post);
 }
 
-__global__ void k_session_init(Session s, const int* __restrict__ src_len, const int* __restrict__ max_tgt, int B,
+static __global__ void k_session_init(Session s, const int* __restrict__ src_len, const int* __restrict__ max_tgt, int B,
                                int max_tgt_cap, int S_max) {
     int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b == 0) {
@@ -936,7 +944,7 @@ __global__ void k_session_init(Session s, const int* __restrict__ src_len, const
     s.src_len[b] = min(max(src_len[b], 1), S_max);
 }
 
-__global__ void k_count_active(Session s, int B) {      // one warp
+static __global__ void k_count_active(Session s, int B) {      // one warp
     int n = 0;
     for (int b = threadIdx.x; b < B; b += 32) n += s.finished[b] ? 0 : 1;
 #pragma unroll
@@ -944,10 +952,11 @@ __global__ void k_count_active(Session s, int B) {      // one warp
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         s.counters[CNT_ACTIVE] = n;
         s.counters[CNT_TICKET] = 0;
+        s.counters[CNT_MAXLEN] = 0;
     }
 }
 
-__global__ void k_copy_out(Session s, int B, int* __restrict__ out, int out_stride, int* __restrict__ out_len,
+static __global__ void k_copy_out(Session s, int B, int* __restrict__ out, int out_stride, int* __restrict__ out_len,
                            int* __restrict__ fin) {
     int b = blockIdx.x;
     if (b >= B) return;
@@ -961,11 +970,11 @@ __global__ void k_copy_out(Session s, int B, int* __restrict__ out, int out_stri
 // Every arena allocation is followed by a 256-byte red zone holding a fixed pattern; a kernel that writes past the end
 // of its buffer damages one.  One warp per zone: report[0] += damaged zones, report[1] = lowest damaged zone index.
 constexpr unsigned long long RED_PATTERN = 0xC5A5C5A5C5A5C5A5ull;
-__global__ void k_red_fill(unsigned char* base, const unsigned long long* __restrict__ zone_off, int n_zones) {
+static __global__ void k_red_fill(unsigned char* base, const unsigned long long* __restrict__ zone_off, int n_zones) {
     const int z = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (z < n_zones) reinterpret_cast<unsigned long long*>(base + zone_off[z])[lane] = RED_PATTERN;
 }
-__global__ void k_red_check(const unsigned char* base, const unsigned long long* __restrict__ zone_off, int n_zones,
+static __global__ void k_red_check(const unsigned char* base, const unsigned long long* __restrict__ zone_off, int n_zones,
                             unsigned long long* report) {
     const int z = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (z >= n_zones) return;
@@ -978,7 +987,7 @@ __global__ void k_red_check(const unsigned char* base, const unsigned long long*
 // Non-finite values (NaN, +-Inf) in activation buffers and caches: blockIdx.y = buffer, blockIdx.x strides over its
 // 16-byte pieces.  report[2] += count, report[3] = lowest buffer index holding one.
 struct ScanBuf { const void* p; unsigned long long n16; int f32; int pad; };   // n16 = whole 16-byte pieces
-__global__ void k_nonfinite_scan(const ScanBuf* __restrict__ bufs, unsigned long long* report) {
+static __global__ void k_nonfinite_scan(const ScanBuf* __restrict__ bufs, unsigned long long* report) {
     const ScanBuf b = bufs[blockIdx.y];
     const uint4* p = reinterpret_cast<const uint4*>(b.p);
     int cnt = 0;

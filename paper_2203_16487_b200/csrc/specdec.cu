@@ -26,7 +26,7 @@
 #include "gemm_tc_splitk.cuh"
 #include "kernels.cuh"
 #include "mma_rate.cuh"
-#include "skinny_gemm.cuh"
+#include "rows_gemm.cuh"
 
 using namespace sd;
 
@@ -89,8 +89,9 @@ struct specdec_handle {
     std::vector<void*> dkc, dvc;
     int drafter_pc = 0;             // option "drafter_prefix_causal", as set
     int drafter_pc_session = 0;     // ... as in force for the running session (latched by specdec_encode)
+    int act_ub = 0;                 // upper bound on the unfinished sequences of the passes being issued
     bool fuse_commit = false;       // the generation loop: the acceptance scan commits its own decision (no commit kernel)
-    bool commit_done = false;       // ... and did so in the verify pass just issued
+    bool commit_done = false;       // ... and did so in the verify pass just issued (with it, verify blocks are packed: unfinished sequences only)
     int dnew_ub = 1;                // upper bound on the prefix positions the next draft pass has to add to that cache
     int* page_table;
     // rows
@@ -110,7 +111,6 @@ struct specdec_handle {
     int use_tc = 1, use_graphs = 1, use_tc_attn = 1, want_lse = 0, use_skinny = 1, use_pdl = 1;
     long long* trace_buf = nullptr; // device [256] in-kernel time stamps (option "trace")
     int want_trace = 0;
-    size_t skinny_smem_cap = 0;
     int poll_lag = -1;              // -1: chosen by batch size
     int stats_timing = 0;           // 1: specdec_generate records an event after every phase (option "stats_timing")
     int use_gate = 1;               // whole iterations as one graph behind a device-side IF node (option "gate")
@@ -125,10 +125,9 @@ struct specdec_handle {
     int zone_cap = 0, n_zones = 0, n_scan = 0;
     std::vector<std::string> scan_names;
     int debug_checks = 0;
-    int enc_skinny = 1;             // option "enc_skinny": 1 = the drafter's encoder (the longer of the two side-by-side chains) uses the weight-streaming GEMM for sources of at most 32 positions (default: 360 -> 340 us for a 29-token source), 2 = both encoders (no better: they get in each other's way), 0 = neither
-    bool enc_skinny_now = false;
+    int enc_skinny = 1;             // option "enc_skinny": the encoders use the few-rows GEMM too
     int use_ln_fuse = 0;            // option "ln_fuse": measured slower than the separate LayerNorm launch, kept for comparison
-    int use_sk_cluster = 1;         // option "sk_cluster": 1 = LayerNorm-fused weight-streaming GEMMs share the normalised rows in clusters of 8; 2 = the plain ones too (measured slower)
+    int use_sk_cluster = 1;         // option "sk_cluster": the few-rows GEMM splits long reductions across a cluster
     bool splitk_ready = false;
     int diag_repeat = 0;            // diagnostics: launch every attention (1) / LayerNorm (2) / non-residual GEMM (4) / vocabulary (8) kernel twice (same result) to
                                     // read its cost inside the pipeline off the step time (option "diag_repeat")
@@ -139,7 +138,6 @@ struct specdec_handle {
     int attn_stream = 1;            // streaming tile attention: 0 never, 1 by rule, 2 always, 3 always with the 2-stage ring (option "attn_stream")
     int attn_stream_keys = 320;     // option "attn_stream_keys"
     int attn_warps = 0;             // 0 = choose per launch, else 4 or 8 warps per tile-attention CTA (option "attn_warps")
-    int skinny_groups = 1;          // 8-row weight groups per CTA of the weight-streaming GEMM (1, 2 or 4)
     // CUDA graphs of whole draft / verify(+commit) steps, keyed by everything their launches depend on
     struct GraphEntry { cudaGraphExec_t exec; long long kernels; };
     std::map<std::vector<long long>, GraphEntry> graphs;
@@ -147,7 +145,7 @@ struct specdec_handle {
     long long launches = 0;
     // polling
     int* h_poll = nullptr;          // pinned
-    unsigned long long* h_post = nullptr;   // pinned, written by k_commit: (commits of this handle so far) << 32 | unfinished sequences
+    unsigned long long* h_post = nullptr;   // pinned, written by k_commit / k_accept (see commit_post)
     unsigned commits_issued = 0;    // commit kernels launched so far: what the posted count reaches once the stream drains
     int poll_flag = 1;              // the generation loop polls h_post instead of copying the counter back (option "poll_flag")
     unsigned long long* h_stats = nullptr;  // pinned [4]
@@ -266,7 +264,7 @@ void layout_rows(Arena& A, Rows& r, int n, int B) {
     auto iv = [&](size_t c) { return (int*)A.take(c * 4); };
     r.tok = iv(n); r.pos = iv(n); r.seq = iv(n); r.nk_self = iv(n); r.nk_cross = iv(n);
     r.src_row = iv(n); r.slot = iv(n);
-    r.kv_off = iv(B); r.kv_off_cross = iv(B); r.q_off = iv(B); r.q_cnt = iv(B);
+    r.kv_off = iv(B); r.kv_off_cross = iv(B); r.q_off = iv(B); r.q_cnt = iv(B); r.slot_seq = iv(B);
 }
 
 void layout_all(specdec_handle* h) {
@@ -327,7 +325,7 @@ void layout_all(specdec_handle* h) {
     s.out = (int*)A.take((size_t)h->B_cap * s.out_stride * 4);
     s.dlen = (int*)A.take((size_t)h->B_cap * 4);
     s.dticket = (int*)A.take(4);
-    s.counters = (int*)A.take(8 * 4);
+    s.counters = (int*)A.take(16 * 4);
     s.stats = (unsigned long long*)A.take(4 * 8);
     // integrity checks: report words, the table of scanned buffers, the table of red-zone offsets (sized by the dry run)
     h->integ_report = (unsigned long long*)A.take(4 * 8);
@@ -413,14 +411,18 @@ cudaError_t launch_pdl(specdec_handle* h, void (*kernel)(KArgs...), dim3 grid, d
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Row count of a pass where the host knows it, else -1 (the kernels read it from the device).
+inline int static_rows(const specdec_handle* h, int cnt, int rows_ub) {
+    return (cnt == CNT_ENC || (cnt == CNT_VERIFY && !(h->fuse_commit && h->B > 1))) ? rows_ub : -1;
+}
+
 template <typename T>
 int ln(specdec_handle* h, const float* x, const float* g, const float* b, int cnt, int rows_ub, void* y, int d,
        cudaStream_t st) {
     if (rows_ub <= 0) return 0;
     {
         cudaError_t e = launch_pdl(h, k_layernorm<T>, dim3(cdiv(rows_ub, 8)), dim3(256), 0, st, x, g, b,
-                                   (const int*)(h->ses.counters + cnt), (T*)y, d, 1e-5f,
-                                   (cnt == CNT_VERIFY || cnt == CNT_ENC) ? rows_ub : -1);
+                                   (const int*)(h->ses.counters + cnt), (T*)y, d, 1e-5f, static_rows(h, cnt, rows_ub));
         if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("layer norm launch: ") + cudaGetErrorString(e));
     }
     KCHECK(h);
@@ -446,73 +448,6 @@ template <typename T> bool tc_usable(const specdec_handle* h, int N, int K) {
 
 // LayerNorm fused in front of a GEMM: x fp32 rows, gain, bias.
 struct LnSpec { const float* x; const float* g; const float* b; };
-
-// The weight-streaming kernel serves bf16 GEMMs over at most 32 rows (see skinny_gemm.cuh; 64-row variants of its
-// row-sharing LayerNorm kernels were tried too: 422 vs 356 us per 2-sequence verify step, and 360 vs 315 us after the
-// kernel's bank conflicts were gone): measured on a
-// verify step, 26 rows take 362 us with it against 391 us with 64-wide tensor-core tiles, but 52 rows take
-// 500 us against 391 us, so anything beyond two 16-row tiles goes to the tile GEMM.
-constexpr int SK_ROWS_MAX = 32;
-template <typename T>
-bool skinny_ok(const specdec_handle* h, int epi, int rows_ub, int N, int K, bool with_ln) {
-    if (!std::is_same<T, bf16>::value || !h->use_skinny || rows_ub > SK_ROWS_MAX) return false;
-    if (epi != EPI_STORE && epi != EPI_RELU && epi != EPI_GELU && epi != EPI_RESID && epi != EPI_QKV) return false;
-    if (K % 32 || (with_ln && (K % 128 || K > 512))) return false;
-    return skinny_smem(2, K) <= h->skinny_smem_cap;
-}
-
-template <int EPI, int MT, int G>
-int skinny_launch_g(specdec_handle* h, SkinnyArgs& a, cudaStream_t st) {
-    const int grid = cdiv(a.g.N, SK_NB * G);
-    const size_t smem = skinny_smem(MT, a.g.K);
-    cudaError_t e;
-    if (G == 1 && h->use_sk_cluster && grid % 8 == 0 && (a.ln_x ? a.g.K % 128 == 0 : (a.g.K % 8 == 0 && a.g.lda % 8 == 0 && (h->use_sk_cluster >= 3 || (h->use_sk_cluster == 2 && a.g.K <= 512))))) {
-        // clusters of 8 CTAs share the (normalised) input rows (see skinny_gemm.cuh)
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(grid); cfg.blockDim = dim3(SK_WARPS * 32); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-        cudaLaunchAttribute attr[2];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 8; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr; cfg.numAttrs = h->use_pdl ? 2 : 1;
-        e = a.ln_x ? cudaLaunchKernelEx(&cfg, k_skinny<EPI, MT, true, 1, true>, a)
-                   : cudaLaunchKernelEx(&cfg, k_skinny<EPI, MT, false, 1, true>, a);
-    } else {
-        e = a.ln_x ? launch_pdl(h, k_skinny<EPI, MT, true, G>, dim3(grid), dim3(SK_WARPS * 32), smem, st, a)
-                   : launch_pdl(h, k_skinny<EPI, MT, false, G>, dim3(grid), dim3(SK_WARPS * 32), smem, st, a);
-    }
-    if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("skinny GEMM launch: ") + cudaGetErrorString(e));
-    KCHECK(h);
-    return 0;
-}
-template <int EPI, int MT>
-int skinny_launch_ln(specdec_handle* h, SkinnyArgs& a, cudaStream_t st) {
-    return skinny_launch_g<EPI, MT, 1>(h, a, st);
-}
-template <int EPI>
-int skinny_launch_mt(specdec_handle* h, SkinnyArgs& a, int rows_ub, cudaStream_t st) {
-    (void)rows_ub;
-    return skinny_launch_ln<EPI, 2>(h, a, st);
-}
-int skinny_launch(specdec_handle* h, int epi, SkinnyArgs& a, int rows_ub, cudaStream_t st) {
-    switch (epi) {
-        case EPI_STORE: return skinny_launch_mt<EPI_STORE>(h, a, rows_ub, st);
-        case EPI_RELU: return skinny_launch_mt<EPI_RELU>(h, a, rows_ub, st);
-        case EPI_GELU: return skinny_launch_mt<EPI_GELU>(h, a, rows_ub, st);
-        case EPI_RESID: return skinny_launch_mt<EPI_RESID>(h, a, rows_ub, st);
-        default: return skinny_launch_mt<EPI_QKV>(h, a, rows_ub, st);
-    }
-}
-template <int EPI, int MT>
-cudaError_t skinny_attr(int bytes) {
-    cudaError_t e = cudaSuccess;
-    auto set = [&](auto* f) { if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
-    set(k_skinny<EPI, MT, true, 1>); set(k_skinny<EPI, MT, false, 1>); set(k_skinny<EPI, MT, true, 1, true>); set(k_skinny<EPI, MT, false, 1, true>);
-    return e;
-}
-template <int EPI>
-cudaError_t skinny_attr_mt(int bytes) { return skinny_attr<EPI, 2>(bytes); }
 
 // out = A W^T (+bias) with one of the epilogues; rows_ub bounds the grid, the live count is on the device.
 template <typename T>
@@ -541,8 +476,11 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
     if (rows_ub <= 0) return 0;
     // (not in the encoders: the two encoders run side by side on two streams, and the weight-streaming kernels' 64-256
     // CTAs per launch get in each other's way there -- 440 us against 386 us with 8-32-CTA tile GEMMs for a 32-token source)
-    const bool skinny = (cnt != CNT_ENC || h->enc_skinny_now) && skinny_ok<T>(h, epi, rows_ub, N, K, lnp != nullptr);
-    if (lnp && !skinny) {           // separate normalisation launch, then a plain GEMM on its output
+    // few rows: the weight-streaming kernel, with the LayerNorm inside where it has one
+    const bool few = std::is_same<T, bf16>::value && h->use_skinny && h->use_tc && rows_ub <= (cnt == CNT_ENC ? (h->enc_skinny ? RG_MAX_ROWS_ENC : 0) : RG_MAX_ROWS) &&
+                     !(epi == EPI_RESID && h->use_ln_fuse) && rg_supported(epi, N, K, lnp ? K : lda, rows_ub, h->use_sk_cluster != 0);
+    const bool ln_inside = few && lnp && rows_ub <= RG_LN_ROWS && rg_ln_width(K);
+    if (lnp && !ln_inside) {           // separate normalisation launch, then a plain GEMM on its output
         TRY(ln_or_fused<T>(h, lnp->x, lnp->g, lnp->b, cnt, rows_ub, h->y, K, st));
         A = h->y; lda = K;
     }
@@ -550,8 +488,8 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
     if (epi == EPI_RESID) { h->fused_x = nullptr; h->next_ln = {nullptr, nullptr, nullptr}; }   // the residual rows change
     GemmArgs<T> g;
     g.A = (const T*)A; g.lda = lda; g.W = (const T*)W; g.bias = bias; g.N = N; g.K = K;
-    g.n_rows = h->ses.counters + cnt; g.rows_static = (cnt == CNT_VERIFY || cnt == CNT_ENC) ? rows_ub : -1; g.out = (T*)out; g.ldo = ldo; g.resid = resid;
-    g.one_m_tile = 0; g.act = h->cfg.ffn_activation;
+    g.n_rows = h->ses.counters + cnt; g.rows_static = static_rows(h, cnt, rows_ub); g.out = (T*)out; g.ldo = ldo; g.resid = resid;
+    g.act = h->cfg.ffn_activation;
     g.ln_g = nullptr; g.ln_b = nullptr; g.ln_eps = 1e-5f; g.ln_out = nullptr;
     g.part = h->part; g.ld = ldv; g.ld_id = ld_id; g.n_tiles = cdiv(N, 64); g.want_sum = h->want_lse;
     g.seq = nullptr; g.pos = nullptr; g.kc = nullptr; g.vc = nullptr; g.kv_d = 0;
@@ -559,12 +497,15 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
     g.trace = (h->want_trace && epi == (h->want_trace >= 10 ? h->want_trace - 10 : EPI_STATS)) ? h->trace_buf + 200 : nullptr;
     if (kv) { g.seq = kv->seq; g.pos = kv->pos; g.kc = (T*)kv->kc; g.vc = (T*)kv->vc; g.kv_d = kv->d; }
     if constexpr (std::is_same<T, bf16>::value) {
-        if (skinny) {
-            SkinnyArgs sa; sa.g = g;
-            sa.ln_x = lnp ? lnp->x : nullptr; sa.ln_g = lnp ? lnp->g : nullptr; sa.ln_b = lnp ? lnp->b : nullptr;
-            sa.ln_eps = 1e-5f; sa.ln_out = nullptr; sa.err_word = h->ses.counters + 7;
-            sa.trace = h->want_trace ? h->trace_buf + 216 + 6 * ((epi == EPI_RELU || epi == EPI_GELU) ? 0 : epi == EPI_RESID ? 1 : epi == EPI_QKV ? 2 : 3) : nullptr;
-            TRY(skinny_launch(h, epi, sa, rows_ub, st));
+        if (few) {
+            RowsArgs ra{};
+            ra.g = g;
+            if (ln_inside) { ra.ln_x = lnp->x; ra.ln_g = lnp->g; ra.ln_b = lnp->b; ra.ln_eps = 1e-5f; }
+            ra.err_word = h->ses.counters + 7;
+            ra.trace = h->want_trace ? h->trace_buf + 216 + 6 * ((epi == EPI_RELU || epi == EPI_GELU) ? 0 : epi == EPI_RESID ? 1 : epi == EPI_QKV ? 2 : 3) : nullptr;
+            const cudaError_t e = rg_launch(epi, ra, rows_ub, h->use_sk_cluster != 0, h->use_pdl, st);
+            if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("row GEMM launch: ") + cudaGetErrorString(e));
+            KCHECK(h);
             return 0;
         }
     }
@@ -619,7 +560,8 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
         // the streaming kernel where the one-shot kernel cannot hold the keys, and where the SMs are full of CTAs
         // and the keys are many (its small footprint keeps the occupancy up; with few CTAs its block-by-block walk
         // is slower than one big request)
-        const long long attn_ctas = (long long)cdiv(q_ub, ATT_Q) * n_heads * h->B;
+        const int n_seq = cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub);
+        const long long attn_ctas = (long long)cdiv(q_ub, ATT_Q) * n_heads * n_seq;
         const bool stream = h->use_tc_attn && d_head == 64 &&
                             (h->attn_stream >= 2 ||
                              (h->attn_stream == 1 && (smem > h->attn_tc_smem_cap ||
@@ -634,7 +576,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             a.scale = 1.0f / sqrtf((float)d_head);
             dim3 grid(cdiv(q_ub, ATT_Q), n_heads, h->B);
             if (stream) {          // key blocks through a ring of stages: shared memory independent of the key count
-                const bool deep = h->attn_stream != 3 && (long long)grid.x * grid.y * grid.z < 4LL * h->tma.n_sm;    // few CTAs: more bytes in flight per CTA
+                const bool deep = h->attn_stream != 3 && attn_ctas < 4LL * h->tma.n_sm;    // few CTAs: more bytes in flight per CTA
                 cudaError_t e = deep ? (paged ? launch_pdl(h, k_attn_stream<true, 4>, grid, dim3(128), (size_t)ats_smem(4), st, a)
                                               : launch_pdl(h, k_attn_stream<false, 4>, grid, dim3(128), (size_t)ats_smem(4), st, a))
                                      : (paged ? launch_pdl(h, k_attn_stream<true, 2>, grid, dim3(128), (size_t)ats_smem(2), st, a)
@@ -645,7 +587,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             }
             // 4 warps when the SMs are saturated with CTAs anyway, 8 when a CTA's own latency chain is what counts;
             // scores stay in registers (smaller shared memory: more CTAs per SM) when the keys fit 6 tiles per warp
-            const long long ctas = (long long)grid.x * grid.y * grid.z;
+            const long long ctas = attn_ctas;
             const int nkp = (max_keys + 15) & ~15;
             auto per_sm_of = [](size_t sm) { return (long long)(227 * 1024) / (long long)(sm + 1024); };
             // (measured: the register variant is slower per CTA, 357 -> 387 us per batch-1 step, and pays off only where
@@ -809,8 +751,6 @@ void use_workset(specdec_handle* h, int i) {
 template <typename T>
 int encode_model(specdec_handle* h, ModelW& m, cudaStream_t st) {
     const int R = h->B * h->S_max, d = m.dm.d_model;
-    h->enc_skinny_now = h->enc_skinny == 2 || (h->enc_skinny == 1 && &m == &h->dra);
-    struct Off { specdec_handle* h; ~Off() { h->enc_skinny_now = false; } } off{h};
     TRY(embed<T>(h, m, h->rows, m.pos_enc, CNT_ENC, R, st));
     for (int l = 0; l < m.dm.enc_layers; ++l) {
         const bool last = l + 1 == m.dm.enc_layers;
@@ -828,7 +768,7 @@ int encode_model(specdec_handle* h, ModelW& m, cudaStream_t st) {
 template <typename T>
 int encode_impl(specdec_handle* h, const int* d_src, const int* d_src_len, const int* d_max_tgt, int B, int S_max,
                 cudaStream_t st) {
-    h->B = B; h->S_max = S_max; h->len_ub = 0;
+    h->B = B; h->S_max = S_max; h->len_ub = 0; h->act_ub = B;
     h->dnew_ub = 1; h->drafter_pc_session = h->drafter_pc;
     h->encoded = false; h->verified = false; h->drafted = false;
     k_session_init<<<cdiv(B, 128), 128, 0, st>>>(h->ses, d_src_len, d_max_tgt, B, h->T_cap, S_max);
@@ -873,7 +813,7 @@ int draft_impl(specdec_handle* h, int k, int* d_draft, cudaStream_t st) {
     // rows of the full pass per sequence: the whole [BOS, committed, MASK x k] input, or (prefix-causal reading) only the
     // prefix positions its K/V cache does not hold yet plus the k [MASK] rows
     const int per_seq = pc ? std::min(h->dnew_ub, len_ub + 1) + k : len_ub + 1 + k;
-    const int R1 = B * per_seq, R2 = B * k, max_keys = len_ub + 1 + k;
+    const int n_seq = std::min(B, h->act_ub), R1 = n_seq * per_seq, R2 = n_seq * k, max_keys = len_ub + 1 + k;
     // row metadata of the pass and the embedding of its rows in one kernel (one block per sequence)
     h->fused_x = nullptr;
     // blocks per sequence: enough to fill the machine at small batches, never fewer than two rows a block
@@ -938,14 +878,16 @@ template <typename T>
 int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float tau, int* d_accepted, int* d_bif,
                 cudaStream_t st) {
     ModelW& m = h->ver;
-    const int B = h->B, d = m.dm.d_model, L = m.dm.dec_layers, M = B * (k + 1);
+    // the generation loop verifies the unfinished sequences only: packed blocks, M an upper bound on their rows
+    const bool compact = h->fuse_commit && h->B > 1;
+    const int B = h->B, slots = compact ? std::min(B, h->act_ub) : B, d = m.dm.d_model, L = m.dm.dec_layers, M = slots * (k + 1);
     const int max_keys = std::min(h->len_ub, h->T_cap) + k + 1;
     if (d_draft != h->v_draft && k > 0)
         CUDA_TRY(h, cudaMemcpyAsync(h->v_draft, d_draft, (size_t)B * k * 4, cudaMemcpyDeviceToDevice, st));
     // row metadata and embedding of the block in one kernel
     h->fused_x = nullptr;
     CUDA_TRY(h, launch_pdl(h, k_verify_prep_embed<T>, dim3(M), dim3(128), 0, st, h->ses, (const int*)h->v_draft, B, k, h->S_max, h->cfg.bos_id,
-                           h->rows, (const T*)m.embed, (const float*)m.pos_dec, h->x, d, sqrtf((float)d), m.dm.vocab, m.dm.max_pos));
+                           h->rows, (const T*)m.embed, (const float*)m.pos_dec, h->x, d, sqrtf((float)d), m.dm.vocab, m.dm.max_pos, compact ? 1 : 0));
     KCHECK(h);
     for (int l = 0; l < L; ++l) {
         const bool last = l + 1 == L;
@@ -961,7 +903,7 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
         cudaError_t e = cudaSuccess;
         const dim3 grid(cdiv(M, 8)), block(256);
 #define LN_LD(NC) e = launch_pdl(h, k_layernorm_ld<T, NC>, grid, block, 0, st, (const float*)h->x, (const float*)m.dec_lnf_g, (const float*)m.dec_lnf_b, (T*)h->y, d, 1e-5f, \
-                                 (const T*)m.embed, (const int*)h->v_draft, B, k, m.dm.vocab, h->ld, h->ld_id)
+                                 (const T*)m.embed, (const int*)h->v_draft, (const int*)h->rows.slot_seq, (const int*)(h->ses.counters + CNT_VERIFY), k, m.dm.vocab, h->ld, h->ld_id)
         switch (d / 128) {
             case 1: LN_LD(1); break; case 2: LN_LD(2); break; case 3: LN_LD(3); break; case 4: LN_LD(4); break;
             case 5: LN_LD(5); break; case 6: LN_LD(6); break; case 7: LN_LD(7); break; default: LN_LD(8); break;
@@ -972,7 +914,7 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
     } else {
         TRY(ln_or_fused<T>(h, h->x, m.dec_lnf_g, m.dec_lnf_b, CNT_VERIFY, M, h->y, d, st));
         CUDA_TRY(h, launch_pdl(h, k_draft_logit<T>, dim3(cdiv(M, 4)), dim3(128), 0, st, (const T*)h->y, (const T*)m.embed,
-                               (const int*)h->v_draft, B, k, d, m.dm.vocab, h->ld, h->ld_id));
+                               (const int*)h->v_draft, (const int*)h->rows.slot_seq, (const int*)(h->ses.counters + CNT_VERIFY), k, d, m.dm.vocab, h->ld, h->ld_id));
         KCHECK(h);
     }
     int n_tiles = 0;
@@ -981,8 +923,8 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
                 h->ld_id, &n_tiles));
     prof_mark(h, st);
     FusedCommit fc{h->ses, h->v_draft, h->cfg.eos_id, h->h_post, h->fuse_commit ? 1 : 0};
-    CUDA_TRY(h, launch_pdl(h, k_accept, dim3(B), dim3(1024), (size_t)(k + 1) * sizeof(RowPart), st, (const RowPart*)h->part, n_tiles,
-                           (const float*)h->ld, (const int*)h->ld_id, k, beta, tau, h->accepted, h->bif, h->row_stats, h->want_lse, fc));
+    CUDA_TRY(h, launch_pdl(h, k_accept, dim3(slots), dim3(1024), (size_t)(k + 1) * sizeof(RowPart), st, (const RowPart*)h->part, n_tiles,
+                           (const float*)h->ld, (const int*)h->ld_id, k, beta, tau, h->accepted, h->bif, h->row_stats, h->want_lse, (const int*)h->rows.slot_seq, fc));
     KCHECK(h);
     h->commit_done = h->fuse_commit;
     if (d_accepted) CUDA_TRY(h, cudaMemcpyAsync(d_accepted, h->accepted, (size_t)B * 4, cudaMemcpyDeviceToDevice, st));
@@ -1036,8 +978,8 @@ inline void graph_key_tail(const specdec_handle* h, std::vector<long long>& key)
     for (long long v : {(long long)h->use_tc, (long long)h->use_tc_attn, (long long)h->want_lse, (long long)h->use_skinny,
                         (long long)h->use_pdl, (long long)h->use_ln_fuse, (long long)h->use_sk_cluster,
                         (long long)h->use_pair, (long long)h->diag_repeat, (long long)h->use_splitk, (long long)h->attn_stream, (long long)h->attn_stream_keys, (long long)h->attn_warps, (long long)h->attn_rs,
-                        (long long)h->skinny_groups, (long long)h->want_trace,
-                        (long long)(h->script_on ? 1 : 0), (long long)h->B, (long long)h->S_max, (long long)h->drafter_pc_session, (long long)(h->fuse_commit ? 1 : 0), (long long)h->enc_skinny})
+                        (long long)h->want_trace,
+                        (long long)(h->script_on ? 1 : 0), (long long)h->B, (long long)h->S_max, (long long)h->drafter_pc_session, (long long)(h->fuse_commit ? 1 : 0), (long long)h->enc_skinny, (long long)h->act_ub})
         key.push_back(v);
 }
 
@@ -1127,15 +1069,21 @@ int encode_staged(specdec_handle* h, const int* d_src, const int* d_src_len, con
     if (d_src != h->stage_src) CUDA_TRY(h, cudaMemcpyAsync(h->stage_src, d_src, (size_t)B * S_max * 4, cudaMemcpyDeviceToDevice, st));
     if (d_src_len != h->stage_len) CUDA_TRY(h, cudaMemcpyAsync(h->stage_len, d_src_len, (size_t)B * 4, cudaMemcpyDeviceToDevice, st));
     if (d_max_tgt && d_max_tgt != h->stage_mt) CUDA_TRY(h, cudaMemcpyAsync(h->stage_mt, d_max_tgt, (size_t)B * 4, cudaMemcpyDeviceToDevice, st));
-    h->B = B; h->S_max = S_max;
+    h->B = B; h->S_max = S_max; h->act_ub = B;
     h->drafter_pc_session = h->drafter_pc;
     TRY(graph_call(h, {5, d_max_tgt ? 1 : 0}, st, [&]() {
         return encode_impl<T>(h, h->stage_src, h->stage_len, d_max_tgt ? h->stage_mt : nullptr, B, S_max, st); }));
-    h->len_ub = 0; h->encoded = true; h->verified = false; h->drafted = false;
+    h->len_ub = 0; h->act_ub = B; h->encoded = true; h->verified = false; h->drafted = false;
     h->dnew_ub = 1;
     return 0;
 }
 
+// Smallest power of two that covers the unfinished sequences (at most the batch).
+inline int act_bucket(int B, int active) {
+    int n = 1;
+    while (n < active) n *= 2;
+    return std::min(B, n);
+}
 inline int len_bucket(const specdec_handle* h, int len_ub) { return std::min(h->T_cap, (len_ub + 31) / 32 * 32); }
 
 template <typename T>
@@ -1144,7 +1092,7 @@ int generate_loop(specdec_handle* h, const int* d_src, const int* d_src_len, con
                   cudaStream_t st) {
     const bool timed = hs != nullptr, phases = timed && h->stats_timing;
     // the acceptance scan commits its own decision (one kernel less per iteration) unless the phases are timed apart
-    struct FuseGuard { specdec_handle* h; ~FuseGuard() { h->fuse_commit = false; h->commit_done = false; } } fuse_guard{h};
+    struct FuseGuard { specdec_handle* h; ~FuseGuard() { h->fuse_commit = false; h->commit_done = false; h->act_ub = h->B; } } fuse_guard{h};
     h->fuse_commit = !phases;
     size_t ev = 0;
     auto mark_always = [&]() { if (timed && ev < h->time_ev.size()) cudaEventRecord(h->time_ev[ev++], st); };
@@ -1168,12 +1116,16 @@ int generate_loop(specdec_handle* h, const int* d_src, const int* d_src_len, con
     if (flag && cudaStreamQuery(st) == cudaSuccess) h->commits_issued = (unsigned)(*(volatile unsigned long long*)h->h_post >> 32);
     const unsigned commits_base = h->commits_issued;
     std::vector<long long> it_kernels;
+    int act_seen = B;
     int tau_bits; memcpy(&tau_bits, &tau, 4);
     // the drafter writes its block straight into the verifier's draft buffer: no copy between the two steps
     for (; it < max_iters; ++it) {
         if (graphs) {
             // the launches depend on the host-side length bound only through its 32-token bucket
+            // (what the last post showed bounds them: the longest length it saw plus what the iterations since can add,
+            // the sequences it saw unfinished, rounded up to a power of two so that few graphs exist)
             const int true_ub = h->len_ub, lb = len_bucket(h, true_ub);
+            h->act_ub = act_bucket(B, act_seen);
             // (prefix-causal drafter: the pass is also sized by how many prefix positions its cache still lacks)
             const int dn = h->dnew_ub, dkey = (h->drafter_pc_session && k > 0) ? dn : -1;
             bool done = false;
@@ -1228,7 +1180,12 @@ int generate_loop(specdec_handle* h, const int* d_src, const int* d_src_len, con
             it_kernels.push_back(0);
         }
         mark();
-        int active_seen = 1;
+        int active_seen = 1, longest_seen = 65535;
+        auto take_post = [&](unsigned long long v) {
+            active_seen = (int)((unsigned)v >> 16);
+            if (active_seen == 65535) active_seen = B;
+            longest_seen = (int)((unsigned)v & 0xffffu);
+        };
         if (flag) {
             // spin on the word k_commit posts; a look at the stream now and then surfaces a failed launch
             if (it >= lag) {
@@ -1236,13 +1193,13 @@ int generate_loop(specdec_handle* h, const int* d_src, const int* d_src_len, con
                 const auto t0 = std::chrono::steady_clock::now();
                 for (unsigned spins = 1;; ++spins) {
                     const unsigned long long v = *(volatile unsigned long long*)h->h_post;
-                    if ((int)((unsigned)(v >> 32) - want) >= 0) { active_seen = (int)(unsigned)v; break; }
+                    if ((int)((unsigned)(v >> 32) - want) >= 0) { take_post(v); break; }
                     if ((spins & 0xfffu) == 0) {
                         cudaError_t q = cudaStreamQuery(st);
                         if (q != cudaSuccess && q != cudaErrorNotReady) return fail(h, SPECDEC_ERR_CUDA, std::string("generate: ") + cudaGetErrorString(q));
                         if (q == cudaSuccess) {       // the stream drained: the word must be there now
                             const unsigned long long v2 = *(volatile unsigned long long*)h->h_post;
-                            if ((int)((unsigned)(v2 >> 32) - want) >= 0) { active_seen = (int)(unsigned)v2; break; }
+                            if ((int)((unsigned)(v2 >> 32) - want) >= 0) { take_post(v2); break; }
                             // behind a gate no commit kernel runs once nothing is left to decode (for instance when
                             // every budget was zero from the start): ask the device
                             int active_now = -1;
@@ -1265,6 +1222,9 @@ int generate_loop(specdec_handle* h, const int* d_src, const int* d_src_len, con
             }
         }
         if (it >= lag) {
+            act_seen = std::min(act_seen, active_seen);
+            if (longest_seen < 65535)                // after iteration it - lag; the lag iterations behind it add at most k + 1 each
+                h->len_ub = (int)std::min<long long>(h->len_ub, longest_seen + (long long)lag * (k + 1));
             if (active_seen == 0) {
                 // iterations it - lag + 1 .. it found nothing to do: behind a gate only the gate kernel ran
                 for (int j = it - lag + 1; j <= it; ++j)
@@ -1319,7 +1279,7 @@ int generate_impl(specdec_handle* h, const int* d_src, const int* d_src_len, con
         h->commits_issued = (unsigned)(*(volatile unsigned long long*)h->h_post >> 32);
         cudaMemsetAsync(h->ses.counters + 7, 0, 4, st);
         h->h_poll[ERRW_SLOT] = 0; h->errw_pending = false;
-        h->encoded = false; h->verified = false; h->drafted = false;
+        h->encoded = false; h->verified = false; h->drafted = false; h->act_ub = h->B;
         h->err = msg;
     }
     return rc;
@@ -1537,17 +1497,6 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
             cudaGetLastError();
             h->attn_tc_smem_cap = 48 * 1024;
         }
-        {
-            const int kmax = std::max(h->d_max, h->f_max);
-            size_t need = std::min<size_t>(skinny_smem(2, kmax), 227 * 1024);
-            cudaError_t e = skinny_attr_mt<EPI_STORE>((int)need);
-            if (e == cudaSuccess) e = skinny_attr_mt<EPI_GELU>((int)need);
-            if (e == cudaSuccess) e = skinny_attr_mt<EPI_RELU>((int)need);
-            if (e == cudaSuccess) e = skinny_attr_mt<EPI_RESID>((int)need);
-            if (e == cudaSuccess) e = skinny_attr_mt<EPI_QKV>((int)need);
-            if (e != cudaSuccess) { cudaGetLastError(); need = 48 * 1024; }
-            h->skinny_smem_cap = need;
-        }
         if (sd::tc_init(h->tma, h->ses.counters + 7) != 0) h->use_tc = 0;     // reported through specdec_last_error; SIMT GEMM still runs on the GPU
         h->splitk_ready = h->use_tc && sd::spk_init() == cudaSuccess;
         if (!h->splitk_ready) cudaGetLastError();
@@ -1606,7 +1555,7 @@ int specdec_set_option(specdec_handle* h, const char* name, int value) {
     if (!strcmp(name, "poll_flag")) { h->poll_flag = value ? 1 : 0; return SPECDEC_OK; }
     if (!strcmp(name, "gate")) { h->use_gate = value; return SPECDEC_OK; }
     if (!strcmp(name, "tc_bn")) { h->tma.force_bn = value; return SPECDEC_OK; }
-    if (!strcmp(name, "sk_cluster")) { h->use_sk_cluster = value < 0 ? 0 : value; return SPECDEC_OK; }   // 0 off, 1 LayerNorm-fused kernels, 2 + plain ones with K <= 512, 3 all
+    if (!strcmp(name, "sk_cluster")) { h->use_sk_cluster = value < 0 ? 0 : value; return SPECDEC_OK; }
     if (!strcmp(name, "ln_fuse")) { h->use_ln_fuse = value ? 1 : 0; return SPECDEC_OK; }
     if (!strcmp(name, "enc_skinny")) { h->enc_skinny = value < 0 ? 0 : (value > 2 ? 2 : value); return SPECDEC_OK; }
     if (!strcmp(name, "debug_checks")) { h->debug_checks = value ? 1 : 0; return SPECDEC_OK; }

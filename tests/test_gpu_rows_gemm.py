@@ -1,0 +1,42 @@
+"""The few-rows GEMM against the oracle, in lock step, at the row counts where its launch rule changes (16-row tiles, LayerNorm inside
+or in front, the hand-over to the 128-row tensor-core tiles) and at widths that are not whole MMA steps of its K slices,
+have no LayerNorm inside, or split long reductions across a cluster (K = 1024 and more)."""
+import numpy as np
+import pytest
+
+from oracle import specdec_oracle as O
+from paper_2203_16487_b200 import workloads as W
+from tests import lockstep
+
+pytestmark = pytest.mark.gpu
+
+
+# (d, heads, ffn, batch, k): batch * (k + 1) rows in a verify block
+@pytest.mark.parametrize("d,H,f,B,k", [
+    (256, 4, 1040, 1, 15),          # 16 rows; K = 1040: two slices that end inside an MMA step
+    (512, 8, 2048, 3, 10),          # 33 rows
+    (768, 12, 3072, 12, 11),        # 144 rows: the last with the LayerNorm inside
+    (256, 4, 1024, 29, 4),          # 145 rows: LayerNorm in front, four slices
+    (320, 5, 1312, 24, 15),         # 384 rows: the last of the few-rows kernel; no LayerNorm width
+    (128, 2, 192, 35, 10),          # 385 rows: tensor-core tiles
+])
+def test_rows_gemm_edges(d, H, f, B, k):
+    from paper_2203_16487_b200 import binding
+    V = 515
+    dims = W.ModelDims(d, H, f, V, 1, 1, 64)
+    wv, wd = W.make_weights(dims, 40 + d, True), W.make_weights(dims, 41 + d, True)
+    mv, md = O.model_from(dims, wv, mode="bf16"), O.model_from(dims, wd, mode="bf16")
+    rng = np.random.default_rng(B)
+    srcs = [W.zipf_ids(rng, int(n), V) for n in rng.integers(2, 13, size=B)]
+    sd = binding.SpecDec(dims, wv, dims, wd, k_max=k, max_batch=B, max_src=12, max_tgt=16, bf16=True)
+    sd.set_option("debug_checks", 1)
+    rep = lockstep.run(sd, mv, md, srcs, [10] * B, k, 3, 1.0, margin=1e-3, check_logits_every=1, max_iters=2)
+    assert rep.ok, rep.notes
+    assert rep.max_logit_err < 2e-2 and rep.max_stat_err < 2e-2
+    # packed blocks: budgets that end at different iterations
+    tgt = [1 + b % 9 for b in range(B)]
+    out, n, _ = sd.generate(*W.pad_batch(srcs), np.array(tgt, np.int32), k, 1, 0.0)
+    out, n = out.cpu().numpy(), n.cpu().numpy()
+    for b in range(0, B, 7):
+        assert out[b, :n[b]].tolist() == O.greedy_decode(mv, srcs[b], tgt[b], W.BOS_ID, W.EOS_ID), b
+    sd.close()
