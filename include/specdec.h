@@ -278,10 +278,10 @@ int specdec_profile_read(specdec_handle* h, double* h_ms, long long* h_launches)
  * "tc_bn"        0 choose (default), else the column width of the tensor-core tiles (64 / 128 / 256)
  * "pdl"          0/1 programmatic dependent launch between the kernels of a step (default 1)
  * "graphs"       0/1 replay steps from CUDA graphs (default 1)
- * "gate"         0 never / 1 above batch 4 (default) / 2 always: each iteration of specdec_generate is one graph
+ * "gate"         0 never (default) / 1 above batch 4 / 2 always: each iteration of specdec_generate is one graph
  *                behind a device-side IF node, so the host can queue iterations ahead of the counter it reads
  * "poll_flag"    0/1 specdec_generate learns of each commit from a word in pinned host memory (default 1)
- * "poll_lag"     n: specdec_generate reads the unfinished-sequences counter n iterations late (default: by batch)
+ * "poll_lag"     n: specdec_generate reads the unfinished-sequences counter n iterations late (default 0; 2 behind a gate)
  * "stats_timing" 0/1 fill ms_draft / ms_verify / ms_commit of specdec_stats (default 0; turns the gate off)
  * "profile"      0/1 see specdec_profile_read
  * "row_lse"      0/1 also accumulate the log-sum-exp of every verifier row (reported by specdec_debug_row_stats)

@@ -124,7 +124,7 @@ static __global__ void k_enc_prep(const int* __restrict__ src, const int* __rest
 template <typename T>
 __global__ void k_verify_prep_embed(Session s, const int* __restrict__ draft, int B, int k, int S_max, int bos, Rows r,
                                     const T* __restrict__ E, const float* __restrict__ P, float* __restrict__ x, int d,
-                                    float scale, int vocab, int max_pos, int compact) {
+                                    float scale, int vocab, int max_pos, int compact, int* __restrict__ keep) {
     __shared__ int s_b, s_live;
     const int i = blockIdx.x;                      // row slot * (k + 1) + c
     pdl_wait();                                    // session state comes from the previous step's commit
@@ -161,6 +161,7 @@ __global__ void k_verify_prep_embed(Session s, const int* __restrict__ draft, in
             r.seq[i] = b;
             r.nk_self[i] = j + c + 1;     // causal: positions 0..j+c
             r.nk_cross[i] = s.src_len[b];
+            if (keep && c > 0) keep[b * k + c - 1] = tok;      // the caller's drafts, for the commit that follows
         } else if (c == 0) {
             r.slot_seq[slot] = -1;
         }
@@ -807,7 +808,8 @@ struct FusedCommit { Session s; const int* draft; int eos; unsigned long long* p
 // finds the first rejected draft.  row_stats (optional) receives 6 floats per row.
 static __global__ void k_accept(const RowPart* __restrict__ part, int n_tiles, const float* __restrict__ ld,
                          const int* __restrict__ ld_id, int k, int beta, float tau, int* __restrict__ accepted,
-                         int* __restrict__ bif, float* __restrict__ row_stats, int want_sum, const int* __restrict__ slot_seq, FusedCommit fc) {
+                         int* __restrict__ bif, int* __restrict__ accepted2, int* __restrict__ bif2, float* __restrict__ row_stats,
+                         int want_sum, const int* __restrict__ slot_seq, FusedCommit fc) {
     extern __shared__ unsigned char sm_acc[];
     RowPart* rs = reinterpret_cast<RowPart*>(sm_acc);       // [k+1]
     __shared__ unsigned char ok_s[256];                     // row c passes both tests (k <= 255 rows take this path)
@@ -864,6 +866,8 @@ static __global__ void k_accept(const RowPart* __restrict__ part, int n_tiles, c
         }
         accepted[sq] = a;
         bif[sq] = rs[a].arg;
+        if (accepted2) accepted2[sq] = a;                    // the caller's arrays
+        if (bif2) bif2[sq] = rs[a].arg;
         if (fc.on) commit_sequence(fc.s, sq, fc.draft, a, rs[a].arg, k, fc.eos);
     }
     if (row_stats)

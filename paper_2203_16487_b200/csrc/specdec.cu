@@ -113,7 +113,7 @@ struct specdec_handle {
     int want_trace = 0;
     int poll_lag = -1;              // -1: chosen by batch size
     int stats_timing = 0;           // 1: specdec_generate records an event after every phase (option "stats_timing")
-    int use_gate = 1;               // whole iterations as one graph behind a device-side IF node (option "gate")
+    int use_gate = 0;               // whole iterations as one graph behind a device-side IF node (option "gate")
     bool gate_ok = true;            // false once building such a graph failed: the plain graphs are used from then on
     // LayerNorm fused into the residual GEMM that feeds it (tensor-core path): what the next residual GEMM should
     // also produce, and what the last one did produce
@@ -882,12 +882,12 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
     const bool compact = h->fuse_commit && h->B > 1;
     const int B = h->B, slots = compact ? std::min(B, h->act_ub) : B, d = m.dm.d_model, L = m.dm.dec_layers, M = slots * (k + 1);
     const int max_keys = std::min(h->len_ub, h->T_cap) + k + 1;
-    if (d_draft != h->v_draft && k > 0)
-        CUDA_TRY(h, cudaMemcpyAsync(h->v_draft, d_draft, (size_t)B * k * 4, cudaMemcpyDeviceToDevice, st));
+    // (the caller's drafts and result arrays are read and written by the kernels themselves: a copy node costs 2 us of the step)
+    int* keep = (d_draft != h->v_draft && k > 0) ? h->v_draft : nullptr;
     // row metadata and embedding of the block in one kernel
     h->fused_x = nullptr;
-    CUDA_TRY(h, launch_pdl(h, k_verify_prep_embed<T>, dim3(M), dim3(128), 0, st, h->ses, (const int*)h->v_draft, B, k, h->S_max, h->cfg.bos_id,
-                           h->rows, (const T*)m.embed, (const float*)m.pos_dec, h->x, d, sqrtf((float)d), m.dm.vocab, m.dm.max_pos, compact ? 1 : 0));
+    CUDA_TRY(h, launch_pdl(h, k_verify_prep_embed<T>, dim3(M), dim3(128), 0, st, h->ses, d_draft, B, k, h->S_max, h->cfg.bos_id,
+                           h->rows, (const T*)m.embed, (const float*)m.pos_dec, h->x, d, sqrtf((float)d), m.dm.vocab, m.dm.max_pos, compact ? 1 : 0, keep));
     KCHECK(h);
     for (int l = 0; l < L; ++l) {
         const bool last = l + 1 == L;
@@ -903,7 +903,7 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
         cudaError_t e = cudaSuccess;
         const dim3 grid(cdiv(M, 8)), block(256);
 #define LN_LD(NC) e = launch_pdl(h, k_layernorm_ld<T, NC>, grid, block, 0, st, (const float*)h->x, (const float*)m.dec_lnf_g, (const float*)m.dec_lnf_b, (T*)h->y, d, 1e-5f, \
-                                 (const T*)m.embed, (const int*)h->v_draft, (const int*)h->rows.slot_seq, (const int*)(h->ses.counters + CNT_VERIFY), k, m.dm.vocab, h->ld, h->ld_id)
+                                 (const T*)m.embed, d_draft, (const int*)h->rows.slot_seq, (const int*)(h->ses.counters + CNT_VERIFY), k, m.dm.vocab, h->ld, h->ld_id)
         switch (d / 128) {
             case 1: LN_LD(1); break; case 2: LN_LD(2); break; case 3: LN_LD(3); break; case 4: LN_LD(4); break;
             case 5: LN_LD(5); break; case 6: LN_LD(6); break; case 7: LN_LD(7); break; default: LN_LD(8); break;
@@ -914,7 +914,7 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
     } else {
         TRY(ln_or_fused<T>(h, h->x, m.dec_lnf_g, m.dec_lnf_b, CNT_VERIFY, M, h->y, d, st));
         CUDA_TRY(h, launch_pdl(h, k_draft_logit<T>, dim3(cdiv(M, 4)), dim3(128), 0, st, (const T*)h->y, (const T*)m.embed,
-                               (const int*)h->v_draft, (const int*)h->rows.slot_seq, (const int*)(h->ses.counters + CNT_VERIFY), k, d, m.dm.vocab, h->ld, h->ld_id));
+                               d_draft, (const int*)h->rows.slot_seq, (const int*)(h->ses.counters + CNT_VERIFY), k, d, m.dm.vocab, h->ld, h->ld_id));
         KCHECK(h);
     }
     int n_tiles = 0;
@@ -924,11 +924,9 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
     prof_mark(h, st);
     FusedCommit fc{h->ses, h->v_draft, h->cfg.eos_id, h->h_post, h->fuse_commit ? 1 : 0};
     CUDA_TRY(h, launch_pdl(h, k_accept, dim3(slots), dim3(1024), (size_t)(k + 1) * sizeof(RowPart), st, (const RowPart*)h->part, n_tiles,
-                           (const float*)h->ld, (const int*)h->ld_id, k, beta, tau, h->accepted, h->bif, h->row_stats, h->want_lse, (const int*)h->rows.slot_seq, fc));
+                           (const float*)h->ld, (const int*)h->ld_id, k, beta, tau, h->accepted, h->bif, d_accepted, d_bif, h->row_stats, h->want_lse, (const int*)h->rows.slot_seq, fc));
     KCHECK(h);
     h->commit_done = h->fuse_commit;
-    if (d_accepted) CUDA_TRY(h, cudaMemcpyAsync(d_accepted, h->accepted, (size_t)B * 4, cudaMemcpyDeviceToDevice, st));
-    if (d_bif) CUDA_TRY(h, cudaMemcpyAsync(d_bif, h->bif, (size_t)B * 4, cudaMemcpyDeviceToDevice, st));
     h->last_k = k; h->verified = true; h->drafted = false;
     return 0;
 }
@@ -1102,14 +1100,13 @@ int generate_loop(specdec_handle* h, const int* d_src, const int* d_src_len, con
     mark_always();
     const int max_iters = h->T_cap;            // every iteration commits >= 1 token per unfinished sequence
     const bool graphs = h->use_graphs && !h->profile;
-    // the conditional node costs more per iteration than the bubble it removes: worth it only where the host ran
-    // ahead anyway (larger batches), to make the iterations queued after the last sequence finished free
     bool gated = graphs && h->gate_ok && !phases && (h->use_gate == 1 ? B > 4 : h->use_gate == 2);
-    // how many iterations the host runs ahead of the "unfinished sequences" counter it reads back.  Plain graphs:
-    // every iteration launched after the last sequence finished is wasted work, every wait for the counter is a
-    // bubble.  Gated graphs: an iteration too many costs one small kernel, so the host always runs ahead.
+    // How many iterations the host runs ahead of the post it reads.  The default waits for each post: the few microseconds until the
+    // next launch arrives cost less than what running ahead does -- an iteration queued after the last sequence finished is a
+    // wasted pass, launches are sized by an older count of unfinished sequences, and a conditional node in front of the iteration (option
+    // "gate") adds some 40 us to it (32 sequences: 7.75 ms waiting, 8.07 one ahead, 8.43 two ahead, 8.38 two ahead and gated).
     const int slots = (int)h->poll_ev.size();
-    int lag = h->poll_lag >= 0 ? std::min(h->poll_lag, slots - 1) : (gated ? 2 : (B <= 4 ? 0 : 2));
+    int lag = h->poll_lag >= 0 ? std::min(h->poll_lag, slots - 1) : (gated ? 2 : 0);
     int it = 0, skipped = 0;
     long long skipped_kernels = 0;
     const bool flag = h->poll_flag != 0;
@@ -1138,7 +1135,7 @@ int generate_loop(specdec_handle* h, const int* d_src, const int* d_src_len, con
                     if (!r) r = verify_impl<T>(h, h->v_draft, k, beta, tau, nullptr, nullptr, st);
                     return r ? r : commit_impl(h, nullptr, nullptr, st);
                 }, &nk);
-                if (rc == 1) { gated = false; if (h->poll_lag < 0) lag = std::min(lag, B <= 4 ? 0 : 2); }
+                if (rc == 1) { gated = false; if (h->poll_lag < 0) lag = 0; }
                 else if (rc != 0) return rc;
                 else { done = true; it_kernels.push_back(nk); }
             }
