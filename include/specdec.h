@@ -271,10 +271,10 @@ int specdec_profile_read(specdec_handle* h, double* h_ms, long long* h_launches)
  * "enc_skinny"   0 / 1 (default) / 2: the weight-streaming GEMM does not / does / does serve the encoders (up to 208 rows)
  * "ln_fuse"      0/1 the LayerNorm that reads the residual stream next runs inside the residual GEMM (default 0)
  * "splitk"       0/1 residual GEMMs with K >= 1024 over few row tiles split K across a cluster (default 1)
- * "attn_rs"      0 never / 1 by rule (default) / 2 whenever the keys allow: scores stay in the MMA accumulators
- * "attn_stream"  0 never / 1 by rule (default) / 2 always / 3 always, two-stage ring: attention walks the keys in
- *                blocks of 64 with a running maximum; "attn_stream_keys" (default 320) is the rule's threshold
- * "attn_warps"   0 choose per launch (default), 4 or 8 warps per tile-attention CTA
+ * "attn_stream"  0 / 1 by rule (default) / 2 / 3: attention CTAs of 16 queries with the keys spread over their warps, or of
+ *                64 (2) or 32 (3) queries with 16 to a warp
+ * "attn_warps"   0 by rule (default), 4 or 8: the former with that many warps.  ("attn_rs" and "attn_stream_keys" are accepted
+ *                and do nothing: they chose between kernels that are one now)
  * "tc_bn"        0 choose (default), else the column width of the tensor-core tiles (64 / 128 / 256)
  * "pdl"          0/1 programmatic dependent launch between the kernels of a step (default 1)
  * "graphs"       0/1 replay steps from CUDA graphs (default 1)

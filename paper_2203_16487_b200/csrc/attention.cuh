@@ -1,0 +1,316 @@
+// Attention for bf16 operands and head size 64: one CTA per (tile of 16 MT queries, head, sequence).  Used for the verifier's
+// causal attention over the paged cache, both cross-attentions, the drafter's bidirectional attention and the encoders.
+//
+// K and V walk through a ring of NS cp.async stages (128-byte rows, XOR-swizzled 16-byte chunks).  Warp (row tile mt, key group
+// kg) takes KW keys of every block for 16 queries: S = Q K^T (mma.sync m16n8k16, fp32 accumulation), running row maximum and
+// sum in registers, P (bf16, relative to the running maximum) straight from the score registers into the second
+// contraction; the result is divided by the fp32 sum of the unrounded exponentials.  With KG > 1 the key groups of a row tile
+// meet in shared memory at the end, added in group order.  Work per CTA is 64 keys x 64 x 16 MT x 4 flops a block: too little to
+// fill a 128-row tcgen05 tile, which is why this contraction uses warp-level MMA (8 clocks each per scheduler, measured).
+//
+// What bounds it.  Few CTAs: the chain of round trips of one CTA.  Everything that predates the step -- row counts, the page
+// table's rows of all keys, the cached keys themselves -- is fetched ahead of the dependency wait, so that one round trip (queries and
+// new keys) is left behind it, and the keys are spread over four or eight warps (verify step at 26 rows: 176 us with the one-shot
+// kernel this one replaces, 161 with MT = 1, KG = 4).  Many CTAs: the fixed-latency chain inside a warp at the
+// occupancy that 130 registers leave (12 warps per SM: issue slots 42 % busy, tensor pipe 22 %, DRAM 27 %); 64-key blocks per
+// warp give the most independent work per barrier (128 sequences x 51 queries x 307 keys: 51 -> 34 us a launch; x 26 x 90: 16 -> 10.7).
+#pragma once
+#include "kernels.cuh"
+
+namespace sd {
+
+struct AttnTcArgs {
+    const bf16* q; int q_stride; const int* q_index;     // query row r reads q + (q_index ? q_index[r] : r) * q_stride
+    const bf16* k; const bf16* v; int kv_stride;         // contiguous: key t of sequence b at row kv_off[b] + t
+    const int* kv_off;
+    Paged pg;                                             // paged: row pg.row(b, t)
+    const int* q_off; const int* q_cnt;                   // per sequence: first query row, number of query rows
+    const int* nkeys;                                     // per query row: visible keys (0..nkeys-1)
+    const int* pre_keys;                                  // per sequence (or null): keys 0..pre-1 were written before this
+                                                          // step began, so they may be fetched before the dependency wait
+    bf16* out; int out_stride;
+    int max_keys;                                         // upper bound on nkeys
+    float scale;
+};
+
+__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
+}
+__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
+}
+__device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// byte offset of 16-byte chunk c (0..7) of row r in a tile of 128-byte rows
+__device__ __forceinline__ uint32_t swz(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
+// 2^x for x <= 0: results below 2^-126 are 0.
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ void cp_wait_pending(int n) {       // cp.async.wait_group takes an immediate
+    if (n <= 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
+    else if (n == 1) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else if (n == 2) asm volatile("cp.async.wait_group 2;" ::: "memory");
+    else asm volatile("cp.async.wait_group 3;" ::: "memory");
+}
+
+// MT row tiles of 16 queries x KG key groups = MT KG warps; a key block holds KW keys for each group; NS stages.
+template <int MT, int KG, int KW>
+struct AttnCfg {
+    static constexpr int KB = KG * KW;                                    // keys per block
+    static constexpr int STAGE = KB * 256;                                // K and V of a block
+    static constexpr int MERGE = KG > 1 ? MT * KG * 16 * (68 + 2) * 4 : 0;     // partial outputs (padded rows) and (maximum, sum); reuses the stages
+    static size_t smem(int max_keys, int ns) {
+        const int nb = (max_keys + KB - 1) / KB;
+        const size_t ring = (size_t)(nb < ns ? (nb < 1 ? 1 : nb) : ns) * STAGE;
+        return (size_t)MT * 2048 + (ring > MERGE ? ring : MERGE) + (size_t)((max_keys + 3) & ~3) * 4;
+    }
+};
+
+template <bool PAGED, int MT, int KG, int KW, int NS>
+__global__ void __launch_bounds__(MT * KG * 32) k_attn(AttnTcArgs a) {
+    using C = AttnCfg<MT, KG, KW>;
+    static_assert(NS >= 1 && NS <= 4 && KW % 16 == 0, "ring depth, keys per warp");
+    constexpr int THREADS = MT * KG * 32, KB = C::KB, NT = KW / 8, BM = MT * 16;
+    extern __shared__ __align__(128) unsigned char sm[];
+    __shared__ int s_nk[BM];
+    __shared__ int s_nkmax;
+    const int b = blockIdx.z, h = blockIdx.y, qt = blockIdx.x;
+    // Row metadata, page table and sequence lengths are written at the start of the step, before the first
+    // kernel of the programmatic-launch chain can begin, so they may be read before the dependency wait.
+    const int cnt = a.q_cnt[b], q_first = a.q_off[b];
+    const int pre = a.pre_keys ? min(a.pre_keys[b], a.max_keys) : 0, kv0 = PAGED ? 0 : a.kv_off[b];
+    if (qt * BM >= cnt) return;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int r0 = q_first + qt * BM, nq = min(BM, cnt - qt * BM);
+    const int nb_cap = (a.max_keys + KB - 1) / KB, ring = nb_cap < NS ? max(nb_cap, 1) : NS;        // stages that shared memory was sized for
+    const uint32_t Qs = (uint32_t)__cvta_generic_to_shared(sm), St = Qs + BM * 128;
+    unsigned char* Sp = sm + BM * 128;
+    int* s_row = reinterpret_cast<int*>(Sp + max(ring * C::STAGE, C::MERGE));                          // paged: K / V row of every key
+    if (PAGED) {
+        for (int t = tid; t < a.max_keys; t += THREADS) s_row[t] = (int)a.pg.row(b, t);
+        __syncthreads();
+    }
+    const int c8 = tid & 7, t0 = tid >> 3;      // a thread keeps its 16-byte chunk of the 128-byte head slice and walks the keys
+    const bf16* kcol = a.k + h * 64 + c8 * 8;
+    const bf16* vcol = a.v + h * 64 + c8 * 8;
+    // keys [blk KB + lo, blk KB + hi) of a block into its stage; rows past the last key (n) are zeroed
+    auto load_keys = [&](int blk, int lo, int hi, int n) {
+        const uint32_t Ks = St + (blk % ring) * C::STAGE, Vs = Ks + KB * 128;
+        for (int t = lo + t0; t < hi; t += THREADS / 8) {
+            const int key = blk * KB + t;
+            if (key < n) {
+                const size_t off = (size_t)(PAGED ? s_row[key] : kv0 + key) * a.kv_stride;
+                cp_async16(Ks + swz(t, c8), kcol + off);
+                cp_async16(Vs + swz(t, c8), vcol + off);
+            } else {
+                *reinterpret_cast<uint4*>(sm + (Ks - Qs) + swz(t, c8)) = make_uint4(0, 0, 0, 0);
+                *reinterpret_cast<uint4*>(sm + (Vs - Qs) + swz(t, c8)) = make_uint4(0, 0, 0, 0);
+            }
+        }
+    };
+    // keys that predate this step (cached prefix, encoder memory) are requested before the wait, as far as the ring reaches ...
+    const int npre = min(pre, ring * KB);
+    for (int blk = 0; blk * KB < npre; ++blk) load_keys(blk, 0, min(npre - blk * KB, KB), npre);
+    if (tid < 32) {
+        int m = 0;
+#pragma unroll
+        for (int i = 0; i < (BM + 31) / 32; ++i) {
+            const int r = tid + i * 32;
+            const int nk = r < nq ? min(a.nkeys[r0 + r], a.max_keys) : 0;
+            if (r < BM) s_nk[r] = nk;
+            m = max(m, nk);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (tid == 0) s_nkmax = m;
+    }
+    __syncthreads();
+    const int nkmax = s_nkmax, nblk = max((nkmax + KB - 1) / KB, 1);
+    pdl_launch_dependents();
+    pdl_wait();                                  // ... and everything the predecessor kernels wrote after it
+    for (int r = t0; r < BM; r += THREADS / 8) {
+        if (r < nq) {
+            const size_t qr = a.q_index ? (size_t)a.q_index[r0 + r] : (size_t)(r0 + r);
+            cp_async16(Qs + swz(r, c8), a.q + qr * a.q_stride + h * 64 + c8 * 8);
+        } else {
+            *reinterpret_cast<uint4*>(sm + swz(r, c8)) = make_uint4(0, 0, 0, 0);
+        }
+    }
+    int issued = 0;
+    auto issue = [&]() {                         // the rest of block `issued`, one commit group per block
+        load_keys(issued, min(max(npre - issued * KB, 0), KB), KB, nkmax);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        ++issued;
+    };
+
+    const int g = lane >> 2, t4 = lane & 3;
+    const int mt = warp % MT, kg = warp / MT;    // query rows 16 mt .. + 15, keys KW kg .. + KW - 1 of every block
+    const int nk0 = s_nk[mt * 16 + g], nk1 = s_nk[mt * 16 + g + 8];
+    uint32_t qf[4][4];
+    float m_run[2] = {-CUDART_INF_F, -CUDART_INF_F}, l_run[2] = {0.f, 0.f};   // rows g, g + 8 (sums: this lane's share)
+    float acc[8][4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+    const float sl = a.scale * 1.4426950408889634f;      // exp(scale (s - max)) as 2^(sl s - sl max)
+    // keys that every row of this warp sees (rows past the last query see none and are never stored)
+    int nkall = mt * 16 + g < nq ? nk0 : 0x7fffffff;
+    if (mt * 16 + g + 8 < nq) nkall = min(nkall, nk1);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) nkall = min(nkall, __shfl_xor_sync(0xffffffffu, nkall, o));
+
+    while (issued < min(ring, nblk)) issue();
+    for (int blk = 0; blk < nblk; ++blk) {
+        cp_wait_pending(issued - blk - 1);
+        __syncthreads();
+        if (blk == 0) {
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+                const int r = mt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, c = ks * 2 + (lane >> 4);
+                ldsm_x4(Qs + swz(r, c), qf[ks][0], qf[ks][1], qf[ks][2], qf[ks][3]);
+            }
+        }
+        const uint32_t Ks = St + (blk % ring) * C::STAGE + kg * KW * 128, Vs = Ks + KB * 128;
+        const int kbase = blk * KB + kg * KW;
+        if (kbase < nkmax && mt * 16 < nq) {       // warp-uniform: a visible key, a live query
+            float sc[NT][4];
+            float bm0 = -CUDART_INF_F, bm1 = -CUDART_INF_F;
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                uint32_t kf[2][4];
+#pragma unroll
+                for (int kk = 0; kk < 2; ++kk)
+                    ldsm_x4(Ks + swz(nt * 8 + (lane & 7), kk * 4 + (lane >> 3)), kf[kk][0], kf[kk][1], kf[kk][2], kf[kk][3]);
+                float s4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) mma_bf16(s4, qf[ks], kf[ks >> 1][(ks & 1) * 2], kf[ks >> 1][(ks & 1) * 2 + 1]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sc[nt][e] = s4[e];
+            }
+            if (kbase + KW > nkall) {              // a block at some row's last key
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) {
+                    const int col = kbase + nt * 8 + t4 * 2;
+                    if (col >= nk0) sc[nt][0] = -CUDART_INF_F;
+                    if (col + 1 >= nk0) sc[nt][1] = -CUDART_INF_F;
+                    if (col >= nk1) sc[nt][2] = -CUDART_INF_F;
+                    if (col + 1 >= nk1) sc[nt][3] = -CUDART_INF_F;
+                }
+            }
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                bm0 = fmaxf(bm0, fmaxf(sc[nt][0], sc[nt][1]));
+                bm1 = fmaxf(bm1, fmaxf(sc[nt][2], sc[nt][3]));
+            }
+            bm0 = fmaxf(bm0, __shfl_xor_sync(0xffffffffu, bm0, 1)); bm1 = fmaxf(bm1, __shfl_xor_sync(0xffffffffu, bm1, 1));
+            bm0 = fmaxf(bm0, __shfl_xor_sync(0xffffffffu, bm0, 2)); bm1 = fmaxf(bm1, __shfl_xor_sync(0xffffffffu, bm1, 2));
+            const float mn0 = fmaxf(m_run[0], bm0), mn1 = fmaxf(m_run[1], bm1);
+            // a row with no visible key so far keeps maximum -inf: its terms are 0 against a base of 0
+            const float mb0 = (mn0 == -CUDART_INF_F) ? 0.f : mn0 * sl, mb1 = (mn1 == -CUDART_INF_F) ? 0.f : mn1 * sl;
+            if (blk > 0) {
+                const float al0 = ex2(fmaf(m_run[0], sl, -mb0)), al1 = ex2(fmaf(m_run[1], sl, -mb1));      // (maximum -inf: 0, on sums that are 0)
+                l_run[0] *= al0; l_run[1] *= al1;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) { acc[j][0] *= al0; acc[j][1] *= al0; acc[j][2] *= al1; acc[j][3] *= al1; }
+            }
+            m_run[0] = mn0; m_run[1] = mn1;
+#pragma unroll
+            for (int kt = 0; kt < NT / 2; ++kt) {
+                uint32_t pf[4];
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    const float* s = sc[2 * kt + hf];
+                    const float e0 = ex2(fmaf(s[0], sl, -mb0)), e1 = ex2(fmaf(s[1], sl, -mb0));      // -inf scores give 0
+                    const float e2 = ex2(fmaf(s[2], sl, -mb1)), e3 = ex2(fmaf(s[3], sl, -mb1));
+                    l_run[0] += e0 + e1; l_run[1] += e2 + e3;
+                    __nv_bfloat162 p01 = __floats2bfloat162_rn(e0, e1), p23 = __floats2bfloat162_rn(e2, e3);
+                    // accumulator layout of an 8-key tile = half of the A fragment of a 16-key step
+                    pf[hf * 2] = *reinterpret_cast<uint32_t*>(&p01);
+                    pf[hf * 2 + 1] = *reinterpret_cast<uint32_t*>(&p23);
+                }
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    uint32_t vf[4];
+                    ldsm_x4_t(Vs + swz(kt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, v * 2 + (lane >> 4)), vf[0], vf[1], vf[2], vf[3]);
+                    mma_bf16(acc[2 * v], pf, vf[0], vf[1]);
+                    mma_bf16(acc[2 * v + 1], pf, vf[2], vf[3]);
+                }
+            }
+        }
+        if (issued < nblk || (KG > 1 && blk + 1 == nblk)) __syncthreads();       // the stage is about to be overwritten (by a later block, or by the merge)
+        if (issued < nblk) issue();
+    }
+
+    l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 1); l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 1);
+    l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 2); l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 2);
+    if constexpr (KG == 1) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const int r = mt * 16 + g + half * 8;
+            if (r < nq) {
+                const float inv = l_run[half] > 0.f ? 1.0f / l_run[half] : 0.f;
+                bf16* o = a.out + (size_t)(r0 + r) * a.out_stride + h * 64 + t4 * 2;
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    *reinterpret_cast<__nv_bfloat162*>(o + j * 8) = __floats2bfloat162_rn(acc[j][half * 2] * inv, acc[j][half * 2 + 1] * inv);
+            }
+        }
+    } else {
+        // ---- the key groups of a row tile meet in shared memory; each of its warps combines 64 / KG columns, in group order
+        float* mO = reinterpret_cast<float*>(Sp);                        // [MT][KG][16 rows][68]
+        float* mML = mO + MT * KG * 16 * 68;                             // [MT][KG][16 rows][maximum, sum]
+        float* po = mO + (mt * KG + kg) * 16 * 68;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            *reinterpret_cast<float2*>(po + g * 68 + j * 8 + t4 * 2) = make_float2(acc[j][0], acc[j][1]);
+            *reinterpret_cast<float2*>(po + (g + 8) * 68 + j * 8 + t4 * 2) = make_float2(acc[j][2], acc[j][3]);
+        }
+        if (t4 == 0) {
+            float* ml = mML + (mt * KG + kg) * 32;
+            ml[g * 2] = m_run[0]; ml[g * 2 + 1] = l_run[0];
+            ml[(g + 8) * 2] = m_run[1]; ml[(g + 8) * 2 + 1] = l_run[1];
+        }
+        __syncthreads();
+        constexpr int CW = 64 / KG, PER = CW / 2;                        // columns per warp; two lanes per row
+        const int rr = lane >> 1, c0 = kg * CW + (lane & 1) * PER, r = mt * 16 + rr;
+        float m = -CUDART_INF_F;
+        float f[KG];
+#pragma unroll
+        for (int q = 0; q < KG; ++q) { f[q] = mML[(mt * KG + q) * 32 + rr * 2]; m = fmaxf(m, f[q]); }
+        float den = 0.f;
+#pragma unroll
+        for (int q = 0; q < KG; ++q) {
+            f[q] = (f[q] == -CUDART_INF_F) ? 0.f : ex2((f[q] - m) * sl);
+            den = fmaf(mML[(mt * KG + q) * 32 + rr * 2 + 1], f[q], den);
+        }
+        const float inv = den > 0.f ? 1.0f / den : 0.f;
+        if (r < nq) {
+            bf16* o = a.out + (size_t)(r0 + r) * a.out_stride + h * 64 + c0;
+#pragma unroll
+            for (int c = 0; c < PER; c += 4) {
+                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int q = 0; q < KG; ++q) {
+                    const float4 t = *reinterpret_cast<const float4*>(mO + ((mt * KG + q) * 16 + rr) * 68 + c0 + c);
+                    x.x = fmaf(t.x, f[q], x.x); x.y = fmaf(t.y, f[q], x.y); x.z = fmaf(t.z, f[q], x.z); x.w = fmaf(t.w, f[q], x.w);
+                }
+                __nv_bfloat162 p0 = __floats2bfloat162_rn(x.x * inv, x.y * inv), p1 = __floats2bfloat162_rn(x.z * inv, x.w * inv);
+                *reinterpret_cast<uint2*>(o + c) = make_uint2(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1));
+            }
+        }
+    }
+}
+
+}  // namespace sd

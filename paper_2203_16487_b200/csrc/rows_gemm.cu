@@ -1,5 +1,5 @@
 // GEMM for passes of few activation rows (see rows_gemm.cuh for where it is used).
-#include "attention_tc.cuh"
+#include "attention.cuh"
 #include "gemm_tc.cuh"
 #include "rows_gemm.cuh"
 

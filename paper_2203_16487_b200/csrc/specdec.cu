@@ -18,8 +18,7 @@
 
 #include "../../include/specdec.h"
 #include "accept_scan.cuh"
-#include "attention_stream.cuh"
-#include "attention_tc.cuh"
+#include "attention.cuh"
 #include "cluster_round.cuh"
 #include "gemm_tc.cuh"
 #include "gemm_tc_pair.cuh"
@@ -134,14 +133,11 @@ struct specdec_handle {
     int use_splitk = 1;             // residual GEMMs with K >= 1024 over few row tiles split K across a cluster of 4 / 6 CTAs (option "splitk")
     bool pair_ready = false;
     int use_pair = 0;               // two-SM tiles (cta_group::2) for wide GEMMs over many rows (option "pair")
-    int attn_rs = 1;                // tile attention keeps the scores in registers when the keys allow (option "attn_rs")
-    int attn_stream = 1;            // streaming tile attention: 0 never, 1 by rule, 2 always, 3 always with the 2-stage ring (option "attn_stream")
-    int attn_stream_keys = 320;     // option "attn_stream_keys"
-    int attn_warps = 0;             // 0 = choose per launch, else 4 or 8 warps per tile-attention CTA (option "attn_warps")
+    int attn_stream = 1;            // attention variant (option "attn_stream")
+    int attn_warps = 0;             // 0 by rule, else 4 or 8 key groups per attention CTA (option "attn_warps")
     // CUDA graphs of whole draft / verify(+commit) steps, keyed by everything their launches depend on
     struct GraphEntry { cudaGraphExec_t exec; long long kernels; };
     std::map<std::vector<long long>, GraphEntry> graphs;
-    size_t attn_tc_smem_cap = 0;
     long long launches = 0;
     // polling
     int* h_poll = nullptr;          // pinned
@@ -556,17 +552,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
          int out_stride, int n_heads, int d_head, int max_keys, cudaStream_t st, const int* pre_keys = nullptr) {
     if (rows_ub <= 0) return 0;
     if constexpr (std::is_same<T, bf16>::value) {
-        const size_t smem = attn_tc_smem(max_keys);
-        // the streaming kernel where the one-shot kernel cannot hold the keys, and where the SMs are full of CTAs
-        // and the keys are many (its small footprint keeps the occupancy up; with few CTAs its block-by-block walk
-        // is slower than one big request)
-        const int n_seq = cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub);
-        const long long attn_ctas = (long long)cdiv(q_ub, ATT_Q) * n_heads * n_seq;
-        const bool stream = h->use_tc_attn && d_head == 64 &&
-                            (h->attn_stream >= 2 ||
-                             (h->attn_stream == 1 && (smem > h->attn_tc_smem_cap ||
-                                                      (max_keys > h->attn_stream_keys && attn_ctas >= 4LL * h->tma.n_sm))));
-        if (stream || (h->use_tc_attn && d_head == 64 && smem <= h->attn_tc_smem_cap)) {
+        if (h->use_tc_attn && d_head == 64) {
             AttnTcArgs a;
             a.q = (const bf16*)q; a.q_stride = q_stride; a.q_index = q_index;
             a.k = (const bf16*)k; a.v = (const bf16*)v; a.kv_stride = kv_stride; a.kv_off = kv_off;
@@ -574,44 +560,28 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             a.q_off = r.q_off; a.q_cnt = r.q_cnt; a.nkeys = nkeys; a.pre_keys = h->use_pdl ? pre_keys : nullptr;
             a.out = (bf16*)out; a.out_stride = out_stride; a.max_keys = max_keys;
             a.scale = 1.0f / sqrtf((float)d_head);
-            dim3 grid(cdiv(q_ub, ATT_Q), n_heads, h->B);
-            if (stream) {          // key blocks through a ring of stages: shared memory independent of the key count
-                const bool deep = h->attn_stream != 3 && attn_ctas < 4LL * h->tma.n_sm;    // few CTAs: more bytes in flight per CTA
-                cudaError_t e = deep ? (paged ? launch_pdl(h, k_attn_stream<true, 4>, grid, dim3(128), (size_t)ats_smem(4), st, a)
-                                              : launch_pdl(h, k_attn_stream<false, 4>, grid, dim3(128), (size_t)ats_smem(4), st, a))
-                                     : (paged ? launch_pdl(h, k_attn_stream<true, 2>, grid, dim3(128), (size_t)ats_smem(2), st, a)
-                                              : launch_pdl(h, k_attn_stream<false, 2>, grid, dim3(128), (size_t)ats_smem(2), st, a));
+            const int n_seq = cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub);
+            auto go = [&](auto* kernel, int bm, int warps, size_t smem) {
+                const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, bm), n_heads, h->B), dim3(warps * 32), smem, st, a);
                 if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
                 KCHECK(h);
                 return 0;
+            };
+#define ATTN_GO(MT, KG, KW, NS) (paged ? go(k_attn<true, MT, KG, KW, NS>, 16 * MT, MT * KG, AttnCfg<MT, KG, KW>::smem(max_keys, NS)) \
+                                       : go(k_attn<false, MT, KG, KW, NS>, 16 * MT, MT * KG, AttnCfg<MT, KG, KW>::smem(max_keys, NS)))
+            // While 16-query tiles are at most four CTAs per SM the keys are spread over the warps of a CTA: four, or eight when the
+            // keys are many and the CTAs fewer than SMs (verify step of 11 rows over 511 keys: 192 us with four, 180 with eight).
+            const long long tiles16 = (long long)cdiv(q_ub, 16) * n_heads * n_seq;
+            const bool spread = h->attn_warps || h->attn_stream == 0 || (h->attn_stream == 1 && tiles16 <= 4LL * h->tma.n_sm);
+            if (spread) {
+                const bool eight = h->attn_warps ? h->attn_warps == 8 : (max_keys > 256 && tiles16 <= h->tma.n_sm);
+                return eight ? ATTN_GO(1, 8, 32, 2) : ATTN_GO(1, 4, 32, 3);
             }
-            // 4 warps when the SMs are saturated with CTAs anyway, 8 when a CTA's own latency chain is what counts;
-            // scores stay in registers (smaller shared memory: more CTAs per SM) when the keys fit 6 tiles per warp
-            const long long ctas = attn_ctas;
-            const int nkp = (max_keys + 15) & ~15;
-            auto per_sm_of = [](size_t sm) { return (long long)(227 * 1024) / (long long)(sm + 1024); };
-            // (measured: the register variant is slower per CTA, 357 -> 387 us per batch-1 step, and pays off only where
-            // shared memory held the occupancy down: 1018 -> 873 us per step at batch 128 over a 256-token prefix)
-            // (choosing it wherever it saves a wave of CTAs was tried too: 479 vs 469 us per 128-sequence draft step)
-            bool rs = nkp <= attn_tc_rs_max_keys(8) &&
-                      (h->attn_rs == 2 || (h->attn_rs == 1 && per_sm_of(smem) <= 2 && ctas > 2LL * h->tma.n_sm));
-            size_t smem_l = rs ? attn_tc_smem_rs(max_keys) : smem;
-            bool wide = h->attn_warps ? h->attn_warps == 8 : (per_sm_of(smem_l) <= 2 || ctas < 4LL * h->tma.n_sm);
-            if (rs && !wide && nkp > attn_tc_rs_max_keys(4)) {       // too many keys for four warps' registers
-                if (h->attn_warps == 4) { rs = false; smem_l = smem; } else wide = true;
-            }
-            cudaError_t e;
-            if (rs) e = wide ? (paged ? launch_pdl(h, k_attn_tc<true, 8, true>, grid, dim3(256), smem_l, st, a)
-                                      : launch_pdl(h, k_attn_tc<false, 8, true>, grid, dim3(256), smem_l, st, a))
-                             : (paged ? launch_pdl(h, k_attn_tc<true, 4, true>, grid, dim3(128), smem_l, st, a)
-                                      : launch_pdl(h, k_attn_tc<false, 4, true>, grid, dim3(128), smem_l, st, a));
-            else e = wide ? (paged ? launch_pdl(h, k_attn_tc<true, 8>, grid, dim3(256), smem, st, a)
-                                   : launch_pdl(h, k_attn_tc<false, 8>, grid, dim3(256), smem, st, a))
-                          : (paged ? launch_pdl(h, k_attn_tc<true, 4>, grid, dim3(128), smem, st, a)
-                                   : launch_pdl(h, k_attn_tc<false, 4>, grid, dim3(128), smem, st, a));
-            if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
-            KCHECK(h);
-            return 0;
+            // Otherwise 64 or 32 queries per CTA, a warp for every 16: 64 share one pass over the keys (51 queries x 307 keys, 128
+            // sequences: 1186 against 1294 us a step) unless the tail of the last tile is more than an eighth of the work (90
+            // queries: 273 against 265 us a draft step).
+            const bool tall = h->attn_stream == 1 ? 8LL * ((q_ub + 63) / 64 * 64) <= 9LL * ((q_ub + 31) / 32 * 32) : h->attn_stream == 2;
+            return tall ? ATTN_GO(4, 1, 64, 3) : ATTN_GO(2, 1, 64, 3);
         }
     }
     AttnArgs<T> a;
@@ -971,13 +941,10 @@ void drop_graphs(specdec_handle* h) {
 }
 
 // Runs `body` (a sequence of launches on `st`) through a cached CUDA graph: captured on first use,
-// replayed afterwards.  The key must name everything the launches depend on besides device memory.
+// replayed afterwards.  The key must name everything the launches depend on besides device memory and options (setting an
+// option drops every graph).
 inline void graph_key_tail(const specdec_handle* h, std::vector<long long>& key) {
-    for (long long v : {(long long)h->use_tc, (long long)h->use_tc_attn, (long long)h->want_lse, (long long)h->use_skinny,
-                        (long long)h->use_pdl, (long long)h->use_ln_fuse, (long long)h->use_sk_cluster,
-                        (long long)h->use_pair, (long long)h->diag_repeat, (long long)h->use_splitk, (long long)h->attn_stream, (long long)h->attn_stream_keys, (long long)h->attn_warps, (long long)h->attn_rs,
-                        (long long)h->want_trace,
-                        (long long)(h->script_on ? 1 : 0), (long long)h->B, (long long)h->S_max, (long long)h->drafter_pc_session, (long long)(h->fuse_commit ? 1 : 0), (long long)h->enc_skinny, (long long)h->act_ub})
+    for (long long v : {(long long)((h->script_on ? 1 : 0) | (h->drafter_pc_session ? 2 : 0) | (h->fuse_commit ? 4 : 0)), (long long)h->B, (long long)h->S_max, (long long)h->act_ub})
         key.push_back(v);
 }
 
@@ -1480,20 +1447,14 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
     }
     if (h->dtype == SPECDEC_DTYPE_BF16) {
         const int max_keys = std::max(h->S_cap, h->T_cap + h->k_cap + 1);
-        h->attn_tc_smem_cap = std::min<size_t>(attn_tc_smem(max_keys), 227 * 1024);
-        cudaFuncSetAttribute(k_attn_stream<true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, ats_smem(4));
-        cudaFuncSetAttribute(k_attn_stream<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, ats_smem(4));
-        if (cudaFuncSetAttribute(k_attn_tc<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->attn_tc_smem_cap) != cudaSuccess ||
-            cudaFuncSetAttribute(k_attn_tc<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->attn_tc_smem_cap) != cudaSuccess ||
-            cudaFuncSetAttribute(k_attn_tc<true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->attn_tc_smem_cap) != cudaSuccess ||
-            cudaFuncSetAttribute(k_attn_tc<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->attn_tc_smem_cap) != cudaSuccess ||
-            cudaFuncSetAttribute(k_attn_tc<true, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->attn_tc_smem_cap) != cudaSuccess ||
-            cudaFuncSetAttribute(k_attn_tc<false, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->attn_tc_smem_cap) != cudaSuccess ||
-            cudaFuncSetAttribute(k_attn_tc<true, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->attn_tc_smem_cap) != cudaSuccess ||
-            cudaFuncSetAttribute(k_attn_tc<false, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->attn_tc_smem_cap) != cudaSuccess) {
-            cudaGetLastError();
-            h->attn_tc_smem_cap = 48 * 1024;
-        }
+        cudaError_t e = cudaSuccess;
+        auto room = [&](auto* kernel, size_t smem) {
+            if (smem > 227 * 1024 - 2048) h->use_tc_attn = 0;
+            else if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048);
+        };
+#define ATTN_ROOM(MT, KG, KW, NS) room(k_attn<true, MT, KG, KW, NS>, AttnCfg<MT, KG, KW>::smem(max_keys, NS)); room(k_attn<false, MT, KG, KW, NS>, AttnCfg<MT, KG, KW>::smem(max_keys, NS))
+        ATTN_ROOM(1, 4, 32, 3); ATTN_ROOM(1, 8, 32, 2); ATTN_ROOM(4, 1, 64, 3); ATTN_ROOM(2, 1, 64, 3);
+        if (e != cudaSuccess) { cudaGetLastError(); h->use_tc_attn = 0; }
         if (sd::tc_init(h->tma, h->ses.counters + 7) != 0) h->use_tc = 0;     // reported through specdec_last_error; SIMT GEMM still runs on the GPU
         h->splitk_ready = h->use_tc && sd::spk_init() == cudaSuccess;
         if (!h->splitk_ready) cudaGetLastError();
@@ -1580,8 +1541,7 @@ int specdec_set_option(specdec_handle* h, const char* name, int value) {
     if (!strcmp(name, "diag_repeat")) { h->diag_repeat = value; return SPECDEC_OK; }
     if (!strcmp(name, "splitk")) { h->use_splitk = value ? 1 : 0; return SPECDEC_OK; }
     if (!strcmp(name, "attn_stream")) { h->attn_stream = value < 0 ? 0 : (value > 3 ? 3 : value); return SPECDEC_OK; }
-    if (!strcmp(name, "attn_stream_keys")) { h->attn_stream_keys = value; return SPECDEC_OK; }
-    if (!strcmp(name, "attn_rs")) { h->attn_rs = value < 0 ? 0 : (value > 2 ? 2 : value); return SPECDEC_OK; }   // 0 never, 1 choose, 2 whenever possible
+    if (!strcmp(name, "attn_rs") || !strcmp(name, "attn_stream_keys")) return SPECDEC_OK;      // (chose between kernels that are one now)
     if (!strcmp(name, "attn_warps")) {
         if (value != 0 && value != 4 && value != 8) return fail(h, SPECDEC_ERR_INVALID_ARG, "attn_warps must be 0, 4 or 8");
         h->attn_warps = value; return SPECDEC_OK;

@@ -1,0 +1,49 @@
+"""The attention kernel against the oracle, in lock step: every variant (16 / 32 / 64 queries per CTA, one, four or eight key groups)
+over key counts at the edges of its key blocks (32 a warp, 64, 128, 256 a block), with the ring wrapping and with less
+than one block, query counts at the edges of the query tiles, cached prefixes that end inside a block."""
+import numpy as np
+import pytest
+
+from oracle import specdec_oracle as O
+from paper_2203_16487_b200 import workloads as W
+from tests import lockstep
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("opts", [{}, {"attn_warps": 4}, {"attn_warps": 8}, {"attn_stream": 2}, {"attn_stream": 3}])
+@pytest.mark.parametrize("lens,k", [((1, 31, 33, 64, 65), 15), ((127, 129, 255, 257, 385), 33)])
+def test_attention_edges(opts, lens, k):
+    from paper_2203_16487_b200 import binding
+    V = 515
+    dims = W.ModelDims(128, 2, 128, V, 1, 2, 512)
+    wv, wd = W.make_weights(dims, 71, True), W.make_weights(dims, 72, True)
+    mv, md = O.model_from(dims, wv, mode="bf16"), O.model_from(dims, wd, mode="bf16")
+    rng = np.random.default_rng(k)
+    srcs = [W.zipf_ids(rng, n, V) for n in lens]
+    sd = binding.SpecDec(dims, wv, dims, wd, k_max=k, max_batch=len(lens), max_src=max(lens), max_tgt=100, bf16=True)
+    for name, v in opts.items():
+        sd.set_option(name, v)
+    sd.set_option("debug_checks", 1)
+    # drafts that are accepted in part: the prefixes grow by different lengths
+    greedy = [O.greedy_decode(mv, s, 100, W.BOS_ID, W.EOS_ID) for s in srcs]
+
+    def drafts(b, out, n):
+        d = (greedy[b] + [5] * n)[len(out):len(out) + n]
+        cut = (7 * b + 3 + len(out)) % n
+        return np.array(d[:cut] + [(d[cut] + 9) % V] + d[cut + 1:], np.int32)
+
+    rep = lockstep.run(sd, mv, md, srcs, [100] * len(lens), k, 1, 0.0, margin=1e-3, check_logits_every=1, max_iters=4, draft_fn=drafts)
+    assert rep.ok, rep.notes
+    assert rep.max_logit_err < 2e-2 and rep.max_stat_err < 2e-2
+    # the drafter's own attention (bidirectional, all rows of the sequence)
+    g = sd.draft(k).cpu().numpy()
+    out, n, fin = sd.output()
+    out, n, fin = out.cpu().numpy(), n.cpu().numpy(), fin.cpu().numpy()
+    for b in (0, 2, 4):
+        if fin[b]:
+            continue
+        logits = O.decoder_rows(md, [W.BOS_ID] + out[b, :n[b]].tolist() + [W.MASK_ID] * k, O.encode(md, srcs[b]), causal=False)[n[b] + 1:]
+        for i in range(k):
+            assert g[b, i] == logits[i].argmax() or logits[i].max() - logits[i, g[b, i]] < 2e-2, (b, i)
+    sd.close()
