@@ -74,6 +74,7 @@ struct Session {
     int* finished;     // [B]
     int* max_tgt;      // [B]
     int* src_len;      // [B]
+    int* src_off;      // [B] first row of the sequence in the packed encoder pass and in the cross-attention K/V
     int* out;          // [B, out_stride] committed ids
     int out_stride;
     int* counters;     // [16]: 0 rows of the drafter's full pass, 1 rows of its mask-only pass,
@@ -101,19 +102,46 @@ struct Rows {
 };
 
 // ------------------------------------------------------------------ row preparation
-// Encoder: rows are the padded [B,S_max] grid.
-static __global__ void k_enc_prep(const int* __restrict__ src, const int* __restrict__ src_len, int B, int S_max,
-                           Rows r, int* counters) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) counters[CNT_ENC] = B * S_max;
-    if (i < B) { r.kv_off[i] = i * S_max; r.kv_off_cross[i] = i * S_max; r.q_off[i] = i * S_max; r.q_cnt[i] = src_len[i]; }
-    if (i >= B * S_max) return;
-    int b = i / S_max, t = i % S_max;
-    r.tok[i] = src[i];
-    r.pos[i] = t;
-    r.seq[i] = b;
-    r.nk_self[i] = src_len[b];
-    r.nk_cross[i] = src_len[b];
+// Starts a session and prepares the encoder pass, one block per sequence.  Encoder rows are packed: sequence b's source
+// positions follow those of the sequences before it (a ragged batch of 10..80 ids would be 44 % padding), and so do the rows of
+// the cross-attention K/V.  Every block sums the lengths before its own.
+static __global__ void k_enc_prep(Session s, const int* __restrict__ src, const int* __restrict__ src_len, const int* __restrict__ max_tgt,
+                                  int B, int S_max, int max_tgt_cap, Rows r) {
+    __shared__ int red[3][32];
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    int before = 0, total = 0, active = 0;
+    for (int o = tid; o < B; o += blockDim.x) {
+        const int n = min(max(src_len[o], 1), S_max);
+        total += n;
+        if (o < b) before += n;
+        active += (max_tgt ? min(max(max_tgt[o], 0), max_tgt_cap) : max_tgt_cap) > 0 ? 1 : 0;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        before += __shfl_xor_sync(0xffffffffu, before, o);
+        total += __shfl_xor_sync(0xffffffffu, total, o);
+        active += __shfl_xor_sync(0xffffffffu, active, o);
+    }
+    if (lane == 0) { red[0][warp] = before; red[1][warp] = total; red[2][warp] = active; }
+    __syncthreads();
+    before = total = active = 0;
+    for (int w = 0; w < nw; ++w) { before += red[0][w]; total += red[1][w]; active += red[2][w]; }
+    const int n = min(max(src_len[b], 1), S_max);
+    if (tid == 0) {
+        const int mt = max_tgt ? min(max(max_tgt[b], 0), max_tgt_cap) : max_tgt_cap;
+        s.len[b] = 0; s.dlen[b] = 0; s.max_tgt[b] = mt; s.finished[b] = mt <= 0 ? 1 : 0; s.src_len[b] = n; s.src_off[b] = before;
+        r.kv_off[b] = before; r.kv_off_cross[b] = before; r.q_off[b] = before; r.q_cnt[b] = n;
+        if (b == 0) {
+            for (int i = 0; i < 4; ++i) s.stats[i] = 0ull;
+            *s.dticket = 0;
+            s.counters[CNT_ENC] = total; s.counters[CNT_ACTIVE] = active; s.counters[CNT_TICKET] = 0; s.counters[CNT_MAXLEN] = 0;
+        }
+    }
+    for (int t = tid; t < n; t += blockDim.x) {
+        const int i = before + t;
+        r.tok[i] = src[(size_t)b * S_max + t]; r.pos[i] = t; r.seq[i] = b; r.nk_self[i] = n; r.nk_cross[i] = n;
+    }
+    __threadfence();
 }
 
 // Verify block: row slot * (k+1) + c holds [last committed token (BOS if none), drafts] at positions j..j+k of the slot's
@@ -122,7 +150,7 @@ static __global__ void k_enc_prep(const int* __restrict__ src, const int* __rest
 // more than half of all blocks would belong to sequences that ended iterations ago.  The row metadata is complete before the
 // block lets its successors start, because kernels further down the chain read it ahead of their own dependency waits.
 template <typename T>
-__global__ void k_verify_prep_embed(Session s, const int* __restrict__ draft, int B, int k, int S_max, int bos, Rows r,
+__global__ void k_verify_prep_embed(Session s, const int* __restrict__ draft, int B, int k, int bos, Rows r,
                                     const T* __restrict__ E, const float* __restrict__ P, float* __restrict__ x, int d,
                                     float scale, int vocab, int max_pos, int compact, int* __restrict__ keep) {
     __shared__ int s_b, s_live;
@@ -155,7 +183,7 @@ __global__ void k_verify_prep_embed(Session s, const int* __restrict__ draft, in
     if (threadIdx.x == 0) {
         if (i == 0) s.counters[CNT_VERIFY] = (compact ? s_live : B) * (k + 1);
         if (b >= 0) {
-            if (c == 0) { r.kv_off_cross[b] = b * S_max; r.q_off[b] = slot * (k + 1); r.q_cnt[b] = k + 1; r.slot_seq[slot] = b; }
+            if (c == 0) { r.kv_off_cross[b] = s.src_off[b]; r.q_off[b] = slot * (k + 1); r.q_cnt[b] = k + 1; r.slot_seq[slot] = b; }
             r.tok[i] = tok;
             r.pos[i] = j + c;
             r.seq[i] = b;
@@ -199,7 +227,7 @@ __device__ __forceinline__ void embed_rows(const Rows& all, int r0, int n, const
 // 90-row pass a 26 us serial walk).  Every block completes its metadata before it lets the successors start, because
 // kernels further down the chain read it ahead of their dependency waits.
 template <typename T>
-__global__ void k_draft_prep(Session s, int B, int k, int S_max, int bos, int mask, Rows all, Rows msk,
+__global__ void k_draft_prep(Session s, int B, int k, int bos, int mask, Rows all, Rows msk,
                              const T* __restrict__ E, const float* __restrict__ P, float* __restrict__ x, int d, float scale,
                              int vocab, int max_pos) {
     __shared__ int red_a[32], red_m[32], tot_a[32], tot_l[32];
@@ -224,8 +252,8 @@ __global__ void k_draft_prep(Session s, int B, int k, int S_max, int bos, int ma
     const int j = s.len[b], n = fin ? 0 : j + 1 + k, sl = s.src_len[b];
     const int chunk = (n + (int)gridDim.y - 1) / (int)gridDim.y, t0 = min(n, part * chunk), t1 = min(n, t0 + chunk);
     if (tid == 0 && part == 0) {
-        all.kv_off[b] = off; all.kv_off_cross[b] = b * S_max;
-        msk.kv_off[b] = off; msk.kv_off_cross[b] = b * S_max;
+        all.kv_off[b] = off; all.kv_off_cross[b] = s.src_off[b];
+        msk.kv_off[b] = off; msk.kv_off_cross[b] = s.src_off[b];
         all.q_off[b] = off; all.q_cnt[b] = n;
         msk.q_off[b] = moff; msk.q_cnt[b] = fin ? 0 : k;
         if (b == 0) {
@@ -261,7 +289,7 @@ __global__ void k_draft_prep(Session s, int B, int k, int S_max, int bos, int ma
 // hold yet, c..j of [BOS, committed...], then k [MASK] rows at positions j+1..j+k.  Position p sees keys 0..p when it is
 // a prefix row and every key 0..j+k when it is a [MASK] row.  The last block to finish records the new cache length.
 template <typename T>
-__global__ void k_draft_prep_pc(Session s, int B, int k, int S_max, int bos, int mask, Rows all, Rows msk,
+__global__ void k_draft_prep_pc(Session s, int B, int k, int bos, int mask, Rows all, Rows msk,
                                 const T* __restrict__ E, const float* __restrict__ P, float* __restrict__ x, int d, float scale,
                                 int vocab, int max_pos) {
     __shared__ int red_a[32], red_m[32], tot_a[32], tot_l[32];
@@ -287,8 +315,8 @@ __global__ void k_draft_prep_pc(Session s, int B, int k, int S_max, int bos, int
     const int j = s.len[b], c = min(s.dlen[b], j + 1), n_new = j + 1 - c, n = fin ? 0 : n_new + k, sl = s.src_len[b];
     const int chunk = (n + (int)gridDim.y - 1) / (int)gridDim.y, t0 = min(n, part * chunk), t1 = min(n, t0 + chunk);
     if (tid == 0 && part == 0) {
-        all.kv_off[b] = off; all.kv_off_cross[b] = b * S_max;
-        msk.kv_off[b] = off; msk.kv_off_cross[b] = b * S_max;
+        all.kv_off[b] = off; all.kv_off_cross[b] = s.src_off[b];
+        msk.kv_off[b] = off; msk.kv_off_cross[b] = s.src_off[b];
         all.q_off[b] = off; all.q_cnt[b] = n;
         msk.q_off[b] = moff; msk.q_cnt[b] = fin ? 0 : k;
         if (b == 0) {
@@ -932,31 +960,12 @@ static __global__ void k_commit(Session s, const int* __restrict__ draft, const 
     commit_post(s, post);
 }
 
-static __global__ void k_session_init(Session s, const int* __restrict__ src_len, const int* __restrict__ max_tgt, int B,
-                               int max_tgt_cap, int S_max) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b == 0) {
-        for (int i = 0; i < 4; ++i) s.stats[i] = 0ull;
-    }
-    if (b >= B) return;
-    int mt = max_tgt ? min(max(max_tgt[b], 0), max_tgt_cap) : max_tgt_cap;
-    s.len[b] = 0;
-    s.dlen[b] = 0;
-    if (b == 0) *s.dticket = 0;
-    s.max_tgt[b] = mt;
-    s.finished[b] = (mt <= 0) ? 1 : 0;
-    s.src_len[b] = min(max(src_len[b], 1), S_max);
-}
-
-static __global__ void k_count_active(Session s, int B) {      // one warp
-    int n = 0;
-    for (int b = threadIdx.x; b < B; b += 32) n += s.finished[b] ? 0 : 1;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        s.counters[CNT_ACTIVE] = n;
-        s.counters[CNT_TICKET] = 0;
-        s.counters[CNT_MAXLEN] = 0;
+// The caller's sources, lengths and budgets into the handle's own buffers, in one launch.
+static __global__ void k_stage_inputs(const int* __restrict__ src, const int* __restrict__ len, const int* __restrict__ mt, int n_src, int B,
+                                      int* __restrict__ o_src, int* __restrict__ o_len, int* __restrict__ o_mt) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_src; i += gridDim.x * blockDim.x) {
+        o_src[i] = src[i];
+        if (i < B) { o_len[i] = len[i]; if (mt) o_mt[i] = mt[i]; }
     }
 }
 

@@ -317,6 +317,7 @@ void layout_all(specdec_handle* h) {
     s.finished = (int*)A.take((size_t)h->B_cap * 4);
     s.max_tgt = (int*)A.take((size_t)h->B_cap * 4);
     s.src_len = (int*)A.take((size_t)h->B_cap * 4);
+    s.src_off = (int*)A.take((size_t)h->B_cap * 4);
     s.out_stride = h->T_cap > 0 ? h->T_cap : 1;
     s.out = (int*)A.take((size_t)h->B_cap * s.out_stride * 4);
     s.dlen = (int*)A.take((size_t)h->B_cap * 4);
@@ -409,7 +410,7 @@ cudaError_t launch_pdl(specdec_handle* h, void (*kernel)(KArgs...), dim3 grid, d
 
 // Row count of a pass where the host knows it, else -1 (the kernels read it from the device).
 inline int static_rows(const specdec_handle* h, int cnt, int rows_ub) {
-    return (cnt == CNT_ENC || (cnt == CNT_VERIFY && !(h->fuse_commit && h->B > 1))) ? rows_ub : -1;
+    return (cnt == CNT_VERIFY && !(h->fuse_commit && h->B > 1)) ? rows_ub : -1;
 }
 
 template <typename T>
@@ -741,15 +742,8 @@ int encode_impl(specdec_handle* h, const int* d_src, const int* d_src_len, const
     h->B = B; h->S_max = S_max; h->len_ub = 0; h->act_ub = B;
     h->dnew_ub = 1; h->drafter_pc_session = h->drafter_pc;
     h->encoded = false; h->verified = false; h->drafted = false;
-    k_session_init<<<cdiv(B, 128), 128, 0, st>>>(h->ses, d_src_len, d_max_tgt, B, h->T_cap, S_max);
+    k_enc_prep<<<B, 128, 0, st>>>(h->ses, d_src, d_src_len, d_max_tgt, B, S_max, h->T_cap, h->rows);
     KCHECK(h);
-    k_count_active<<<1, 32, 0, st>>>(h->ses, B);
-    KCHECK(h);
-    {
-        const int R = B * S_max;
-        k_enc_prep<<<cdiv(R, 256), 256, 0, st>>>(d_src, h->ses.src_len, B, S_max, h->rows, h->ses.counters);
-        KCHECK(h);
-    }
     // the two encoders are independent: the drafter's runs on a second stream in its own workspace
     const bool side = h->enc_stream != nullptr;
     cudaStream_t st2 = side ? h->enc_stream : st;
@@ -788,9 +782,9 @@ int draft_impl(specdec_handle* h, int k, int* d_draft, cudaStream_t st) {
     h->fused_x = nullptr;
     // blocks per sequence: enough to fill the machine at small batches, never fewer than two rows a block
     const int parts = std::max(1, std::min(cdiv(592, B), cdiv(h->T_cap + k + 1, 2)));
-    if (pc) CUDA_TRY(h, launch_pdl(h, k_draft_prep_pc<T>, dim3(B, parts), dim3(128), 0, st, h->ses, B, k, h->S_max, h->cfg.bos_id, h->cfg.mask_id, h->rows, h->mrows,
+    if (pc) CUDA_TRY(h, launch_pdl(h, k_draft_prep_pc<T>, dim3(B, parts), dim3(128), 0, st, h->ses, B, k, h->cfg.bos_id, h->cfg.mask_id, h->rows, h->mrows,
                                    (const T*)m.embed, (const float*)m.pos_dec, h->x, d, sqrtf((float)d), m.dm.vocab, m.dm.max_pos));
-    else CUDA_TRY(h, launch_pdl(h, k_draft_prep<T>, dim3(B, parts), dim3(128), 0, st, h->ses, B, k, h->S_max, h->cfg.bos_id, h->cfg.mask_id, h->rows, h->mrows,
+    else CUDA_TRY(h, launch_pdl(h, k_draft_prep<T>, dim3(B, parts), dim3(128), 0, st, h->ses, B, k, h->cfg.bos_id, h->cfg.mask_id, h->rows, h->mrows,
                                 (const T*)m.embed, (const float*)m.pos_dec, h->x, d, sqrtf((float)d), m.dm.vocab, m.dm.max_pos));
     KCHECK(h);
     for (int l = 0; l + 1 < L; ++l) {
@@ -856,7 +850,7 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
     int* keep = (d_draft != h->v_draft && k > 0) ? h->v_draft : nullptr;
     // row metadata and embedding of the block in one kernel
     h->fused_x = nullptr;
-    CUDA_TRY(h, launch_pdl(h, k_verify_prep_embed<T>, dim3(M), dim3(128), 0, st, h->ses, d_draft, B, k, h->S_max, h->cfg.bos_id,
+    CUDA_TRY(h, launch_pdl(h, k_verify_prep_embed<T>, dim3(M), dim3(128), 0, st, h->ses, d_draft, B, k, h->cfg.bos_id,
                            h->rows, (const T*)m.embed, (const float*)m.pos_dec, h->x, d, sqrtf((float)d), m.dm.vocab, m.dm.max_pos, compact ? 1 : 0, keep));
     KCHECK(h);
     for (int l = 0; l < L; ++l) {
@@ -1031,9 +1025,10 @@ template <typename T>
 int encode_staged(specdec_handle* h, const int* d_src, const int* d_src_len, const int* d_max_tgt, int B, int S_max,
                   cudaStream_t st) {
     if (!h->use_graphs || h->profile) return encode_impl<T>(h, d_src, d_src_len, d_max_tgt, B, S_max, st);
-    if (d_src != h->stage_src) CUDA_TRY(h, cudaMemcpyAsync(h->stage_src, d_src, (size_t)B * S_max * 4, cudaMemcpyDeviceToDevice, st));
-    if (d_src_len != h->stage_len) CUDA_TRY(h, cudaMemcpyAsync(h->stage_len, d_src_len, (size_t)B * 4, cudaMemcpyDeviceToDevice, st));
-    if (d_max_tgt && d_max_tgt != h->stage_mt) CUDA_TRY(h, cudaMemcpyAsync(h->stage_mt, d_max_tgt, (size_t)B * 4, cudaMemcpyDeviceToDevice, st));
+    if (d_src != h->stage_src) {
+        k_stage_inputs<<<std::min(cdiv(B * S_max, 256), 64), 256, 0, st>>>(d_src, d_src_len, d_max_tgt, B * S_max, B, h->stage_src, h->stage_len, h->stage_mt);
+        KCHECK(h);
+    }
     h->B = B; h->S_max = S_max; h->act_ub = B;
     h->drafter_pc_session = h->drafter_pc;
     TRY(graph_call(h, {5, d_max_tgt ? 1 : 0}, st, [&]() {
