@@ -25,6 +25,7 @@
 #include "gemm_tc_splitk.cuh"
 #include "kernels.cuh"
 #include "mma_rate.cuh"
+#include "rows_f32.cuh"
 #include "rows_gemm.cuh"
 
 using namespace sd;
@@ -439,8 +440,10 @@ int ln_or_fused(specdec_handle* h, const float* x, const float* g, const float* 
 // Where the K and V columns of a fused QKV projection go (the verifier's paged cache).
 struct KvDest { const int* seq; const int* pos; void* kc; void* vc; int d; };
 
-template <typename T> bool tc_usable(const specdec_handle* h, int N, int K) {
-    return std::is_same<T, bf16>::value && h->use_tc && sd::tc_supported(N, K);
+// Whether the QKV projection of a pass stores K and V in the paged cache itself.
+template <typename T> bool kv_in_gemm(const specdec_handle* h, int d, int rows_ub) {
+    if (std::is_same<T, float>::value) return h->use_skinny && rf_supported(EPI_QKV, 3 * d, d, d, rows_ub);
+    return h->use_tc && sd::tc_supported(3 * d, d) && d % 32 == 0;
 }
 
 // LayerNorm fused in front of a GEMM: x fp32 rows, gain, bias.
@@ -477,7 +480,9 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
     const bool few = std::is_same<T, bf16>::value && h->use_skinny && h->use_tc && rows_ub <= (cnt == CNT_ENC ? (h->enc_skinny ? RG_MAX_ROWS_ENC : 0) : RG_MAX_ROWS) &&
                      !(epi == EPI_RESID && h->use_ln_fuse) && rg_supported(epi, N, K, lnp ? K : lda, rows_ub, h->use_sk_cluster != 0);
     const bool ln_inside = few && lnp && rows_ub <= RG_LN_ROWS && rg_ln_width(K);
-    if (lnp && !ln_inside) {           // separate normalisation launch, then a plain GEMM on its output
+    const bool few32 = std::is_same<T, float>::value && h->use_skinny && rf_supported(epi, N, K, lnp ? K : lda, rows_ub);
+    const bool ln32 = few32 && lnp && rf_ln_width(K);
+    if (lnp && !ln_inside && !ln32) {  // separate normalisation launch, then a plain GEMM on its output
         TRY(ln_or_fused<T>(h, lnp->x, lnp->g, lnp->b, cnt, rows_ub, h->y, K, st));
         A = h->y; lda = K;
     }
@@ -532,6 +537,16 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
         }
     }
     if (n_tiles_out) *n_tiles_out = g.n_tiles;
+    if constexpr (std::is_same<T, float>::value) {
+        if (few32) {
+            if (ln32 && epi == EPI_STATS) g.ln_out = (T*)h->y;     // specdec_debug_logits replays the projection from there
+            RowsF32Args ra{g, ln32 ? lnp->x : nullptr, ln32 ? lnp->g : nullptr, ln32 ? lnp->b : nullptr, 1e-5f};
+            const cudaError_t e = rf_launch(epi, ra, rows_ub, h->use_pdl, st);
+            if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("row GEMM launch: ") + cudaGetErrorString(e));
+            KCHECK(h);
+            return 0;
+        }
+    }
     dim3 grid(cdiv(N, 64), cdiv(rows_ub, 64));
     switch (epi) {
         case EPI_STORE: k_gemm_simt<T, EPI_STORE><<<grid, 256, 0, st>>>(g); break;
@@ -583,6 +598,21 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             // queries: 273 against 265 us a draft step).
             const bool tall = h->attn_stream == 1 ? 8LL * ((q_ub + 63) / 64 * 64) <= 9LL * ((q_ub + 31) / 32 * 32) : h->attn_stream == 2;
             return tall ? ATTN_GO(4, 1, 64, 3) : ATTN_GO(2, 1, 64, 3);
+        }
+    }
+    if constexpr (std::is_same<T, float>::value) {
+        if (h->use_tc_attn && af_supported(d_head, max_keys)) {
+            AttnF32Args a;
+            a.q = (const float*)q; a.q_stride = q_stride; a.q_index = q_index;
+            a.k = (const float*)k; a.v = (const float*)v; a.kv_stride = kv_stride; a.kv_off = kv_off;
+            a.pg.table = h->page_table; a.pg.page_tokens = h->cfg.page_tokens; a.pg.max_pages = h->pages_per_seq;
+            a.q_off = r.q_off; a.q_cnt = r.q_cnt; a.nkeys = nkeys; a.pre_keys = h->use_pdl ? pre_keys : nullptr;
+            a.out = (float*)out; a.out_stride = out_stride; a.max_keys = max_keys; a.d_head = d_head;
+            a.scale = 1.0f / sqrtf((float)d_head);
+            const cudaError_t e = af_launch(paged, a, q_ub, n_heads, h->B, h->use_pdl, st);
+            if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
+            KCHECK(h);
+            return 0;
         }
     }
     AttnArgs<T> a;
@@ -647,7 +677,7 @@ int block_self(specdec_handle* h, const ModelW& m, const LayerW& w, float* x, co
     const size_t e = h->esz;
     const bool verify = kc != nullptr;
     const LnSpec l1{x, w.ln1_g, w.ln1_b};
-    if (verify && tc_usable<T>(h, 3 * d, d) && d % 32 == 0) {
+    if (verify && kv_in_gemm<T>(h, d, rows_ub)) {
         // K and V columns leave the GEMM epilogue straight into the paged cache
         KvDest kv{r.seq, r.pos, kc, vc, d};
         TRY(gemm<T>(h, EPI_QKV, h->y, d, w.qkv_w, w.qkv_b, 3 * d, d, cnt, rows_ub, h->qkv, 3 * d, nullptr, st, nullptr,
@@ -796,7 +826,7 @@ int draft_impl(specdec_handle* h, int k, int* d_draft, cudaStream_t st) {
     // last layer: K/V from every row, queries and everything after them from the k mask rows only
     const LayerW& w = m.dec[L - 1];
     const LnSpec l1{h->x, w.ln1_g, w.ln1_b};
-    const bool scatter_in_gemm = pc && tc_usable<T>(h, 3 * d, d) && d % 32 == 0;
+    const bool scatter_in_gemm = pc && kv_in_gemm<T>(h, d, R1);
     if (scatter_in_gemm) {
         KvDest kv{h->rows.seq, h->rows.pos, h->dkc[L - 1], h->dvc[L - 1], d};
         TRY(gemm<T>(h, EPI_QKV, h->y, d, w.qkv_w, w.qkv_b, 3 * d, d, CNT_DRAFT_ALL, R1, h->qkv, 3 * d, nullptr, st, nullptr,
@@ -823,10 +853,10 @@ int draft_impl(specdec_handle* h, int k, int* d_draft, cudaStream_t st) {
     TRY(gemm<T>(h, EPI_RESID, h->att, d, w.o_w, w.o_b, d, d, CNT_DRAFT_MASK, R2, nullptr, 0, h->x2, st));
     TRY(block_cross<T>(h, m, w, h->x2, h->mrows, CNT_DRAFT_MASK, R2, k, L - 1, st));
     TRY(block_ffn<T>(h, m, w, h->x2, CNT_DRAFT_MASK, R2, st, m.dec_lnf_g, m.dec_lnf_b));
-    TRY(ln_or_fused<T>(h, h->x2, m.dec_lnf_g, m.dec_lnf_b, CNT_DRAFT_MASK, R2, h->y, d, st));
+    const LnSpec lf{h->x2, m.dec_lnf_g, m.dec_lnf_b};
     int n_tiles = 0;
     TRY(gemm<T>(h, EPI_STATS, h->y, d, m.embed, nullptr, m.dm.vocab, d, CNT_DRAFT_MASK, R2, nullptr, 0, nullptr, st,
-                nullptr, nullptr, &n_tiles));
+                nullptr, nullptr, &n_tiles, nullptr, &lf));
     CUDA_TRY(h, launch_pdl(h, k_draft_argmax, dim3(cdiv(R2, 4)), dim3(128), 0, st, (const RowPart*)h->part, n_tiles,
                            (const int*)(h->ses.counters + CNT_DRAFT_MASK), (const int*)h->mrows.slot, d_draft,
                            (const int*)(h->script_on ? h->script : nullptr), h->T_cap + h->k_cap, (const int*)h->ses.len, k));
@@ -862,13 +892,13 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
                          last ? m.dec_lnf_b : m.dec[l + 1].ln1_b));
     }
     const bool ln_pending = !(h->x == h->fused_x && m.dec_lnf_g == h->fused_g && h->y == h->fused_out);
-    if (ln_pending && d % 128 == 0 && d <= 1024 && !(h->diag_repeat & 2)) {
+    if (ln_pending && d <= 1024 && !(h->diag_repeat & 2)) {
         // final LayerNorm and the pre-pass logit of every row's draft in one kernel
         cudaError_t e = cudaSuccess;
         const dim3 grid(cdiv(M, 8)), block(256);
 #define LN_LD(NC) e = launch_pdl(h, k_layernorm_ld<T, NC>, grid, block, 0, st, (const float*)h->x, (const float*)m.dec_lnf_g, (const float*)m.dec_lnf_b, (T*)h->y, d, 1e-5f, \
                                  (const T*)m.embed, d_draft, (const int*)h->rows.slot_seq, (const int*)(h->ses.counters + CNT_VERIFY), k, m.dm.vocab, h->ld, h->ld_id)
-        switch (d / 128) {
+        switch (cdiv(d, 128)) {
             case 1: LN_LD(1); break; case 2: LN_LD(2); break; case 3: LN_LD(3); break; case 4: LN_LD(4); break;
             case 5: LN_LD(5); break; case 6: LN_LD(6); break; case 7: LN_LD(7); break; default: LN_LD(8); break;
         }
@@ -887,8 +917,8 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
                 h->ld_id, &n_tiles));
     prof_mark(h, st);
     FusedCommit fc{h->ses, h->v_draft, h->cfg.eos_id, h->h_post, h->fuse_commit ? 1 : 0};
-    CUDA_TRY(h, launch_pdl(h, k_accept, dim3(slots), dim3(1024), (size_t)(k + 1) * sizeof(RowPart), st, (const RowPart*)h->part, n_tiles,
-                           (const float*)h->ld, (const int*)h->ld_id, k, beta, tau, h->accepted, h->bif, d_accepted, d_bif, h->row_stats, h->want_lse, (const int*)h->rows.slot_seq, fc));
+    CUDA_TRY(h, launch_pdl(h, k_accept, dim3(slots), dim3(32 * std::min(32, std::max(k + 1, 4))), (size_t)(k + 1) * sizeof(RowPart), st, (const RowPart*)h->part, n_tiles,
+                           (const float*)h->ld, (const int*)h->ld_id, k, beta, tau, h->accepted, h->bif, d_accepted, d_bif, h->fuse_commit ? nullptr : h->row_stats, h->want_lse, (const int*)h->rows.slot_seq, fc));
     KCHECK(h);
     h->commit_done = h->fuse_commit;
     h->last_k = k; h->verified = true; h->drafted = false;
