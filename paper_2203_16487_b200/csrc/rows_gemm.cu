@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(RG_THREADS, NC > 4 ? 2 : 3) k_rows(RowsArgs a)
         // A: rows lane % 16, k half lane / 16.  B: with two column tiles, rows (lane & 7) + 8 (lane >> 4), k half (lane >> 3) & 1
         uint32_t ap = As + (lane & 15) * pitch + wk * steps * 32 + (lane >> 4) * 16;
         uint32_t bp = Ws + (wn * TN * 8 + (lane & 7) + (TN > 1 ? (lane >> 4) * 8 : 0)) * pitch + wk * steps * 32 + ((lane >> 3) & 1) * 16;
-#pragma unroll 2
+#pragma unroll 8
         for (int s = 0; s < steps; ++s, ap += 32, bp += 32) {
             uint32_t af[MT][4], bf[TN][2];
 #pragma unroll

@@ -565,7 +565,7 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
 template <typename T>
 int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const int* q_index, const void* k, const void* v,
          int kv_stride, const int* kv_off, const Rows& r, const int* nkeys, int cnt, int rows_ub, int q_ub, void* out,
-         int out_stride, int n_heads, int d_head, int max_keys, cudaStream_t st, const int* pre_keys = nullptr) {
+         int out_stride, int n_heads, int d_head, int max_keys, cudaStream_t st, const int* pre_keys = nullptr, const QueryArgs* qp = nullptr) {
     if (rows_ub <= 0) return 0;
     if constexpr (std::is_same<T, bf16>::value) {
         if (h->use_tc_attn && d_head == 64) {
@@ -577,14 +577,29 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             a.out = (bf16*)out; a.out_stride = out_stride; a.max_keys = max_keys;
             a.scale = 1.0f / sqrtf((float)d_head);
             const int n_seq = cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub);
+            QueryArgs qa{};
+            if (qp) {
+                qa = *qp;
+                auto goq = [&](auto* kernel, int bytes) {
+                    const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, 16), n_heads, h->B), dim3(256), AttnCfg<1, 8, 16>::smem(max_keys, 3, false, bytes), st, a, qa);
+                    if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
+                    KCHECK(h);
+                    return 0;
+                };
+                switch (n_heads) {                           // (64-wide heads: the width is 64 n_heads)
+                    case 4: return goq(k_attn<false, 1, 8, 16, 3, 2>, QueryCfg<2>::OPS);
+                    case 8: return goq(k_attn<false, 1, 8, 16, 3, 4>, QueryCfg<4>::OPS);
+                    default: return goq(k_attn<false, 1, 8, 16, 3, 6>, QueryCfg<6>::OPS);
+                }
+            }
             auto go = [&](auto* kernel, int bm, int warps, size_t smem) {
-                const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, bm), n_heads, h->B), dim3(warps * 32), smem, st, a);
+                const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, bm), n_heads, h->B), dim3(warps * 32), smem, st, a, qa);
                 if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
                 KCHECK(h);
                 return 0;
             };
-#define ATTN_GO(MT, KG, KW, NS) (paged ? go(k_attn<true, MT, KG, KW, NS>, 16 * MT, MT * KG, AttnCfg<MT, KG, KW>::smem(max_keys, NS)) \
-                                       : go(k_attn<false, MT, KG, KW, NS>, 16 * MT, MT * KG, AttnCfg<MT, KG, KW>::smem(max_keys, NS)))
+#define ATTN_GO(MT, KG, KW, NS) (paged ? go(k_attn<true, MT, KG, KW, NS>, 16 * MT, MT * KG, AttnCfg<MT, KG, KW>::smem(max_keys, NS, true)) \
+                                       : go(k_attn<false, MT, KG, KW, NS>, 16 * MT, MT * KG, AttnCfg<MT, KG, KW>::smem(max_keys, NS, false)))
             // While 16-query tiles are at most four CTAs per SM the keys are spread over the warps of a CTA: four, or eight when the
             // keys are many and the CTAs fewer than SMs (verify step of 11 rows over 511 keys: 192 us with four, 180 with eight).
             const long long tiles16 = (long long)cdiv(q_ub, 16) * n_heads * n_seq;
@@ -637,12 +652,12 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
 template <typename T>
 int attn(specdec_handle* h, bool paged, const void* q, int q_stride, const int* q_index, const void* k, const void* v,
          int kv_stride, const int* kv_off, const Rows& r, const int* nkeys, int cnt, int rows_ub, int q_ub, void* out,
-         int out_stride, int n_heads, int d_head, int max_keys, cudaStream_t st, const int* pre_keys = nullptr) {
+         int out_stride, int n_heads, int d_head, int max_keys, cudaStream_t st, const int* pre_keys = nullptr, const QueryArgs* qp = nullptr) {
     TRY(attn_once<T>(h, paged, q, q_stride, q_index, k, v, kv_stride, kv_off, r, nkeys, cnt, rows_ub, q_ub, out, out_stride,
-                     n_heads, d_head, max_keys, st, pre_keys));
+                     n_heads, d_head, max_keys, st, pre_keys, qp));
     if (h->diag_repeat & 1)
         TRY(attn_once<T>(h, paged, q, q_stride, q_index, k, v, kv_stride, kv_off, r, nkeys, cnt, rows_ub, q_ub, out, out_stride,
-                         n_heads, d_head, max_keys, st, pre_keys));
+                         n_heads, d_head, max_keys, st, pre_keys, qp));
     return 0;
 }
 
@@ -704,16 +719,26 @@ int block_self(specdec_handle* h, const ModelW& m, const LayerW& w, float* x, co
     return 0;
 }
 
+// Whether the cross-attention kernel projects its queries itself: while its CTAs (16 queries of a head with the head's 64 rows of Wq, over 100 KB
+// of shared memory) fill the SMs once, or twice over at most 128 keys (verify step of 208 rows 262 / 241 us, 416 rows 364 / 358; 832 rows 396 / 453).
+bool query_inside(const specdec_handle* h, int d, int d_head, int q_ub, int n_heads, int max_keys) {
+    return h->use_tc && h->use_skinny && h->use_tc_attn && !h->use_ln_fuse && d_head == 64 && rg_ln_width(d) &&
+           (long long)cdiv(q_ub, 16) * n_heads * std::min(h->B, h->act_ub) <= (max_keys <= 128 ? 2 : 1) * h->tma.n_sm;
+}
+
 template <typename T>
 int block_cross(specdec_handle* h, const ModelW& m, const LayerW& w, float* x, const Rows& r, int cnt, int rows_ub,
                 int q_ub, int layer, cudaStream_t st) {
     const int d = m.dm.d_model, H = m.dm.n_heads, dh = d / H;
     const size_t e = h->esz;
     const LnSpec lc{x, w.lnc_g, w.lnc_b};
-    TRY(gemm<T>(h, EPI_STORE, h->y, d, w.cq_w, w.cq_b, d, d, cnt, rows_ub, h->q, d, nullptr, st, nullptr, nullptr, nullptr,
-                nullptr, &lc));
+    QueryArgs qa{};
+    const bool inside = std::is_same<T, bf16>::value && query_inside(h, d, dh, q_ub, H, h->S_max);
+    if (inside) qa = QueryArgs{x, w.lnc_g, w.lnc_b, 1e-5f, (const bf16*)w.cq_w, w.cq_b};
+    else TRY(gemm<T>(h, EPI_STORE, h->y, d, w.cq_w, w.cq_b, d, d, cnt, rows_ub, h->q, d, nullptr, st, nullptr, nullptr, nullptr,
+                     nullptr, &lc));
     TRY(attn<T>(h, false, h->q, d, nullptr, m.ckv[layer], (char*)m.ckv[layer] + (size_t)d * e, m.ckv_stride, r.kv_off_cross,
-                r, r.nk_cross, cnt, rows_ub, q_ub, h->att, d, H, dh, h->S_max, st, h->ses.src_len));   // encoder K/V: all of it
+                r, r.nk_cross, cnt, rows_ub, q_ub, h->att, d, H, dh, h->S_max, st, h->ses.src_len, inside ? &qa : nullptr));   // encoder K/V: all of it
     h->next_ln = {w.ln2_g, w.ln2_b, h->y};           // the feed-forward sublayer's LayerNorm comes next
     TRY(gemm<T>(h, EPI_RESID, h->att, d, w.co_w, w.co_b, d, d, cnt, rows_ub, nullptr, 0, x, st));
     return 0;
@@ -1477,7 +1502,8 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
             if (smem > 227 * 1024 - 2048) h->use_tc_attn = 0;
             else if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048);
         };
-#define ATTN_ROOM(MT, KG, KW, NS) room(k_attn<true, MT, KG, KW, NS>, AttnCfg<MT, KG, KW>::smem(max_keys, NS)); room(k_attn<false, MT, KG, KW, NS>, AttnCfg<MT, KG, KW>::smem(max_keys, NS))
+#define ATTN_ROOM(MT, KG, KW, NS) room(k_attn<true, MT, KG, KW, NS>, AttnCfg<MT, KG, KW>::smem(max_keys, NS, true)); room(k_attn<false, MT, KG, KW, NS>, 0)
+        room(k_attn<false, 1, 8, 16, 3, 2>, 0); room(k_attn<false, 1, 8, 16, 3, 4>, 0); room(k_attn<false, 1, 8, 16, 3, 6>, 0);   // (at most 222 KB: no table of rows)
         ATTN_ROOM(1, 4, 32, 3); ATTN_ROOM(1, 8, 32, 2); ATTN_ROOM(4, 1, 64, 3); ATTN_ROOM(2, 1, 64, 3);
         if (e != cudaSuccess) { cudaGetLastError(); h->use_tc_attn = 0; }
         if (sd::tc_init(h->tma, h->ses.counters + 7) != 0) h->use_tc = 0;     // reported through specdec_last_error; SIMT GEMM still runs on the GPU

@@ -47,3 +47,21 @@ def test_attention_edges(opts, lens, k):
         for i in range(k):
             assert g[b, i] == logits[i].argmax() or logits[i].max() - logits[i, g[b, i]] < 2e-2, (b, i)
     sd.close()
+
+
+@pytest.mark.parametrize("d,f,B,k,S", [(256, 256, 1, 15, 12), (512, 128, 3, 16, 130), (768, 128, 2, 31, 400)])
+def test_queries_projected_inside_the_attention(d, f, B, k, S):
+    """Cross-attention of few rows: one and two 16-row tiles with a ragged end, key rings of one stage and more, the three widths."""
+    from paper_2203_16487_b200 import binding
+    V = 515
+    dims = W.ModelDims(d, d // 64, f, V, 1, 1, 512)
+    wv, wd = W.make_weights(dims, 81, True), W.make_weights(dims, 82, True)
+    mv, md = O.model_from(dims, wv, mode="bf16"), O.model_from(dims, wd, mode="bf16")
+    rng = np.random.default_rng(d)
+    srcs = [W.zipf_ids(rng, n, V) for n in ([S] + [max(S // 2, 1), 7])[:B]]
+    sd = binding.SpecDec(dims, wv, dims, wd, k_max=k, max_batch=B, max_src=S, max_tgt=40, bf16=True)
+    sd.set_option("debug_checks", 1)
+    rep = lockstep.run(sd, mv, md, srcs, [40] * B, k, 3, 1.0, margin=1e-3, check_logits_every=1, max_iters=2)
+    assert rep.ok, rep.notes
+    assert rep.max_logit_err < 2e-2 and rep.max_stat_err < 2e-2
+    sd.close()
