@@ -59,6 +59,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         }
     }
 }
+// The same for a converged warp: every lane gets the same answer, as an elected instruction behind it needs all of them there.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err_word, int code) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, err_word, code));
+}
 constexpr int TC_BM = 128, TC_BK = 64;
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, uint32_t bar) {
     asm volatile(
@@ -80,6 +84,15 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint6
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
+}
+// One lane of a converged warp.  The threads that feed the tensor pipe run their loops as whole warps and elect a lane only around
+// the instructions themselves: barrier addresses, descriptors and loop counters then stay in uniform registers, where tcgen05.mma and
+// the TMA take them.  (A loop inside `if (lane == 0)` moves every operand over before every instruction: a 128 x 256 k-block then
+// took 0.44 us instead of 0.33, the verify step of 3328 rows 636 us instead of 563.)
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t pred;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
+    return pred;
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -254,17 +267,18 @@ __device__ __forceinline__ void tc_epilogue_tile(const GemmArgs<bf16>& g, int R,
     float ln_s1[8], ln_s2[8];                        // LNF: per pass, sum and sum of squares of row 4 ps + lane / 8 over this lane's columns
 #pragma unroll
     for (int ps = 0; ps < 8; ++ps) { ln_s1[ps] = 0.f; ln_s2[ps] = 0.f; }
-    // ... and so are this lane's bias columns, its cache row and its draft logit
-    float4 bzv[NCH][2];
+    // ... and so are this lane's bias columns (bf16 outputs: the warp's, into its buffer), its cache row and its draft logit
+    float4 bzv[bf_out ? 1 : NCH];
+    float* bias_s = stg + 512;
     if (EPI != EPI_STATS && vec_ok && g.bias) {
+        if (bf_out) {
 #pragma unroll
-        for (int c = 0; c < NCH; ++c) {
-            const int nb = n0 + c * CW;
-            if (nb + CW <= g.N) {
-                const float4* bp = reinterpret_cast<const float4*>(g.bias + nb);
-                if (bf_out) { bzv[c][0] = __ldg(bp + 2 * (lane & 3)); bzv[c][1] = __ldg(bp + 2 * (lane & 3) + 1); }
-                else bzv[c][0] = __ldg(bp + (lane & 7));
-            }
+            for (int c = 0; c < NCH; ++c) bias_s[c * 32 + lane] = n0 + c * 32 + lane < g.N ? __ldg(g.bias + n0 + c * 32 + lane) : 0.f;
+            __syncwarp();
+        } else {
+#pragma unroll
+            for (int c = 0; c < NCH; ++c)
+                if (n0 + c * CW + CW <= g.N) bzv[c] = __ldg(reinterpret_cast<const float4*>(g.bias + n0 + c * CW) + (lane & 7));
         }
     }
     long long my_cache_row = 0;                          // EPI_QKV: cache row of this lane's output row
@@ -324,6 +338,9 @@ __device__ __forceinline__ void tc_epilogue_tile(const GemmArgs<bf16>& g, int R,
         }
         if (r < R) g.part[(size_t)r * g.n_tiles + n_tile * 2 + half] = p;
     } else if (warp_live) {
+        // (bf16 outputs: the next chunk's tensor-memory load runs under this chunk's arithmetic)
+        uint32_t vr[2][bf_out ? CW : 1];
+        if constexpr (bf_out) tmem_ld_issue<CW>(trow, vr[0]);
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
             const int nb = n0 + c * CW;
@@ -334,20 +351,47 @@ __device__ __forceinline__ void tc_epilogue_tile(const GemmArgs<bf16>& g, int R,
                     xin[c & 1][ps] = gr < R ? *reinterpret_cast<const float4*>(g.resid + (size_t)gr * g.N + nb + (lane & 7) * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }
-            tmem_ld<CW>(trow + c * CW, v);
+            if constexpr (bf_out) {
+                tmem_ld_done<CW>(vr[c & 1]);
+                if (c + 1 < NCH) tmem_ld_issue<CW>(trow + (c + 1) * CW, vr[(c + 1) & 1]);
+#pragma unroll
+                for (int j = 0; j < CW; ++j) v[j] = __uint_as_float(vr[c & 1][j]);
+            } else {
+                tmem_ld<CW>(trow + c * CW, v);
+            }
             if (CW == 32 && vec_ok && nb + CW <= g.N) {
                 // Transpose through shared memory: a thread owns one output ROW in tensor memory, but global
                 // memory wants neighbouring lanes on neighbouring addresses.  The 32 x 32 block is written row-wise
                 // with its 16-byte chunks XOR-swizzled by the row, then read back 16 bytes of output per lane.
-                float* srow = stg + lane * 32;
+                // bf16 outputs are finished (bias, activation, rounding) before the transpose: half the shared-memory traffic.
+                if (!bf_out) {
+                    float* srow = stg + lane * 32;
 #pragma unroll
-                for (int j4 = 0; j4 < 8; ++j4)
-                    *reinterpret_cast<float4*>(srow + ((j4 ^ (lane & 7)) << 2)) = make_float4(v[j4 * 4], v[j4 * 4 + 1], v[j4 * 4 + 2], v[j4 * 4 + 3]);
+                    for (int j4 = 0; j4 < 8; ++j4)
+                        *reinterpret_cast<float4*>(srow + ((j4 ^ (lane & 7)) << 2)) = make_float4(v[j4 * 4], v[j4 * 4 + 1], v[j4 * 4 + 2], v[j4 * 4 + 3]);
+                } else {
+#pragma unroll
+                    for (int j8 = 0; j8 < 4; ++j8) {
+                        float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
+                        if (g.bias) { b0 = *reinterpret_cast<const float4*>(bias_s + c * 32 + j8 * 8); b1 = *reinterpret_cast<const float4*>(bias_s + c * 32 + j8 * 8 + 4); }
+                        float y[8] = {v[j8 * 8] + b0.x, v[j8 * 8 + 1] + b0.y, v[j8 * 8 + 2] + b0.z, v[j8 * 8 + 3] + b0.w,
+                                      v[j8 * 8 + 4] + b1.x, v[j8 * 8 + 5] + b1.y, v[j8 * 8 + 6] + b1.z, v[j8 * 8 + 7] + b1.w};
+                        uint32_t pk[4];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            if (EPI == EPI_RELU) y[e] = fmaxf(y[e], 0.f);
+                            if (EPI == EPI_GELU) y[e] = ffn_act(y[e], 1);
+                        }
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) { __nv_bfloat162 h2 = __floats2bfloat162_rn(y[2 * e], y[2 * e + 1]); pk[e] = *reinterpret_cast<uint32_t*>(&h2); }
+                        *reinterpret_cast<uint4*>(reinterpret_cast<char*>(stg) + lane * 64 + ((j8 ^ ((lane >> 1) & 3)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    }
+                }
                 __syncwarp();
                 if (!bf_out) {
                     // fp32 rows: 8 lanes per row (4 columns each), 4 rows per pass
                     const int l8 = lane & 7, rsub = lane >> 3;
-                    const float4 bz = g.bias ? bzv[c][0] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const float4 bz = g.bias ? bzv[bf_out ? 0 : c] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                     for (int ps = 0; ps < 8; ++ps) {
                         const int rr = ps * 4 + rsub, gr = rbase + rr;
@@ -363,35 +407,17 @@ __device__ __forceinline__ void tc_epilogue_tile(const GemmArgs<bf16>& g, int R,
                 } else {
                     // bf16 rows: 4 lanes per row (8 columns = 16 bytes each), 8 rows per pass
                     const int c4 = lane & 3, rsub = lane >> 2;
-                    float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
-                    if (g.bias) { b0 = bzv[c][0]; b1 = bzv[c][1]; }
 #pragma unroll
                     for (int ps = 0; ps < 4; ++ps) {
                         const int rr = ps * 8 + rsub, gr = rbase + rr;
                         const long long row_of = (EPI == EPI_QKV) ? __shfl_sync(0xffffffffu, my_cache_row, rr) : 0;
-                        float4 a0 = *reinterpret_cast<const float4*>(stg + rr * 32 + (((2 * c4) ^ (rr & 7)) << 2));
-                        float4 a1 = *reinterpret_cast<const float4*>(stg + rr * 32 + (((2 * c4 + 1) ^ (rr & 7)) << 2));
-                        a0.x += b0.x; a0.y += b0.y; a0.z += b0.z; a0.w += b0.w;
-                        a1.x += b1.x; a1.y += b1.y; a1.z += b1.z; a1.w += b1.w;
-                        if (EPI == EPI_RELU) {
-                            a0.x = fmaxf(a0.x, 0.f); a0.y = fmaxf(a0.y, 0.f); a0.z = fmaxf(a0.z, 0.f); a0.w = fmaxf(a0.w, 0.f);
-                            a1.x = fmaxf(a1.x, 0.f); a1.y = fmaxf(a1.y, 0.f); a1.z = fmaxf(a1.z, 0.f); a1.w = fmaxf(a1.w, 0.f);
-                        }
-                        if (EPI == EPI_GELU) {
-                            a0.x = ffn_act(a0.x, 1); a0.y = ffn_act(a0.y, 1); a0.z = ffn_act(a0.z, 1); a0.w = ffn_act(a0.w, 1);
-                            a1.x = ffn_act(a1.x, 1); a1.y = ffn_act(a1.y, 1); a1.z = ffn_act(a1.z, 1); a1.w = ffn_act(a1.w, 1);
-                        }
+                        const uint4 pk = *reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(stg) + rr * 64 + ((c4 ^ ((rr >> 1) & 3)) << 4));
                         if (gr < R) {
                             bf16* o = g.out + (size_t)gr * g.ldo + nb;
                             if (EPI == EPI_QKV && nb >= g.kv_d) {          // K or V part: straight into the paged cache
                                 const size_t row = (size_t)row_of;
                                 o = (nb < 2 * g.kv_d ? g.kc + row * g.kv_d + (nb - g.kv_d) : g.vc + row * g.kv_d + (nb - 2 * g.kv_d));
                             }
-                            __nv_bfloat162 p0 = __floats2bfloat162_rn(a0.x, a0.y), p1 = __floats2bfloat162_rn(a0.z, a0.w);
-                            __nv_bfloat162 p2 = __floats2bfloat162_rn(a1.x, a1.y), p3 = __floats2bfloat162_rn(a1.z, a1.w);
-                            uint4 pk;
-                            pk.x = *reinterpret_cast<uint32_t*>(&p0); pk.y = *reinterpret_cast<uint32_t*>(&p1);
-                            pk.z = *reinterpret_cast<uint32_t*>(&p2); pk.w = *reinterpret_cast<uint32_t*>(&p3);
                             *reinterpret_cast<uint4*>(o + c4 * 8) = pk;
                         }
                     }
@@ -478,7 +504,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     __shared__ float ln_mr_s[LNF ? TC_BM * 2 : 1];                   // [row][mean, 1 / std]
     __shared__ __align__(8) uint64_t bar_ln;                         // LNF: counts the peers' statistics as they arrive
     const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int nkb = g.K / TC_BK;
     float* stg = reinterpret_cast<float*>(smem_raw + (tiles - smem_u32(smem_raw)) + STAGES * Cfg::STAGE_BYTES) + (warp >= 2 ? warp - 2 : 0) * 1024;
 
@@ -504,81 +530,67 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         __syncthreads();
     }
     tc_fence_after();
-    const uint32_t tmem_d = tmem_base_s;
+    const uint32_t tmem_d = __shfl_sync(0xffffffffu, tmem_base_s, 0);
     volatile int* abort_flag = &abort_s;
-    if (threadIdx.x == 0 && tmem_d != 0xffffffffu) tc_stamp(g.trace, 1);   // (the test pins the stamp behind the read)
-    int pre = 0;                                       // stages whose weight half was requested before the wait
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0) tc_stamp(g.trace, 1);
+    const uint32_t full0 = smem_u32(&bar_full[0]), empty0 = smem_u32(&bar_empty[0]);
+    const int pre = min(STAGES, nkb);                  // stages whose weight half is requested before the wait
+    if (warp == 0) {
         const int n0 = (LNF ? (int)blockIdx.x % n_tiles : (int)blockIdx.x / m_tiles) * BN;
-        for (; pre < STAGES && pre < nkb; ++pre) {
-            const uint32_t bar = smem_u32(&bar_full[pre]);
-            mbar_expect_tx(bar, Cfg::STAGE_BYTES);
-            tma_load_2d(tiles + pre * Cfg::STAGE_BYTES + A_BYTES, &tmW, pre * TC_BK, n0, bar);
-        }
+        for (int st = 0; st < pre; ++st)
+            if (elect_one()) {
+                mbar_expect_tx(full0 + 8 * st, Cfg::STAGE_BYTES);
+                tma_load_2d(tiles + st * Cfg::STAGE_BYTES + A_BYTES, &tmW, st * TC_BK, n0, full0 + 8 * st);
+            }
     }
     pdl_launch_dependents();
     pdl_wait();                                        // activations, residual and outputs belong to the predecessors until here
+    if (threadIdx.x == 0) tc_stamp(g.trace, 2);
 
     if (warp == 0) {
-        if (lane == 0) {
-            int kbi = 0;                               // k-blocks issued so far, over all tiles
-            // ring position kept incrementally and the abort flag read only when a wait gave up: this thread's own
-            // instructions are part of every stage's turnaround (freed -> requested again)
-            int ps = 0; uint32_t ppar = 0; bool wrapped = false, dead = false;
-            for (int t = blockIdx.x; t < total && !dead && !*abort_flag; t += gridDim.x) {
-                const int m0 = (LNF ? t / n_tiles : t % m_tiles) * TC_BM, n0 = (LNF ? t % n_tiles : t / m_tiles) * BN;
-                for (int kb = 0; kb < nkb; ++kb, ++kbi) {
-                    if (wrapped && !mbar_wait(smem_u32(&bar_empty[ps]), ppar, abort_flag, err_word, 1)) { dead = true; break; }
-                    const uint32_t a_dst = tiles + ps * Cfg::STAGE_BYTES, w_dst = a_dst + A_BYTES;
-                    const uint32_t bar = smem_u32(&bar_full[ps]);
+        int kbi = 0, ps = 0; uint32_t ppar = 1; bool ok = true;          // (a fresh barrier counts as past the phase before its first)
+        for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+            const int m0 = (LNF ? t / n_tiles : t % m_tiles) * TC_BM, n0 = (LNF ? t % n_tiles : t / m_tiles) * BN;
+            for (int kb = 0; kb < nkb; ++kb, ++kbi) {
+                ok = mbar_wait_warp(empty0 + 8 * ps, ppar, abort_flag, err_word, 1);
+                if (!ok) break;
+                const uint32_t a_dst = tiles + ps * Cfg::STAGE_BYTES, bar = full0 + 8 * ps;
+                if (elect_one()) {
                     if (kbi >= pre) {
                         mbar_expect_tx(bar, Cfg::STAGE_BYTES);
-                        tma_load_2d(w_dst, &tmW, kb * TC_BK, n0, bar);
+                        tma_load_2d(a_dst + A_BYTES, &tmW, kb * TC_BK, n0, bar);
                     }
                     tma_load_2d(a_dst, &tmA, kb * TC_BK, m0, bar);
-                    if (++ps == STAGES) { ps = 0; if (wrapped) ppar ^= 1u; wrapped = true; }
                 }
+                if (++ps == STAGES) { ps = 0; ppar ^= 1u; }
             }
-            tc_stamp(g.trace, 3);
         }
+        if (lane == 0) tc_stamp(g.trace, 3);
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, BN);
-            int kbi = 0, i = 0;
-            int s = 0; uint32_t par = 0;                     // ring position of k-block kbi: stage and phase parity, kept incrementally
-            const bool stamps = g.trace != nullptr && blockIdx.x == 0;
-            for (int t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x, ++i) {
-                const int ab = i & 1;
-                if (i >= 2) mbar_wait(smem_u32(&bar_acc_empty[ab]), ((i >> 1) - 1) & 1, abort_flag, err_word, 4);
-                tc_fence_after();
-                const uint32_t acc = tmem_d + ab * BN;
-                // The tensor pipe takes one MMA at a time from this thread and the thread stalls in each issue until the
-                // pipe accepts it, so whatever the thread does BETWEEN two issues is free while whatever it does between
-                // the last MMA of a k-block and the first of the next leaves the pipe idle (measured: ~300 clocks of
-                // bookkeeping per MMA throttle the pipe to exactly that).  All bookkeeping for the next k-block -- its
-                // ring position, descriptors and the test of its barrier -- therefore sits between this k-block's issues.
-                bool ok = mbar_wait(smem_u32(&bar_full[s]), par, abort_flag, err_word, 2);
-                if (stamps && kbi == 0) tc_stamp(g.trace, 4);
-                for (int kb = 0; kb < nkb && ok; ++kb, ++kbi) {
-                    const uint32_t a_src = tiles + s * Cfg::STAGE_BYTES, w_src = a_src + A_BYTES;
-                    const uint64_t ad = umma_desc_k_sw128(a_src), wd = umma_desc_k_sw128(w_src);
-                    umma_bf16(acc, ad, wd, idesc, kb ? 1u : 0u);
-                    int sn = s + 1; uint32_t parn = par;
-                    if (sn == STAGES) { sn = 0; parn ^= 1u; }
-                    const uint32_t next_bar = smem_u32(&bar_full[sn]);
-                    umma_bf16(acc, ad + 2, wd + 2, idesc, 1u);       // +32 bytes along K per instruction: 2 address units
-                    const uint32_t early_ok = (kb + 1 < nkb) ? mbar_try_wait(next_bar, parn) : 1u;
-                    umma_bf16(acc, ad + 4, wd + 4, idesc, 1u);
-                    if (stamps && kbi < 16) tc_stamp(g.trace, 40 + kbi);          // landing cadence of the first k-blocks
-                    umma_bf16(acc, ad + 6, wd + 6, idesc, 1u);
-                    umma_commit(smem_u32(&bar_empty[s]));        // stage reusable once these MMAs have read it
-                    if (!early_ok) ok = mbar_wait(next_bar, parn, abort_flag, err_word, 2);
-                    s = sn; par = parn;
-                }
+        constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, BN);
+        int i = 0, s = 0; uint32_t par = 0; bool ok = true;
+        for (int t = blockIdx.x; t < total; t += gridDim.x, ++i) {
+            const int ab = i & 1;
+            if (i >= 2) ok = mbar_wait_warp(smem_u32(&bar_acc_empty[ab]), ((i >> 1) - 1) & 1, abort_flag, err_word, 4);
+            tc_fence_after();
+            const uint32_t acc = tmem_d + ab * BN;
+            for (int kb = 0; kb < nkb && ok; ++kb) {
+                ok = mbar_wait_warp(full0 + 8 * s, par, abort_flag, err_word, 2);
                 if (!ok) break;
-                umma_commit(smem_u32(&bar_acc_full[ab]));        // accumulator of this tile complete
-                if (stamps) tc_stamp(g.trace, 5 + (i > 0));
+                const uint32_t a_src = tiles + s * Cfg::STAGE_BYTES, bar = empty0 + 8 * s;
+                if (elect_one()) {
+                    const uint64_t ad = umma_desc_k_sw128(a_src), wd = umma_desc_k_sw128(a_src + A_BYTES);
+                    umma_bf16(acc, ad, wd, idesc, kb ? 1u : 0u);
+                    umma_bf16(acc, ad + 2, wd + 2, idesc, 1u);           // +32 bytes along K per instruction: 2 address units
+                    umma_bf16(acc, ad + 4, wd + 4, idesc, 1u);
+                    umma_bf16(acc, ad + 6, wd + 6, idesc, 1u);
+                    umma_commit(bar);                                    // stage reusable once these MMAs have read it
+                }
+                if (++s == STAGES) { s = 0; par ^= 1u; }
             }
+            if (!ok) break;
+            if (elect_one()) umma_commit(smem_u32(&bar_acc_full[ab]));   // accumulator of this tile complete
+            if (lane == 0) tc_stamp(g.trace, 5 + (i > 0));
         }
     } else {
         const int q = warp & 3;                                  // TMEM lane quadrant this warp may read

@@ -97,7 +97,7 @@ k_gemm_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
     const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t rank = pair_cta_rank();
     const bool leader = rank == 0;
     const int nkb = g.K / TC_BK;
@@ -114,9 +114,9 @@ k_gemm_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tc_fence_before();
     pair_sync();                                     // both CTAs' barriers and tensor memory exist from here on
     tc_fence_after();
-    const uint32_t tmem_d = tmem_base_s;
+    const uint32_t tmem_d = __shfl_sync(0xffffffffu, tmem_base_s, 0);
     volatile int* abort_flag = &abort_s;
-    if (threadIdx.x == 0 && tmem_d != 0xffffffffu) tc_stamp(g.trace, 1);
+    if (threadIdx.x == 0) tc_stamp(g.trace, 1);
     int pre = 0;                                     // stages whose weight halves were requested before the wait
     if (early) {
         if (threadIdx.x == 0) {
@@ -130,60 +130,56 @@ k_gemm_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         pdl_wait();                                  // activations, residual and outputs belong to the predecessors until here
     }
 
+    // (loops of whole warps, electing a lane only around the instructions: see elect_one)
+    const uint32_t full0 = smem_u32(&bar_full[0]), empty0 = smem_u32(&bar_empty[0]), full_lead = pair_map(full0, 0);
     if (warp == 0) {
-        if (lane == 0) {
-            int kbi = 0;
-            int ps = 0; uint32_t ppar = 0; bool wrapped = false, dead = false;   // producer's ring position (incremental: see k_vocab_pair)
-            for (int t = pair; t < total && !dead && !*abort_flag; t += pairs) {
-                const int m0 = (t % m_pairs) * 2 * TC_BM + (int)rank * TC_BM, n0 = (t / m_pairs) * BN + (int)rank * BNH;
-                for (int kb = 0; kb < nkb; ++kb, ++kbi) {
-                    if (wrapped && !mbar_wait(smem_u32(&bar_empty[ps]), ppar, abort_flag, err_word, 1)) { dead = true; break; }
-                    const uint32_t a_dst = tiles + ps * Cfg::STAGE_BYTES, w_dst = a_dst + A_BYTES;
-                    const uint32_t bar = pair_map(smem_u32(&bar_full[ps]), 0);
-                    if (kbi >= pre) {
-                        if (leader) mbar_expect_tx(smem_u32(&bar_full[ps]), 2 * Cfg::STAGE_BYTES);
-                        tma_load_2d_pair(w_dst, &tmW, kb * TC_BK, n0, bar);
+        const int npre = early ? min(STAGES, nkb) : 0;
+        int kbi = 0, ps = 0; uint32_t ppar = 1; bool ok = true;          // (a fresh barrier counts as past the phase before its first)
+        for (int t = pair; t < total && ok; t += pairs) {
+            const int m0 = (t % m_pairs) * 2 * TC_BM + (int)rank * TC_BM, n0 = (t / m_pairs) * BN + (int)rank * BNH;
+            for (int kb = 0; kb < nkb; ++kb, ++kbi) {
+                ok = mbar_wait_warp(empty0 + 8 * ps, ppar, abort_flag, err_word, 1);
+                if (!ok) break;
+                const uint32_t a_dst = tiles + ps * Cfg::STAGE_BYTES, bar = full_lead + 8 * ps;
+                if (elect_one()) {
+                    if (kbi >= npre) {
+                        if (leader) mbar_expect_tx(full0 + 8 * ps, 2 * Cfg::STAGE_BYTES);
+                        tma_load_2d_pair(a_dst + A_BYTES, &tmW, kb * TC_BK, n0, bar);
                     }
                     tma_load_2d_pair(a_dst, &tmA, kb * TC_BK, m0, bar);
-                    if (++ps == STAGES) { ps = 0; if (wrapped) ppar ^= 1u; wrapped = true; }
                 }
+                if (++ps == STAGES) { ps = 0; ppar ^= 1u; }
             }
-            tc_stamp(g.trace, 3);
         }
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
+        if (leader) {
             constexpr uint32_t idesc = umma_idesc_bf16(2 * TC_BM, BN);
-            int kbi = 0, i = 0;
-            int s = 0; uint32_t par = 0;                      // ring position kept incrementally; bookkeeping between the issues (see k_gemm_tc)
-            const bool stamps = g.trace != nullptr && blockIdx.x == 0;
-            for (int t = pair; t < total && !*abort_flag; t += pairs, ++i) {
+            int i = 0, s = 0; uint32_t par = 0; bool ok = true;
+            for (int t = pair; t < total; t += pairs, ++i) {
                 const int ab = i & 1;
-                if (i >= 2) mbar_wait(smem_u32(&bar_acc_empty[ab]), ((i >> 1) - 1) & 1, abort_flag, err_word, 4);
+                if (i >= 2) ok = mbar_wait_warp(smem_u32(&bar_acc_empty[ab]), ((i >> 1) - 1) & 1, abort_flag, err_word, 4);
                 tc_fence_after();
                 const uint32_t acc = tmem_d + ab * BN;
-                bool ok = mbar_wait(smem_u32(&bar_full[s]), par, abort_flag, err_word, 2);
-                if (stamps && kbi == 0) tc_stamp(g.trace, 4);
-                for (int kb = 0; kb < nkb && ok; ++kb, ++kbi) {
-                    const uint32_t a_src = tiles + s * Cfg::STAGE_BYTES, w_src = a_src + A_BYTES;
-                    const uint64_t ad = umma_desc_k_sw128(a_src), wd = umma_desc_k_sw128(w_src);
-                    umma_bf16_pair(acc, ad, wd, idesc, kb ? 1u : 0u);
-                    int sn = s + 1; uint32_t parn = par;
-                    if (sn == STAGES) { sn = 0; parn ^= 1u; }
-                    const uint32_t next_bar = smem_u32(&bar_full[sn]);
-                    umma_bf16_pair(acc, ad + 2, wd + 2, idesc, 1u);
-                    const uint32_t early_ok = (kb + 1 < nkb) ? mbar_try_wait(next_bar, parn) : 1u;
-                    umma_bf16_pair(acc, ad + 4, wd + 4, idesc, 1u);
-                    if (stamps && kbi < 16) tc_stamp(g.trace, 40 + kbi);
-                    umma_bf16_pair(acc, ad + 6, wd + 6, idesc, 1u);
-                    umma_commit_pair(smem_u32(&bar_empty[s]));       // both CTAs may refill the stage
-                    if (!early_ok) ok = mbar_wait(next_bar, parn, abort_flag, err_word, 2);
-                    s = sn; par = parn;
+                for (int kb = 0; kb < nkb && ok; ++kb) {
+                    ok = mbar_wait_warp(full0 + 8 * s, par, abort_flag, err_word, 2);
+                    if (!ok) break;
+                    const uint32_t a_src = tiles + s * Cfg::STAGE_BYTES, bar = empty0 + 8 * s;
+                    if (elect_one()) {
+                        const uint64_t ad = umma_desc_k_sw128(a_src), wd = umma_desc_k_sw128(a_src + A_BYTES);
+                        umma_bf16_pair(acc, ad, wd, idesc, kb ? 1u : 0u);
+                        umma_bf16_pair(acc, ad + 2, wd + 2, idesc, 1u);
+                        umma_bf16_pair(acc, ad + 4, wd + 4, idesc, 1u);
+                        umma_bf16_pair(acc, ad + 6, wd + 6, idesc, 1u);
+                        umma_commit_pair(bar);                           // both CTAs may refill the stage
+                    }
+                    if (++s == STAGES) { s = 0; par ^= 1u; }
                 }
                 if (!ok) break;
-                umma_commit_pair(smem_u32(&bar_acc_full[ab]));       // both CTAs' halves of the accumulator are complete
-                if (stamps) tc_stamp(g.trace, 5 + (i > 0));
+                if (elect_one()) umma_commit_pair(smem_u32(&bar_acc_full[ab]));       // both CTAs' halves of the accumulator are complete
+                if (lane == 0) tc_stamp(g.trace, 5 + (i > 0));
             }
         }
+        __syncwarp();
     } else {
         const int q = warp & 3;
         const int half = (warp - 2) >> 2;
@@ -251,7 +247,7 @@ k_vocab_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         bar_acc_full[2], bar_acc_empty[2];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t rank = pair_cta_rank();
     const bool leader = rank == 0;
     const int nkb = g.K / TC_BK;
@@ -269,9 +265,9 @@ k_vocab_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     tc_fence_before();
     pair_sync();
     tc_fence_after();
-    const uint32_t tmem_d = tmem_base_s;
+    const uint32_t tmem_d = __shfl_sync(0xffffffffu, tmem_base_s, 0);
     volatile int* abort_flag = &abort_s;
-    if (threadIdx.x == 0 && tmem_d != 0xffffffffu) tc_stamp(g.trace, 1);
+    if (threadIdx.x == 0) tc_stamp(g.trace, 1);
     int pre = 0;                                     // ring stages requested before the wait (weights only)
     if (early) {
         if (threadIdx.x == 0) {
@@ -287,76 +283,72 @@ k_vocab_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         pdl_wait();
     }
 
+    const uint32_t full0 = smem_u32(&bar_w_full[0]), empty0 = smem_u32(&bar_w_empty[0]), full_lead = pair_map(full0, 0);
     if (warp == 0) {
-        if (lane == 0) {
-            int kbi = 0, a_loads = 0;
-            int ps = 0; uint32_t ppar = 0; bool wrapped = false, dead = false;   // producer's ring position; ppar = parity of the empty phase awaited
-            for (int u = pair; u < units && !dead && !*abort_flag; u += pairs) {
-                VP_UNIT(u, m_pair, nb, ne);
-                // this unit's activation rows replace the resident ones
-                if (a_loads > 0 && !mbar_wait(smem_u32(&bar_a_empty), (a_loads - 1) & 1, abort_flag, err_word, 5)) break;
-                if (leader) mbar_expect_tx(smem_u32(&bar_a_full), 2 * nkb * VP_KB_BYTES);
-                const uint32_t abar = pair_map(smem_u32(&bar_a_full), 0);
-                for (int kb = 0; kb < nkb; ++kb)
-                    tma_load_2d_pair(a_base + kb * VP_KB_BYTES, &tmA, kb * TC_BK, m_pair * 2 * TC_BM + (int)rank * TC_BM, abar);
-                ++a_loads;
-                if (a_loads == 1) tc_stamp(g.trace, 2);
-                for (int n = nb; n < ne && !dead; ++n) {
-                    const int n0 = n * VP_BN + (int)rank * VP_BNH;
-                    for (int kb = 0; kb < nkb; ++kb, ++kbi) {
-                        if (wrapped && !mbar_wait(smem_u32(&bar_w_empty[ps]), ppar, abort_flag, err_word, 1)) { dead = true; break; }
-                        if (kbi >= pre) {
-                            if (leader) mbar_expect_tx(smem_u32(&bar_w_full[ps]), 2 * VP_KB_BYTES);
-                            tma_load_2d_pair(w_base + ps * VP_KB_BYTES, &tmW, kb * TC_BK, n0, pair_map(smem_u32(&bar_w_full[ps]), 0));
-                        }
-                        if (++ps == stages) { ps = 0; if (wrapped) ppar ^= 1u; wrapped = true; }
+        const int npre = early ? min(stages, nkb) : 0;
+        int kbi = 0, a_loads = 0, ps = 0; uint32_t ppar = 1; bool ok = true;
+        const uint32_t abar = pair_map(smem_u32(&bar_a_full), 0);
+        for (int u = pair; u < units && ok; u += pairs) {
+            VP_UNIT(u, m_pair, nb, ne);
+            // this unit's activation rows replace the resident ones
+            if (a_loads > 0) ok = mbar_wait_warp(smem_u32(&bar_a_empty), (a_loads - 1) & 1, abort_flag, err_word, 5);
+            if (!ok) break;
+            if (leader && elect_one()) mbar_expect_tx(smem_u32(&bar_a_full), 2 * nkb * VP_KB_BYTES);
+            __syncwarp();
+            for (int kb = 0; kb < nkb; ++kb)
+                if (elect_one()) tma_load_2d_pair(a_base + kb * VP_KB_BYTES, &tmA, kb * TC_BK, m_pair * 2 * TC_BM + (int)rank * TC_BM, abar);
+            ++a_loads;
+            for (int n = nb; n < ne && ok; ++n) {
+                const int n0 = n * VP_BN + (int)rank * VP_BNH;
+                for (int kb = 0; kb < nkb; ++kb, ++kbi) {
+                    ok = mbar_wait_warp(empty0 + 8 * ps, ppar, abort_flag, err_word, 1);
+                    if (!ok) break;
+                    if (kbi >= npre && elect_one()) {
+                        if (leader) mbar_expect_tx(full0 + 8 * ps, 2 * VP_KB_BYTES);
+                        tma_load_2d_pair(w_base + ps * VP_KB_BYTES, &tmW, kb * TC_BK, n0, full_lead + 8 * ps);
                     }
+                    if (++ps == stages) { ps = 0; ppar ^= 1u; }
                 }
             }
-            tc_stamp(g.trace, 3);
         }
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
+        if (leader) {
             constexpr uint32_t idesc = umma_idesc_bf16(2 * TC_BM, VP_BN);
-            int kbi = 0, i = 0, a_uses = 0;
-            int s = 0; uint32_t par = 0;                      // ring position kept incrementally; bookkeeping between the issues (see k_gemm_tc)
-            const bool stamps = g.trace != nullptr && blockIdx.x == 0;
-            bool ok = true;
-            for (int u = pair; u < units && ok && !*abort_flag; u += pairs) {
+            int i = 0, a_uses = 0, s = 0; uint32_t par = 0; bool ok = true;
+            for (int u = pair; u < units && ok; u += pairs) {
                 VP_UNIT(u, m_pair, nb, ne);
                 (void)m_pair;
-                ok = mbar_wait(smem_u32(&bar_a_full), a_uses & 1, abort_flag, err_word, 6);
+                ok = mbar_wait_warp(smem_u32(&bar_a_full), a_uses & 1, abort_flag, err_word, 6);
                 ++a_uses;
                 for (int n = nb; n < ne && ok; ++n, ++i) {
                     const int ab = i & 1;
-                    if (i >= 2) ok = mbar_wait(smem_u32(&bar_acc_empty[ab]), ((i >> 1) - 1) & 1, abort_flag, err_word, 4);
-                    if (!ok) break;
+                    if (i >= 2) ok = mbar_wait_warp(smem_u32(&bar_acc_empty[ab]), ((i >> 1) - 1) & 1, abort_flag, err_word, 4);
                     tc_fence_after();
                     const uint32_t acc = tmem_d + ab * VP_BN;
-                    ok = mbar_wait(smem_u32(&bar_w_full[s]), par, abort_flag, err_word, 2);
-                    if (stamps && kbi == 0) tc_stamp(g.trace, 4);
-                    for (int kb = 0; kb < nkb && ok; ++kb, ++kbi) {
-                        const uint64_t ad = umma_desc_k_sw128(a_base + kb * VP_KB_BYTES), wd = umma_desc_k_sw128(w_base + s * VP_KB_BYTES);
-                        umma_bf16_pair(acc, ad, wd, idesc, kb ? 1u : 0u);
-                        int sn = s + 1; uint32_t parn = par;
-                        if (sn == stages) { sn = 0; parn ^= 1u; }
-                        const uint32_t next_bar = smem_u32(&bar_w_full[sn]);
-                        umma_bf16_pair(acc, ad + 2, wd + 2, idesc, 1u);
-                        const uint32_t early_ok = (kb + 1 < nkb) ? mbar_try_wait(next_bar, parn) : 1u;
-                        umma_bf16_pair(acc, ad + 4, wd + 4, idesc, 1u);
-                        if (stamps && kbi < 16) tc_stamp(g.trace, 40 + kbi);
-                        umma_bf16_pair(acc, ad + 6, wd + 6, idesc, 1u);
-                        umma_commit_pair(smem_u32(&bar_w_empty[s]));
-                        if (!early_ok) ok = mbar_wait(next_bar, parn, abort_flag, err_word, 2);
-                        s = sn; par = parn;
+                    for (int kb = 0; kb < nkb && ok; ++kb) {
+                        ok = mbar_wait_warp(full0 + 8 * s, par, abort_flag, err_word, 2);
+                        if (!ok) break;
+                        const uint32_t a_src = a_base + kb * VP_KB_BYTES, w_src = w_base + s * VP_KB_BYTES, bar = empty0 + 8 * s;
+                        if (elect_one()) {
+                            const uint64_t ad = umma_desc_k_sw128(a_src), wd = umma_desc_k_sw128(w_src);
+                            umma_bf16_pair(acc, ad, wd, idesc, kb ? 1u : 0u);
+                            umma_bf16_pair(acc, ad + 2, wd + 2, idesc, 1u);
+                            umma_bf16_pair(acc, ad + 4, wd + 4, idesc, 1u);
+                            umma_bf16_pair(acc, ad + 6, wd + 6, idesc, 1u);
+                            umma_commit_pair(bar);
+                        }
+                        if (++s == stages) { s = 0; par ^= 1u; }
                     }
                     if (!ok) break;
-                    if (n + 1 == ne) umma_commit_pair(smem_u32(&bar_a_empty));   // the unit's rows may be replaced
-                    umma_commit_pair(smem_u32(&bar_acc_full[ab]));
-                    if (stamps) tc_stamp(g.trace, 5 + (i > 0));
+                    if (elect_one()) {
+                        if (n + 1 == ne) umma_commit_pair(smem_u32(&bar_a_empty));   // the unit's rows may be replaced
+                        umma_commit_pair(smem_u32(&bar_acc_full[ab]));
+                    }
+                    if (lane == 0) tc_stamp(g.trace, 5 + (i > 0));
                 }
             }
         }
+        __syncwarp();
     } else {
         const int q = warp & 3;
         const int half = (warp - 2) >> 2;
@@ -448,7 +440,7 @@ inline int gemm_tc_pair_launch(TmaEncoder& enc, int epi, GemmArgs<bf16>& g, int 
         case EPI_STATS:
             g.n_tiles = 2 * ((g.N + 255) / 256);
             if (n_tiles_out) *n_tiles_out = g.n_tiles;
-            if (g.K <= 512 && vp_stages(g.K) >= 4) return vocab_pair_launch(enc, g, rows_ub, st);
+            if (!enc.force_bn && g.K <= 512 && vp_stages(g.K) >= 4) return vocab_pair_launch(enc, g, rows_ub, st);
             return tc_pair_launch_one<EPI_STATS, 256>(enc, g, rows_ub, st);
         default: return -2;
     }

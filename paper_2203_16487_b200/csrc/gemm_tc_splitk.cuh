@@ -48,7 +48,7 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     __shared__ int abort_s;
     const uint32_t a_base = (smem_u32(smem_raw) + 1023u) & ~1023u, w_base = a_base + nkb * SPK_A_KB;
     uint8_t* base_ptr = smem_raw + (a_base - smem_u32(smem_raw));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     uint32_t rank;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     const int n_tile = blockIdx.x / SPLIT, kb0 = (int)rank * nkb, m0 = blockIdx.y * TC_BM;
@@ -65,22 +65,24 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     tc_fence_before();
     tc_cluster_sync();                               // rank 0's barrier exists before anybody sends
     tc_fence_after();
-    const uint32_t tmem_d = tmem_base_s;
+    const uint32_t tmem_d = __shfl_sync(0xffffffffu, tmem_base_s, 0);
     volatile int* abort_flag = &abort_s;
-    if (threadIdx.x == 0) {                          // this CTA's slice of the weights: before the dependency wait
-        for (int kb = 0; kb < nkb; ++kb) {
-            mbar_expect_tx(smem_u32(&bar_full[kb]), SPK_A_KB + SPK_W_KB);
-            tma_load_2d(w_base + kb * SPK_W_KB, &tmW, (kb0 + kb) * TC_BK, n_tile * SPK_BN, smem_u32(&bar_full[kb]));
-        }
+    const uint32_t full0 = smem_u32(&bar_full[0]);
+    if (warp == 0) {                                 // this CTA's slice of the weights: before the dependency wait
+        for (int kb = 0; kb < nkb; ++kb)
+            if (elect_one()) {
+                mbar_expect_tx(full0 + 8 * kb, SPK_A_KB + SPK_W_KB);
+                tma_load_2d(w_base + kb * SPK_W_KB, &tmW, (kb0 + kb) * TC_BK, n_tile * SPK_BN, full0 + 8 * kb);
+            }
     }
     pdl_launch_dependents();
     pdl_wait();
     // rows of this CTA's 128-row tile (none: the tile still runs, on zero-filled rows, and stores nothing)
     const int R = min(max((g.rows_static >= 0 ? g.rows_static : *g.n_rows) - m0, 0), TC_BM);
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
         for (int kb = 0; kb < nkb; ++kb)
-            tma_load_2d(a_base + kb * SPK_A_KB, &tmA, (kb0 + kb) * TC_BK, m0, smem_u32(&bar_full[kb]));
-        if (rank == 0) mbar_expect_tx(smem_u32(&bar_part), (uint32_t)(SPLIT - 1) * R * SPK_BN * 4);
+            if (elect_one()) tma_load_2d(a_base + kb * SPK_A_KB, &tmA, (kb0 + kb) * TC_BK, m0, full0 + 8 * kb);
+        if (rank == 0 && elect_one()) mbar_expect_tx(smem_u32(&bar_part), (uint32_t)(SPLIT - 1) * R * SPK_BN * 4);
     }
     const int q = warp & 3, half = (warp - 2) >> 2, row = q * 32 + lane;
     const int n0 = n_tile * SPK_BN + half * 32;
@@ -95,19 +97,20 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
     bool ok = true;
     if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, SPK_BN);
-            for (int kb = 0; kb < nkb && ok; ++kb) {
-                ok = mbar_wait(smem_u32(&bar_full[kb]), 0, abort_flag, err_word, 2);
-                if (!ok) break;
-                tc_fence_after();
-                const uint64_t ad = umma_desc_k_sw128(a_base + kb * SPK_A_KB), wd = umma_desc_k_sw128(w_base + kb * SPK_W_KB);
+        constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, SPK_BN);
+        for (int kb = 0; kb < nkb; ++kb) {
+            ok = mbar_wait_warp(full0 + 8 * kb, 0, abort_flag, err_word, 2);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t a_src = a_base + kb * SPK_A_KB, w_src = w_base + kb * SPK_W_KB;
+            if (elect_one()) {
+                const uint64_t ad = umma_desc_k_sw128(a_src), wd = umma_desc_k_sw128(w_src);
 #pragma unroll
                 for (int k4 = 0; k4 < TC_BK / 16; ++k4)
                     umma_bf16(tmem_d, ad + (uint64_t)(k4 * 2), wd + (uint64_t)(k4 * 2), idesc, (kb | k4) ? 1u : 0u);
             }
-            umma_commit(smem_u32(&bar_acc));
         }
+        if (elect_one()) umma_commit(smem_u32(&bar_acc));
     } else if (warp >= 2) {
         ok = mbar_wait(smem_u32(&bar_acc), 0, abort_flag, err_word, 3);      // this CTA's MMAs are done: its operand tiles are dead
         tc_fence_after();

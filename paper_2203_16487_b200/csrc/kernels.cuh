@@ -385,37 +385,64 @@ static __global__ void k_gather_rows(const float* __restrict__ x, const int* __r
     for (int e = threadIdx.x; e < d; e += blockDim.x) out[(size_t)row * d + e] = s[e];
 }
 
-// Register-resident row of up to NC * 128 elements (one warp per row).  gm / bt = this lane's gain and bias columns,
-// fetched by the caller before the dependency wait (they are weights).
-template <typename T, int NC>
-__device__ __forceinline__ void ln_row_regs(const float* __restrict__ xr, const float4* gm, const float4* bt,
-                                            T* __restrict__ y, int row, int d, float eps, int lane, bool store = true) {
-    float4 v[NC];
+// LayerNorm of rows of d = 128 NC elements, ROWS rows per warp held in registers; biased variance, eps inside the square root.
+// Bound by one round trip to L2 and the launch itself: gain and bias are fetched and the row count is read ahead of the dependency wait
+// (3328 rows of 512: 3.6 -> 2.7 us a launch inside the verify step against the kernel that chose the width at run time and read the
+// count behind the wait).  Two rows per warp beyond 512 columns (1560 rows of 768, whole first-tokens call: 1212 -> 1189 us; 512
+// columns: 560 with one, 563 with two).
+template <typename T, int NC, int ROWS>
+__global__ void __launch_bounds__(256) k_layernorm_rows(const float* __restrict__ x, const float* __restrict__ g, const float* __restrict__ b,
+                                                        const int* __restrict__ n_rows, T* __restrict__ y, int d, float eps, int rows_static) {
+    const int lane = threadIdx.x & 31, row0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * ROWS;
+    float4 gm[NC], bt[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-        const int e = lane * 4 + c * 128;
-        v[c] = e < d ? *reinterpret_cast<const float4*>(xr + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+        gm[c] = __ldg(reinterpret_cast<const float4*>(g + lane * 4 + c * 128));
+        bt[c] = __ldg(reinterpret_cast<const float4*>(b + lane * 4 + c * 128));
     }
-    float s = 0.f;
+    const int R = rows_static >= 0 ? rows_static : *n_rows;      // (a device-side count predates the step's kernel chain)
+    pdl_launch_dependents();
+    pdl_wait();
+    float4 v[ROWS][NC];
+    float s[ROWS], q[ROWS];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) s += v[c].x + v[c].y + v[c].z + v[c].w;
-    const float mu = warp_sum(s) / d;
-    float q = 0.f;
+    for (int r = 0; r < ROWS; ++r)
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-        if (lane * 4 + c * 128 < d) {
-            const float c0 = v[c].x - mu, c1 = v[c].y - mu, c2 = v[c].z - mu, c3 = v[c].w - mu;
-            q += c0 * c0 + c1 * c1 + c2 * c2 + c3 * c3;
+        for (int c = 0; c < NC; ++c)
+            v[r][c] = row0 + r < R ? *reinterpret_cast<const float4*>(x + (size_t)(row0 + r) * d + lane * 4 + c * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        s[r] = 0.f;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[r] += v[r][c].x + v[r][c].y + v[r][c].z + v[r][c].w;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) s[r] += __shfl_xor_sync(0xffffffffu, s[r], o);
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        s[r] /= d; q[r] = 0.f;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            v[r][c].x -= s[r]; v[r][c].y -= s[r]; v[r][c].z -= s[r]; v[r][c].w -= s[r];
+            q[r] += v[r][c].x * v[r][c].x + v[r][c].y * v[r][c].y + v[r][c].z * v[r][c].z + v[r][c].w * v[r][c].w;
         }
-    const float rstd = 1.0f / sqrtf(warp_sum(q) / d + eps);
+    }
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        const int e = lane * 4 + c * 128;
-        if (e < d && store) {
-            T* o = y + (size_t)row * d + e;
-            const float r0 = (v[c].x - mu) * rstd * gm[c].x + bt[c].x, r1 = (v[c].y - mu) * rstd * gm[c].y + bt[c].y;
-            const float r2 = (v[c].z - mu) * rstd * gm[c].z + bt[c].z, r3 = (v[c].w - mu) * rstd * gm[c].w + bt[c].w;
-            if constexpr (sizeof(T) == 2) {          // bf16: one 8-byte store per lane and chunk
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) q[r] += __shfl_xor_sync(0xffffffffu, q[r], o);
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        const float rstd = 1.0f / sqrtf(q[r] / d + eps);
+        if (row0 + r >= R) continue;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            T* o = y + (size_t)(row0 + r) * d + lane * 4 + c * 128;
+            const float r0 = v[r][c].x * rstd * gm[c].x + bt[c].x, r1 = v[r][c].y * rstd * gm[c].y + bt[c].y;
+            const float r2 = v[r][c].z * rstd * gm[c].z + bt[c].z, r3 = v[r][c].w * rstd * gm[c].w + bt[c].w;
+            if constexpr (sizeof(T) == 2) {
                 __nv_bfloat162 p0 = __floats2bfloat162_rn(r0, r1), p1 = __floats2bfloat162_rn(r2, r3);
                 *reinterpret_cast<uint2*>(o) = make_uint2(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1));
             } else {
@@ -425,32 +452,15 @@ __device__ __forceinline__ void ln_row_regs(const float* __restrict__ xr, const 
     }
 }
 
-// One warp per row; biased variance, eps inside the square root.  Rows of up to 1024 elements
-// (a multiple of 128) are held in registers, so the row is read from memory once.
+// Any other width: one warp per row, the row read three times.
 template <typename T>
 __global__ void k_layernorm(const float* __restrict__ x, const float* __restrict__ g, const float* __restrict__ b,
                             const int* __restrict__ n_rows, T* __restrict__ y, int d, float eps, int rows_static) {
-    // rows_static >= 0: the row count is known on the host (saves the dependent load of n_rows in front of the row's own)
-    int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    int lane = threadIdx.x & 31;
-    const bool regs4 = d % 128 == 0 && d <= 512, regs8 = d % 128 == 0 && d <= 1024;
-    float4 gm[8], bt[8];                             // gain and bias are weights: fetched before the dependency wait
-    if (regs8) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int e = lane * 4 + c * 128;
-            if (c < 4 || !regs4) {
-                gm[c] = e < d ? __ldg(reinterpret_cast<const float4*>(g + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                bt[c] = e < d ? __ldg(reinterpret_cast<const float4*>(b + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-        }
-    }
+    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     pdl_launch_dependents();
     pdl_wait();
     if (row >= (rows_static >= 0 ? rows_static : *n_rows)) return;
     const float* xr = x + (size_t)row * d;
-    if (regs4) { ln_row_regs<T, 4>(xr, gm, bt, y, row, d, eps, lane); return; }
-    if (regs8) { ln_row_regs<T, 8>(xr, gm, bt, y, row, d, eps, lane); return; }
     float s = 0.f;
     for (int e = lane; e < d; e += 32) s += xr[e];
     float mu = warp_sum(s) / d;

@@ -418,11 +418,17 @@ template <typename T>
 int ln(specdec_handle* h, const float* x, const float* g, const float* b, int cnt, int rows_ub, void* y, int d,
        cudaStream_t st) {
     if (rows_ub <= 0) return 0;
-    {
-        cudaError_t e = launch_pdl(h, k_layernorm<T>, dim3(cdiv(rows_ub, 8)), dim3(256), 0, st, x, g, b,
-                                   (const int*)(h->ses.counters + cnt), (T*)y, d, 1e-5f, static_rows(h, cnt, rows_ub));
-        if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("layer norm launch: ") + cudaGetErrorString(e));
+    cudaError_t e;
+#define LN_ROWS(NC, ROWS) e = launch_pdl(h, k_layernorm_rows<T, NC, ROWS>, dim3(cdiv(rows_ub, 8 * ROWS)), dim3(256), 0, st, x, g, b, \
+                                         (const int*)(h->ses.counters + cnt), (T*)y, d, 1e-5f, static_rows(h, cnt, rows_ub))
+    switch (d % 128 ? 0 : d / 128) {
+        case 1: LN_ROWS(1, 1); break; case 2: LN_ROWS(2, 1); break; case 3: LN_ROWS(3, 1); break; case 4: LN_ROWS(4, 1); break;
+        case 5: LN_ROWS(5, 2); break; case 6: LN_ROWS(6, 2); break; case 7: LN_ROWS(7, 2); break; case 8: LN_ROWS(8, 2); break;
+        default: e = launch_pdl(h, k_layernorm<T>, dim3(cdiv(rows_ub, 8)), dim3(256), 0, st, x, g, b,
+                                (const int*)(h->ses.counters + cnt), (T*)y, d, 1e-5f, static_rows(h, cnt, rows_ub));
     }
+#undef LN_ROWS
+    if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("layer norm launch: ") + cudaGetErrorString(e));
     KCHECK(h);
     return 0;
 }
