@@ -25,7 +25,8 @@ template <typename T> __device__ __forceinline__ float round_as(float v) { retur
 // Programmatic dependent launch: a kernel launched with the stream-serialization attribute may start
 // while its predecessor is still running.  pdl_wait() blocks until the predecessor grids have completed
 // and their writes are visible; everything a kernel does before it must not depend on them (weights and
-// constants only) and must not write global memory.  Without the attribute both are no-ops.
+// constants only) and must not write global memory.  Without the attribute both are no-ops.  Pointers to what a predecessor
+// writes are never `const __restrict__`: the compiler may fetch through those at any point of the kernel, the wait notwithstanding.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -150,7 +151,7 @@ static __global__ void k_enc_prep(Session s, const int* __restrict__ src, const 
 // more than half of all blocks would belong to sequences that ended iterations ago.  The row metadata is complete before the
 // block lets its successors start, because kernels further down the chain read it ahead of their own dependency waits.
 template <typename T>
-__global__ void k_verify_prep_embed(Session s, const int* __restrict__ draft, int B, int k, int bos, Rows r,
+__global__ void k_verify_prep_embed(Session s, const int* draft, int B, int k, int bos, Rows r,
                                     const T* __restrict__ E, const float* __restrict__ P, float* __restrict__ x, int d,
                                     float scale, int vocab, int max_pos, int compact, int* __restrict__ keep) {
     __shared__ int s_b, s_live;
@@ -363,7 +364,7 @@ __global__ void k_draft_prep_pc(Session s, int B, int k, int bos, int mask, Rows
 // ------------------------------------------------------------------ embedding, gather, layer norm
 // x[row] = sqrt(d) * E[tok] + P[pos]
 template <typename T>
-__global__ void k_embed(const int* __restrict__ tok, const int* __restrict__ pos, const int* __restrict__ n_rows,
+__global__ void k_embed(const int* tok, const int* pos, const int* n_rows,
                         const T* __restrict__ E, const float* __restrict__ P, float* __restrict__ x, int d,
                         float scale, int vocab, int max_pos) {
     int row = blockIdx.x;
@@ -375,8 +376,8 @@ __global__ void k_embed(const int* __restrict__ tok, const int* __restrict__ pos
         x[(size_t)row * d + e] = scale * to_f(E[(size_t)t * d + e]) + P[(size_t)p * d + e];
 }
 
-static __global__ void k_gather_rows(const float* __restrict__ x, const int* __restrict__ src_row,
-                              const int* __restrict__ n_rows, float* __restrict__ out, int d) {
+static __global__ void k_gather_rows(const float* x, const int* src_row,
+                              const int* n_rows, float* __restrict__ out, int d) {
     int row = blockIdx.x;
     pdl_launch_dependents();
     pdl_wait();
@@ -391,8 +392,8 @@ static __global__ void k_gather_rows(const float* __restrict__ x, const int* __r
 // count behind the wait).  Two rows per warp beyond 512 columns (1560 rows of 768, whole first-tokens call: 1212 -> 1189 us; 512
 // columns: 560 with one, 563 with two).
 template <typename T, int NC, int ROWS>
-__global__ void __launch_bounds__(256) k_layernorm_rows(const float* __restrict__ x, const float* __restrict__ g, const float* __restrict__ b,
-                                                        const int* __restrict__ n_rows, T* __restrict__ y, int d, float eps, int rows_static) {
+__global__ void __launch_bounds__(256) k_layernorm_rows(const float* x, const float* __restrict__ g, const float* __restrict__ b,
+                                                        const int* n_rows, T* __restrict__ y, int d, float eps, int rows_static) {
     const int lane = threadIdx.x & 31, row0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * ROWS;
     float4 gm[NC], bt[NC];
 #pragma unroll
@@ -454,8 +455,8 @@ __global__ void __launch_bounds__(256) k_layernorm_rows(const float* __restrict_
 
 // Any other width: one warp per row, the row read three times.
 template <typename T>
-__global__ void k_layernorm(const float* __restrict__ x, const float* __restrict__ g, const float* __restrict__ b,
-                            const int* __restrict__ n_rows, T* __restrict__ y, int d, float eps, int rows_static) {
+__global__ void k_layernorm(const float* x, const float* __restrict__ g, const float* __restrict__ b,
+                            const int* n_rows, T* __restrict__ y, int d, float eps, int rows_static) {
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     pdl_launch_dependents();
     pdl_wait();
@@ -473,9 +474,9 @@ __global__ void k_layernorm(const float* __restrict__ x, const float* __restrict
 // Final LayerNorm of the verify rows together with the pre-pass logit of each row's draft (the dot product of the
 // normalised, operand-rounded row with the draft's embedding row): one warp per row, rows of up to 128 NC elements in registers.
 template <typename T, int NC>
-__global__ void k_layernorm_ld(const float* __restrict__ x, const float* __restrict__ g, const float* __restrict__ b,
-                               T* __restrict__ y, int d, float eps, const T* __restrict__ E, const int* __restrict__ draft,
-                               const int* __restrict__ slot_seq, const int* __restrict__ n_rows, int k, int vocab,
+__global__ void k_layernorm_ld(const float* x, const float* __restrict__ g, const float* __restrict__ b,
+                               T* __restrict__ y, int d, float eps, const T* __restrict__ E, const int* draft,
+                               const int* slot_seq, const int* n_rows, int k, int vocab,
                                float* __restrict__ ld, int* __restrict__ ld_id) {
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     float4 gm[NC], bt[NC];
@@ -756,8 +757,8 @@ __global__ void __launch_bounds__(256) k_gemm_simt(GemmArgs<T> g) {
 // Row c < k of a sequence checks draft c+1: its logit is the dot product of the row's
 // normalised hidden state with the draft's embedding row.  Row k (bonus) has no draft.
 template <typename T>
-__global__ void k_draft_logit(const T* __restrict__ y, const T* __restrict__ E, const int* __restrict__ draft,
-                              const int* __restrict__ slot_seq, const int* __restrict__ n_rows, int k, int d, int vocab,
+__global__ void k_draft_logit(const T* y, const T* __restrict__ E, const int* draft,
+                              const int* slot_seq, const int* n_rows, int k, int d, int vocab,
                               float* __restrict__ ld, int* __restrict__ ld_id) {
     int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     int lane = threadIdx.x & 31;
@@ -800,7 +801,7 @@ __global__ void k_draft_logit(const T* __restrict__ y, const T* __restrict__ E, 
 // ------------------------------------------------------------------ commit / rollback (Eq. 3)
 // Appends drafts[0..keep) and the next token to sequence b, cuts after the first EOS and at max_tgt.
 // Cache rows beyond the new length are simply dead: the next block overwrites them.
-__device__ __forceinline__ void commit_sequence(const Session& s, int b, const int* __restrict__ draft, int keep, int next,
+__device__ __forceinline__ void commit_sequence(const Session& s, int b, const int* draft, int keep, int next,
                                                 int k, int eos) {
     if (s.finished[b]) return;
     int j = s.len[b];
@@ -827,10 +828,10 @@ __device__ __forceinline__ void commit_sequence(const Session& s, int b, const i
 // The same for one warp, which holds the sequence's state and (lane c) draft c from before: one pass instead of a chain of dependent
 // loads per token (4 us of a 237 us iteration at six accepted drafts).  Returns whether the sequence ended here.
 struct CommitState { int finished, len, max_tgt, tok; };
-__device__ __forceinline__ CommitState commit_fetch(const Session& s, int b, const int* __restrict__ draft, int k, int lane) {
+__device__ __forceinline__ CommitState commit_fetch(const Session& s, int b, const int* draft, int k, int lane) {
     return CommitState{s.finished[b], s.len[b], s.max_tgt[b], lane < k ? draft[b * k + lane] : -1};
 }
-__device__ __forceinline__ bool commit_sequence_warp(const Session& s, int b, const int* __restrict__ draft, int a, int next, int k, int eos,
+__device__ __forceinline__ bool commit_sequence_warp(const Session& s, int b, const int* draft, int a, int next, int k, int eos,
                                                      const CommitState& st, int lane, int& len) {
     len = st.len;
     if (st.finished) return false;
@@ -883,10 +884,10 @@ struct FusedCommit { Session s; const int* draft; int eos; unsigned long long* p
 // ------------------------------------------------------------------ acceptance scan (Eq. 7-9)
 // One block per slot (verify block): warps merge the per-tile statistics of the k+1 rows, thread 0
 // finds the first rejected draft.  row_stats (optional) receives 6 floats per row.
-static __global__ void k_accept(const RowPart* __restrict__ part, int n_tiles, const float* __restrict__ ld,
-                         const int* __restrict__ ld_id, int k, int beta, float tau, int* __restrict__ accepted,
+static __global__ void k_accept(const RowPart* part, int n_tiles, const float* ld,
+                         const int* ld_id, int k, int beta, float tau, int* __restrict__ accepted,
                          int* __restrict__ bif, int* __restrict__ accepted2, int* __restrict__ bif2, float* __restrict__ row_stats,
-                         int want_sum, const int* __restrict__ slot_seq, FusedCommit fc) {
+                         int want_sum, const int* slot_seq, FusedCommit fc) {
     extern __shared__ unsigned char sm_acc[];
     RowPart* rs = reinterpret_cast<RowPart*>(sm_acc);       // [k+1]
     __shared__ unsigned char ok_s[256];                     // row c passes both tests (k <= 255 rows take this path)
@@ -981,9 +982,9 @@ static __global__ void k_accept(const RowPart* __restrict__ part, int n_tiles, c
 // ------------------------------------------------------------------ drafter argmax
 // script (optional; benchmark / test hook): draft i of a sequence with j committed tokens is replaced by
 // script[b * stride + j + i] wherever that entry is >= 0 (len = the committed lengths, k = drafts per sequence).
-static __global__ void k_draft_argmax(const RowPart* __restrict__ part, int n_tiles, const int* __restrict__ n_rows,
-                               const int* __restrict__ slot, int* __restrict__ draft, const int* __restrict__ script,
-                               int stride, const int* __restrict__ len, int k) {
+static __global__ void k_draft_argmax(const RowPart* part, int n_tiles, const int* n_rows,
+                               const int* slot, int* __restrict__ draft, const int* __restrict__ script,
+                               int stride, const int* len, int k) {
     int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     int lane = threadIdx.x & 31;
     pdl_launch_dependents();
