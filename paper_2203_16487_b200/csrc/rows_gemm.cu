@@ -296,15 +296,15 @@ constexpr int RG_MAX_SMEM = 227 * 1024 - 1024;
 
 // K slices (CTAs of a cluster) per output tile: reductions of 1024 and more are split (26 rows, K = 2048: 2 slices 180 us per verify step,
 // 4 slices 186, 1 slice of 32 rows 186; 208 rows: 4 slices 284, 2 slices 304).
-static int rg_split(int K, int rows_ub, bool cluster) {
+static int rg_split(int N, int K, int rows_ub, bool cluster) {
     if (K < 1024 || !cluster) return 1;
-    if (rows_ub > RG_LN_ROWS && K % 32 == 0) return 4;
+    if (rows_ub > rg_ln_rows(min(N, K)) && K % 32 == 0) return 4;
     return K % 16 == 0 ? 2 : 1;
 }
 bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster) {
     if (rows_ub > RG_MAX_ROWS || K % 16 || N % 16 || lda % 8) return false;
     if (epi != EPI_STORE && epi != EPI_RELU && epi != EPI_GELU && epi != EPI_RESID && epi != EPI_QKV) return false;
-    const int Kc = K / (epi == EPI_RESID ? rg_split(K, rows_ub, cluster) : 1);
+    const int Kc = K / (epi == EPI_RESID ? rg_split(N, K, rows_ub, cluster) : 1);
     return (int)RgCfg<2, 8, 2, 4>::smem(Kc) <= RG_MAX_SMEM;                     // (the largest tile any of the launches below uses)
 }
 
@@ -313,7 +313,7 @@ bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster) {
 template <int EPI, int NC>
 inline cudaError_t rg_launch_out(const RowsArgs& a, int rows_ub, bool pdl, cudaStream_t st) {
     const bool wide = a.g.N >= 1024;
-    if (NC == 0 && rows_ub > RG_LN_ROWS) {
+    if (NC == 0 && rows_ub > rg_ln_rows(min(a.g.N, a.g.K))) {
         return rg_launch_one<EPI, 0, 2, 8, 2, 1>(a, rows_ub, pdl, st);
     }
     if (wide) return rg_launch_one<EPI, NC, 1, 8, 2, 1>(a, rows_ub, pdl, st);
@@ -321,8 +321,8 @@ inline cudaError_t rg_launch_out(const RowsArgs& a, int rows_ub, bool pdl, cudaS
     return rg_launch_one<EPI, NC, 1, 2, 1, 1>(a, rows_ub, pdl, st);
 }
 static cudaError_t rg_launch_resid(const RowsArgs& a, int rows_ub, bool cluster, bool pdl, cudaStream_t st) {
-    const int split = rg_split(a.g.K, rows_ub, cluster);
-    if (rows_ub > RG_LN_ROWS) {
+    const int split = rg_split(a.g.N, a.g.K, rows_ub, cluster);
+    if (rows_ub > rg_ln_rows(min(a.g.N, a.g.K))) {
         if (split == 4) return rg_launch_one<EPI_RESID, 0, 2, 8, 2, 4>(a, rows_ub, pdl, st);
         return rg_launch_one<EPI_RESID, 0, 2, 8, 2, 1>(a, rows_ub, pdl, st);
     }

@@ -12,14 +12,18 @@ struct RowsArgs {
     int* err_word;               // raised when a bounded wait gives up
 };
 
-// Up to here this kernel beats the 128-row tensor-core tiles (verify step, us, before / after: 26 rows 220 / 178, 52 rows 310 / 186, 104 rows
-// 346 / 211, 208 rows 363 / 278, 312 rows 373 / 339, 364 rows 378 / 354; 416 rows 381 / 389).  Every CTA reads all of its
-// operands from L2 once, so the traffic grows with rows x columns while a tile of 128 rows shares its weights.
-constexpr int RG_MAX_ROWS = 384;
-// The two encoders run side by side on two streams and fill the SMs sooner (time to the first tokens: 160 rows 757 / 683, 320 rows 828 / 856).
-constexpr int RG_MAX_ROWS_ENC = 208;
-// Up to here the LayerNorm in front runs inside the GEMM (16-row tiles; 130 rows 260 / 232), beyond it is a launch of its own (156 rows 264 / 274).
-constexpr int RG_LN_ROWS = 144;
+// Row limits, by the width of the model (the smaller side of a weight matrix).  Every CTA reads all of its operands from L2 once, so the
+// traffic grows with rows x columns, while a tensor-core tile of 128 rows shares its weights among them.
+constexpr int RG_MAX_ROWS = 384;                             // in general; shapes that the tensor-core tiles serve too go over to them at
+// (verify step, us, this kernel / tiles: width 512: 104 rows 191 / 241, 208 rows 238 / 253, 260 rows 295 / 294, 364 rows 343 / 298;
+// width 768: 78 rows 272 / 298, 104 rows 304 / 306, 156 rows 363 / 342)
+__host__ __device__ constexpr int rg_tile_rows(int width) { return width <= 512 ? 256 : 112; }
+// ... and in the encoders, two of which run side by side on two streams and fill the SMs sooner (first tokens: width 512: 60 rows
+// 497 / 560, 180 rows 650 / 656, 240 rows 684 / 684; width 768: 60 rows 577 / 543).
+__host__ __device__ constexpr int rg_tile_rows_enc(int width) { return width <= 512 ? 208 : 48; }
+// Up to here the LayerNorm in front runs inside the GEMM, on 16-row tiles; beyond it is a launch of its own (inside / in front: width 512,
+// 130 rows 202 / 218; width 768, 104 rows 330 / 304).
+__host__ __device__ constexpr int rg_ln_rows(int width) { return width <= 512 ? 144 : 80; }
 
 bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster);
 inline bool rg_ln_width(int K) { return K == 256 || K == 512 || K == 768; }    // widths that the LayerNorm prologue exists for

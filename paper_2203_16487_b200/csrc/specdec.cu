@@ -480,12 +480,11 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
               int rows_ub, void* out, int ldo, float* resid, cudaStream_t st, const float* ldv, const int* ld_id,
               int* n_tiles_out, const KvDest* kv, const LnSpec* lnp) {
     if (rows_ub <= 0) return 0;
-    // (not in the encoders: the two encoders run side by side on two streams, and the weight-streaming kernels' 64-256
-    // CTAs per launch get in each other's way there -- 440 us against 386 us with 8-32-CTA tile GEMMs for a 32-token source)
     // few rows: the weight-streaming kernel, with the LayerNorm inside where it has one
-    const bool few = std::is_same<T, bf16>::value && h->use_skinny && h->use_tc && rows_ub <= (cnt == CNT_ENC ? (h->enc_skinny ? RG_MAX_ROWS_ENC : 0) : RG_MAX_ROWS) &&
+    const int width = std::min(N, K), tile_rows = sd::tc_supported(N, K) ? (cnt == CNT_ENC ? rg_tile_rows_enc(width) : rg_tile_rows(width)) : RG_MAX_ROWS;
+    const bool few = std::is_same<T, bf16>::value && h->use_skinny && h->use_tc && rows_ub <= tile_rows && (cnt != CNT_ENC || h->enc_skinny) &&
                      !(epi == EPI_RESID && h->use_ln_fuse) && rg_supported(epi, N, K, lnp ? K : lda, rows_ub, h->use_sk_cluster != 0);
-    const bool ln_inside = few && lnp && rows_ub <= RG_LN_ROWS && rg_ln_width(K);
+    const bool ln_inside = few && lnp && rows_ub <= rg_ln_rows(width) && rg_ln_width(K);
     const bool few32 = std::is_same<T, float>::value && h->use_skinny && rf_supported(epi, N, K, lnp ? K : lda, rows_ub);
     const bool ln32 = few32 && lnp && rf_ln_width(K);
     if (lnp && !ln_inside && !ln32) {  // separate normalisation launch, then a plain GEMM on its output
