@@ -71,8 +71,65 @@ struct QueryArgs {
     const bf16* w; const float* b;                        // [n_heads * 64, K]
 };
 template <int QNC> struct QueryCfg {                      // K = 128 QNC
-    static constexpr int K = 128 * QNC, PITCH = K * 2 + 16, RP = 72;              // bytes per row; floats per row of partial sums
+    static constexpr int K = 128 * QNC, PITCH = K * 2 + 16;                           // bytes per row
     static constexpr int OPS = QNC ? (16 + 64) * PITCH : 0;
+};
+
+// The output projection and the residual sum inside the attention kernel (few rows): x_out[r] = x_in[x_index ? x_index[r] : r] + O Wo^T + bo.
+struct OutArgs {
+    const bf16* w; const float* b;                        // [K, K], K = 64 n_heads
+    const float* x_in; const int* x_index; float* x_out;  // fp32 rows [rows, K]
+};
+// Bytes behind the ring: 16 rows and 64 rows of weights for each projection that runs inside.
+template <int QNC, int ON> struct ProjCfg { static constexpr int OPS = QueryCfg<QNC>::OPS + QueryCfg<ON / 2>::OPS; };
+
+__device__ __forceinline__ void attn_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void attn_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// 16 x 64 partial products of a CTA's eight warps: warp = (K slice of four, half of the columns); A: 16 rows, W: 64 rows of PITCH bytes.
+// The slices meet in `red` ([4][16][72] floats); thread t then holds row t / 16, columns 4 (t % 16) .. + 3 of the sum.
+template <int K>
+struct Proj64 {
+    static constexpr int PITCH = K * 2 + 16, RP = 72, STEPS = K / 64;
+    uint32_t bfr[STEPS][4][2];
+    __device__ __forceinline__ void load_w(uint32_t ws, int warp, int lane) {
+        const uint32_t bp = ws + ((warp & 1) * 32 + (lane & 7) + (lane >> 4) * 8) * PITCH + (warp >> 1) * STEPS * 32 + ((lane >> 3) & 1) * 16;
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s) {
+            ldsm_x4(bp + s * 32, bfr[s][0][0], bfr[s][0][1], bfr[s][1][0], bfr[s][1][1]);
+            ldsm_x4(bp + 16 * PITCH + s * 32, bfr[s][2][0], bfr[s][2][1], bfr[s][3][0], bfr[s][3][1]);
+        }
+    }
+    __device__ __forceinline__ void multiply(uint32_t as, float* red, int warp, int lane) {
+        float c[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) c[j][e] = 0.f;
+        const uint32_t ap = as + (lane & 15) * PITCH + (warp >> 1) * STEPS * 32 + (lane >> 4) * 16;
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s) {
+            uint32_t af[4];
+            ldsm_x4(ap + s * 32, af[0], af[1], af[2], af[3]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) mma_bf16(c[j], af, bfr[s][j][0], bfr[s][j][1]);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float* p = red + ((warp >> 1) * 16 + (lane >> 2)) * RP + (warp & 1) * 32 + j * 8 + (lane & 3) * 2;
+            *reinterpret_cast<float2*>(p) = make_float2(c[j][0], c[j][1]);
+            *reinterpret_cast<float2*>(p + 8 * RP) = make_float2(c[j][2], c[j][3]);
+        }
+    }
+    static __device__ __forceinline__ float4 sum(const float* red, int tid) {
+        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const float4 u = *reinterpret_cast<const float4*>(red + (s * 16 + (tid >> 4)) * RP + (tid & 15) * 4);
+            t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+        }
+        return t;
+    }
 };
 
 // MT row tiles of 16 queries x KG key groups = MT KG warps; a key block holds KW keys for each group; NS stages.
@@ -91,10 +148,17 @@ struct AttnCfg {
 
 // QNC > 0: the queries are projected here (QueryArgs; MT = 1, KG = 8).  The CTA's 64 rows of Wq are requested ahead of the wait, the
 // 16 rows normalised behind it; one launch and its round trip through memory less per layer (26 rows, K = 512: 5.5 -> 4.4 us).
-template <bool PAGED, int MT, int KG, int KW, int NS, int QNC = 0>
-__global__ void __launch_bounds__(MT * KG * 32) k_attn(AttnTcArgs a, QueryArgs qa) {
+//
+// ON > 0: the heads of a query tile are a cluster of ON CTAs, and the output projection runs here too (OutArgs).  Bound by the same chain of round trips:
+// every CTA sends its head's 16 rows (bf16, as they would go to memory) to the shared memory of all, multiplies the 16 whole rows by its own 64 rows
+// of Wo and adds the residual.  Wo is requested ahead of the wait and turned into register fragments while the queries are on their way, so
+// that only the exchange (0.5 us), 32 MMAs a warp and the sum of four K slices follow the attention: a launch and its round trip less
+// (verify step of 26 rows, both attentions of six layers: 156.5 -> 147.2 us; with Wo fetched behind the wait 155.2).
+template <bool PAGED, int MT, int KG, int KW, int NS, int QNC = 0, int ON = 0>
+__global__ void __launch_bounds__(MT * KG * 32) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {
     using C = AttnCfg<MT, KG, KW>;
-    static_assert(QNC == 0 || (MT == 1 && KG == 8), "the projection is laid out for eight warps and 16 rows");
+    static_assert((QNC == 0 && ON == 0) || (MT == 1 && KG == 8), "the projections are laid out for eight warps and 16 rows");
+    static_assert(QNC == 0 || ON == 0 || ON == 2 * QNC, "one width");
     static_assert(NS >= 1 && NS <= 4 && KW % 16 == 0, "ring depth, keys per warp");
     constexpr int THREADS = MT * KG * 32, KB = C::KB, NT = KW / 8, BM = MT * 16;
     extern __shared__ __align__(128) unsigned char sm[];
@@ -127,7 +191,20 @@ __global__ void __launch_bounds__(MT * KG * 32) k_attn(AttnTcArgs a, QueryArgs q
             lbet[c] = ldg_pinned(reinterpret_cast<const float4*>(qa.ln_b + lane * 4 + c * 128));
         }
     }
-    int* s_row = reinterpret_cast<int*>(qops + QC::OPS);                          // paged: K / V row of every key
+    using OC = QueryCfg<ON ? ON / 2 : 2>;
+    const uint32_t oops = (uint32_t)__cvta_generic_to_shared(qops) + QC::OPS;   // ON: 16 rows that the cluster's CTAs fill, this head's 64 rows of Wo
+    Proj64<OC::K> wo;
+    float4 res = make_float4(0.f, 0.f, 0.f, 0.f), ob = res;              // ON: the residual and the bias of this thread's four outputs
+    if constexpr (ON > 0) {
+        const bf16* w = oa.w + (size_t)h * 64 * OC::K;
+        for (int i = tid; i < 64 * (OC::K / 8); i += THREADS) {
+            const int r = i / (OC::K / 8), c = i % (OC::K / 8);
+            cp_async16(oops + (16 + r) * OC::PITCH + c * 16, w + (size_t)r * OC::K + c * 8);
+        }
+        attn_cluster_arrive();
+        ob = ldg_pinned(reinterpret_cast<const float4*>(oa.b + h * 64 + (tid & 15) * 4));
+    }
+    int* s_row = reinterpret_cast<int*>(qops + ProjCfg<QNC, ON>::OPS);            // paged: K / V row of every key
     if (PAGED) {
         for (int t = tid; t < a.max_keys; t += THREADS) s_row[t] = (int)a.pg.row(b, t);
         __syncthreads();
@@ -166,10 +243,15 @@ __global__ void __launch_bounds__(MT * KG * 32) k_attn(AttnTcArgs a, QueryArgs q
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (tid == 0) s_nkmax = m;
     }
+    if constexpr (ON > 0 && QNC == 0) asm volatile("cp.async.commit_group;" ::: "memory");
     __syncthreads();
     const int nkmax = s_nkmax, nblk = max((nkmax + KB - 1) / KB, 1);
     pdl_launch_dependents();
     pdl_wait();                                  // ... and everything the predecessor kernels wrote after it
+    if constexpr (ON > 0) {
+        const int r = tid >> 4;
+        if (r < nq) res = *reinterpret_cast<const float4*>(oa.x_in + (size_t)(oa.x_index ? oa.x_index[r0 + r] : r0 + r) * OC::K + h * 64 + (tid & 15) * 4);
+    }
     if constexpr (QNC == 0) {
         for (int r = t0; r < BM; r += THREADS / 8) {
             if (r < nq) {
@@ -189,6 +271,13 @@ __global__ void __launch_bounds__(MT * KG * 32) k_attn(AttnTcArgs a, QueryArgs q
                 const int m = warp + 8 * s;
                 xv[s][c] = m < nq ? *reinterpret_cast<const float4*>(qa.x + (size_t)(r0 + m) * QC::K + lane * 4 + c * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
+        const float4 v = __ldg(reinterpret_cast<const float4*>(qa.b + h * 64 + (tid & 15) * 4));
+        // while the rows are on their way: the weights, requested before the wait, become fragments
+        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        Proj64<QC::K> pj;
+        pj.load_w((uint32_t)__cvta_generic_to_shared(qops) + 16 * QC::PITCH, warp, lane);
+        if constexpr (ON > 0) wo.load_w(oops + 16 * OC::PITCH, warp, lane);
         float mu[2] = {0.f, 0.f}, rs[2] = {0.f, 0.f};
 #pragma unroll
         for (int s = 0; s < 2; ++s)
@@ -221,45 +310,13 @@ __global__ void __launch_bounds__(MT * KG * 32) k_attn(AttnTcArgs a, QueryArgs q
                     m < nq ? make_uint2(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1)) : make_uint2(0u, 0u);
             }
         }
-        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");       // weights (and the keys before the wait)
         __syncthreads();
-        // warp = (K slice of four, half of the head's columns)
-        const int wk = warp >> 1, wn = warp & 1;
-        constexpr int STEPS = QC::K / 64;
-        float qc[4][4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) qc[j][e] = 0.f;
         const uint32_t ops = (uint32_t)__cvta_generic_to_shared(qops);
-        const uint32_t ap = ops + (lane & 15) * QC::PITCH + wk * STEPS * 32 + (lane >> 4) * 16;
-        const uint32_t bp = ops + (16 + wn * 32 + (lane & 7) + (lane >> 4) * 8) * QC::PITCH + wk * STEPS * 32 + ((lane >> 3) & 1) * 16;
-#pragma unroll
-        for (int s = 0; s < STEPS; ++s) {
-            uint32_t af[4], bfr[4][2];
-            ldsm_x4(ap + s * 32, af[0], af[1], af[2], af[3]);
-            ldsm_x4(bp + s * 32, bfr[0][0], bfr[0][1], bfr[1][0], bfr[1][1]);
-            ldsm_x4(bp + 16 * QC::PITCH + s * 32, bfr[2][0], bfr[2][1], bfr[3][0], bfr[3][1]);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) mma_bf16(qc[j], af, bfr[j][0], bfr[j][1]);
-        }
-        __syncthreads();                                  // the operands are dead: partial sums take their place
-        float* red = reinterpret_cast<float*>(qops);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            float* p = red + (wk * 16 + (lane >> 2)) * QC::RP + wn * 32 + j * 8 + (lane & 3) * 2;
-            *reinterpret_cast<float2*>(p) = make_float2(qc[j][0], qc[j][1]);
-            *reinterpret_cast<float2*>(p + 8 * QC::RP) = make_float2(qc[j][2], qc[j][3]);
-        }
+        float* red = reinterpret_cast<float*>(Sp + max(ring * C::STAGE, C::MERGE) + 16 * QC::PITCH);        // (weights that are dead by then)
+        pj.multiply(ops, red, warp, lane);
         __syncthreads();
         const int r = tid >> 4, c = (tid & 15) * 4;
-        float4 v = __ldg(reinterpret_cast<const float4*>(qa.b + h * 64 + c));
-        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            const float4 u = *reinterpret_cast<const float4*>(red + (s * 16 + r) * QC::RP + c);
-            t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
-        }
+        const float4 t = Proj64<QC::K>::sum(red, tid);
         __nv_bfloat162 p0 = __floats2bfloat162_rn(t.x + v.x, t.y + v.y), p1 = __floats2bfloat162_rn(t.z + v.z, t.w + v.w);
         *reinterpret_cast<uint2*>(sm + swz(r, c >> 3) + (c & 7) * 2) = make_uint2(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1));
     }
@@ -288,6 +345,11 @@ __global__ void __launch_bounds__(MT * KG * 32) k_attn(AttnTcArgs a, QueryArgs q
     for (int o = 4; o < 32; o <<= 1) nkall = min(nkall, __shfl_xor_sync(0xffffffffu, nkall, o));
 
     while (issued < min(ring, nblk)) issue();
+    if constexpr (ON > 0 && QNC == 0) {          // while the queries are on their way: the weights, requested before the wait, become fragments
+        cp_wait_pending(issued);
+        __syncthreads();
+        wo.load_w(oops + 16 * OC::PITCH, warp, lane);
+    }
     for (int blk = 0; blk < nblk; ++blk) {
         cp_wait_pending(issued - blk - 1);
         __syncthreads();
@@ -412,7 +474,37 @@ __global__ void __launch_bounds__(MT * KG * 32) k_attn(AttnTcArgs a, QueryArgs q
             den = fmaf(mML[(mt * KG + q) * 32 + rr * 2 + 1], f[q], den);
         }
         const float inv = den > 0.f ? 1.0f / den : 0.f;
-        if (r < nq) {
+        if constexpr (ON > 0) {
+            static_assert(PER == 4, "eight key groups");
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < KG; ++q) {
+                const float4 t = *reinterpret_cast<const float4*>(mO + ((mt * KG + q) * 16 + rr) * 68 + c0);
+                x.x = fmaf(t.x, f[q], x.x); x.y = fmaf(t.y, f[q], x.y); x.z = fmaf(t.z, f[q], x.z); x.w = fmaf(t.w, f[q], x.w);
+            }
+            __nv_bfloat162 p0 = __floats2bfloat162_rn(x.x * inv, x.y * inv), p1 = __floats2bfloat162_rn(x.z * inv, x.w * inv);
+            const uint32_t u0 = *reinterpret_cast<uint32_t*>(&p0), u1 = *reinterpret_cast<uint32_t*>(&p1);
+            const uint32_t w0 = __shfl_xor_sync(0xffffffffu, u0, 1), w1 = __shfl_xor_sync(0xffffffffu, u1, 1);
+            const bool odd = lane & 1;
+            // eight columns of a row: the even lane sends them to the lower half of the cluster, the odd lane to the upper
+            const uint32_t dst = oops + rr * OC::PITCH + (h * 64 + kg * CW) * 2;
+            attn_cluster_wait();                          // every CTA of the cluster has begun and its 16 rows are free
+#pragma unroll
+            for (int i = 0; i < ON / 2; ++i) {
+                uint32_t ra;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(dst), "r"((odd ? ON / 2 : 0) + i));
+                asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
+                             ::"r"(ra), "r"(odd ? w0 : u0), "r"(odd ? w1 : u1), "r"(odd ? u0 : w0), "r"(odd ? u1 : w1) : "memory");
+            }
+            attn_cluster_arrive();
+            attn_cluster_wait();
+            wo.multiply(oops, mO, warp, lane);             // (the partial outputs of the key groups are dead)
+            __syncthreads();
+            const float4 t = Proj64<OC::K>::sum(mO, tid);
+            if ((tid >> 4) < nq)
+                *reinterpret_cast<float4*>(oa.x_out + (size_t)(r0 + (tid >> 4)) * OC::K + h * 64 + (tid & 15) * 4) =
+                    make_float4(t.x + ob.x + res.x, t.y + ob.y + res.y, t.z + ob.z + res.z, t.w + ob.w + res.w);
+        } else if (r < nq) {
             bf16* o = a.out + (size_t)(r0 + r) * a.out_stride + h * 64 + c0;
 #pragma unroll
             for (int c = 0; c < PER; c += 4) {

@@ -408,6 +408,20 @@ cudaError_t launch_pdl(specdec_handle* h, void (*kernel)(KArgs...), dim3 grid, d
     cfg.attrs = attr; cfg.numAttrs = h->use_pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
+// ... in clusters of grid.y CTAs
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_heads(specdec_handle* h, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = grid.y; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = h->use_pdl ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 // Row count of a pass where the host knows it, else -1 (the kernels read it from the device).
 inline int static_rows(const specdec_handle* h, int cnt, int rows_ub) {
@@ -570,7 +584,7 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
 template <typename T>
 int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const int* q_index, const void* k, const void* v,
          int kv_stride, const int* kv_off, const Rows& r, const int* nkeys, int cnt, int rows_ub, int q_ub, void* out,
-         int out_stride, int n_heads, int d_head, int max_keys, cudaStream_t st, const int* pre_keys = nullptr, const QueryArgs* qp = nullptr) {
+         int out_stride, int n_heads, int d_head, int max_keys, cudaStream_t st, const int* pre_keys = nullptr, const QueryArgs* qp = nullptr, const OutArgs* op = nullptr) {
     if (rows_ub <= 0) return 0;
     if constexpr (std::is_same<T, bf16>::value) {
         if (h->use_tc_attn && d_head == 64) {
@@ -583,10 +597,22 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             a.scale = 1.0f / sqrtf((float)d_head);
             const int n_seq = cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub);
             QueryArgs qa{};
+            OutArgs oa{};
+            if (qp) qa = *qp;
+            if (op) {                                        // the heads of a tile as one cluster (4 or 8)
+                oa = *op;
+                auto goo = [&](auto* kernel, int bytes) {
+                    const cudaError_t e = launch_pdl_heads(h, kernel, dim3(cdiv(q_ub, 16), n_heads, h->B), dim3(256), AttnCfg<1, 8, 16>::smem(max_keys, 3, paged, bytes), st, a, qa, oa);
+                    if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
+                    KCHECK(h);
+                    return 0;
+                };
+                if (n_heads == 4) return goo(qp ? k_attn<false, 1, 8, 16, 3, 2, 4> : paged ? k_attn<true, 1, 8, 16, 3, 0, 4> : k_attn<false, 1, 8, 16, 3, 0, 4>, qp ? ProjCfg<2, 4>::OPS : ProjCfg<0, 4>::OPS);
+                return goo(qp ? k_attn<false, 1, 8, 16, 3, 4, 8> : paged ? k_attn<true, 1, 8, 16, 3, 0, 8> : k_attn<false, 1, 8, 16, 3, 0, 8>, qp ? ProjCfg<4, 8>::OPS : ProjCfg<0, 8>::OPS);
+            }
             if (qp) {
-                qa = *qp;
                 auto goq = [&](auto* kernel, int bytes) {
-                    const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, 16), n_heads, h->B), dim3(256), AttnCfg<1, 8, 16>::smem(max_keys, 3, false, bytes), st, a, qa);
+                    const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, 16), n_heads, h->B), dim3(256), AttnCfg<1, 8, 16>::smem(max_keys, 3, false, bytes), st, a, qa, oa);
                     if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
                     KCHECK(h);
                     return 0;
@@ -598,7 +624,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
                 }
             }
             auto go = [&](auto* kernel, int bm, int warps, size_t smem) {
-                const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, bm), n_heads, h->B), dim3(warps * 32), smem, st, a, qa);
+                const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, bm), n_heads, h->B), dim3(warps * 32), smem, st, a, qa, oa);
                 if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
                 KCHECK(h);
                 return 0;
@@ -657,10 +683,10 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
 template <typename T>
 int attn(specdec_handle* h, bool paged, const void* q, int q_stride, const int* q_index, const void* k, const void* v,
          int kv_stride, const int* kv_off, const Rows& r, const int* nkeys, int cnt, int rows_ub, int q_ub, void* out,
-         int out_stride, int n_heads, int d_head, int max_keys, cudaStream_t st, const int* pre_keys = nullptr, const QueryArgs* qp = nullptr) {
+         int out_stride, int n_heads, int d_head, int max_keys, cudaStream_t st, const int* pre_keys = nullptr, const QueryArgs* qp = nullptr, const OutArgs* op = nullptr) {
     TRY(attn_once<T>(h, paged, q, q_stride, q_index, k, v, kv_stride, kv_off, r, nkeys, cnt, rows_ub, q_ub, out, out_stride,
-                     n_heads, d_head, max_keys, st, pre_keys, qp));
-    if (h->diag_repeat & 1)
+                     n_heads, d_head, max_keys, st, pre_keys, qp, op));
+    if ((h->diag_repeat & 1) && !op)
         TRY(attn_once<T>(h, paged, q, q_stride, q_index, k, v, kv_stride, kv_off, r, nkeys, cnt, rows_ub, q_ub, out, out_stride,
                          n_heads, d_head, max_keys, st, pre_keys, qp));
     return 0;
@@ -682,6 +708,21 @@ void prof_collect(specdec_handle* h) {
         if (cudaEventElapsedTime(&t, h->prof_ev[i], h->prof_ev[i + 1]) == cudaSuccess) { h->prof_ms += t; ++h->prof_launches; }
     }
     h->prof_n = 0;
+}
+
+// Whether the attention kernel goes on to the output projection and the residual sum: for the two head counts that are one cluster, and few CTAs, since each
+// wants an SM of its own next to the GEMMs before and after it.  With the queries projected too (200 KB a CTA): 32 CTAs and 48 rows, the GEMMs in turn being
+// 128 CTAs beyond (verify step, us, without / with: 26 rows 151 / 147, 44 rows 156 / 151, 52 rows 162 / 164, 88 rows 183 / 188).  Otherwise 64 CTAs
+// (10 rows 149 / 146, 26 rows 157 / 151, 52 rows 163 / 162; 80 CTAs 203 / 205, 128 CTAs 158 / 196), or 96 where a gathering launch goes with it (drafts
+// of 6 x 25 rows 108 / 103).  Blocks of a few rows leave nothing to gain (greedy steps 2 % slower).
+enum OutUse { OUT_SELF, OUT_GATHERS, OUT_QUERIES };
+bool out_inside(const specdec_handle* h, int d_head, int q_ub, int n_heads, int cnt, int rows_ub, int max_keys, OutUse use) {
+    if (!h->use_tc || !h->use_skinny || !h->use_tc_attn || !h->use_sk_cluster || h->use_ln_fuse || (h->diag_repeat & 1)) return false;
+    if (d_head != 64 || (n_heads != 4 && n_heads != 8) || q_ub <= 4) return false;
+    const long long ctas = (long long)cdiv(q_ub, 16) * n_heads * (cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub));
+    if (ctas > (use == OUT_QUERIES ? 32 : use == OUT_GATHERS ? 96 : 64) || (use == OUT_QUERIES && rows_ub > 48)) return false;
+    const int ops = use == OUT_QUERIES ? ProjCfg<4, 8>::OPS : ProjCfg<0, 8>::OPS;
+    return AttnCfg<1, 8, 16>::smem(max_keys, 3, use != OUT_QUERIES, ops) <= 227 * 1024 - 2048;      // (with the queries: up to 128 keys)
 }
 
 // One pre-LN block on `rows_ub` rows of the residual stream x (encoder: no cross-attention).
@@ -712,13 +753,16 @@ int block_self(specdec_handle* h, const ModelW& m, const LayerW& w, float* x, co
             KCHECK(h);
         }
     }
+    const bool inside = std::is_same<T, bf16>::value && out_inside(h, dh, q_ub, H, cnt, rows_ub, max_keys, OUT_SELF);
+    const OutArgs oa{(const bf16*)w.o_w, w.o_b, x, nullptr, x};
     if (verify) {
         TRY(attn<T>(h, true, h->qkv, 3 * d, nullptr, kc, vc, d, nullptr, r, r.nk_self, cnt,
-                    rows_ub, q_ub, h->att, d, H, dh, max_keys, st, pre_keys));
+                    rows_ub, q_ub, h->att, d, H, dh, max_keys, st, pre_keys, nullptr, inside ? &oa : nullptr));
     } else {
         TRY(attn<T>(h, false, h->qkv, 3 * d, nullptr, (char*)h->qkv + (size_t)d * e, (char*)h->qkv + (size_t)2 * d * e,
-                    3 * d, r.kv_off, r, r.nk_self, cnt, rows_ub, q_ub, h->att, d, H, dh, max_keys, st));
+                    3 * d, r.kv_off, r, r.nk_self, cnt, rows_ub, q_ub, h->att, d, H, dh, max_keys, st, nullptr, nullptr, inside ? &oa : nullptr));
     }
+    if (inside) return 0;
     h->next_ln = {next_g, next_b, h->y};             // the LayerNorm that reads the residual stream next
     TRY(gemm<T>(h, EPI_RESID, h->att, d, w.o_w, w.o_b, d, d, cnt, rows_ub, nullptr, 0, x, st));
     return 0;
@@ -739,11 +783,14 @@ int block_cross(specdec_handle* h, const ModelW& m, const LayerW& w, float* x, c
     const LnSpec lc{x, w.lnc_g, w.lnc_b};
     QueryArgs qa{};
     const bool inside = std::is_same<T, bf16>::value && query_inside(h, d, dh, q_ub, H, h->S_max);
+    const bool out = inside && out_inside(h, dh, q_ub, H, cnt, rows_ub, h->S_max, OUT_QUERIES);
+    const OutArgs oa{(const bf16*)w.co_w, w.co_b, x, nullptr, x};
     if (inside) qa = QueryArgs{x, w.lnc_g, w.lnc_b, 1e-5f, (const bf16*)w.cq_w, w.cq_b};
     else TRY(gemm<T>(h, EPI_STORE, h->y, d, w.cq_w, w.cq_b, d, d, cnt, rows_ub, h->q, d, nullptr, st, nullptr, nullptr, nullptr,
                      nullptr, &lc));
     TRY(attn<T>(h, false, h->q, d, nullptr, m.ckv[layer], (char*)m.ckv[layer] + (size_t)d * e, m.ckv_stride, r.kv_off_cross,
-                r, r.nk_cross, cnt, rows_ub, q_ub, h->att, d, H, dh, h->S_max, st, h->ses.src_len, inside ? &qa : nullptr));   // encoder K/V: all of it
+                r, r.nk_cross, cnt, rows_ub, q_ub, h->att, d, H, dh, h->S_max, st, h->ses.src_len, inside ? &qa : nullptr, out ? &oa : nullptr));   // encoder K/V: all of it
+    if (out) return 0;
     h->next_ln = {w.ln2_g, w.ln2_b, h->y};           // the feed-forward sublayer's LayerNorm comes next
     TRY(gemm<T>(h, EPI_RESID, h->att, d, w.co_w, w.co_b, d, d, cnt, rows_ub, nullptr, 0, x, st));
     return 0;
@@ -871,16 +918,18 @@ int draft_impl(specdec_handle* h, int k, int* d_draft, cudaStream_t st) {
             KCHECK(h);
         }
     }
-    CUDA_TRY(h, launch_pdl(h, k_gather_rows, dim3(R2), dim3(128), 0, st, (const float*)h->x, (const int*)h->mrows.src_row, (const int*)(h->ses.counters + CNT_DRAFT_MASK), h->x2, d));
+    const bool inside = std::is_same<T, bf16>::value && out_inside(h, dh, k, H, CNT_DRAFT_MASK, R2, max_keys, OUT_GATHERS);
+    const OutArgs oa{(const bf16*)w.o_w, w.o_b, h->x, h->mrows.src_row, h->x2};       // (takes the [MASK] rows of the residual stream itself)
+    if (!inside) CUDA_TRY(h, launch_pdl(h, k_gather_rows, dim3(R2), dim3(128), 0, st, (const float*)h->x, (const int*)h->mrows.src_row, (const int*)(h->ses.counters + CNT_DRAFT_MASK), h->x2, d));
     KCHECK(h);
     if (pc)
         TRY(attn<T>(h, true, h->qkv, 3 * d, h->mrows.src_row, h->dkc[L - 1], h->dvc[L - 1], d, nullptr, h->mrows, h->mrows.nk_self,
-                    CNT_DRAFT_MASK, R2, k, h->att, d, H, dh, max_keys, st));
+                    CNT_DRAFT_MASK, R2, k, h->att, d, H, dh, max_keys, st, nullptr, nullptr, inside ? &oa : nullptr));
     else
         TRY(attn<T>(h, false, h->qkv, 3 * d, h->mrows.src_row, (char*)h->qkv + (size_t)d * e,
                     (char*)h->qkv + (size_t)2 * d * e, 3 * d, h->mrows.kv_off, h->mrows, h->mrows.nk_self,
-                    CNT_DRAFT_MASK, R2, k, h->att, d, H, dh, max_keys, st));
-    TRY(gemm<T>(h, EPI_RESID, h->att, d, w.o_w, w.o_b, d, d, CNT_DRAFT_MASK, R2, nullptr, 0, h->x2, st));
+                    CNT_DRAFT_MASK, R2, k, h->att, d, H, dh, max_keys, st, nullptr, nullptr, inside ? &oa : nullptr));
+    if (!inside) TRY(gemm<T>(h, EPI_RESID, h->att, d, w.o_w, w.o_b, d, d, CNT_DRAFT_MASK, R2, nullptr, 0, h->x2, st));
     TRY(block_cross<T>(h, m, w, h->x2, h->mrows, CNT_DRAFT_MASK, R2, k, L - 1, st));
     TRY(block_ffn<T>(h, m, w, h->x2, CNT_DRAFT_MASK, R2, st, m.dec_lnf_g, m.dec_lnf_b));
     const LnSpec lf{h->x2, m.dec_lnf_g, m.dec_lnf_b};
@@ -1509,6 +1558,8 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
         };
 #define ATTN_ROOM(MT, KG, KW, NS) room(k_attn<true, MT, KG, KW, NS>, AttnCfg<MT, KG, KW>::smem(max_keys, NS, true)); room(k_attn<false, MT, KG, KW, NS>, 0)
         room(k_attn<false, 1, 8, 16, 3, 2>, 0); room(k_attn<false, 1, 8, 16, 3, 4>, 0); room(k_attn<false, 1, 8, 16, 3, 6>, 0);   // (at most 222 KB: no table of rows)
+        room(k_attn<false, 1, 8, 16, 3, 2, 4>, 0); room(k_attn<true, 1, 8, 16, 3, 0, 4>, 0); room(k_attn<false, 1, 8, 16, 3, 0, 4>, 0);
+        room(k_attn<false, 1, 8, 16, 3, 4, 8>, 0); room(k_attn<true, 1, 8, 16, 3, 0, 8>, 0); room(k_attn<false, 1, 8, 16, 3, 0, 8>, 0);
         ATTN_ROOM(1, 4, 32, 3); ATTN_ROOM(1, 8, 32, 2); ATTN_ROOM(4, 1, 64, 3); ATTN_ROOM(2, 1, 64, 3);
         if (e != cudaSuccess) { cudaGetLastError(); h->use_tc_attn = 0; }
         if (sd::tc_init(h->tma, h->ses.counters + 7) != 0) h->use_tc = 0;     // reported through specdec_last_error; SIMT GEMM still runs on the GPU

@@ -65,3 +65,27 @@ def test_queries_projected_inside_the_attention(d, f, B, k, S):
     assert rep.ok, rep.notes
     assert rep.max_logit_err < 2e-2 and rep.max_stat_err < 2e-2
     sd.close()
+
+
+@pytest.mark.parametrize("d,B,k,S,cached", [
+    (256, 1, 4, 12, False),          # 5 rows of one tile: the fewest
+    (512, 2, 16, 128, False),        # a tile and one row; as many keys as fit beside the queries' projection
+    (512, 1, 47, 129, True),         # 48 rows; one key too many for it
+    (256, 3, 16, 300, True),         # three stages of keys
+])
+def test_output_projected_inside_the_attention(d, B, k, S, cached):
+    """Attention of few rows that goes on to the output projection and the residual, self- and cross-attention, the drafter's [MASK] rows among them."""
+    from paper_2203_16487_b200 import binding
+    V = 515
+    dims = W.ModelDims(d, d // 64, 128, V, 1, 2, 512)
+    wv, wd = W.make_weights(dims, 83, True), W.make_weights(dims, 84, True)
+    mv, md = O.model_from(dims, wv, mode="bf16"), O.model_from(dims, wd, mode="bf16")
+    rng = np.random.default_rng(d + S)
+    srcs = [W.zipf_ids(rng, n, V) for n in ([S] + [max(S // 2, 1), 7])[:B]]
+    sd = binding.SpecDec(dims, wv, dims, wd, k_max=k, max_batch=B, max_src=S, max_tgt=60, bf16=True)
+    sd.set_option("debug_checks", 1)
+    rep = lockstep.run(sd, mv, md, srcs, [60] * B, k, 3, 1.0, margin=1e-3, check_logits_every=1, max_iters=2,
+                       drafter_reading="prefix_causal" if cached else "bidirectional")
+    assert rep.ok, rep.notes
+    assert rep.max_logit_err < 2e-2 and rep.max_stat_err < 2e-2
+    sd.close()
