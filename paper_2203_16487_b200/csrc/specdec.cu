@@ -131,7 +131,7 @@ struct specdec_handle {
     bool splitk_ready = false;
     int diag_repeat = 0;            // diagnostics: launch every attention (1) / LayerNorm (2) / non-residual GEMM (4) / vocabulary (8) kernel twice (same result) to
                                     // read its cost inside the pipeline off the step time (option "diag_repeat")
-    int use_splitk = 1;             // residual GEMMs with K >= 1024 over few row tiles split K across a cluster of 4 / 6 CTAs (option "splitk")
+    int use_splitk = 1;             // residual GEMMs with K >= 1024 over few row tiles split K across a cluster of 4 / 2 CTAs (option "splitk")
     bool pair_ready = false;
     int use_pair = 0;               // two-SM tiles (cta_group::2) for wide GEMMs over many rows (option "pair")
     int attn_stream = 1;            // attention variant (option "attn_stream")
@@ -540,8 +540,9 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
                 ++h->launches;
                 return 0;
             }
-            if (epi == EPI_RESID && h->use_splitk && h->splitk_ready && sd::spk_supported(N, K, rows_ub, h->tma.n_sm)) {
-                if (sd::spk_launch(h->tma, g, rows_ub, st) != 0)
+            const int split = epi == EPI_RESID && h->use_splitk && h->splitk_ready ? sd::spk_split(h->tma, N, K, rows_ub) : 0;
+            if (split) {
+                if (sd::spk_launch(h->tma, split, g, rows_ub, st) != 0)
                     return fail(h, SPECDEC_ERR_CUDA, "tensor-core GEMM launch failed: " + h->tma.err);
                 ++h->launches;
                 return 0;
@@ -1563,7 +1564,7 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
         ATTN_ROOM(1, 4, 32, 3); ATTN_ROOM(1, 8, 32, 2); ATTN_ROOM(4, 1, 64, 3); ATTN_ROOM(2, 1, 64, 3);
         if (e != cudaSuccess) { cudaGetLastError(); h->use_tc_attn = 0; }
         if (sd::tc_init(h->tma, h->ses.counters + 7) != 0) h->use_tc = 0;     // reported through specdec_last_error; SIMT GEMM still runs on the GPU
-        h->splitk_ready = h->use_tc && sd::spk_init() == cudaSuccess;
+        h->splitk_ready = h->use_tc && sd::spk_init(h->tma) == cudaSuccess;
         if (!h->splitk_ready) cudaGetLastError();
         h->pair_ready = h->use_tc && sd::tc_pair_init() == cudaSuccess;
         if (!h->pair_ready) cudaGetLastError();

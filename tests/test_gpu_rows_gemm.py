@@ -16,13 +16,16 @@ pytestmark = pytest.mark.gpu
     (256, 4, 1040, 1, 15),          # 16 rows; K = 1040: two slices that end inside an MMA step
     (512, 8, 2048, 3, 10),          # 33 rows
     (768, 12, 3072, 8, 9),          # 80 rows: the last with the LayerNorm inside
-    (768, 12, 3072, 16, 6),         # 112 rows: the last of the few-rows kernel at this width
+    (768, 12, 3072, 16, 5),         # 96 rows: the last of the few-rows kernel at this width
     (768, 12, 3072, 16, 7),         # 128 rows: tensor-core tiles, four K slices for the output projections
     (512, 8, 2048, 16, 8),          # 144 rows: the last with the LayerNorm inside at this width
     (256, 4, 1024, 29, 4),          # 145 rows: LayerNorm in front, four slices
-    (320, 5, 1312, 32, 7),          # 256 rows: the last of the few-rows kernel; no LayerNorm width, an FFN that has no tiles
+    (320, 5, 1312, 16, 10),         # 176 rows: the last of the few-rows kernel; no LayerNorm width, an FFN that has no tiles
     (320, 5, 1312, 24, 15),         # 384 rows: the FFN's output projection stays with the few-rows kernel
     (128, 2, 192, 35, 10),          # 385 rows: tensor-core tiles
+    (512, 8, 2048, 32, 15),         # 512 rows: the last four K slices of a tile at this width, the last row tile full
+    (512, 8, 2048, 27, 18),         # 513 rows: two K slices, one row in the last tile
+    (256, 4, 1152, 20, 14),         # 300 rows: two slices of nine K blocks, more than the ring holds
 ])
 def test_rows_gemm_edges(d, H, f, B, k):
     from paper_2203_16487_b200 import binding
