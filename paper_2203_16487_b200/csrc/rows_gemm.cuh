@@ -15,12 +15,12 @@ struct RowsArgs {
 // Row limits, by the width of the model (the smaller side of a weight matrix).  Every CTA reads all of its operands from L2 once, so the
 // traffic grows with rows x columns, while a tensor-core tile of 128 rows shares its weights among them.
 constexpr int RG_MAX_ROWS = 384;                             // in general; shapes that the tensor-core tiles serve too go over to them at
-// (verify step, us, this kernel / tiles: width 512: 104 rows 191 / 241, 208 rows 238 / 253, 260 rows 295 / 294, 364 rows 343 / 298;
-// width 768: 78 rows 272 / 298, 104 rows 304 / 306, 156 rows 363 / 342)
-__host__ __device__ constexpr int rg_tile_rows(int width) { return width <= 512 ? 256 : 112; }
+// (verify step, us, this kernel / tiles: width 512: 130 rows 200 / 221, 160 rows 217 / 224, 182 rows 229 / 227, 208 rows 237 / 228;
+// width 768: 78 rows 262 / 294, 96 rows 285 / 294, 104 rows 309 / 291)
+__host__ __device__ constexpr int rg_tile_rows(int width) { return width <= 512 ? 176 : 96; }
 // ... and in the encoders, two of which run side by side on two streams and fill the SMs sooner (first tokens: width 512: 60 rows
-// 497 / 560, 180 rows 650 / 656, 240 rows 684 / 684; width 768: 60 rows 577 / 543).
-__host__ __device__ constexpr int rg_tile_rows_enc(int width) { return width <= 512 ? 208 : 48; }
+// 497 / 560, 80 rows 531 / 526, 120 rows 651 / 582; width 768: 40 rows 527 / 527, 60 rows 561 / 524).
+__host__ __device__ constexpr int rg_tile_rows_enc(int width) { return width <= 512 ? 72 : 40; }
 // Up to here the LayerNorm in front runs inside the GEMM, on 16-row tiles; beyond it is a launch of its own (inside / in front: width 512,
 // 130 rows 202 / 218; width 768, 104 rows 330 / 304).
 __host__ __device__ constexpr int rg_ln_rows(int width) { return width <= 512 ? 144 : 80; }
