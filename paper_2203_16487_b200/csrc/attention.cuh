@@ -11,9 +11,10 @@
 // What bounds it.  Few CTAs: the chain of round trips of one CTA.  Everything that predates the step -- row counts, the page
 // table's rows of all keys, the cached keys themselves -- is fetched ahead of the dependency wait, so that one round trip (queries and
 // new keys) is left behind it, and the keys are spread over four or eight warps (verify step at 26 rows: 176 us with the one-shot
-// kernel this one replaces, 161 with MT = 1, KG = 4).  Many CTAs: the fixed-latency chain inside a warp at the
-// occupancy that 130 registers leave (12 warps per SM: issue slots 42 % busy, tensor pipe 22 %, DRAM 27 %); 64-key blocks per
-// warp give the most independent work per barrier (128 sequences x 51 queries x 307 keys: 51 -> 34 us a launch; x 26 x 90: 16 -> 10.7).
+// kernel this one replaces, 161 with MT = 1, KG = 4).  Many CTAs: the fixed-latency chain inside a warp, so
+// warps per SM and whole waves count: 16 of them, in CTAs of 64 queries with a ring of two 64-key blocks (128 sequences x 51 queries x 307 keys, verify
+// step with 12 warps and a ring of three 1107 us, now 1055-1075) or of 32 queries with 32-key blocks (x 26 x 90: 555 with 8 warps and
+// 64-key blocks, now 514).  Below four CTAs an SM there is nothing to fill the SMs with, and 64-key blocks have more independent work per barrier.
 #pragma once
 #include "kernels.cuh"
 
@@ -155,7 +156,7 @@ struct AttnCfg {
 // that only the exchange (0.5 us), 32 MMAs a warp and the sum of four K slices follow the attention: a launch and its round trip less
 // (verify step of 26 rows, both attentions of six layers: 156.5 -> 147.2 us; with Wo fetched behind the wait 155.2).
 template <bool PAGED, int MT, int KG, int KW, int NS, int QNC = 0, int ON = 0>
-__global__ void __launch_bounds__(MT * KG * 32) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {
+__global__ void __launch_bounds__(MT * KG * 32, KG > 1 ? 1 : MT == 4 ? 4 : KW == 32 ? 8 : 1) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {
     using C = AttnCfg<MT, KG, KW>;
     static_assert((QNC == 0 && ON == 0) || (MT == 1 && KG == 8), "the projections are laid out for eight warps and 16 rows");
     static_assert(QNC == 0 || ON == 0 || ON == 2 * QNC, "one width");

@@ -612,16 +612,20 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
                 return goo(qp ? k_attn<false, 1, 8, 16, 3, 4, 8> : paged ? k_attn<true, 1, 8, 16, 3, 0, 8> : k_attn<false, 1, 8, 16, 3, 0, 8>, qp ? ProjCfg<4, 8>::OPS : ProjCfg<0, 8>::OPS);
             }
             if (qp) {
-                auto goq = [&](auto* kernel, int bytes) {
-                    const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, 16), n_heads, h->B), dim3(256), AttnCfg<1, 8, 16>::smem(max_keys, 3, false, bytes), st, a, qa, oa);
+                auto goq = [&](auto* kernel, size_t bytes) {
+                    const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, 16), n_heads, h->B), dim3(256), bytes, st, a, qa, oa);
                     if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
                     KCHECK(h);
                     return 0;
                 };
-                switch (n_heads) {                           // (64-wide heads: the width is 64 n_heads)
-                    case 4: return goq(k_attn<false, 1, 8, 16, 3, 2>, QueryCfg<2>::OPS);
-                    case 8: return goq(k_attn<false, 1, 8, 16, 3, 4>, QueryCfg<4>::OPS);
-                    default: return goq(k_attn<false, 1, 8, 16, 3, 6>, QueryCfg<6>::OPS);
+                // (64-wide heads: the width is 64 n_heads.)  More than 128 keys in blocks of 256 where shared memory has room for two: sources of 512 tokens, 8
+                // sequences decoded 7834 -> 7757 us, 2 sequences 5660 -> 5528; verify step over 233 keys 236 -> 234.
+                switch (n_heads) {
+#define QUERY_GO(KW, NS, QNC) goq(k_attn<false, 1, 8, KW, NS, QNC>, AttnCfg<1, 8, KW>::smem(max_keys, NS, false, QueryCfg<QNC>::OPS))
+                    case 4: return max_keys > 128 ? QUERY_GO(32, 2, 2) : QUERY_GO(16, 3, 2);
+                    case 8: return max_keys > 128 ? QUERY_GO(32, 2, 4) : QUERY_GO(16, 3, 4);
+                    default: return QUERY_GO(16, 3, 6);
+#undef QUERY_GO
                 }
             }
             auto go = [&](auto* kernel, int bm, int warps, size_t smem) {
@@ -644,7 +648,11 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             // sequences: 1186 against 1294 us a step) unless the tail of the last tile is more than an eighth of the work (90
             // queries: 273 against 265 us a draft step).
             const bool tall = h->attn_stream == 1 ? 8LL * ((q_ub + 63) / 64 * 64) <= 9LL * ((q_ub + 31) / 32 * 32) : h->attn_stream == 2;
-            return tall ? ATTN_GO(4, 1, 64, 3) : ATTN_GO(2, 1, 64, 3);
+            if (tall) return ATTN_GO(4, 1, 64, 2);
+            // 32 queries: up to four CTAs an SM, as many as fit with three 64-key blocks each, those (64 sequences x 26 queries: 388 against 397 us a verify
+            // step); more CTAs take 32-key blocks and are eight to an SM (128 sequences: 514 against 555).
+            const bool dense = h->attn_stream == 1 ? (long long)cdiv(q_ub, 32) * n_heads * n_seq > 4LL * h->tma.n_sm : h->attn_stream == 4;
+            return dense ? ATTN_GO(2, 1, 32, 3) : ATTN_GO(2, 1, 64, 3);
         }
     }
     if constexpr (std::is_same<T, float>::value) {
@@ -1559,9 +1567,10 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
         };
 #define ATTN_ROOM(MT, KG, KW, NS) room(k_attn<true, MT, KG, KW, NS>, AttnCfg<MT, KG, KW>::smem(max_keys, NS, true)); room(k_attn<false, MT, KG, KW, NS>, 0)
         room(k_attn<false, 1, 8, 16, 3, 2>, 0); room(k_attn<false, 1, 8, 16, 3, 4>, 0); room(k_attn<false, 1, 8, 16, 3, 6>, 0);   // (at most 222 KB: no table of rows)
+        room(k_attn<false, 1, 8, 32, 2, 2>, 0); room(k_attn<false, 1, 8, 32, 2, 4>, 0);
         room(k_attn<false, 1, 8, 16, 3, 2, 4>, 0); room(k_attn<true, 1, 8, 16, 3, 0, 4>, 0); room(k_attn<false, 1, 8, 16, 3, 0, 4>, 0);
         room(k_attn<false, 1, 8, 16, 3, 4, 8>, 0); room(k_attn<true, 1, 8, 16, 3, 0, 8>, 0); room(k_attn<false, 1, 8, 16, 3, 0, 8>, 0);
-        ATTN_ROOM(1, 4, 32, 3); ATTN_ROOM(1, 8, 32, 2); ATTN_ROOM(4, 1, 64, 3); ATTN_ROOM(2, 1, 64, 3);
+        ATTN_ROOM(1, 4, 32, 3); ATTN_ROOM(1, 8, 32, 2); ATTN_ROOM(4, 1, 64, 2); ATTN_ROOM(2, 1, 64, 3); ATTN_ROOM(2, 1, 32, 3);
         if (e != cudaSuccess) { cudaGetLastError(); h->use_tc_attn = 0; }
         if (sd::tc_init(h->tma, h->ses.counters + 7) != 0) h->use_tc = 0;     // reported through specdec_last_error; SIMT GEMM still runs on the GPU
         h->splitk_ready = h->use_tc && sd::spk_init(h->tma) == cudaSuccess;
@@ -1648,7 +1657,7 @@ int specdec_set_option(specdec_handle* h, const char* name, int value) {
     }
     if (!strcmp(name, "diag_repeat")) { h->diag_repeat = value; return SPECDEC_OK; }
     if (!strcmp(name, "splitk")) { h->use_splitk = value ? 1 : 0; return SPECDEC_OK; }
-    if (!strcmp(name, "attn_stream")) { h->attn_stream = value < 0 ? 0 : (value > 3 ? 3 : value); return SPECDEC_OK; }
+    if (!strcmp(name, "attn_stream")) { h->attn_stream = value < 0 ? 0 : (value > 4 ? 4 : value); return SPECDEC_OK; }
     if (!strcmp(name, "attn_rs") || !strcmp(name, "attn_stream_keys")) return SPECDEC_OK;      // (chose between kernels that are one now)
     if (!strcmp(name, "attn_warps")) {
         if (value != 0 && value != 4 && value != 8) return fail(h, SPECDEC_ERR_INVALID_ARG, "attn_warps must be 0, 4 or 8");

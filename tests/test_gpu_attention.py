@@ -11,7 +11,7 @@ from tests import lockstep
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("opts", [{}, {"attn_warps": 4}, {"attn_warps": 8}, {"attn_stream": 2}, {"attn_stream": 3}])
+@pytest.mark.parametrize("opts", [{}, {"attn_warps": 4}, {"attn_warps": 8}, {"attn_stream": 2}, {"attn_stream": 3}, {"attn_stream": 4}])
 @pytest.mark.parametrize("lens,k", [((1, 31, 33, 64, 65), 15), ((127, 129, 255, 257, 385), 33)])
 def test_attention_edges(opts, lens, k):
     from paper_2203_16487_b200 import binding
@@ -49,7 +49,7 @@ def test_attention_edges(opts, lens, k):
     sd.close()
 
 
-@pytest.mark.parametrize("d,f,B,k,S", [(256, 256, 1, 15, 12), (512, 128, 3, 16, 130), (768, 128, 2, 31, 400)])
+@pytest.mark.parametrize("d,f,B,k,S", [(256, 256, 1, 15, 12), (512, 128, 3, 16, 130), (256, 128, 2, 15, 300), (768, 128, 2, 31, 400)])
 def test_queries_projected_inside_the_attention(d, f, B, k, S):
     """Cross-attention of few rows: one and two 16-row tiles with a ragged end, key rings of one stage and more, the three widths."""
     from paper_2203_16487_b200 import binding
