@@ -147,6 +147,10 @@ struct AttnCfg {
     }
 };
 
+// CTAs per SM that the registers are cut for; 0 leaves it to the compiler (told 1, it takes 148 registers for MT = 1, KG = 4 where 100 do, and the
+// verify step of 832 rows 334 us instead of 316).
+constexpr int attn_ctas(int mt, int kg, int kw) { return kg > 1 ? 0 : mt == 4 ? 4 : kw == 32 ? 8 : 0; }
+
 // QNC > 0: the queries are projected here (QueryArgs; MT = 1, KG = 8).  The CTA's 64 rows of Wq are requested ahead of the wait, the
 // 16 rows normalised behind it; one launch and its round trip through memory less per layer (26 rows, K = 512: 5.5 -> 4.4 us).
 //
@@ -156,7 +160,7 @@ struct AttnCfg {
 // that only the exchange (0.5 us), 32 MMAs a warp and the sum of four K slices follow the attention: a launch and its round trip less
 // (verify step of 26 rows, both attentions of six layers: 156.5 -> 147.2 us; with Wo fetched behind the wait 155.2).
 template <bool PAGED, int MT, int KG, int KW, int NS, int QNC = 0, int ON = 0>
-__global__ void __launch_bounds__(MT * KG * 32, KG > 1 ? 1 : MT == 4 ? 4 : KW == 32 ? 8 : 1) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {
+__global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {
     using C = AttnCfg<MT, KG, KW>;
     static_assert((QNC == 0 && ON == 0) || (MT == 1 && KG == 8), "the projections are laid out for eight warps and 16 rows");
     static_assert(QNC == 0 || ON == 0 || ON == 2 * QNC, "one width");
