@@ -20,14 +20,15 @@ constexpr int SPK_RECV = TC_BM * SPK_BN * 4;                   // SPLIT slices o
 constexpr int SPK_SMEM = SPK_STAGES * SPK_STAGE + SPK_RECV + 1024;
 static_assert(SPK_STAGES * SPK_STAGE >= TC_EPI_WARPS * 4096, "the outgoing blocks reuse the ring");
 
-// CTAs per tile: 4 while all clusters run at once, else 2, else none (0).  (Clusters of 4 do not use every SM: 36 of them on 148 SMs took two waves,
+// CTAs per tile: 4 while all clusters run at once, else 2, else none (0).  Shorter reductions gain less than the exchange costs (verify step, us, unsplit / split:
+// K = 768 in four 208 rows 318 / 310, in two 520 rows 399 / 403; K = 512 416 rows 279 / 286).  (Clusters of 4 do not use every SM: 36 of them on 148 SMs took two waves,
 // 392 us a verify
 // step of 312 rows at 768 columns where clusters of 2 take 361.)
 inline int spk_split(const TmaEncoder& enc, int N, int K, int rows_ub) {
-    if (N % SPK_BN || K < 1024) return 0;
+    if (N % SPK_BN || K < 768) return 0;
     const long long tiles = (long long)((rows_ub + TC_BM - 1) / TC_BM) * (N / SPK_BN);
     if (K % (4 * TC_BK) == 0 && tiles <= enc.spk_clusters4) return 4;
-    return K % (2 * TC_BK) == 0 && tiles <= enc.spk_clusters2 ? 2 : 0;
+    return K % (2 * TC_BK) == 0 && K >= 1024 && tiles <= enc.spk_clusters2 ? 2 : 0;
 }
 
 template <int SPLIT>
