@@ -148,8 +148,8 @@ struct AttnCfg {
 };
 
 // CTAs per SM that the registers are cut for; 0 leaves it to the compiler (told 1, it takes 148 registers for MT = 1, KG = 4 where 100 do, and the
-// verify step of 832 rows 334 us instead of 316).
-constexpr int attn_ctas(int mt, int kg, int kw) { return kg > 1 ? 0 : mt == 4 ? 4 : kw == 32 ? 8 : 0; }
+// verify step of 832 rows 334 us instead of 316; MT = 2 with 64-key blocks is better with its 174 than with 129: 1664 rows 388 / 400 us).
+constexpr int attn_ctas(int mt, int kg, int kw) { return kg > 1 ? 0 : mt == 4 ? 4 : kw == 32 ? 8 : 1; }
 
 // QNC > 0: the queries are projected here (QueryArgs; MT = 1, KG = 8).  The CTA's 64 rows of Wq are requested ahead of the wait, the
 // 16 rows normalised behind it; one launch and its round trip through memory less per layer (26 rows, K = 512: 5.5 -> 4.4 us).
