@@ -68,7 +68,7 @@ template <int CS>
 inline cudaError_t cluster_round_run(int rounds, int bytes_per_cta_per_peer, long long* d_scratch, int* err_word, cudaStream_t st, double* ns_per_round) {
     const int n16 = bytes_per_cta_per_peer / 16;
     const int smem = CS * (n16 > 0 ? n16 : 1) * 16;
-    cudaError_t e = cudaFuncSetAttribute(k_cluster_round<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(k_cluster_round<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, CS * 8192);     // (the most that a call may ask for)
     if (e == cudaSuccess && CS > 8) e = cudaFuncSetAttribute(k_cluster_round<CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};

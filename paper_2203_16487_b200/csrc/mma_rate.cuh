@@ -112,8 +112,9 @@ inline cudaError_t mma_rate_run(int n_sm, int n_mma, long long* d_scratch, int* 
     if (bg_stages < 0 || bg_stages > 6 || (bg_stages > 0 && (!bg_src || bg_window < (8ll << 20)))) return cudaErrorInvalidValue;
     if (op_stages < 1) return cudaErrorInvalidValue;
     const int smem = op_stages * (TC_BM * TC_BK * 2 + BNL * TC_BK * 2) + bg_stages * 16384 + 1024;
-    if (smem > 232448 - 1024) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_mma_rate<BN, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    constexpr int limit = 232448 - 1024;
+    if (smem > limit) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(k_mma_rate<BN, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
     if (e != cudaSuccess) return e;
     const int ctas = PAIR ? (n_sm / 2) * 2 : n_sm, groups = PAIR ? ctas / 2 : ctas;
     cudaLaunchConfig_t cfg = {};

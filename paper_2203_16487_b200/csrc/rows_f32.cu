@@ -220,11 +220,7 @@ template <int EPI, int BN, int LN>
 static cudaError_t rf_go(const RowsF32Args& a, int rows_ub, bool pdl, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((a.g.N + BN - 1) / BN, (rows_ub + RF_BM - 1) / RF_BM); cfg.blockDim = dim3(RF_THREADS);
-    cfg.dynamicSmemBytes = rf_smem(BN, a.g.K); cfg.stream = st;
-    if (cfg.dynamicSmemBytes > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_rows_f32<EPI, BN, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
-        if (e != cudaSuccess) return e;
-    }
+    cfg.dynamicSmemBytes = rf_smem(BN, a.g.K); cfg.stream = st;        // (allowed by rf_init)
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -357,11 +353,7 @@ cudaError_t af_launch(bool paged, const AttnF32Args& a, int q_ub, int n_heads, i
     auto go = [&](auto* kernel) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((q_ub + AF_Q - 1) / AF_Q, n_heads, B); cfg.blockDim = dim3(AF_WARPS * 32);
-        cfg.dynamicSmemBytes = af_smem(a.d_head, a.max_keys); cfg.stream = st;
-        if (cfg.dynamicSmemBytes > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
-            if (e != cudaSuccess) return e;
-        }
+        cfg.dynamicSmemBytes = af_smem(a.d_head, a.max_keys); cfg.stream = st;      // (allowed by rf_init)
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -369,6 +361,18 @@ cudaError_t af_launch(bool paged, const AttnF32Args& a, int q_ub, int n_heads, i
         return cudaLaunchKernelEx(&cfg, kernel, a);
     };
     return paged ? go(k_attn_f32<true>) : go(k_attn_f32<false>);
+}
+
+// Shared-memory limits of everything launched above: the same for every handle, since they belong to the kernels in the whole process.
+cudaError_t rf_init() {
+    cudaError_t e = cudaSuccess;
+    auto room = [&](auto* kernel) { if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RF_MAX_SMEM); };
+#define RF_ROOM(EPI, BN) room(k_rows_f32<EPI, BN, 0>); room(k_rows_f32<EPI, BN, 4>); room(k_rows_f32<EPI, BN, 16>)
+    RF_ROOM(EPI_STORE, 32); RF_ROOM(EPI_RELU, 32); RF_ROOM(EPI_QKV, 32); RF_ROOM(EPI_STATS, 64);
+#undef RF_ROOM
+    room(k_rows_f32<EPI_RESID, 32, 0>);
+    room(k_attn_f32<true>); room(k_attn_f32<false>);
+    return e;
 }
 
 }  // namespace sd

@@ -11,6 +11,7 @@ struct RowsF32Args {
 };
 inline bool rf_ln_width(int K) { return K <= 512; }          // widths that the LayerNorm prologue exists for
 bool rf_supported(int epi, int N, int K, int lda, int rows_ub);
+cudaError_t rf_init();           // once per handle, before the first launch of either kernel
 cudaError_t rf_launch(int epi, const RowsF32Args& a, int rows_ub, bool pdl, cudaStream_t st);
 
 struct AttnF32Args {

@@ -279,11 +279,7 @@ inline cudaError_t rg_launch_one(const RowsArgs& a, int rows_ub, bool pdl, cudaS
     using C = RgCfg<MT, NT, WN, CS>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((a.g.N + C::NB - 1) / C::NB * CS, (rows_ub + C::BM - 1) / C::BM); cfg.blockDim = dim3(RG_THREADS);
-    cfg.dynamicSmemBytes = C::smem(a.g.K / CS); cfg.stream = st;
-    if (cfg.dynamicSmemBytes > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_rows<EPI, NC, MT, NT, WN, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
-        if (e != cudaSuccess) return e;
-    }
+    cfg.dynamicSmemBytes = C::smem(a.g.K / CS); cfg.stream = st;       // (allowed by rg_init)
     cudaLaunchAttribute attr[2];
     int n = 0;
     if (CS > 1) { attr[n].id = cudaLaunchAttributeClusterDimension; attr[n].val.clusterDim.x = CS; attr[n].val.clusterDim.y = 1; attr[n].val.clusterDim.z = 1; ++n; }
@@ -347,6 +343,30 @@ cudaError_t rg_launch(int epi, const RowsArgs& a, int rows_ub, bool cluster, boo
         case EPI_QKV: return rg_launch_nc<EPI_QKV>(a, rows_ub, pdl, st);
         default: return rg_launch_resid(a, rows_ub, cluster, pdl, st);
     }
+}
+
+
+// Shared-memory limits of everything launched above.  The limit belongs to the kernel in the whole process: one that followed the launch would
+// be another handle's by the time of the launch, if that handle decodes on another host thread.
+template <int EPI, int NC, int MT, int NT, int WN, int CS>
+static void rg_room(cudaError_t& e) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rows<EPI, NC, MT, NT, WN, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, RG_MAX_SMEM);
+}
+template <int EPI, int NC>
+static void rg_room_out(cudaError_t& e) {
+    if (NC == 0) rg_room<EPI, 0, 2, 8, 2, 1>(e);
+    rg_room<EPI, NC, 1, 8, 2, 1>(e);
+    if (EPI == EPI_STORE) rg_room<EPI, NC, 1, 4, 1, 1>(e);
+    rg_room<EPI, NC, 1, 2, 1, 1>(e);
+}
+template <int EPI>
+static void rg_room_nc(cudaError_t& e) { rg_room_out<EPI, 0>(e); rg_room_out<EPI, 2>(e); rg_room_out<EPI, 4>(e); rg_room_out<EPI, 6>(e); }
+cudaError_t rg_init() {
+    cudaError_t e = cudaSuccess;
+    rg_room_nc<EPI_STORE>(e); rg_room_nc<EPI_RELU>(e); rg_room_nc<EPI_GELU>(e); rg_room_nc<EPI_QKV>(e);
+    rg_room<EPI_RESID, 0, 2, 8, 2, 4>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1>(e);
+    rg_room<EPI_RESID, 0, 1, 4, 1, 2>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1>(e); rg_room<EPI_RESID, 0, 1, 2, 1, 1>(e);
+    return e;
 }
 
 }  // namespace sd

@@ -27,6 +27,7 @@ __host__ __device__ constexpr int rg_ln_rows(int width) { return width <= 512 ? 
 
 bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster);
 inline bool rg_ln_width(int K) { return K == 256 || K == 512 || K == 768; }    // widths that the LayerNorm prologue exists for
+cudaError_t rg_init();           // once per handle, before the first launch
 cudaError_t rg_launch(int epi, const RowsArgs& a, int rows_ub, bool cluster, bool pdl, cudaStream_t st);
 
 }  // namespace sd

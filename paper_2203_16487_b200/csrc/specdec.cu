@@ -1526,6 +1526,23 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
     ce = cudaStreamSynchronize(st);
     if (ce == cudaSuccess) ce = cudaGetLastError();
     if (ce != cudaSuccess) return bail(SPECDEC_ERR_CUDA, std::string("weight repacking: ") + cudaGetErrorString(ce));
+    // warp-per-row attention keeps one row of scores per warp in shared memory.  (What a kernel may take is set for the whole process: never to
+    // what this handle needs, or a later handle with fewer keys would take it away from this one.)
+    {
+        const int max_keys = std::max(h->S_cap, h->T_cap + h->k_cap + 1);
+        const int dh = std::max(cfg->verifier.d_model / cfg->verifier.n_heads, cfg->drafter.d_model / cfg->drafter.n_heads);
+        constexpr int limit = 200 * 1024;
+        if (4 * (max_keys + dh) * 4 > limit) return bail(SPECDEC_ERR_CAPACITY, "max_src / max_tgt too large for the attention kernel");
+        auto room = [&](auto* kernel) { if (ce == cudaSuccess) ce = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit); };
+        if (h->dtype == SPECDEC_DTYPE_BF16) {
+            room(k_attention<bf16, true>); room(k_attention<bf16, false>);
+            if (ce == cudaSuccess) ce = sd::rg_init();
+        } else {
+            room(k_attention<float, true>); room(k_attention<float, false>);
+            if (ce == cudaSuccess) ce = sd::rf_init();
+        }
+        if (ce != cudaSuccess) return bail(SPECDEC_ERR_CUDA, std::string("shared memory of the kernels: ") + cudaGetErrorString(ce));
+    }
     if (cudaMallocHost((void**)&h->h_post, 64) != cudaSuccess) return bail(SPECDEC_ERR_CUDA, "pinned host allocation failed");
     *h->h_post = 0ull;
     if (cudaMallocHost((void**)&h->h_poll, 64 * 4) != cudaSuccess || cudaMallocHost((void**)&h->h_stats, 64) != cudaSuccess)
@@ -1542,22 +1559,6 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
     for (auto& e : h->poll_ev) cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
     h->time_ev.resize((size_t)3 * h->T_cap + 8);
     for (auto& e : h->time_ev) cudaEventCreate(&e);
-    // attention keeps one row of scores per warp in shared memory
-    {
-        const int max_keys = std::max(h->S_cap, h->T_cap + h->k_cap + 1);
-        const int dh = std::max(cfg->verifier.d_model / cfg->verifier.n_heads, cfg->drafter.d_model / cfg->drafter.n_heads);
-        const int smem = 4 * (max_keys + dh) * 4;
-        if (smem > 200 * 1024) return bail(SPECDEC_ERR_CAPACITY, "max_src / max_tgt too large for the attention kernel");
-        if (smem > 48 * 1024) {
-            if (h->dtype == SPECDEC_DTYPE_BF16) {
-                cudaFuncSetAttribute(k_attention<bf16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                cudaFuncSetAttribute(k_attention<bf16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            } else {
-                cudaFuncSetAttribute(k_attention<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                cudaFuncSetAttribute(k_attention<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            }
-        }
-    }
     if (h->dtype == SPECDEC_DTYPE_BF16) {
         const int max_keys = std::max(h->S_cap, h->T_cap + h->k_cap + 1);
         cudaError_t e = cudaSuccess;
