@@ -929,8 +929,10 @@ int draft_impl(specdec_handle* h, int k, int* d_draft, cudaStream_t st) {
     }
     const bool inside = std::is_same<T, bf16>::value && out_inside(h, dh, k, H, CNT_DRAFT_MASK, R2, max_keys, OUT_GATHERS);
     const OutArgs oa{(const bf16*)w.o_w, w.o_b, h->x, h->mrows.src_row, h->x2};       // (takes the [MASK] rows of the residual stream itself)
-    if (!inside) CUDA_TRY(h, launch_pdl(h, k_gather_rows, dim3(R2), dim3(128), 0, st, (const float*)h->x, (const int*)h->mrows.src_row, (const int*)(h->ses.counters + CNT_DRAFT_MASK), h->x2, d));
-    KCHECK(h);
+    if (!inside) {
+        CUDA_TRY(h, launch_pdl(h, k_gather_rows, dim3(R2), dim3(128), 0, st, (const float*)h->x, (const int*)h->mrows.src_row, (const int*)(h->ses.counters + CNT_DRAFT_MASK), h->x2, d));
+        KCHECK(h);
+    }
     if (pc)
         TRY(attn<T>(h, true, h->qkv, 3 * d, h->mrows.src_row, h->dkc[L - 1], h->dvc[L - 1], d, nullptr, h->mrows, h->mrows.nk_self,
                     CNT_DRAFT_MASK, R2, k, h->att, d, H, dh, max_keys, st, nullptr, nullptr, inside ? &oa : nullptr));
@@ -1070,6 +1072,8 @@ int graph_call(specdec_handle* h, std::vector<long long> key, cudaStream_t st, F
         int rc = body();
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(st, &g);
+        const long long kernels = h->launches - before;
+        h->launches = before;                          // (captured, not launched)
         if (rc != 0) { if (g) cudaGraphDestroy(g); return rc; }
         if (e != cudaSuccess || !g) return fail(h, SPECDEC_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
         cudaGraphExec_t ex = nullptr;
@@ -1077,8 +1081,7 @@ int graph_call(specdec_handle* h, std::vector<long long> key, cudaStream_t st, F
         cudaGraphDestroy(g);
         if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
         if (h->graphs.size() > 256) drop_graphs(h);
-        specdec_handle::GraphEntry ge{ex, h->launches - before};
-        h->launches = before;
+        specdec_handle::GraphEntry ge{ex, kernels};
         it = h->graphs.emplace(std::move(key), ge).first;
     }
     CUDA_TRY(h, cudaGraphLaunch(it->second.exec, st));
@@ -1378,8 +1381,11 @@ int integrity_run(specdec_handle* h, cudaStream_t st, specdec_integrity* rep) {
     const unsigned long long init[4] = {0ull, ~0ull, 0ull, ~0ull};
     CUDA_TRY(h, cudaMemcpyAsync(h->integ_report, init, sizeof(init), cudaMemcpyHostToDevice, st));
     k_red_check<<<cdiv(h->n_zones, 8), 256, 0, st>>>((const unsigned char*)h->arena.base, h->zone_tab, h->n_zones, h->integ_report);
-    if (h->n_scan > 0) k_nonfinite_scan<<<dim3(2 * h->tma.n_sm, h->n_scan), 256, 0, st>>>(h->integ_bufs, h->integ_report);
     KCHECK(h);
+    if (h->n_scan > 0) {
+        k_nonfinite_scan<<<dim3(2 * h->tma.n_sm, h->n_scan), 256, 0, st>>>(h->integ_bufs, h->integ_report);
+        KCHECK(h);
+    }
     unsigned long long out[4];
     CUDA_TRY(h, cudaMemcpyAsync(out, h->integ_report, sizeof(out), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(h, cudaStreamSynchronize(st));
@@ -1475,6 +1481,7 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
         h->n_zones = (int)h->arena.zones.size();
         cudaMemcpyAsync(h->zone_tab, h->arena.zones.data(), (size_t)h->n_zones * 8, cudaMemcpyHostToDevice, st);
         k_red_fill<<<cdiv(h->n_zones, 8), 256, 0, st>>>((unsigned char*)base, h->zone_tab, h->n_zones);
+        ++h->launches;
         std::vector<ScanBuf> sb;
         auto add = [&](const char* name, const void* p, size_t bytes, bool f32) {
             if (!p || bytes < 16 || sb.size() >= 128) return;
@@ -1643,6 +1650,7 @@ int specdec_set_option(specdec_handle* h, const char* name, int value) {
     }
     if (!strcmp(name, "heal_zones")) {                // test hook: restore every red zone
         k_red_fill<<<cdiv(h->n_zones, 8), 256>>>((unsigned char*)h->arena.base, h->zone_tab, h->n_zones);
+        KCHECK(h);
         CUDA_TRY(h, cudaDeviceSynchronize());
         return SPECDEC_OK;
     }
