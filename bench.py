@@ -325,10 +325,36 @@ def tokens_leg(torch, binding, B: int, K_: int, W_: int, rank: int, world: int, 
     return leg
 
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of the verify microbenchmark, keyed by
-# (batch, what): one whole verify step, or the vocabulary kernel alone.  ncu measures every kernel with cold caches, so at
-# batch 128 the step figure counts activations that normally stay in L2 (an upper bound); cells never captured are absent.
-NCU_TRAFFIC = {(1, "step"): 84391168, (1, "vocabulary"): 33608960, (128, "step"): 817641984, (128, "vocabulary"): 37020000}
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of the verify microbenchmark, by batch: the
+# number of kernels of the step that was captured, one whole step, and the vocabulary kernel alone.  ncu measures every kernel with cold
+# caches, so at batch 128 the step figure counts activations that normally stay in L2 (an upper bound).
+NCU_TRAFFIC = {}
+
+
+def ncu_traffic(B: int, launches_per_step: int, what: str):
+    """A captured figure, as long as the step still consists of as many kernels as the one that was captured."""
+    c = NCU_TRAFFIC.get(B)
+    return c[what] if c and c["launches"] == launches_per_step else None
+
+
+def step_classes(dims, k: int, j: int, S: int, B: int, total: int, extra: dict) -> list:
+    """The kernel classes of a verify step: (diag_repeat bit, label, launches, algorithmic bytes); the last, without a bit, is the rest.
+    total = launches of the step, extra[bit] = launches that the option adds, which is the class's number of launches.  The attention kernels of
+    a step of few rows also do the cross-attention's query projection and the output projections: what is not launched as a GEMM runs there, and
+    its weights are that class's bytes."""
+    L, d, f, V = dims.dec_layers, dims.d_model, dims.d_ffn, dims.vocab
+    rows = B * (k + 1)
+    n_attn, n_ln, n_gemm, n_voc = (extra[b] for b in (1, 2, 4, 8))
+    n_resid = total - n_attn - n_ln - n_gemm - n_voc - 2             # (2: the block's rows with their embedding, and the acceptance scan)
+    q_inside, o_inside = 3 * L - n_gemm, 3 * L - n_resid             # of QKV, cross-Q, FFN1 and of two output projections, FFN2 a layer
+    inside = f", {q_inside} query and {o_inside} output projections inside" if q_inside or o_inside else ""
+    return [(1, "attention (self + cross" + inside + ")", n_attn,
+             B * L * (j + k + 1 + S) * 2 * d * 2 + (q_inside + o_inside) * d * d * 2),
+            (2, "LayerNorm launches (the last one with the logits of the drafts)", n_ln, None),
+            (4, "layer GEMMs without residual (QKV, FFN1" + (", cross-Q)" if q_inside < L else ")"), n_gemm,
+             (L * (3 * d * d + f * d) + (L - q_inside) * d * d) * 2),
+            (8, "vocabulary projection + row statistics", n_voc, V * d * 2 + rows * d * 2),
+            (0, "residual GEMMs (FFN2" + (", attention out" if o_inside < 2 * L else "") + "), embedding, accept scan", n_resid + 2, None)]
 
 
 def verify_step_roofline(torch, binding, B: int, local: int, opts, reps: int = 50):
@@ -349,40 +375,33 @@ def verify_step_roofline(torch, binding, B: int, local: int, opts, reps: int = 5
         opt_name, _, val = kv.partition("=")
         sd.set_option(opt_name, int(val))
     flush = torch.empty(256 * 1024 * 1024, dtype=torch.uint8, device=f"cuda:{local}")
-    l0 = sd.launch_count()
     us, us_min, mean_a = MB.measure(sd, wl, B, k, j, S, reps, 5, flush)
-    n_calls = None
     params, bytes_, flops = MB.algorithmic_work(B, k, j, S, wl.verifier)
-    # launches of one step: count them on one extra call
-    c0 = sd.launch_count()
     d = torch.zeros((B, k), dtype=torch.int32, device=f"cuda:{local}")
     acc_t = torch.zeros(B, dtype=torch.int32, device=f"cuda:{local}"); bif_t = torch.zeros_like(acc_t)
-    sd.verify_raw(d, BETA, TAU, acc_t, bif_t)
-    torch.cuda.synchronize()
-    launches_per_step = sd.launch_count() - c0
-    by_kernel = []
-    d_model, V = wl.verifier.d_model, wl.verifier.vocab
-    rows = B * (k + 1)
-    classes = [(1, "attention (self + cross)", 2 * wl.verifier.dec_layers, B * wl.verifier.dec_layers * (j + k + 1 + S) * 2 * d_model * 2),
-               (2, "LayerNorm launches", None, None),
-               (4, "layer GEMMs without residual (QKV, cross-Q, FFN1)", 3 * wl.verifier.dec_layers,
-                wl.verifier.dec_layers * (3 * d_model * d_model + d_model * d_model + wl.verifier.d_ffn * d_model) * 2),
-               (8, "vocabulary projection + row statistics", 1, V * d_model * 2 + rows * d_model * 2)]
-    for bit, label, n_launch, cls_bytes in classes:
+
+    def launches_of_a_step():
+        c0 = sd.launch_count()
+        sd.verify_raw(d, BETA, TAU, acc_t, bif_t)
+        torch.cuda.synchronize()
+        return sd.launch_count() - c0
+
+    launches_per_step = launches_of_a_step()
+    extra, us_with = {}, {}
+    for bit in (1, 2, 4, 8):
         sd.set_option("diag_repeat", bit)
-        us_c, _, _ = MB.measure(sd, wl, B, k, j, S, max(reps // 2, 10), 3, flush)
+        us_with[bit], _, _ = MB.measure(sd, wl, B, k, j, S, max(reps // 2, 10), 3, flush)
+        extra[bit] = launches_of_a_step() - launches_per_step
         sd.set_option("diag_repeat", 0)
-        cost = max(us_c - us, 0.0)
-        e = {"class": label, "launches": n_launch, "us_in_step": cost, "share_of_step": cost / us}
+    by_kernel = []
+    for bit, label, n_launch, cls_bytes in step_classes(wl.verifier, k, j, S, B, launches_per_step, extra):
+        cost = max(us_with[bit] - us, 0.0) if bit else us - sum(e["us_in_step"] for e in by_kernel)
+        e = {"class": label, "launches": int(n_launch), "us_in_step": cost, "share_of_step": cost / us}
         if cls_bytes:
             e["algorithmic_bytes"] = int(cls_bytes)
-            e["hbm_frac"] = (cls_bytes / (cost * 1e-6) / 1e9 / hbm_peak) if cost > 0 else None
         if bit == 8:
-            e["traffic"] = NCU_TRAFFIC.get((B, "vocabulary"))
+            e["traffic"] = ncu_traffic(B, launches_per_step, "vocabulary")
         by_kernel.append(e)
-    rest = us - sum(e["us_in_step"] for e in by_kernel)
-    by_kernel.append({"class": "residual GEMMs (attention out x2, FFN2), embedding, accept scan, the rest", "launches": None,
-                      "us_in_step": rest, "share_of_step": rest / us})
     link_us = sd.link_cost(64, 148)
     round_ns = sd.cluster_round(16, 2048, 64)
     sd.close()
@@ -398,11 +417,12 @@ def verify_step_roofline(torch, binding, B: int, local: int, opts, reps: int = 5
         if sus:
             roof["frac_of_sustained_peak"] = achieved / float(sus)
     roof.update({
-        "traffic": NCU_TRAFFIC.get((B, "step")),
+        "traffic": ncu_traffic(B, launches_per_step, "step"),
         "traffic_note": "one whole step under ncu (every kernel measured with cold caches: activations that stay in L2 in a real step are counted)",
         "kernel": f"verify step (all {launches_per_step} launches): B={B}, k={k}, committed prefix {j}, source {S}, L2 flushed between repetitions",
         "peak_kind": f"of {peak_kind}", "us_per_step_median": us, "us_per_step_min": us_min, "repetitions": reps,
         "launches_per_step": int(launches_per_step), "algorithmic_bytes_per_launch": int(bytes_), "algorithmic_flops_per_launch": flops,
+        "by_kernel_note": "cost of a class = what the step grows by when each of its launches is issued twice; the second finds its weights in L2",
         "roofline_us": max(bytes_ / (hbm_peak * 1e9), flops / (tc_peak * 1e12)) * 1e6, "mean_accepted": mean_a, "by_kernel": by_kernel,
         # the step is a chain of dependent launches: what the chain alone costs, from the library's own probes
         "latency_floor": {"launches_per_step": int(launches_per_step), "us_per_kernel_boundary": link_us,

@@ -288,8 +288,9 @@ int specdec_profile_read(specdec_handle* h, double* h_ms, long long* h_launches)
  * "stats_timing" 0/1 fill ms_draft / ms_verify / ms_commit of specdec_stats (default 0; turns the gate off)
  * "profile"      0/1 see specdec_profile_read
  * "row_lse"      0/1 also accumulate the log-sum-exp of every verifier row (reported by specdec_debug_row_stats)
- * "diag_repeat"  bit mask: launch every attention (1), LayerNorm (2), non-residual GEMM (4), vocabulary kernel (8)
- *                twice in a row (same result), so the step time rises by that class's cost inside the pipeline
+ * "diag_repeat"  bit mask: launch every attention (1; with the projections that run inside it), LayerNorm (2), non-residual GEMM (4),
+ *                vocabulary kernel (8) of the path twice in a row (same result), so the step time rises by that class's cost inside
+ *                the pipeline and the launch count by its launches
  * "trace"        see specdec_debug_trace
  * "debug_checks" 0/1 see specdec_debug_integrity (default 0: the check synchronises)
  * "poke_zone" i / "heal_zones" / "poke_nan" 0|1: test hooks for that check -- damage red zone i from the host, restore

@@ -129,8 +129,8 @@ struct specdec_handle {
     int use_ln_fuse = 0;            // option "ln_fuse": measured slower than the separate LayerNorm launch, kept for comparison
     int use_sk_cluster = 1;         // option "sk_cluster": the few-rows GEMM splits long reductions across a cluster
     bool splitk_ready = false;
-    int diag_repeat = 0;            // diagnostics: launch every attention (1) / LayerNorm (2) / non-residual GEMM (4) / vocabulary (8) kernel twice (same result) to
-                                    // read its cost inside the pipeline off the step time (option "diag_repeat")
+    int diag_repeat = 0;            // diagnostics: launch every attention (1) / LayerNorm (2) / non-residual GEMM (4) / vocabulary (8) kernel of the path once more (same
+                                    // result) to read its cost inside the pipeline off the step time (option "diag_repeat")
     int use_splitk = 1;             // residual GEMMs with K >= 1024 over few row tiles split K across a cluster of 4 / 2 CTAs (option "splitk")
     bool pair_ready = false;
     int use_pair = 0;               // two-SM tiles (cta_group::2) for wide GEMMs over many rows (option "pair")
@@ -473,7 +473,7 @@ struct LnSpec { const float* x; const float* g; const float* b; };
 template <typename T>
 int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W, const float* bias, int N, int K, int cnt,
               int rows_ub, void* out, int ldo, float* resid, cudaStream_t st, const float* ldv, const int* ld_id,
-              int* n_tiles_out, const KvDest* kv, const LnSpec* lnp);
+              int* n_tiles_out, const KvDest* kv, const LnSpec* lnp, bool again = false);
 
 template <typename T>
 int gemm(specdec_handle* h, int epi, const void* A, int lda, const void* W, const float* bias, int N, int K, int cnt,
@@ -482,17 +482,15 @@ int gemm(specdec_handle* h, int epi, const void* A, int lda, const void* W, cons
          const LnSpec* lnp = nullptr) {
     TRY(gemm_once<T>(h, epi, A, lda, W, bias, N, K, cnt, rows_ub, out, ldo, resid, st, ldv, ld_id, n_tiles_out, kv, lnp));
     // diagnostics: GEMMs that only write outputs (no residual accumulation) can run twice with the same result
-    if ((h->diag_repeat & 4) && epi != EPI_RESID && epi != EPI_STATS)
-        TRY(gemm_once<T>(h, epi, A, lda, W, bias, N, K, cnt, rows_ub, out, ldo, resid, st, ldv, ld_id, n_tiles_out, kv, lnp));
-    if ((h->diag_repeat & 8) && epi == EPI_STATS)
-        TRY(gemm_once<T>(h, epi, A, lda, W, bias, N, K, cnt, rows_ub, out, ldo, resid, st, ldv, ld_id, n_tiles_out, kv, lnp));
+    if (h->diag_repeat & (epi == EPI_RESID ? 0 : epi == EPI_STATS ? 8 : 4))
+        TRY(gemm_once<T>(h, epi, A, lda, W, bias, N, K, cnt, rows_ub, out, ldo, resid, st, ldv, ld_id, n_tiles_out, kv, lnp, true));
     return 0;
 }
 
 template <typename T>
 int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W, const float* bias, int N, int K, int cnt,
               int rows_ub, void* out, int ldo, float* resid, cudaStream_t st, const float* ldv, const int* ld_id,
-              int* n_tiles_out, const KvDest* kv, const LnSpec* lnp) {
+              int* n_tiles_out, const KvDest* kv, const LnSpec* lnp, bool again) {
     if (rows_ub <= 0) return 0;
     // few rows: the weight-streaming kernel, with the LayerNorm inside where it has one
     const int width = std::min(N, K), tile_rows = sd::tc_supported(N, K) ? (cnt == CNT_ENC ? rg_tile_rows_enc(width) : rg_tile_rows(width)) : RG_MAX_ROWS;
@@ -502,7 +500,7 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
     const bool few32 = std::is_same<T, float>::value && h->use_skinny && rf_supported(epi, N, K, lnp ? K : lda, rows_ub);
     const bool ln32 = few32 && lnp && rf_ln_width(K);
     if (lnp && !ln_inside && !ln32) {  // separate normalisation launch, then a plain GEMM on its output
-        TRY(ln_or_fused<T>(h, lnp->x, lnp->g, lnp->b, cnt, rows_ub, h->y, K, st));
+        if (!again) TRY(ln_or_fused<T>(h, lnp->x, lnp->g, lnp->b, cnt, rows_ub, h->y, K, st));      // (again: the same GEMM once more, its rows are there)
         A = h->y; lda = K;
     }
     const specdec_handle::NextLn want_ln = h->next_ln;
@@ -693,12 +691,14 @@ template <typename T>
 int attn(specdec_handle* h, bool paged, const void* q, int q_stride, const int* q_index, const void* k, const void* v,
          int kv_stride, const int* kv_off, const Rows& r, const int* nkeys, int cnt, int rows_ub, int q_ub, void* out,
          int out_stride, int n_heads, int d_head, int max_keys, cudaStream_t st, const int* pre_keys = nullptr, const QueryArgs* qp = nullptr, const OutArgs* op = nullptr) {
-    TRY(attn_once<T>(h, paged, q, q_stride, q_index, k, v, kv_stride, kv_off, r, nkeys, cnt, rows_ub, q_ub, out, out_stride,
-                     n_heads, d_head, max_keys, st, pre_keys, qp, op));
-    if ((h->diag_repeat & 1) && !op)
+    if (h->diag_repeat & 1) {                          // (with the output projection inside, the extra launch leaves its rows where the feed-forward rows go later)
+        OutArgs aside{};
+        if (op) { aside = *op; aside.x_out = (float*)h->hbuf; }
         TRY(attn_once<T>(h, paged, q, q_stride, q_index, k, v, kv_stride, kv_off, r, nkeys, cnt, rows_ub, q_ub, out, out_stride,
-                         n_heads, d_head, max_keys, st, pre_keys, qp));
-    return 0;
+                         n_heads, d_head, max_keys, st, pre_keys, qp, op ? &aside : nullptr));
+    }
+    return attn_once<T>(h, paged, q, q_stride, q_index, k, v, kv_stride, kv_off, r, nkeys, cnt, rows_ub, q_ub, out, out_stride,
+                        n_heads, d_head, max_keys, st, pre_keys, qp, op);
 }
 
 // With the "profile" option on, the vocabulary-projection launches are bracketed by event pairs.
@@ -726,7 +726,8 @@ void prof_collect(specdec_handle* h) {
 // of 6 x 25 rows 108 / 103).  Blocks of a few rows leave nothing to gain (greedy steps 2 % slower).
 enum OutUse { OUT_SELF, OUT_GATHERS, OUT_QUERIES };
 bool out_inside(const specdec_handle* h, int d_head, int q_ub, int n_heads, int cnt, int rows_ub, int max_keys, OutUse use) {
-    if (!h->use_tc || !h->use_skinny || !h->use_tc_attn || !h->use_sk_cluster || h->use_ln_fuse || (h->diag_repeat & 1)) return false;
+    if (!h->use_tc || !h->use_skinny || !h->use_tc_attn || !h->use_sk_cluster || h->use_ln_fuse) return false;
+    if ((h->diag_repeat & 1) && 2 * n_heads * d_head > std::min(h->cfg.verifier.d_ffn, h->cfg.drafter.d_ffn)) return false;    // (no room for the extra launch's rows)
     if (d_head != 64 || (n_heads != 4 && n_heads != 8) || q_ub <= 4) return false;
     const long long ctas = (long long)cdiv(q_ub, 16) * n_heads * (cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub));
     if (ctas > (use == OUT_QUERIES ? 32 : use == OUT_GATHERS ? 96 : 64) || (use == OUT_QUERIES && rows_ub > 48)) return false;
@@ -982,19 +983,21 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
                          last ? m.dec_lnf_b : m.dec[l + 1].ln1_b));
     }
     const bool ln_pending = !(h->x == h->fused_x && m.dec_lnf_g == h->fused_g && h->y == h->fused_out);
-    if (ln_pending && d <= 1024 && !(h->diag_repeat & 2)) {
+    if (ln_pending && d <= 1024) {
         // final LayerNorm and the pre-pass logit of every row's draft in one kernel
-        cudaError_t e = cudaSuccess;
-        const dim3 grid(cdiv(M, 8)), block(256);
+        for (int i = 0; i < (h->diag_repeat & 2 ? 2 : 1); ++i) {
+            cudaError_t e = cudaSuccess;
+            const dim3 grid(cdiv(M, 8)), block(256);
 #define LN_LD(NC) e = launch_pdl(h, k_layernorm_ld<T, NC>, grid, block, 0, st, (const float*)h->x, (const float*)m.dec_lnf_g, (const float*)m.dec_lnf_b, (T*)h->y, d, 1e-5f, \
-                                 (const T*)m.embed, d_draft, (const int*)h->rows.slot_seq, (const int*)(h->ses.counters + CNT_VERIFY), k, m.dm.vocab, h->ld, h->ld_id)
-        switch (cdiv(d, 128)) {
-            case 1: LN_LD(1); break; case 2: LN_LD(2); break; case 3: LN_LD(3); break; case 4: LN_LD(4); break;
-            case 5: LN_LD(5); break; case 6: LN_LD(6); break; case 7: LN_LD(7); break; default: LN_LD(8); break;
-        }
+                                     (const T*)m.embed, d_draft, (const int*)h->rows.slot_seq, (const int*)(h->ses.counters + CNT_VERIFY), k, m.dm.vocab, h->ld, h->ld_id)
+            switch (cdiv(d, 128)) {
+                case 1: LN_LD(1); break; case 2: LN_LD(2); break; case 3: LN_LD(3); break; case 4: LN_LD(4); break;
+                case 5: LN_LD(5); break; case 6: LN_LD(6); break; case 7: LN_LD(7); break; default: LN_LD(8); break;
+            }
 #undef LN_LD
-        if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("final layer norm launch: ") + cudaGetErrorString(e));
-        KCHECK(h);
+            if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("final layer norm launch: ") + cudaGetErrorString(e));
+            KCHECK(h);
+        }
     } else {
         TRY(ln_or_fused<T>(h, h->x, m.dec_lnf_g, m.dec_lnf_b, CNT_VERIFY, M, h->y, d, st));
         CUDA_TRY(h, launch_pdl(h, k_draft_logit<T>, dim3(cdiv(M, 4)), dim3(128), 0, st, (const T*)h->y, (const T*)m.embed,
