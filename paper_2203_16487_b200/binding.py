@@ -346,7 +346,7 @@ def accept_scan(logits: torch.Tensor, drafts: torch.Tensor, beta: int, tau: floa
 def accept_scan_static(logits: torch.Tensor, drafts: torch.Tensor, beta: int, tau: float,
                        acc: Optional[torch.Tensor] = None, bif: Optional[torch.Tensor] = None):
     """specdec_accept_scan_static: the acceptance rule for callers that cannot allocate device memory
-    (the partial statistics sit in an array compiled into the library).  Pass preallocated `acc` and
+    (its partial statistics stay in shared memory).  Pass preallocated `acc` and
     `bif` [B] int32 device tensors to keep the call itself free of any allocation."""
     assert logits.is_cuda and logits.dtype == torch.float32 and logits.is_contiguous()
     B, k1, V = logits.shape

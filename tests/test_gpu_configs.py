@@ -85,14 +85,15 @@ def test_config3_batch32_all_nine_cells(base):
 def test_config3_batch128_sampled_sequences(base, pair):
     """Config 3, batch 128 at (beta, tau) = (3, 1): twelve sequences over their whole length against the oracle, and
     batch invariance on the device.  pair = 1: the wide GEMMs over many rows (QKV, FFN1, vocabulary, encoder K/V) run as
-    two-SM tiles, and every LayerNorm is applied inside the residual GEMM before it (clusters of four CTAs per row tile)."""
+    two-SM tiles, every LayerNorm is applied inside the residual GEMM before it (clusters of four CTAs per row tile), and
+    attention takes 64 queries to a CTA at every size."""
     binding, wv, wd, mv, md = base
     wl = W.config3_batched(128)
     smax, tmax = max(len(s) for s in wl.src), max(wl.max_tgt)
     sd = binding.SpecDec(W.BASE_V, wv, W.BASE_D, wd, k_max=25, max_batch=128, max_src=smax, max_tgt=tmax, bf16=True)
     sd.set_option("pair", pair)
     sd.set_option("ln_fuse", pair)
-    sd.set_option("attn_rs", 2 if pair else 1)             # 2: attention scores stay in registers wherever the keys allow
+    sd.set_option("attn_stream", 2 if pair else 1)
     src, lens = W.pad_batch(wl.src)
     out, n, st = sd.generate(src, lens, wl.max_tgt, 25, 3, 1.0)
     out, n = out.cpu().numpy(), n.cpu().numpy()

@@ -320,8 +320,8 @@ def test_bf16_mid_lockstep(gemm, attn):
 
 @pytest.mark.parametrize("nseq,skinny", [(2, 1), (4, 1), (2, 0), (4, 2)])
 def test_bf16_mid_small_batches_weight_streaming_gemm(nseq, skinny):
-    """Passes of at most 32 rows run the weight-streaming GEMM with fused LayerNorm (26 rows: two 16-row
-    tiles); 52 rows run one 128-row tile of the tensor-core GEMM with 64-wide column tiles."""
+    """Verify blocks of 26 and 52 rows (two and four 16-row tiles of the few-rows GEMM, LayerNorm inside); 26 rows on one 128-row tile of
+    the tensor-core GEMM; and 52 rows with every LayerNorm inside the residual GEMM before it and attention CTAs of 32 queries."""
     wv, wd = W.make_weights(MID_V, 21, True), W.make_weights(MID_D, 22, True)
     mv, md = O.model_from(MID_V, wv, mode="bf16"), O.model_from(MID_D, wd, mode="bf16")
     rng = np.random.default_rng(8)
@@ -329,7 +329,7 @@ def test_bf16_mid_small_batches_weight_streaming_gemm(nseq, skinny):
     sd = _handle(MID_V, wv, MID_D, wd, True, k_max=12, max_batch=4, max_src=40, max_tgt=24)
     sd.set_option("skinny", min(skinny, 1))
     sd.set_option("ln_fuse", 1 if skinny == 2 else 0)      # 2: also fuse each LayerNorm into the residual GEMM before it
-    sd.set_option("attn_rs", 2 if skinny == 2 else 1)      # ... and keep attention scores in registers wherever possible
+    sd.set_option("attn_stream", 3 if skinny == 2 else 1)  # ... and let every attention warp take 16 queries and all keys
     rep = lockstep.run(sd, mv, md, srcs, [24, 18, 9, 20][:nseq], 12, 3, 1.0, margin=1e-3, check_logits_every=2)
     print(rep.iterations, rep.draft_near_ties, rep.verify_near_ties, rep.max_logit_err, rep.max_stat_err)
     assert rep.ok, rep.notes
@@ -339,7 +339,7 @@ def test_bf16_mid_small_batches_weight_streaming_gemm(nseq, skinny):
 
 @pytest.mark.parametrize("long_keys,mode", [(False, 2), (True, 2), (True, 3)])
 def test_bf16_streaming_attention(long_keys, mode):
-    """The streaming tile attention (key blocks of 64 through a two-stage ring, running maximum) against the
+    """Attention with all keys of a query in one warp (blocks of 64 keys through a ring, running maximum) against the
     oracle's one-pass softmax: forced on for the short case (a single, partly filled block), and over sources of
     up to 200 tokens and targets past 64 (several blocks, ragged last block, causal mask crossing a block edge)."""
     dv = W.ModelDims(128, 2, 512, 2000, 2, 2, 256)
@@ -353,7 +353,7 @@ def test_bf16_streaming_attention(long_keys, mode):
         lens, tgts, max_src, max_tgt = (20, 7, 33, 12), [24, 18, 9, 20], 40, 24
     srcs = [W.zipf_ids(rng, n, 2000) for n in lens]
     sd = _handle(dv, wv, dd, wd, True, k_max=12, max_batch=4, max_src=max_src, max_tgt=max_tgt)
-    sd.set_option("attn_stream", mode)                       # 2: four-stage ring here (few CTAs), 3: the two-stage ring
+    sd.set_option("attn_stream", mode)                       # 2: 64 queries to a CTA, a ring of two blocks; 3: 32 queries, three blocks
     rep = lockstep.run(sd, mv, md, srcs, tgts, 12, 3, 1.0, margin=1e-3, check_logits_every=2)
     print(rep.iterations, rep.draft_near_ties, rep.verify_near_ties, rep.max_logit_err, rep.max_stat_err)
     assert rep.ok, rep.notes
@@ -363,8 +363,8 @@ def test_bf16_streaming_attention(long_keys, mode):
 
 @pytest.mark.parametrize("sk_cluster", [1, 0])
 def test_base_shapes_batch1_lockstep(sk_cluster):
-    """One config-2 sentence at batch 1 (26-row verify block): per-operation kernels with the weight-streaming GEMM,
-    its LayerNorm prologue shared across clusters of 8 CTAs (the default) or computed by every CTA."""
+    """One config-2 sentence at batch 1 (26-row verify block): the few-rows kernels with the output projections inside the attention and
+    FFN2 split along K (clusters of 8 and of 2 CTAs, the default), or with neither."""
     wl = W.config2_translation(1)
     wv = W.make_weights(wl.verifier, wl.seed_verifier, True)
     wd = W.make_weights(wl.drafter, wl.seed_drafter, True)

@@ -1,8 +1,7 @@
 """specdec_accept_scan_static -- the acceptance rule for callers that cannot allocate device memory
-(for example inside a server whose pool already owns all of HBM): its intermediate statistics sit in a
-fixed array inside the library.  Checked through the C ABI against the oracle's rule row by row and against
-specdec_accept_scan, on two calls in a row that share that array, the second smaller than the first so stale
-entries would show.  Collected last on purpose, so a run that stops at the first failure has already run
+(for example inside a server whose pool already owns all of HBM): its intermediate statistics sit in shared
+memory.  Checked through the C ABI against the oracle's rule row by row and against specdec_accept_scan, on two
+calls in a row into the same outputs, the second smaller than the first.  Collected last on purpose, so a run that stops at the first failure has already run
 everything else."""
 import numpy as np
 import pytest
@@ -47,7 +46,7 @@ def test_static_scratch_variant_matches_on_two_calls_in_a_row():
 
 
 def test_static_scratch_variant_long_blocks():
-    """Blocks of more than 256 rows per sequence take the scan's second code path (no per-row flag byte)."""
+    """Blocks of more than 256 rows per sequence: many groups of rows, a rejection far behind the first."""
     from paper_2203_16487_b200 import binding
     rng = np.random.default_rng(7)
     B, k, V = 2, 300, 700
