@@ -7,7 +7,7 @@
 // itself; the rows of later groups are never read.  32 x 26 x 32768 logits: 994 -> 22 us (one CTA per sequence, a row at a time,
 // 4 bytes a load, before); 128 sequences: 1010 -> 47 us.
 #pragma once
-#include "gemm_tc.cuh"
+#include "barriers.cuh"
 #include "kernels.cuh"
 
 namespace sd {

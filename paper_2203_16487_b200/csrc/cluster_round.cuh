@@ -3,7 +3,7 @@
 // rounds (every CTA sends its share of a small operand tile to every peer, then all wait for all): this measures
 // what a round costs, empty and with data, so the two can be compared.
 #pragma once
-#include "gemm_tc.cuh"
+#include "barriers.cuh"
 
 namespace sd {
 

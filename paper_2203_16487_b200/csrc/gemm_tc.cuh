@@ -21,48 +21,12 @@
 #include <string>
 #include <tuple>
 
+#include "barriers.cuh"
 #include "kernels.cuh"
 
 namespace sd {
 
 // ------------------------------------------------------------------ PTX wrappers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok;
-}
-// Bounded wait: gives up after ~2e8 clocks, raises the CTA-wide abort flag and the global error word.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err_word,
-                                          int code) {
-    if (mbar_try_wait(bar, parity)) return true;      // fast path: no other shared-memory access
-    if (*abort_flag) return false;
-    const long long t0 = clock64();
-    while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > 200000000LL) {
-            *abort_flag = 1;
-            atomicExch(err_word, code);
-            return false;
-        }
-    }
-}
-// The same for a converged warp: every lane gets the same answer, as an elected instruction behind it needs all of them there.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err_word, int code) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, err_word, code));
-}
 constexpr int TC_BM = 128, TC_BK = 64;
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, uint32_t bar) {
     asm volatile(
@@ -149,9 +113,6 @@ template <int BN, int AR = 128, bool STG = true, bool LNF = false> struct TcCfg 
     static constexpr int TMEM_COLS = 2 * BN <= 32 ? 32 : (2 * BN <= 64 ? 64 : (2 * BN <= 128 ? 128 : (2 * BN <= 256 ? 256 : 512)));  // two accumulators, power of two
 };
 
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 // CW consecutive fp32 columns (CW = 16 or 32) of this thread's TMEM lane.
 template <int CW>
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, float* v) {
@@ -209,9 +170,6 @@ __device__ __forceinline__ void tmem_ld_done(uint32_t* r) {
     }
 }
 
-__device__ __forceinline__ void tc_cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ uint32_t tc_cluster_nctas() {
     uint32_t n;
     asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n));

@@ -2,7 +2,7 @@
 // pair is a chain of some forty launches over kilobytes -- so, as in the bf16 path, everything that predates the
 // predecessor (weights, page rows, cached keys) is requested before the dependency wait, the LayerNorm in front runs inside, K and V
 // leave the QKV epilogue for the cache, and the work of a launch is spread over enough warps for one short round trip.
-#include "gemm_tc.cuh"
+#include "barriers.cuh"
 #include "rows_f32.cuh"
 #include "attention.cuh"
 

@@ -1,6 +1,6 @@
 // GEMM for passes of few activation rows (see rows_gemm.cuh for where it is used).
 #include "attention.cuh"
-#include "gemm_tc.cuh"
+#include "barriers.cuh"
 #include "rows_gemm.cuh"
 
 namespace sd {
