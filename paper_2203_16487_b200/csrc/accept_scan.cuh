@@ -12,7 +12,6 @@
 
 namespace sd {
 
-
 __device__ __forceinline__ void as_take(RowPart& m, float x, int v, float ld) {
     if (x > m.mx || (x == m.mx && v < m.arg)) { m.mx = x; m.arg = v; }
     m.cnt += (x > ld) ? 1 : 0;
@@ -28,6 +27,7 @@ k_accept_scan(const float* __restrict__ logits, const int* __restrict__ draft, i
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint32_t rank = 0;
     if (CL > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    if (CL > 1) cluster_arrive();                // waited for before anything is sent: a peer's shared memory is there once the peer has begun
     const int b = blockIdx.x / CL, part = (int)rank * WPR + warp % WPR, parts = CL * WPR;
     // the draft of this warp's row in the next group is fetched a group ahead, so that its logit does not wait for it
     int tok_next = (warp / WPR < k) ? draft[b * k + warp / WPR] : -1;
@@ -76,6 +76,8 @@ k_accept_scan(const float* __restrict__ logits, const int* __restrict__ draft, i
         }
         m.sum = ld;                                      // (the unused field carries the draft's logit)
         RowPart* slot = &inbox[it & 1][part][warp / WPR];
+        __syncwarp();
+        if (CL > 1 && it == 0) cluster_wait();
         if (lane < CL) {                                 // one lane per peer
             if (CL == 1) *slot = m;
             else {
@@ -85,6 +87,7 @@ k_accept_scan(const float* __restrict__ logits, const int* __restrict__ draft, i
                              ::"r"(ra), "r"(__float_as_uint(m.mx)), "r"(m.arg), "r"(__float_as_uint(m.sum)), "r"(m.cnt) : "memory");
             }
         }
+        __syncwarp();
         if (CL > 1) tc_cluster_sync(); else __syncthreads();
         // every warp merges the group by itself: 32 / GR lanes per row, each over its share of the senders
         constexpr int LPR = 32 / GR;

@@ -16,6 +16,7 @@
 // step with 12 warps and a ring of three 1107 us, now 1055-1075) or of 32 queries with 32-key blocks (x 26 x 90: 555 with 8 warps and
 // 64-key blocks, now 514).  Below four CTAs an SM there is nothing to fill the SMs with, and 64-key blocks have more independent work per barrier.
 #pragma once
+#include "barriers.cuh"
 #include "kernels.cuh"
 
 namespace sd {
@@ -83,9 +84,6 @@ struct OutArgs {
 };
 // Bytes behind the ring: 16 rows and 64 rows of weights for each projection that runs inside.
 template <int QNC, int ON> struct ProjCfg { static constexpr int OPS = QueryCfg<QNC>::OPS + QueryCfg<ON / 2>::OPS; };
-
-__device__ __forceinline__ void attn_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void attn_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // 16 x 64 partial products of a CTA's eight warps: warp = (K slice of four, half of the columns); A: 16 rows, W: 64 rows of PITCH bytes.
 // The slices meet in `red` ([4][16][72] floats); thread t then holds row t / 16, columns 4 (t % 16) .. + 3 of the sum.
@@ -206,7 +204,7 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
             const int r = i / (OC::K / 8), c = i % (OC::K / 8);
             cp_async16(oops + (16 + r) * OC::PITCH + c * 16, w + (size_t)r * OC::K + c * 8);
         }
-        attn_cluster_arrive();
+        cluster_arrive();
         ob = ldg_pinned(reinterpret_cast<const float4*>(oa.b + h * 64 + (tid & 15) * 4));
     }
     int* s_row = reinterpret_cast<int*>(qops + ProjCfg<QNC, ON>::OPS);            // paged: K / V row of every key
@@ -493,7 +491,7 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
             const bool odd = lane & 1;
             // eight columns of a row: the even lane sends them to the lower half of the cluster, the odd lane to the upper
             const uint32_t dst = oops + rr * OC::PITCH + (h * 64 + kg * CW) * 2;
-            attn_cluster_wait();                          // every CTA of the cluster has begun and its 16 rows are free
+            cluster_wait();                          // every CTA of the cluster has begun and its 16 rows are free
 #pragma unroll
             for (int i = 0; i < ON / 2; ++i) {
                 uint32_t ra;
@@ -501,8 +499,8 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
                 asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
                              ::"r"(ra), "r"(odd ? w0 : u0), "r"(odd ? w1 : u1), "r"(odd ? u0 : w0), "r"(odd ? u1 : w1) : "memory");
             }
-            attn_cluster_arrive();
-            attn_cluster_wait();
+            cluster_arrive();
+            cluster_wait();
             wo.multiply(oops, mO, warp, lane);             // (the partial outputs of the key groups are dead)
             __syncthreads();
             const float4 t = Proj64<OC::K>::sum(mO, tid);

@@ -27,6 +27,12 @@ def test_accept_scan_edges(B, k, V):
         drafts[2, 0] = V + 3                                                 # not a token: rejected
     lg, dr = torch.from_numpy(logits).cuda(), torch.from_numpy(drafts).cuda()
     for beta, tau in ((3, 1.0), (1, 0.0)):
+        # (other work holds SMs meanwhile, so that the CTAs of a cluster need not begin together)
+        other = torch.cuda.Stream()
+        with torch.cuda.stream(other):
+            busy = torch.ones((2048, 2048), device="cuda")
+            for _ in range(8):
+                busy = busy @ busy * 1e-4
         a, t = binding.accept_scan(lg, dr, beta, tau)
         for b in range(B):
             row = drafts[b].tolist()
