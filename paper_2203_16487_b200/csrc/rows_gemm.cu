@@ -32,11 +32,11 @@ __device__ __forceinline__ void rg_st_peer16(uint32_t local_addr, uint32_t local
 
 // One CTA = 16 MT rows x 8 NT columns, K walked by the warps side by side (WN warps across the columns, 8 / WN K slices).
 //
-// Bound: latency.  A decoding step is a chain of some fifty such launches, each over 0.5-2 MB of weights, so what counts is the
+// Bound: latency.  A decoding step is a chain of 34 launches, 18 of them these, each over 0.5-2 MB of weights, so what counts is the
 // time from the predecessor's last store to this kernel's.  Hence:
 //   * everything that does not depend on the predecessor -- the CTA's whole weight tile into shared memory, LayerNorm
 //     parameters, cache rows -- is requested before the dependency wait;
-//   * 256 threads of at most 80 registers and 20-100 KB of shared memory, so that the next two kernels of the chain are resident
+//   * 256 threads of at most 80 registers (118 where a LayerNorm of 768 columns runs inside) and 20-100 KB of shared memory, so that the next two kernels of the chain are resident
 //     (their weights landed) while this one runs.  A 512-thread version with the weights in registers had shorter phases and a
 //     longer step (240 against 218 us), because its successors could not start early;
 //   * after the wait one round trip brings the rows; with NC > 0 they are normalised on the way (K = 128 NC, two rows per
@@ -309,11 +309,9 @@ bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster) {
 template <int EPI, int NC>
 inline cudaError_t rg_launch_out(const RowsArgs& a, int rows_ub, bool pdl, cudaStream_t st) {
     const bool wide = a.g.N >= 1024;
-    if (NC == 0 && rows_ub > rg_ln_rows(min(a.g.N, a.g.K))) {
-        return rg_launch_one<EPI, 0, 2, 8, 2, 1>(a, rows_ub, pdl, st);
-    }
+    if constexpr (NC == 0) { if (rows_ub > rg_ln_rows(min(a.g.N, a.g.K))) return rg_launch_one<EPI, 0, 2, 8, 2, 1>(a, rows_ub, pdl, st); }
     if (wide) return rg_launch_one<EPI, NC, 1, 8, 2, 1>(a, rows_ub, pdl, st);
-    if (EPI == EPI_STORE && rows_ub > 32) return rg_launch_one<EPI, NC, 1, 4, 1, 1>(a, rows_ub, pdl, st);
+    if constexpr (EPI == EPI_STORE) { if (rows_ub > 32) return rg_launch_one<EPI, NC, 1, 4, 1, 1>(a, rows_ub, pdl, st); }
     return rg_launch_one<EPI, NC, 1, 2, 1, 1>(a, rows_ub, pdl, st);
 }
 static cudaError_t rg_launch_resid(const RowsArgs& a, int rows_ub, bool cluster, bool pdl, cudaStream_t st) {
@@ -354,9 +352,9 @@ static void rg_room(cudaError_t& e) {
 }
 template <int EPI, int NC>
 static void rg_room_out(cudaError_t& e) {
-    if (NC == 0) rg_room<EPI, 0, 2, 8, 2, 1>(e);
+    if constexpr (NC == 0) rg_room<EPI, 0, 2, 8, 2, 1>(e);
     rg_room<EPI, NC, 1, 8, 2, 1>(e);
-    if (EPI == EPI_STORE) rg_room<EPI, NC, 1, 4, 1, 1>(e);
+    if constexpr (EPI == EPI_STORE) rg_room<EPI, NC, 1, 4, 1, 1>(e);
     rg_room<EPI, NC, 1, 2, 1, 1>(e);
 }
 template <int EPI>
