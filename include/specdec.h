@@ -273,7 +273,7 @@ int specdec_profile_read(specdec_handle* h, double* h_ms, long long* h_launches)
  * "enc_skinny"   0 / 1 (default) / 2: the weight-streaming GEMM does not / does / does serve the encoders (up to 72 rows, wider
  *                than 512 up to 40)
  * "ln_fuse"      0/1 the LayerNorm that reads the residual stream next runs inside the residual GEMM (default 0)
- * "splitk"       0/1 residual GEMMs with K >= 1024 over few row tiles split K across a cluster (default 1)
+ * "splitk"       0/1 residual GEMMs with K >= 768 over few row tiles split K across a cluster (default 1)
  * "attn_stream"  0 / 1 by rule (default) / 2 / 3 / 4: attention CTAs of 16 queries with the keys spread over their warps, or of
  *                64 (2) or 32 (3, 4: 32-key blocks) queries with 16 to a warp
  * "attn_warps"   0 by rule (default), 4 or 8: the former with that many warps.  ("attn_rs" and "attn_stream_keys" are accepted

@@ -4,8 +4,8 @@
 // cluster's CTAs split a row's columns and the warps of a CTA take GR rows at once (W / GR warps to a row), so a lane keeps
 // eight 16-byte loads in flight.  After each group of GR rows every warp sends its (max, argmax, count) to the
 // cluster's shared memories, and behind one cluster barrier each CTA merges them and finds the first rejected draft by
-// itself; the rows of later groups are never read.  32 x 26 x 32768 logits: 994 -> 22 us (one CTA per sequence, a row at a time,
-// 4 bytes a load, before); 128 sequences: 1010 -> 47 us.
+// itself; the rows of later groups are never read.  32 x 26 x 32768 logits, launched from the Python binding one after the other: 1001 -> 22 us
+// (one CTA per sequence, a row at a time, 4 bytes a load, before); 128 sequences: 1010 -> 47 us.
 #pragma once
 #include "barriers.cuh"
 #include "kernels.cuh"
@@ -129,11 +129,16 @@ inline cudaError_t as_launch_one(const float* logits, const int* draft, int B, i
     return cudaLaunchKernelEx(&cfg, k_accept_scan<CL, GR, W>, logits, draft, k, V, beta, tau, acc, bif);
 }
 
-// The split by size (us at k = 25, V = 32768, a draft wrong once in seven; launches 8.5 us apart from the Python binding):
-// short rows are one CTA's work and an exchange would cost more than it saves (128 x 21 x 1000: 8.8 with one CTA, 12.5 with
-// eight); up to 16 sequences the SMs are empty, so 256 warps a sequence (16: 14.5, with 64 warps 24.7); up to 32 half as many
-// (22.5 / 28.7); beyond, groups of 8 rows and 8-warp CTAs, so that the rows read past a rejection stay few (128: 47,
-// with 16-row groups 55-68; all rows of 128 x 26 would be 436 MB = 68 us).
+// The split by size.  us between events around one launch, logits not in L2, a draft wrong once in seven, k = 25; the variants in the order of
+// the rule (one CTA | 256 warps a sequence | 128 warps | 128 in small CTAs with groups of 8 rows), * = taken:
+//   V = 1000    16 sequences  14* 12 10 14      64  16* 23 14 19     128  16* 40 20 31
+//   V = 4096    16            18* 14 12 14      64  23* 25 16 21     128  23* 41 23 31
+//   V = 8192    16  31 13* 12 16    32  32 19 14* 18    33  33 20 14 18*    64  33 29 21 25*    128  33 43 29 33*
+//   V = 32768   16  94 21* 23 25    17  94 21 23* 25    27  96 29 27* 27    33  74 29 28 27*    64  96 45 42 35*    128  99 72 64 55*
+//   V = 50265   16 147 25* 32 33    17 147 27 33* 35    27 147 37 37* 37    33 115 39 39 34*    64 150 60 61 53*    128 154 100 94 78*
+// The wider the row, the longer 256 warps pay, until their CTAs (three of 16 warps to an SM) no longer run at once, from 28 sequences on; the
+// groups of 8 read fewer rows past a rejection, which counts once memory is busy.  Short blocks prefer groups of 16 longer (k = 8, V = 32768:
+// 64 sequences 53 35 27 31*).  Between neighbouring variants the lines cost at most 7 us where they are not best.
 inline cudaError_t as_launch(const float* logits, const int* draft, int B, int k, int V, int beta, float tau, int* acc, int* bif, cudaStream_t st) {
     if (V <= 4096) return as_launch_one<1, 8, 16>(logits, draft, B, k, V, beta, tau, acc, bif, st);
     if (B <= 16) return as_launch_one<16, 16, 16>(logits, draft, B, k, V, beta, tau, acc, bif, st);

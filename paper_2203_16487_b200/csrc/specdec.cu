@@ -131,7 +131,7 @@ struct specdec_handle {
     bool splitk_ready = false;
     int diag_repeat = 0;            // diagnostics: launch every attention (1) / LayerNorm (2) / non-residual GEMM (4) / vocabulary (8) kernel of the path once more (same
                                     // result) to read its cost inside the pipeline off the step time (option "diag_repeat")
-    int use_splitk = 1;             // residual GEMMs with K >= 1024 over few row tiles split K across a cluster of 4 / 2 CTAs (option "splitk")
+    int use_splitk = 1;             // residual GEMMs with K >= 768 over few row tiles split K across a cluster of 4 / 2 CTAs (option "splitk")
     bool pair_ready = false;
     int use_pair = 0;               // two-SM tiles (cta_group::2) for wide GEMMs over many rows (option "pair")
     int attn_stream = 1;            // attention variant (option "attn_stream")
@@ -1189,8 +1189,8 @@ int generate_loop(specdec_handle* h, const int* d_src, const int* d_src_len, con
     bool gated = graphs && h->gate_ok && !phases && (h->use_gate == 1 ? B > 4 : h->use_gate == 2);
     // How many iterations the host runs ahead of the post it reads.  The default waits for each post: the few microseconds until the
     // next launch arrives cost less than what running ahead does -- an iteration queued after the last sequence finished is a
-    // wasted pass, launches are sized by an older count of unfinished sequences, and a conditional node in front of the iteration (option
-    // "gate") adds some 40 us to it (32 sequences: 7.75 ms waiting, 8.07 one ahead, 8.43 two ahead, 8.38 two ahead and gated).
+    // wasted pass, and launches are sized by an older count of unfinished sequences (32 sequences: 7.75 ms waiting, 8.07 one ahead, 8.43 two
+    // ahead).  A conditional node in front of the iteration (option "gate") saves the wasted pass but adds some 40 us to each (8.38 two ahead).
     const int slots = (int)h->poll_ev.size();
     int lag = h->poll_lag >= 0 ? std::min(h->poll_lag, slots - 1) : (gated ? 2 : 0);
     int it = 0, skipped = 0;
