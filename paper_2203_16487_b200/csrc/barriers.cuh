@@ -25,7 +25,9 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok;
 }
-// Bounded wait: gives up after ~2e8 clocks, raises the CTA-wide abort flag and the global error word.
+// Bounded wait: gives up after ~2e8 clocks, raises the CTA-wide abort flag and the global error word.  The warp that gives up then holds the
+// CTA, and with it the shared memory that its copies in flight and its peers still write to, for about a millisecond longer: many times what
+// a copy that was issued before the flag was up can take.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err_word,
                                           int code) {
     if (mbar_try_wait(bar, parity)) return true;      // fast path: no other shared-memory access
@@ -37,6 +39,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         if (clock64() - t0 > 200000000LL) {
             *abort_flag = 1;
             atomicExch(err_word, code);
+            while (clock64() - t0 < 202000000LL) {}
             return false;
         }
     }
