@@ -30,6 +30,7 @@ struct AttnTcArgs {
     const int* kv_off;
     Paged pg;                                             // paged: row pg.row(b, t)
     const int* q_off; const int* q_cnt;                   // per sequence: first query row, number of query rows
+    const int* seq_of;                                    // the sequence of grid slice z (-1: none), or null: slice z is sequence z
     const int* nkeys;                                     // per query row: visible keys (0..nkeys-1)
     const int* pre_keys;                                  // per sequence (or null): keys 0..pre-1 were written before this
                                                           // step began, so they may be fetched before the dependency wait
@@ -170,7 +171,8 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ int s_nk[BM];
     __shared__ int s_nkmax;
-    const int b = blockIdx.z, h = blockIdx.y, qt = blockIdx.x;
+    const int b = a.seq_of ? a.seq_of[blockIdx.z] : (int)blockIdx.z, h = blockIdx.y, qt = blockIdx.x;
+    if (b < 0) return;
     // Row metadata, page table and sequence lengths are written at the start of the step, before the first
     // kernel of the programmatic-launch chain can begin, so they may be read before the dependency wait.
     const int cnt = a.q_cnt[b], q_first = a.q_off[b];
@@ -494,7 +496,7 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
             const bool odd = lane & 1;
             // eight columns of a row: the even lane sends them to the lower half of the cluster, the odd lane to the upper
             const uint32_t dst = oops + rr * OC::PITCH + (h * 64 + kg * CW) * 2;
-            cluster_wait();                          // every CTA of the cluster has begun and its 16 rows are free
+            cluster_wait();                          // every CTA of the cluster has begun and its barrier exists
 #pragma unroll
             for (int i = 0; i < ON / 2; ++i) {
                 uint32_t ra;

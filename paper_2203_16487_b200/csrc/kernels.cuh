@@ -99,7 +99,8 @@ struct Rows {
     int* slot;      // mask-only pass: index into the [B,k] draft array
     int* q_off;     // [B] first row of the sequence in this pass
     int* q_cnt;     // [B] rows of the sequence in this pass (0: none)
-    int* slot_seq;  // [B] verify pass: the sequence whose block starts at row slot * (k + 1)
+    int* slot_seq;  // [B] verify pass: the sequence whose block starts at row slot * (k + 1); mask-only pass: the sequence whose
+                    // [MASK] rows start at row slot * k, for both passes of the drafter (-1: none)
 };
 
 // ------------------------------------------------------------------ row preparation
@@ -257,11 +258,14 @@ __global__ void k_draft_prep(Session s, int B, int k, int bos, int mask, Rows al
         msk.kv_off[b] = off; msk.kv_off_cross[b] = s.src_off[b];
         all.q_off[b] = off; all.q_cnt[b] = n;
         msk.q_off[b] = moff; msk.q_cnt[b] = fin ? 0 : k;
+        if (!fin) msk.slot_seq[moff / k] = b;
         if (b == 0) {
             s.counters[CNT_DRAFT_ALL] = total;
             s.counters[CNT_DRAFT_MASK] = live * k;  // k mask rows per unfinished sequence
         }
     }
+    if (b == 0 && part == 0)
+        for (int o = live + tid; o < B; o += blockDim.x) msk.slot_seq[o] = -1;
     for (int t = t0 + tid; t < t1; t += blockDim.x) {
         const int row = off + t;
         all.tok[row] = (t == 0) ? bos : (t <= j ? s.out[(size_t)b * s.out_stride + t - 1] : mask);
@@ -320,11 +324,14 @@ __global__ void k_draft_prep_pc(Session s, int B, int k, int bos, int mask, Rows
         msk.kv_off[b] = off; msk.kv_off_cross[b] = s.src_off[b];
         all.q_off[b] = off; all.q_cnt[b] = n;
         msk.q_off[b] = moff; msk.q_cnt[b] = fin ? 0 : k;
+        if (!fin) msk.slot_seq[moff / k] = b;
         if (b == 0) {
             s.counters[CNT_DRAFT_ALL] = total;
             s.counters[CNT_DRAFT_MASK] = live * k;
         }
     }
+    if (b == 0 && part == 0)
+        for (int o = live + tid; o < B; o += blockDim.x) msk.slot_seq[o] = -1;
     if (!fin) {
         for (int t = t0 + tid; t < t1; t += blockDim.x) {
             const int row = off + t, p = c + t;

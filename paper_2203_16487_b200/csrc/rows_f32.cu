@@ -255,7 +255,8 @@ static size_t af_smem(int dh, int max_keys) {
 template <bool PAGED>
 __global__ void __launch_bounds__(AF_WARPS * 32) k_attn_f32(AttnF32Args a) {
     extern __shared__ __align__(16) float af_sm[];
-    const int b = blockIdx.z, h = blockIdx.y, qt = blockIdx.x;
+    const int b = a.seq_of ? a.seq_of[blockIdx.z] : (int)blockIdx.z, h = blockIdx.y, qt = blockIdx.x;
+    if (b < 0) return;
     // (row metadata, page table and sequence lengths predate the step's kernel chain: readable before the wait)
     const int cnt = a.q_cnt[b], q_first = a.q_off[b];
     const int pre = a.pre_keys ? min(a.pre_keys[b], a.max_keys) : 0, kv0 = PAGED ? 0 : a.kv_off[b];
@@ -349,10 +350,10 @@ __global__ void __launch_bounds__(AF_WARPS * 32) k_attn_f32(AttnF32Args a) {
 bool af_supported(int d_head, int max_keys) {
     return d_head >= 4 && d_head <= 128 && (d_head & (d_head - 1)) == 0 && af_smem(d_head, max_keys) <= RF_MAX_SMEM;
 }
-cudaError_t af_launch(bool paged, const AttnF32Args& a, int q_ub, int n_heads, int B, bool pdl, cudaStream_t st) {
+cudaError_t af_launch(bool paged, const AttnF32Args& a, int q_ub, int n_heads, int slots, bool pdl, cudaStream_t st) {
     auto go = [&](auto* kernel) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((q_ub + AF_Q - 1) / AF_Q, n_heads, B); cfg.blockDim = dim3(AF_WARPS * 32);
+        cfg.gridDim = dim3((q_ub + AF_Q - 1) / AF_Q, n_heads, slots); cfg.blockDim = dim3(AF_WARPS * 32);
         cfg.dynamicSmemBytes = af_smem(a.d_head, a.max_keys); cfg.stream = st;      // (allowed by rf_init)
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

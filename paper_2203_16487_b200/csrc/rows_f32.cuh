@@ -20,6 +20,7 @@ struct AttnF32Args {
     const int* kv_off;
     Paged pg;                                             // paged: row pg.row(b, t)
     const int* q_off; const int* q_cnt;                   // per sequence: first query row, number of query rows
+    const int* seq_of;                                    // the sequence of grid slice z (-1: none), or null: slice z is sequence z
     const int* nkeys;                                     // per query row: visible keys (0..nkeys-1)
     const int* pre_keys;                                  // per sequence (or null): keys 0..pre-1 were written before this
                                                           // step began, so they may be fetched before the dependency wait
@@ -28,6 +29,6 @@ struct AttnF32Args {
     float scale;
 };
 bool af_supported(int d_head, int max_keys);
-cudaError_t af_launch(bool paged, const AttnF32Args& a, int q_ub, int n_heads, int B, bool pdl, cudaStream_t st);
+cudaError_t af_launch(bool paged, const AttnF32Args& a, int q_ub, int n_heads, int slots, bool pdl, cudaStream_t st);
 
 }  // namespace sd

@@ -423,9 +423,12 @@ cudaError_t launch_pdl_heads(specdec_handle* h, void (*kernel)(KArgs...), dim3 g
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Verify blocks are packed, unfinished sequences only, in the generation loop (the step calls have one for every sequence).
+inline bool packed_blocks(const specdec_handle* h) { return h->fuse_commit && h->B > 1; }
+
 // Row count of a pass where the host knows it, else -1 (the kernels read it from the device).
 inline int static_rows(const specdec_handle* h, int cnt, int rows_ub) {
-    return (cnt == CNT_VERIFY && !(h->fuse_commit && h->B > 1)) ? rows_ub : -1;
+    return (cnt == CNT_VERIFY && !packed_blocks(h)) ? rows_ub : -1;
 }
 
 template <typename T>
@@ -577,6 +580,18 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
     return 0;
 }
 
+// Grid slices of the attention launches of a pass: one for every sequence that may have rows in it, by the pass's slot table (seq_of null: slice =
+// sequence).  An empty CTA takes its shared memory and its turn on an SM (a handful of sequences left of 128, launched as 128: 12.6 us for the
+// cross-attention with both projections, 29 for a draft's self-attention in clusters, where 6 and 6 do; 128 sequences decoded 10.22 -> 9.84 ms).
+// While the empty ones fit beside the others (16-query tiles, one to an SM) the table is left out: it is one more round trip ahead of a CTA's first loads
+// (tiny fp32 pair, 2 sequences: 730 / 738 us).
+struct AttnSlots { int n; const int* seq_of; };
+inline AttnSlots attn_slots(const specdec_handle* h, int cnt, int q_ub, int n_heads) {
+    const int n = cnt == CNT_ENC || (cnt == CNT_VERIFY && !packed_blocks(h)) ? h->B : std::min(h->B, h->act_ub);
+    if (n == h->B || (long long)cdiv(q_ub, 16) * n_heads * h->B <= h->tma.n_sm) return {h->B, nullptr};
+    return {n, cnt == CNT_VERIFY ? h->rows.slot_seq : h->mrows.slot_seq};
+}
+
 // Attention of the pass described by `r`.  bf16 handles with 64-wide heads use the tensor-core tile
 // kernel (one CTA per 32-query tile, head, sequence; q_ub bounds the queries of one sequence);
 // everything else uses the warp-per-(row, head) kernel.
@@ -594,6 +609,8 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             a.q_off = r.q_off; a.q_cnt = r.q_cnt; a.nkeys = nkeys; a.pre_keys = h->use_pdl ? pre_keys : nullptr;
             a.out = (bf16*)out; a.out_stride = out_stride; a.max_keys = max_keys;
             a.scale = 1.0f / sqrtf((float)d_head);
+            const AttnSlots slots = attn_slots(h, cnt, q_ub, n_heads);
+            a.seq_of = slots.seq_of;
             const int n_seq = cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub);
             QueryArgs qa{};
             OutArgs oa{};
@@ -601,7 +618,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             if (op) {                                        // the heads of a tile as one cluster (4 or 8)
                 oa = *op;
                 auto goo = [&](auto* kernel, int bytes) {
-                    const cudaError_t e = launch_pdl_heads(h, kernel, dim3(cdiv(q_ub, 16), n_heads, h->B), dim3(256), AttnCfg<1, 8, 16>::smem(max_keys, 3, paged, bytes), st, a, qa, oa);
+                    const cudaError_t e = launch_pdl_heads(h, kernel, dim3(cdiv(q_ub, 16), n_heads, slots.n), dim3(256), AttnCfg<1, 8, 16>::smem(max_keys, 3, paged, bytes), st, a, qa, oa);
                     if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
                     KCHECK(h);
                     return 0;
@@ -611,7 +628,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             }
             if (qp) {
                 auto goq = [&](auto* kernel, size_t bytes) {
-                    const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, 16), n_heads, h->B), dim3(256), bytes, st, a, qa, oa);
+                    const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, 16), n_heads, slots.n), dim3(256), bytes, st, a, qa, oa);
                     if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
                     KCHECK(h);
                     return 0;
@@ -627,7 +644,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
                 }
             }
             auto go = [&](auto* kernel, int bm, int warps, size_t smem) {
-                const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, bm), n_heads, h->B), dim3(warps * 32), smem, st, a, qa, oa);
+                const cudaError_t e = launch_pdl(h, kernel, dim3(cdiv(q_ub, bm), n_heads, slots.n), dim3(warps * 32), smem, st, a, qa, oa);
                 if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
                 KCHECK(h);
                 return 0;
@@ -662,7 +679,9 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             a.q_off = r.q_off; a.q_cnt = r.q_cnt; a.nkeys = nkeys; a.pre_keys = h->use_pdl ? pre_keys : nullptr;
             a.out = (float*)out; a.out_stride = out_stride; a.max_keys = max_keys; a.d_head = d_head;
             a.scale = 1.0f / sqrtf((float)d_head);
-            const cudaError_t e = af_launch(paged, a, q_ub, n_heads, h->B, h->use_pdl, st);
+            const AttnSlots slots = attn_slots(h, cnt, q_ub, n_heads);
+            a.seq_of = slots.seq_of;
+            const cudaError_t e = af_launch(paged, a, q_ub, n_heads, slots.n, h->use_pdl, st);
             if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
             KCHECK(h);
             return 0;
@@ -964,7 +983,7 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
                 cudaStream_t st) {
     ModelW& m = h->ver;
     // the generation loop verifies the unfinished sequences only: packed blocks, M an upper bound on their rows
-    const bool compact = h->fuse_commit && h->B > 1;
+    const bool compact = packed_blocks(h);
     const int B = h->B, slots = compact ? std::min(B, h->act_ub) : B, d = m.dm.d_model, L = m.dm.dec_layers, M = slots * (k + 1);
     const int max_keys = std::min(h->len_ub, h->T_cap) + k + 1;
     // (the caller's drafts and result arrays are read and written by the kernels themselves: a copy node costs 2 us of the step)

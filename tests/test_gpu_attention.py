@@ -89,3 +89,37 @@ def test_output_projected_inside_the_attention(d, B, k, S, cached):
     assert rep.ok, rep.notes
     assert rep.max_logit_err < 2e-2 and rep.max_stat_err < 2e-2
     sd.close()
+
+
+@pytest.mark.parametrize("bf16,d,H,cached", [(True, 256, 4, False), (True, 256, 4, True), (False, 64, 16, False), (False, 64, 16, True)])
+def test_slices_of_unfinished_sequences(bf16, d, H, cached):
+    """A ragged batch whose sequences end one after another: the attention launches shrink to the unfinished ones (32, 16, ... of 33).
+    Every draft is accepted, so what comes out is what the drafter's passes computed, and each (k + 1)-th token what the verifier's did."""
+    from paper_2203_16487_b200 import binding
+    V, B, k, beta, tau = 515, 33, 17, 515, 1e9
+    dims = W.ModelDims(d, H, 2 * d, V, 1, 2, 128)
+    wv, wd = W.make_weights(dims, 91, bf16), W.make_weights(dims, 92, bf16)
+    for w in (wv, wd):                                   # sublayers that outweigh the embedding: the argmax depends on every key
+        for name in w:
+            if name.endswith((".o.w", ".v.w", ".ffn.w2")):
+                w[name] = w[name] * 8
+        w["pos_dec"] = 4 * np.random.default_rng(5).standard_normal(w["pos_dec"].shape).astype(np.float32)
+    mv, md = (O.model_from(dims, w, mode="bf16" if bf16 else "pure") for w in (wv, wd))
+    rng = np.random.default_rng(4)
+    srcs = [W.zipf_ids(rng, int(n), V) for n in rng.integers(2, 20, size=B)]
+    tgt = [3 + 9 * (b % 9) for b in range(B)]
+    sd = binding.SpecDec(dims, wv, dims, wd, k_max=k, max_batch=B, max_src=20, max_tgt=max(tgt), bf16=bf16)
+    sd.set_option("debug_checks", 1)
+    sd.set_option("drafter_prefix_causal", int(cached))
+    out, n, _ = sd.generate(*W.pad_batch(srcs), np.array(tgt, np.int32), k, beta, tau)
+    out, n = out.cpu().numpy(), n.cpu().numpy()
+    wrong, seen = 0, set()
+    for b in range(B):
+        ref, _ = O.specdec_generate(mv, md, srcs[b], tgt[b], k, beta, tau, W.BOS_ID, W.EOS_ID, W.MASK_ID,
+                                    drafter_reading="prefix_causal" if cached else "bidirectional")
+        wrong += out[b, :n[b]].tolist() != ref
+        seen.update(ref)
+    assert len(seen) > 50                                # (the drafts do vary)
+    # fp32: exact.  bf16: about 1300 arguments of a maximum over 515 logits of spread ~1 that agree to 2e-3: a few near-ties are expected
+    assert wrong <= (4 if bf16 else 0), wrong
+    sd.close()
