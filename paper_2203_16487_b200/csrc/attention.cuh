@@ -85,6 +85,7 @@ template <int QNC> struct QueryCfg {                      // K = 128 QNC
 struct OutArgs {
     const bf16* w; const float* b;                        // [K, K], K = 64 n_heads
     const float* x_in; const int* x_index; float* x_out;  // fp32 rows [rows, K]
+    int* err_word;                                        // raised when the bounded wait for the other heads gives up
 };
 // Bytes behind the ring: 16 rows and 64 rows of weights for each projection that runs inside.
 template <int QNC, int ON> struct ProjCfg { static constexpr int OPS = QueryCfg<QNC>::OPS + QueryCfg<ON / 2>::OPS; };
@@ -159,8 +160,10 @@ constexpr int attn_ctas(int mt, int kg, int kw) { return kg > 1 ? 0 : mt == 4 ? 
 // ON > 0: the heads of a query tile are a cluster of ON CTAs, and the output projection runs here too (OutArgs).  Bound by the same chain of round trips:
 // every CTA sends its head's 16 rows (bf16, as they would go to memory) to the shared memory of all, multiplies the 16 whole rows by its own 64 rows
 // of Wo and adds the residual.  Wo is requested ahead of the wait and turned into register fragments while the queries are on their way, so
-// that only the exchange (0.5 us), 32 MMAs a warp and the sum of four K slices follow the attention: a launch and its round trip less
-// (verify step of 26 rows, both attentions of six layers: 156.5 -> 147.2 us; with Wo fetched behind the wait 155.2).
+// that only the exchange, 32 MMAs a warp and the sum of four K slices follow the attention: a launch and its round trip less
+// (verify step of 26 rows, both attentions of six layers: 156.5 -> 147.2 us; with Wo fetched behind the wait 155.2).  The exchange is counted on
+// the receiver's mbarrier: plain remote stores behind a cluster barrier, whose release and acquire every thread pays, took 0.2 us more a launch
+// (the same step 147.3 -> 145.1).
 template <bool PAGED, int MT, int KG, int KW, int NS, int QNC = 0, int ON = 0>
 __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {
     using C = AttnCfg<MT, KG, KW>;
@@ -171,6 +174,8 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ int s_nk[BM];
     __shared__ int s_nkmax;
+    __shared__ __align__(8) uint64_t heads_bar;               // ON: counts the heads' rows as they arrive
+    __shared__ int abort_s;
     const int b = a.seq_of ? a.seq_of[blockIdx.z] : (int)blockIdx.z, h = blockIdx.y, qt = blockIdx.x;
     if (b < 0) return;
     // Row metadata, page table and sequence lengths are written at the start of the step, before the first
@@ -209,6 +214,13 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
             const int r = i / (OC::K / 8), c = i % (OC::K / 8);
             cp_async16(oops + (16 + r) * OC::PITCH + c * 16, w + (size_t)r * OC::K + c * 8);
         }
+        if (tid == 0) {
+            abort_s = 0;
+            mbar_init(smem_u32(&heads_bar), 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            mbar_expect_tx(smem_u32(&heads_bar), 16 * OC::K * 2);           // all heads' columns of the 16 rows, this CTA's own among them
+        }
+        __syncwarp();
         cluster_arrive();
         ob = ldg_pinned(reinterpret_cast<const float4*>(oa.b + h * 64 + (tid & 15) * 4));
     }
@@ -498,15 +510,11 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
             const uint32_t dst = oops + rr * OC::PITCH + (h * 64 + kg * CW) * 2;
             cluster_wait();                          // every CTA of the cluster has begun and its barrier exists
 #pragma unroll
-            for (int i = 0; i < ON / 2; ++i) {
-                uint32_t ra;
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(dst), "r"((odd ? ON / 2 : 0) + i));
-                asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
-                             ::"r"(ra), "r"(odd ? w0 : u0), "r"(odd ? w1 : u1), "r"(odd ? u0 : w0), "r"(odd ? u1 : w1) : "memory");
-            }
-            cluster_arrive();
-            cluster_wait();
-            wo.multiply(oops, mO, warp, lane);             // (the partial outputs of the key groups are dead)
+            for (int i = 0; i < ON / 2; ++i)
+                st_peer16(dst, smem_u32(&heads_bar), (odd ? ON / 2 : 0) + i, make_uint4(odd ? w0 : u0, odd ? w1 : u1, odd ? u0 : w0, odd ? u1 : w1));
+            mbar_wait(smem_u32(&heads_bar), 0, &abort_s, oa.err_word, 12);
+            __syncthreads();                         // (the partial outputs of the key groups are dead)
+            wo.multiply(oops, mO, warp, lane);
             __syncthreads();
             const float4 t = Proj64<OC::K>::sum(mO, tid);
             if ((tid >> 4) < nq)

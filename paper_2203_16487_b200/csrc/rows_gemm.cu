@@ -21,15 +21,6 @@ struct RgCfg {
     }
 };
 
-// 16 consecutive bytes to the shared memory of CTA `rank` of this cluster, counted on its mbarrier.
-__device__ __forceinline__ void rg_st_peer16(uint32_t local_addr, uint32_t local_bar, uint32_t rank, float4 v) {
-    uint32_t ra, rb;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local_addr), "r"(rank));
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(local_bar), "r"(rank));
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-                 ::"r"(ra), "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)), "r"(__float_as_uint(v.w)), "r"(rb) : "memory");
-}
-
 // One CTA = 16 MT rows x 8 NT columns, K walked by the warps side by side (WN warps across the columns, 8 / WN K slices).
 //
 // Bound: latency.  A decoding step is a chain of 34 launches, 18 of them these, each over 0.5-2 MB of weights, so what counts is the
@@ -254,7 +245,7 @@ __global__ void __launch_bounds__(RG_THREADS, NC > 4 ? 2 : 3) k_rows(RowsArgs a)
             const uint32_t own = cn / OW;
             float* slot = inbox + ((int)rank * BM + r) * OW + cn % OW;
             if (own == rank) *reinterpret_cast<float4*>(slot) = v;
-            else rg_st_peer16(smem_u32(slot), smem_u32(&part_bar), own, v);
+            else st_peer16(smem_u32(slot), smem_u32(&part_bar), own, make_uint4(__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w)));
         }
     }
     if (CS > 1) {

@@ -783,7 +783,7 @@ int block_self(specdec_handle* h, const ModelW& m, const LayerW& w, float* x, co
         }
     }
     const bool inside = std::is_same<T, bf16>::value && out_inside(h, dh, q_ub, H, cnt, rows_ub, max_keys, OUT_SELF);
-    const OutArgs oa{(const bf16*)w.o_w, w.o_b, x, nullptr, x};
+    const OutArgs oa{(const bf16*)w.o_w, w.o_b, x, nullptr, x, h->ses.counters + 7};
     if (verify) {
         TRY(attn<T>(h, true, h->qkv, 3 * d, nullptr, kc, vc, d, nullptr, r, r.nk_self, cnt,
                     rows_ub, q_ub, h->att, d, H, dh, max_keys, st, pre_keys, nullptr, inside ? &oa : nullptr));
@@ -813,7 +813,7 @@ int block_cross(specdec_handle* h, const ModelW& m, const LayerW& w, float* x, c
     QueryArgs qa{};
     const bool inside = std::is_same<T, bf16>::value && query_inside(h, d, dh, q_ub, H, h->S_max);
     const bool out = inside && out_inside(h, dh, q_ub, H, cnt, rows_ub, h->S_max, OUT_QUERIES);
-    const OutArgs oa{(const bf16*)w.co_w, w.co_b, x, nullptr, x};
+    const OutArgs oa{(const bf16*)w.co_w, w.co_b, x, nullptr, x, h->ses.counters + 7};
     if (inside) qa = QueryArgs{x, w.lnc_g, w.lnc_b, 1e-5f, (const bf16*)w.cq_w, w.cq_b};
     else TRY(gemm<T>(h, EPI_STORE, h->y, d, w.cq_w, w.cq_b, d, d, cnt, rows_ub, h->q, d, nullptr, st, nullptr, nullptr, nullptr,
                      nullptr, &lc));
@@ -948,7 +948,7 @@ int draft_impl(specdec_handle* h, int k, int* d_draft, cudaStream_t st) {
         }
     }
     const bool inside = std::is_same<T, bf16>::value && out_inside(h, dh, k, H, CNT_DRAFT_MASK, R2, max_keys, OUT_GATHERS);
-    const OutArgs oa{(const bf16*)w.o_w, w.o_b, h->x, h->mrows.src_row, h->x2};       // (takes the [MASK] rows of the residual stream itself)
+    const OutArgs oa{(const bf16*)w.o_w, w.o_b, h->x, h->mrows.src_row, h->x2, h->ses.counters + 7};       // (takes the [MASK] rows of the residual stream itself)
     if (!inside) {
         CUDA_TRY(h, launch_pdl(h, k_gather_rows, dim3(R2), dim3(128), 0, st, (const float*)h->x, (const int*)h->mrows.src_row, (const int*)(h->ses.counters + CNT_DRAFT_MASK), h->x2, d));
         KCHECK(h);
