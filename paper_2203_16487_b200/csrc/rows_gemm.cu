@@ -15,8 +15,9 @@ struct RgCfg {
     static constexpr int BM = 16 * MT, NB = 8 * NT, WK = RG_WARPS / WN, RP = NB + 8;     // RP: pitch of a partial row (floats)
     static constexpr size_t red_bytes = (size_t)WK * BM * RP * 4;
     static int kpad(int Kc) { return (Kc + 16 * WK - 1) / (16 * WK) * (16 * WK); }               // whole MMA steps for every K slice
-    static size_t smem(int Kc) {
-        const size_t ops = (size_t)(BM + NB) * (kpad(Kc) * 2 + 16);
+    static size_t smem(int Kc, bool fragments = false) {
+        size_t ops = (size_t)(BM + NB) * (kpad(Kc) * 2 + 16);
+        if (fragments && (size_t)BM * (kpad(Kc) * 2 + 16) + red_bytes > ops) ops = (size_t)BM * (kpad(Kc) * 2 + 16) + red_bytes;
         return (ops > red_bytes ? ops : red_bytes) + (CS > 1 ? (size_t)BM * NB * 4 : 0);
     }
 };
@@ -32,22 +33,27 @@ struct RgCfg {
 //     longer step (240 against 218 us), because its successors could not start early;
 //   * after the wait one round trip brings the rows; with NC > 0 they are normalised on the way (K = 128 NC, two rows per
 //     warp: 1.3 us against 2.3 us when a cluster of 8 shared the normalised rows through distributed shared memory);
+//   * where the reduction's length is one of the usual ones (ST > 0: ST MMA steps a warp) the weights have also become register fragments by then,
+//     so that behind the rows there are only ST loads of A and the MMAs: shared memory handed over 96 KB a CTA before (0.39 of the 0.75 us between the
+//     rows' arrival and the partial sums), 16 KB now, and the partial sums go where the weights were, without a barrier in between;
 //   * K is split over the warps (and, for long reductions, over a cluster of CS CTAs whose partial tiles meet in the owner's
 //     shared memory), the slices are added in a fixed order: results do not depend on timing.
-// Measured inside a verify step at 26 rows: 2.4 us per 512 x 512 launch, 3.3 us for QKV and FFN1 with their LayerNorm (5.2-6.0
-// with the kernel this one replaced), 3.9 us for FFN2.
-template <int EPI, int NC, int MT, int NT, int WN, int CS>
-__global__ void __launch_bounds__(RG_THREADS, NC > 4 ? 2 : 3) k_rows(RowsArgs a) {
+// Measured inside a verify step at 26 rows: 2.8 us for QKV and FFN1 with their LayerNorm (3.5 with the weights read from shared memory behind the
+// rows), 2.6 us for FFN2 (3.5); the step 145.1 -> 131, a greedy pass over 16 sequences 6262 -> 5680 us.  The fragments cost registers (up to 165 a
+// thread): beyond three row tiles with a LayerNorm inside too few of the successors' CTAs are resident (52 rows: 154 / 161 us a step), those keep the variant without.
+template <int EPI, int NC, int MT, int NT, int WN, int CS, int ST>
+__global__ void __launch_bounds__(RG_THREADS, NC > 0 && ST >= 8 ? 1 : NC > 4 || ST > 0 ? 2 : 3) k_rows(RowsArgs a) {
     using C = RgCfg<MT, NT, WN, CS>;
     constexpr int BM = C::BM, NB = C::NB, WK = C::WK, RP = C::RP, TN = NT / WN;      // TN = 8-column tiles per warp
     static_assert(TN % 2 == 0 || TN == 1, "B fragments come in pairs");
+    static_assert(ST == 0 || (MT == 1 && TN > 1), "weights as fragments: 16 rows, column tiles in pairs");
     constexpr bool LN = NC > 0;
     extern __shared__ __align__(16) unsigned char rg_sm[];
     __shared__ int s_kv[BM];
     __shared__ __align__(8) uint64_t part_bar;
     __shared__ int abort_s;
     const GemmArgs<bf16>& g = a.g;
-    const int K = LN ? NC * 128 : g.K, N = g.N, Kc = CS > 1 ? K / CS : K;
+    const int K = LN ? NC * 128 : g.K, N = g.N, Kc = ST > 0 ? ST * 16 * WK : CS > 1 ? K / CS : K;
     const int Kp = (Kc + 16 * WK - 1) / (16 * WK) * (16 * WK), pitch = Kp * 2 + 16;                // Kp: padded with zeros; pitch in bytes
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint32_t rank = 0;
@@ -56,8 +62,8 @@ __global__ void __launch_bounds__(RG_THREADS, NC > 4 ? 2 : 3) k_rows(RowsArgs a)
     const int R = min((g.rows_static >= 0 ? g.rows_static : *g.n_rows) - m0, BM);
     if (R <= 0 && blockIdx.y > 0) return;
     const uint32_t As = smem_u32(rg_sm), Ws = As + BM * pitch;
-    float* red = reinterpret_cast<float*>(rg_sm);
-    const size_t ops = (size_t)(BM + NB) * pitch;
+    float* red = reinterpret_cast<float*>(rg_sm + (ST > 0 ? BM * pitch : 0));        // (in place of the operands; with fragments, of the weights)
+    const size_t ops = ST > 0 ? BM * pitch + ((size_t)NB * pitch > C::red_bytes ? (size_t)NB * pitch : C::red_bytes) : (size_t)(BM + NB) * pitch;
     float* inbox = reinterpret_cast<float*>(rg_sm + (ops > C::red_bytes ? ops : C::red_bytes));     // CS > 1: [rank][BM][NB / CS]
     rg_stamp(a.trace, 0);
     // ---- before the dependency wait: weights, bias, LayerNorm parameters, cache rows
@@ -97,6 +103,19 @@ __global__ void __launch_bounds__(RG_THREADS, NC > 4 ? 2 : 3) k_rows(RowsArgs a)
     }
     rg_stamp(a.trace, 1);
     pdl_launch_dependents();
+    const int wk = warp / WN, wn = warp % WN, steps = Kp / (16 * WK);
+    // A: rows lane % 16, k half lane / 16.  B: with two column tiles, rows (lane & 7) + 8 (lane >> 4), k half (lane >> 3) & 1
+    uint32_t ap = As + (lane & 15) * pitch + wk * steps * 32 + (lane >> 4) * 16;
+    uint32_t bp = Ws + (wn * TN * 8 + (lane & 7) + (TN > 1 ? (lane >> 4) * 8 : 0)) * pitch + wk * steps * 32 + ((lane >> 3) & 1) * 16;
+    uint32_t wf[ST > 0 ? ST : 1][TN][2];
+    if constexpr (ST > 0) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+#pragma unroll
+        for (int s = 0; s < ST; ++s)
+#pragma unroll
+            for (int j = 0; j < TN; j += 2) ldsm_x4(bp + s * 32 + j * 8 * pitch, wf[s][j][0], wf[s][j][1], wf[s][j + 1][0], wf[s][j + 1][1]);
+    }
     pdl_wait();
     rg_stamp(a.trace, 2);
     // ---- activation rows
@@ -172,7 +191,6 @@ __global__ void __launch_bounds__(RG_THREADS, NC > 4 ? 2 : 3) k_rows(RowsArgs a)
     __syncthreads();
     rg_stamp(a.trace, 3);
     // ---- products: warp (wk, wn) takes K slice wk and TN column tiles of every row tile
-    const int wk = warp / WN, wn = warp % WN, steps = Kp / (16 * WK);
     float acc[MT][TN][4];
 #pragma unroll
     for (int i = 0; i < MT; ++i)
@@ -180,10 +198,15 @@ __global__ void __launch_bounds__(RG_THREADS, NC > 4 ? 2 : 3) k_rows(RowsArgs a)
         for (int j = 0; j < TN; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
-    {
-        // A: rows lane % 16, k half lane / 16.  B: with two column tiles, rows (lane & 7) + 8 (lane >> 4), k half (lane >> 3) & 1
-        uint32_t ap = As + (lane & 15) * pitch + wk * steps * 32 + (lane >> 4) * 16;
-        uint32_t bp = Ws + (wn * TN * 8 + (lane & 7) + (TN > 1 ? (lane >> 4) * 8 : 0)) * pitch + wk * steps * 32 + ((lane >> 3) & 1) * 16;
+    if constexpr (ST > 0) {
+#pragma unroll
+        for (int s = 0; s < ST; ++s) {
+            uint32_t af[4];
+            ldsm_x4(ap + s * 32, af[0], af[1], af[2], af[3]);
+#pragma unroll
+            for (int j = 0; j < TN; ++j) mma_bf16(acc[0][j], af, wf[s][j][0], wf[s][j][1]);
+        }
+    } else {
 #pragma unroll 8
         for (int s = 0; s < steps; ++s, ap += 32, bp += 32) {
             uint32_t af[MT][4], bf[TN][2];
@@ -199,8 +222,8 @@ __global__ void __launch_bounds__(RG_THREADS, NC > 4 ? 2 : 3) k_rows(RowsArgs a)
 #pragma unroll
                 for (int j = 0; j < TN; ++j) mma_bf16(acc[i][j], af[i], bf[j][0], bf[j][1]);
         }
+        __syncthreads();                                      // the operands are dead: partial sums take their place
     }
-    __syncthreads();                                          // the operands are dead: partial sums take their place
     {
         const int gq = lane >> 2, t4 = lane & 3;
 #pragma unroll
@@ -265,18 +288,18 @@ __global__ void __launch_bounds__(RG_THREADS, NC > 4 ? 2 : 3) k_rows(RowsArgs a)
     rg_stamp(a.trace, 5);
 }
 
-template <int EPI, int NC, int MT, int NT, int WN, int CS>
+template <int EPI, int NC, int MT, int NT, int WN, int CS, int ST = 0>
 inline cudaError_t rg_launch_one(const RowsArgs& a, int rows_ub, bool pdl, cudaStream_t st) {
     using C = RgCfg<MT, NT, WN, CS>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((a.g.N + C::NB - 1) / C::NB * CS, (rows_ub + C::BM - 1) / C::BM); cfg.blockDim = dim3(RG_THREADS);
-    cfg.dynamicSmemBytes = C::smem(a.g.K / CS); cfg.stream = st;       // (allowed by rg_init)
+    cfg.dynamicSmemBytes = C::smem(a.g.K / CS, ST > 0); cfg.stream = st;       // (allowed by rg_init)
     cudaLaunchAttribute attr[2];
     int n = 0;
     if (CS > 1) { attr[n].id = cudaLaunchAttributeClusterDimension; attr[n].val.clusterDim.x = CS; attr[n].val.clusterDim.y = 1; attr[n].val.clusterDim.z = 1; ++n; }
     if (pdl) { attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[n].val.programmaticStreamSerializationAllowed = 1; ++n; }
     cfg.attrs = attr; cfg.numAttrs = n;
-    return cudaLaunchKernelEx(&cfg, k_rows<EPI, NC, MT, NT, WN, CS>, a);
+    return cudaLaunchKernelEx(&cfg, k_rows<EPI, NC, MT, NT, WN, CS, ST>, a);
 }
 
 constexpr int RG_MAX_SMEM = 227 * 1024 - 1024;
@@ -286,7 +309,7 @@ constexpr int RG_MAX_SMEM = 227 * 1024 - 1024;
 static int rg_split(int N, int K, int rows_ub, bool cluster) {
     if (K < 1024 || !cluster) return 1;
     if (rows_ub > rg_ln_rows(min(N, K)) && K % 32 == 0) return 4;
-    return K % 16 == 0 ? 2 : 1;
+    return K % 16 == 0 ? 2 : 1;       // (the reductions whose weights become fragments take four: rg_launch_resid)
 }
 bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster) {
     if (rows_ub > RG_MAX_ROWS || K % 16 || N % 16 || lda % 8) return false;
@@ -300,6 +323,14 @@ bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster) {
 template <int EPI, int NC>
 inline cudaError_t rg_launch_out(const RowsArgs& a, int rows_ub, bool pdl, cudaStream_t st) {
     const bool wide = a.g.N >= 1024;
+    // Weights as fragments.  One row tile: 32 columns a CTA (greedy pass over 16 sequences 6090 -> 5700 us; with two row tiles these are too many CTAs: one
+    // sentence 902 -> 973); up to three: 64 columns (verify step, us, without / with: 26 rows 136.4 / 129.6, 44 rows 139.8 / 136.7, 52 rows 154 / 161).
+    // 768 columns take 96 registers of fragments next to the 96 of the rows: 11 rows 190.6 / 183.6, 26 rows 195 / 201.5, 41 rows 205 / 212.
+    if constexpr (NC == 2 || NC == 4) {
+        if (wide && rows_ub <= 16) return rg_launch_one<EPI, NC, 1, 4, 1, 1, NC>(a, rows_ub, pdl, st);
+        if (wide && rows_ub <= 48) return rg_launch_one<EPI, NC, 1, 8, 2, 1, 2 * NC>(a, rows_ub, pdl, st);
+    }
+    if constexpr (NC == 6) { if (wide && rows_ub <= 16) return rg_launch_one<EPI, NC, 1, 8, 2, 1, 2 * NC>(a, rows_ub, pdl, st); }
     if constexpr (NC == 0) { if (rows_ub > rg_ln_rows(min(a.g.N, a.g.K))) return rg_launch_one<EPI, 0, 2, 8, 2, 1>(a, rows_ub, pdl, st); }
     if (wide) return rg_launch_one<EPI, NC, 1, 8, 2, 1>(a, rows_ub, pdl, st);
     if constexpr (EPI == EPI_STORE) { if (rows_ub > 32) return rg_launch_one<EPI, NC, 1, 4, 1, 1>(a, rows_ub, pdl, st); }
@@ -311,9 +342,24 @@ static cudaError_t rg_launch_resid(const RowsArgs& a, int rows_ub, bool cluster,
         if (split == 4) return rg_launch_one<EPI_RESID, 0, 2, 8, 2, 4>(a, rows_ub, pdl, st);
         return rg_launch_one<EPI_RESID, 0, 2, 8, 2, 1>(a, rows_ub, pdl, st);
     }
-    if (split == 2) return rg_launch_one<EPI_RESID, 0, 1, 4, 1, 2>(a, rows_ub, pdl, st);
-    if (rows_ub > 32) return rg_launch_one<EPI_RESID, 0, 1, 4, 1, 1>(a, rows_ub, pdl, st);
-    return rg_launch_one<EPI_RESID, 0, 1, 2, 1, 1>(a, rows_ub, pdl, st);
+    // Weights as fragments where K is one of these (verify step, us, without / with: K = 2048 26 rows 143 / 137.5 with two slices of 32 columns, 136.7 with
+    // four of 64; 104 rows 188 / 184, 183; K = 3072 26 rows 194.9 / 190 with two slices, 195 with four; 63 rows 247 / 243.6; K = 512 52 rows 154 / 152).
+    if (split == 2) {
+        switch (a.g.K) {
+            case 1024: return rg_launch_one<EPI_RESID, 0, 1, 4, 1, 2, 4>(a, rows_ub, pdl, st);
+            case 2048: return rg_launch_one<EPI_RESID, 0, 1, 8, 2, 4, 8>(a, rows_ub, pdl, st);
+            case 3072: return rg_launch_one<EPI_RESID, 0, 1, 4, 1, 2, 12>(a, rows_ub, pdl, st);
+            default: return rg_launch_one<EPI_RESID, 0, 1, 4, 1, 2>(a, rows_ub, pdl, st);
+        }
+    }
+    switch (split == 1 ? a.g.K : 0) {
+#define RG_RESID(ST) return rows_ub > 32 ? rg_launch_one<EPI_RESID, 0, 1, 4, 1, 1, ST>(a, rows_ub, pdl, st) : rg_launch_one<EPI_RESID, 0, 1, 2, 1, 1, ST>(a, rows_ub, pdl, st)
+        case 256: RG_RESID(2);
+        case 512: RG_RESID(4);
+        case 768: RG_RESID(6);
+        default: RG_RESID(0);
+#undef RG_RESID
+    }
 }
 template <int EPI>
 inline cudaError_t rg_launch_nc(const RowsArgs& a, int rows_ub, bool pdl, cudaStream_t st) {
@@ -337,13 +383,15 @@ cudaError_t rg_launch(int epi, const RowsArgs& a, int rows_ub, bool cluster, boo
 
 // Shared-memory limits of everything launched above.  The limit belongs to the kernel in the whole process: one that followed the launch would
 // be another handle's by the time of the launch, if that handle decodes on another host thread.
-template <int EPI, int NC, int MT, int NT, int WN, int CS>
+template <int EPI, int NC, int MT, int NT, int WN, int CS, int ST = 0>
 static void rg_room(cudaError_t& e) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rows<EPI, NC, MT, NT, WN, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, RG_MAX_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rows<EPI, NC, MT, NT, WN, CS, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, RG_MAX_SMEM);
 }
 template <int EPI, int NC>
 static void rg_room_out(cudaError_t& e) {
     if constexpr (NC == 0) rg_room<EPI, 0, 2, 8, 2, 1>(e);
+    if constexpr (NC == 2 || NC == 4) rg_room<EPI, NC, 1, 4, 1, 1, NC>(e);
+    if constexpr (NC > 0) rg_room<EPI, NC, 1, 8, 2, 1, 2 * NC>(e);
     rg_room<EPI, NC, 1, 8, 2, 1>(e);
     if constexpr (EPI == EPI_STORE) rg_room<EPI, NC, 1, 4, 1, 1>(e);
     rg_room<EPI, NC, 1, 2, 1, 1>(e);
@@ -353,8 +401,10 @@ static void rg_room_nc(cudaError_t& e) { rg_room_out<EPI, 0>(e); rg_room_out<EPI
 cudaError_t rg_init() {
     cudaError_t e = cudaSuccess;
     rg_room_nc<EPI_STORE>(e); rg_room_nc<EPI_RELU>(e); rg_room_nc<EPI_GELU>(e); rg_room_nc<EPI_QKV>(e);
-    rg_room<EPI_RESID, 0, 2, 8, 2, 4>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1>(e);
-    rg_room<EPI_RESID, 0, 1, 4, 1, 2>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1>(e); rg_room<EPI_RESID, 0, 1, 2, 1, 1>(e);
+    rg_room<EPI_RESID, 0, 2, 8, 2, 4>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 2>(e);
+    rg_room<EPI_RESID, 0, 1, 4, 1, 2, 4>(e); rg_room<EPI_RESID, 0, 1, 8, 2, 4, 8>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 2, 12>(e);
+    rg_room<EPI_RESID, 0, 1, 4, 1, 1>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1, 2>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1, 4>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1, 6>(e);
+    rg_room<EPI_RESID, 0, 1, 2, 1, 1>(e); rg_room<EPI_RESID, 0, 1, 2, 1, 1, 2>(e); rg_room<EPI_RESID, 0, 1, 2, 1, 1, 4>(e); rg_room<EPI_RESID, 0, 1, 2, 1, 1, 6>(e);
     return e;
 }
 

@@ -14,7 +14,15 @@ pytestmark = pytest.mark.gpu
 # (d, heads, ffn, batch, k): batch * (k + 1) rows in a verify block
 @pytest.mark.parametrize("d,H,f,B,k", [
     (256, 4, 1040, 1, 15),          # 16 rows; K = 1040: two slices that end inside an MMA step
+    (512, 8, 2048, 1, 15),          # 16 rows: the last with weight fragments of 32 columns
+    (512, 8, 2048, 1, 16),          # 17 rows: a tile and one row, fragments of 64 columns; K = 2048 in four slices
     (512, 8, 2048, 3, 10),          # 33 rows
+    (512, 8, 2048, 3, 15),          # 48 rows: the last with fragments where a LayerNorm runs inside
+    (512, 8, 2048, 7, 6),           # 49 rows
+    (256, 4, 1024, 1, 4),           # 5 rows; K = 1024: two slices, as fragments
+    (256, 4, 1024, 8, 3),           # 32 rows: the last with 16-column output projections
+    (768, 12, 3072, 1, 15),         # 16 rows at this width: fragments of the widest LayerNorm
+    (768, 12, 3072, 1, 16),         # 17 rows: without
     (768, 12, 3072, 8, 9),          # 80 rows: the last with the LayerNorm inside
     (768, 12, 3072, 16, 5),         # 96 rows: the last of the few-rows kernel at this width
     (768, 12, 3072, 16, 7),         # 128 rows: tensor-core tiles, four K slices for the output projections
