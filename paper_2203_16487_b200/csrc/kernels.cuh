@@ -54,6 +54,13 @@ __device__ __forceinline__ float ldg_pinned(const float* p) {
     return v;
 }
 
+// (a plain load that is issued where it is written)
+__device__ __forceinline__ int ld_pinned(const int* p) {
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -1019,6 +1026,14 @@ static __global__ void k_draft_argmax(const RowPart* part, int n_tiles, const in
         for (int i = 0; i < 8; ++i) q[i] = p[t + 32 * i];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
+            if (q[i].mx > mx || (q[i].mx == mx && q[i].arg < arg)) { mx = q[i].mx; arg = q[i].arg; }
+    }
+    for (; t + 96 < n_tiles; t += 128) {
+        RowPart q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = p[t + 32 * i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
             if (q[i].mx > mx || (q[i].mx == mx && q[i].arg < arg)) { mx = q[i].mx; arg = q[i].arg; }
     }
     for (; t < n_tiles; t += 32) {

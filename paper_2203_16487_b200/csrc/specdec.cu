@@ -27,6 +27,7 @@
 #include "mma_rate.cuh"
 #include "rows_f32.cuh"
 #include "rows_gemm.cuh"
+#include "vocab_rows.cuh"
 
 using namespace sd;
 
@@ -128,7 +129,7 @@ struct specdec_handle {
     int enc_skinny = 1;             // option "enc_skinny": the encoders use the few-rows GEMM too
     int use_ln_fuse = 0;            // option "ln_fuse": measured slower than the separate LayerNorm launch, kept for comparison
     int use_sk_cluster = 1;         // option "sk_cluster": the few-rows GEMM splits long reductions across a cluster
-    bool splitk_ready = false;
+    bool splitk_ready = false, vocab_rows_ready = false;
     int diag_repeat = 0;            // diagnostics: launch every attention (1) / LayerNorm (2) / non-residual GEMM (4) / vocabulary (8) kernel of the path once more (same
                                     // result) to read its cost inside the pipeline off the step time (option "diag_repeat")
     int use_splitk = 1;             // residual GEMMs with K >= 768 over few row tiles split K across a cluster of 4 / 2 CTAs (option "splitk")
@@ -837,6 +838,21 @@ int block_ffn(specdec_handle* h, const ModelW& m, const LayerW& w, float* x, int
     return 0;
 }
 
+// The last LayerNorm and the vocabulary projection of a few rows as one kernel.  The rows' drafts are checked where there are any (verify).
+bool vocab_rows_inside(const specdec_handle* h, const ModelW& m, int rows_ub) {
+    return h->vocab_rows_ready && h->use_tc && h->use_skinny && !h->use_ln_fuse && !h->tma.force_bn && vr_supported(h->tma, m.dm.vocab, m.dm.d_model, rows_ub);
+}
+int vocab_rows(specdec_handle* h, const ModelW& m, const float* x, int cnt, int rows_ub, const int* draft, int k, int* n_tiles, cudaStream_t st) {
+    VocabRowsArgs a{x, m.dec_lnf_g, m.dec_lnf_b, 1e-5f, (const bf16*)m.embed, m.dm.vocab, h->ses.counters + cnt, static_rows(h, cnt, rows_ub),
+                    draft, h->rows.slot_seq, k, h->ld, h->ld_id, (bf16*)h->y, h->part, h->want_lse};
+    *n_tiles = cdiv(m.dm.vocab, VR_BN);
+    for (int i = 0; i < (h->diag_repeat & 8 ? 2 : 1); ++i) {
+        if (vr_launch(h->tma, a, rows_ub, st) != 0) return fail(h, SPECDEC_ERR_CUDA, "tensor-core GEMM launch failed: " + h->tma.err);
+        ++h->launches;
+    }
+    return 0;
+}
+
 template <typename T>
 int embed(specdec_handle* h, const ModelW& m, const Rows& r, const float* pos_table, int cnt, int rows_ub,
           cudaStream_t st) {
@@ -965,8 +981,9 @@ int draft_impl(specdec_handle* h, int k, int* d_draft, cudaStream_t st) {
     TRY(block_ffn<T>(h, m, w, h->x2, CNT_DRAFT_MASK, R2, st, m.dec_lnf_g, m.dec_lnf_b));
     const LnSpec lf{h->x2, m.dec_lnf_g, m.dec_lnf_b};
     int n_tiles = 0;
-    TRY(gemm<T>(h, EPI_STATS, h->y, d, m.embed, nullptr, m.dm.vocab, d, CNT_DRAFT_MASK, R2, nullptr, 0, nullptr, st,
-                nullptr, nullptr, &n_tiles, nullptr, &lf));
+    if (std::is_same<T, bf16>::value && vocab_rows_inside(h, m, R2)) TRY(vocab_rows(h, m, h->x2, CNT_DRAFT_MASK, R2, nullptr, k, &n_tiles, st));
+    else TRY(gemm<T>(h, EPI_STATS, h->y, d, m.embed, nullptr, m.dm.vocab, d, CNT_DRAFT_MASK, R2, nullptr, 0, nullptr, st,
+                     nullptr, nullptr, &n_tiles, nullptr, &lf));
     CUDA_TRY(h, launch_pdl(h, k_draft_argmax, dim3(cdiv(R2, 4)), dim3(128), 0, st, (const RowPart*)h->part, n_tiles,
                            (const int*)(h->ses.counters + CNT_DRAFT_MASK), (const int*)h->mrows.slot, d_draft,
                            (const int*)(h->script_on ? h->script : nullptr), h->T_cap + h->k_cap, (const int*)h->ses.len, k));
@@ -1002,7 +1019,10 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
                          last ? m.dec_lnf_b : m.dec[l + 1].ln1_b));
     }
     const bool ln_pending = !(h->x == h->fused_x && m.dec_lnf_g == h->fused_g && h->y == h->fused_out);
-    if (ln_pending && d <= 1024) {
+    const bool inside = std::is_same<T, bf16>::value && ln_pending && vocab_rows_inside(h, m, M);
+    if (inside) {
+        // (normalised and checked against the drafts by the projection itself)
+    } else if (ln_pending && d <= 1024) {
         // final LayerNorm and the pre-pass logit of every row's draft in one kernel
         for (int i = 0; i < (h->diag_repeat & 2 ? 2 : 1); ++i) {
             cudaError_t e = cudaSuccess;
@@ -1025,8 +1045,9 @@ int verify_impl(specdec_handle* h, const int* d_draft, int k, int beta, float ta
     }
     int n_tiles = 0;
     prof_mark(h, st);
-    TRY(gemm<T>(h, EPI_STATS, h->y, d, m.embed, nullptr, m.dm.vocab, d, CNT_VERIFY, M, nullptr, 0, nullptr, st, h->ld,
-                h->ld_id, &n_tiles));
+    if (inside) TRY(vocab_rows(h, m, h->x, CNT_VERIFY, M, d_draft, k, &n_tiles, st));
+    else TRY(gemm<T>(h, EPI_STATS, h->y, d, m.embed, nullptr, m.dm.vocab, d, CNT_VERIFY, M, nullptr, 0, nullptr, st, h->ld,
+                     h->ld_id, &n_tiles));
     prof_mark(h, st);
     FusedCommit fc{h->ses, h->v_draft, h->cfg.eos_id, h->h_post, h->fuse_commit ? 1 : 0};
     CUDA_TRY(h, launch_pdl(h, k_accept, dim3(slots), dim3(32 * std::min(32, std::max(k + 1, 4))), (size_t)(k + 1) * sizeof(RowPart), st, (const RowPart*)h->part, n_tiles,
@@ -1605,6 +1626,8 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
         if (sd::tc_init(h->tma, h->ses.counters + 7) != 0) h->use_tc = 0;     // reported through specdec_last_error; SIMT GEMM still runs on the GPU
         h->splitk_ready = h->use_tc && sd::spk_init(h->tma) == cudaSuccess;
         if (!h->splitk_ready) cudaGetLastError();
+        h->vocab_rows_ready = h->use_tc && sd::vr_init() == cudaSuccess;
+        if (!h->vocab_rows_ready) cudaGetLastError();
         h->pair_ready = h->use_tc && sd::tc_pair_init() == cudaSuccess;
         if (!h->pair_ready) cudaGetLastError();
         if (!h->use_tc) h->err = "tensor-core GEMM unavailable: " + h->tma.err;
