@@ -104,17 +104,20 @@ struct Proj64 {
             ldsm_x4(bp + 16 * PITCH + s * 32, bfr[s][2][0], bfr[s][2][1], bfr[s][3][0], bfr[s][3][1]);
         }
     }
+    // BLOCKED: A as 8-column chunks of 16 rows of 16 bytes, the way the heads send them; else rows of PITCH bytes
+    template <bool BLOCKED>
     __device__ __forceinline__ void multiply(uint32_t as, float* red, int warp, int lane) {
         float c[4][4];
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) c[j][e] = 0.f;
-        const uint32_t ap = as + (lane & 15) * PITCH + (warp >> 1) * STEPS * 32 + (lane >> 4) * 16;
+        const uint32_t ap = BLOCKED ? as + ((warp >> 1) * STEPS * 2 + (lane >> 4)) * 256 + (lane & 15) * 16
+                                    : as + (lane & 15) * PITCH + (warp >> 1) * STEPS * 32 + (lane >> 4) * 16;
 #pragma unroll
         for (int s = 0; s < STEPS; ++s) {
             uint32_t af[4];
-            ldsm_x4(ap + s * 32, af[0], af[1], af[2], af[3]);
+            ldsm_x4(ap + s * (BLOCKED ? 512 : 32), af[0], af[1], af[2], af[3]);
 #pragma unroll
             for (int j = 0; j < 4; ++j) mma_bf16(c[j], af, bfr[s][j][0], bfr[s][j][1]);
         }
@@ -159,11 +162,12 @@ constexpr int attn_ctas(int mt, int kg, int kw) { return kg > 1 ? 0 : mt == 4 ? 
 //
 // ON > 0: the heads of a query tile are a cluster of ON CTAs, and the output projection runs here too (OutArgs).  Bound by the same chain of round trips:
 // every CTA sends its head's 16 rows (bf16, as they would go to memory) to the shared memory of all, multiplies the 16 whole rows by its own 64 rows
-// of Wo and adds the residual.  Wo is requested ahead of the wait and turned into register fragments while the queries are on their way, so
-// that only the exchange, 32 MMAs a warp and the sum of four K slices follow the attention: a launch and its round trip less
-// (verify step of 26 rows, both attentions of six layers: 156.5 -> 147.2 us; with Wo fetched behind the wait 155.2).  The exchange is counted on
-// the receiver's mbarrier: plain remote stores behind a cluster barrier, whose release and acquire every thread pays, took 0.2 us more a launch
-// (the same step 147.3 -> 145.1).
+// of Wo and adds the residual.  A launch and its round trip less (verify step of 26 rows, both attentions of six layers: 156.5 -> 147.2 us).
+//   * Wo, and Wq with QNC, are requested ahead of the wait and are register fragments by the time it returns (fetched behind it 155.2 us; turned into fragments
+//     behind it, while the rows arrive, their 128 KB from shared memory delayed the LayerNorm: rows and LayerNorm 1.5 us, now 1.0);
+//   * every warp sends its eight columns as one bulk copy of 256 bytes to each CTA, counted on the receiver's mbarrier: 0.45 us from the combined rows to the
+//     first MMA, 0.85 with 16-byte asynchronous remote stores, more with plain ones behind a cluster barrier (the step: 147.3, 145.1; both changes, beside
+//     others by then, 125.8 -> 120.4).
 template <bool PAGED, int MT, int KG, int KW, int NS, int QNC = 0, int ON = 0>
 __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {
     using C = AttnCfg<MT, KG, KW>;
@@ -263,10 +267,18 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (tid == 0) s_nkmax = m;
     }
-    if constexpr (ON > 0 && QNC == 0) asm volatile("cp.async.commit_group;" ::: "memory");
+    if constexpr (ON > 0 || QNC > 0) asm volatile("cp.async.commit_group;" ::: "memory");
     __syncthreads();
     const int nkmax = s_nkmax, nblk = max((nkmax + KB - 1) / KB, 1);
     pdl_launch_dependents();
+    // the weights become fragments as soon as they are here, still ahead of the wait
+    Proj64<QNC ? QC::K : 256> pj;
+    if constexpr (ON > 0 || QNC > 0) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if constexpr (QNC > 0) pj.load_w((uint32_t)__cvta_generic_to_shared(qops) + 16 * QC::PITCH, warp, lane);
+        if constexpr (ON > 0) wo.load_w(oops + 16 * OC::PITCH, warp, lane);
+    }
     pdl_wait();                                  // ... and everything the predecessor kernels wrote after it
     if constexpr (ON > 0) {
         const int r = tid >> 4;
@@ -292,12 +304,6 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
                 xv[s][c] = m < nq ? *reinterpret_cast<const float4*>(qa.x + (size_t)(r0 + m) * QC::K + lane * 4 + c * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         const float4 v = __ldg(reinterpret_cast<const float4*>(qa.b + h * 64 + (tid & 15) * 4));
-        // while the rows are on their way: the weights, requested before the wait, become fragments
-        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-        __syncthreads();
-        Proj64<QC::K> pj;
-        pj.load_w((uint32_t)__cvta_generic_to_shared(qops) + 16 * QC::PITCH, warp, lane);
-        if constexpr (ON > 0) wo.load_w(oops + 16 * OC::PITCH, warp, lane);
         float mu[2] = {0.f, 0.f}, rs[2] = {0.f, 0.f};
 #pragma unroll
         for (int s = 0; s < 2; ++s)
@@ -333,7 +339,7 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
         __syncthreads();
         const uint32_t ops = (uint32_t)__cvta_generic_to_shared(qops);
         float* red = reinterpret_cast<float*>(Sp + max(ring * C::STAGE, C::MERGE) + 16 * QC::PITCH);        // (weights that are dead by then)
-        pj.multiply(ops, red, warp, lane);
+        pj.template multiply<false>(ops, red, warp, lane);
         __syncthreads();
         const int r = tid >> 4, c = (tid & 15) * 4;
         const float4 t = Proj64<QC::K>::sum(red, tid);
@@ -365,11 +371,6 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
     for (int o = 4; o < 32; o <<= 1) nkall = min(nkall, __shfl_xor_sync(0xffffffffu, nkall, o));
 
     while (issued < min(ring, nblk)) issue();
-    if constexpr (ON > 0 && QNC == 0) {          // while the queries are on their way: the weights, requested before the wait, become fragments
-        cp_wait_pending(issued);
-        __syncthreads();
-        wo.load_w(oops + 16 * OC::PITCH, warp, lane);
-    }
     for (int blk = 0; blk < nblk; ++blk) {
         cp_wait_pending(issued - blk - 1);
         __syncthreads();
@@ -503,23 +504,27 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
                 x.x = fmaf(t.x, f[q], x.x); x.y = fmaf(t.y, f[q], x.y); x.z = fmaf(t.z, f[q], x.z); x.w = fmaf(t.w, f[q], x.w);
             }
             __nv_bfloat162 p0 = __floats2bfloat162_rn(x.x * inv, x.y * inv), p1 = __floats2bfloat162_rn(x.z * inv, x.w * inv);
-            const uint32_t u0 = *reinterpret_cast<uint32_t*>(&p0), u1 = *reinterpret_cast<uint32_t*>(&p1);
-            const uint32_t w0 = __shfl_xor_sync(0xffffffffu, u0, 1), w1 = __shfl_xor_sync(0xffffffffu, u1, 1);
-            const bool odd = lane & 1;
-            // eight columns of a row: the even lane sends them to the lower half of the cluster, the odd lane to the upper
-            const uint32_t dst = oops + rr * OC::PITCH + (h * 64 + kg * CW) * 2;
+            // this warp's eight columns of the 16 rows, 256 bytes in place of the queries, go to every CTA of the cluster as one copy
+            *reinterpret_cast<uint2*>(sm + kg * 256 + lane * 8) = make_uint2(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1));
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             cluster_wait();                          // every CTA of the cluster has begun and its barrier exists
-#pragma unroll
-            for (int i = 0; i < ON / 2; ++i)
-                st_peer16(dst, smem_u32(&heads_bar), (odd ? ON / 2 : 0) + i, make_uint4(odd ? w0 : u0, odd ? w1 : u1, odd ? u0 : w0, odd ? u1 : w1));
+            if (lane < ON) {
+                uint32_t ra, rb;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(oops + (h * 8 + kg) * 256), "r"(lane));
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_u32(&heads_bar)), "r"(lane));
+                asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], 256, [%2];"
+                             ::"r"(ra), "r"(Qs + kg * 256), "r"(rb) : "memory");
+            }
             mbar_wait(smem_u32(&heads_bar), 0, &abort_s, oa.err_word, 12);
             __syncthreads();                         // (the partial outputs of the key groups are dead)
-            wo.multiply(oops, mO, warp, lane);
+            cluster_arrive_relaxed();                // this CTA has what was sent to it
+            wo.template multiply<true>(oops, mO, warp, lane);
             __syncthreads();
             const float4 t = Proj64<OC::K>::sum(mO, tid);
             if ((tid >> 4) < nq)
                 *reinterpret_cast<float4*>(oa.x_out + (size_t)(r0 + (tid >> 4)) * OC::K + h * 64 + (tid & 15) * 4) =
                     make_float4(t.x + ob.x + res.x, t.y + ob.y + res.y, t.z + ob.z + res.z, t.w + ob.w + res.w);
+            cluster_wait();                          // nobody leaves while a copy from its shared memory may be under way
         } else if (r < nq) {
             bf16* o = a.out + (size_t)(r0 + r) * a.out_stride + h * 64 + c0;
 #pragma unroll
