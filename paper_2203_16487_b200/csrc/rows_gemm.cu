@@ -42,11 +42,11 @@ struct RgCfg {
 // rows), 2.6 us for FFN2 (3.5); the step 145.1 -> 131, a greedy pass over 16 sequences 6262 -> 5680 us.  The fragments cost registers (up to 165 a
 // thread): beyond three row tiles with a LayerNorm inside too few of the successors' CTAs are resident (52 rows: 154 / 161 us a step), those keep the variant without.
 template <int EPI, int NC, int MT, int NT, int WN, int CS, int ST>
-__global__ void __launch_bounds__(RG_THREADS, NC > 0 && ST >= 8 ? 1 : NC > 4 || ST > 0 ? 2 : 3) k_rows(RowsArgs a) {
+__global__ void __launch_bounds__(RG_THREADS, (NC > 0 && ST >= 8) || MT * ST > 16 ? 1 : NC > 4 || ST > 0 ? 2 : 3) k_rows(RowsArgs a) {
     using C = RgCfg<MT, NT, WN, CS>;
     constexpr int BM = C::BM, NB = C::NB, WK = C::WK, RP = C::RP, TN = NT / WN;      // TN = 8-column tiles per warp
     static_assert(TN % 2 == 0 || TN == 1, "B fragments come in pairs");
-    static_assert(ST == 0 || (MT == 1 && TN > 1), "weights as fragments: 16 rows, column tiles in pairs");
+    static_assert(ST == 0 || TN > 1, "weights as fragments: column tiles in pairs");
     constexpr bool LN = NC > 0;
     extern __shared__ __align__(16) unsigned char rg_sm[];
     __shared__ int s_kv[BM];
@@ -216,10 +216,13 @@ __global__ void __launch_bounds__(RG_THREADS, NC > 0 && ST >= 8 ? 1 : NC > 4 || 
     if constexpr (ST > 0) {
 #pragma unroll
         for (int s = 0; s < ST; ++s) {
-            uint32_t af[4];
-            ldsm_x4(ap + s * 32, af[0], af[1], af[2], af[3]);
+            uint32_t af[MT][4];
 #pragma unroll
-            for (int j = 0; j < TN; ++j) mma_bf16(acc[0][j], af, wf[s][j][0], wf[s][j][1]);
+            for (int i = 0; i < MT; ++i) ldsm_x4(ap + i * 16 * pitch + s * 32, af[i][0], af[i][1], af[i][2], af[i][3]);
+#pragma unroll
+            for (int i = 0; i < MT; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) mma_bf16(acc[i][j], af[i], wf[s][j][0], wf[s][j][1]);
         }
     } else {
 #pragma unroll 8
@@ -323,6 +326,19 @@ static int rg_split(int N, int K, int rows_ub, bool cluster) {
     if (rows_ub > rg_ln_rows(min(N, K)) && K % 32 == 0) return 4;
     return K % 16 == 0 ? 2 : 1;       // (the reductions whose weights become fragments take four: rg_launch_resid)
 }
+// 16-row tiles read the weights once more for every 16 rows, so they stop first; what counts is whether all CTAs are resident at once next to their
+// predecessors' and successors', hence limits in CTAs per SM.  Width 512 (84 KB and 100 KB a CTA, two to an SM), verify step, us, tcgen05 tiles / 16 rows / 32 rows
+// of the output projections: 208 rows 223 / 204 / 214, 312 rows 258 / 235 / 244, 416 rows 277 / 269 / 270, 520 rows 289 / 280 / 275, 624 rows 295 / 295 / 291.5, 832 rows
+// 312 / 333 / 312; the QKV projection: 182 rows 203 / - / 195, 208 rows 204 / - / 199.6, 312 rows 235 / - / 245.  Width 768 (50 KB, 32 columns; 149 KB, one to an SM): 130
+// rows 275 / 258 / 265, 156 rows 281 / 265 / 269, 208 rows 307 / 325 / 296, 312 rows 360 / 373 / 350, 364 rows 343 / - / 346.  The two encoders share the SMs (512: 144 rows
+// 316 / 273, 200 rows 324 / 299, 400 rows 380 / 392 on 16 rows, 496 rows 422 / 419, 640 rows 430 / 439; 768: 96 rows 203 / 193, 200 rows 270 / 260, 296 rows 303 / 314).
+int rg_frag_rows(int epi, int N, int K, int rows_ub, int n_sm, bool enc) {
+    const bool resid = epi == EPI_RESID;
+    if (N % 64 || !(K == 512 || (K == 768 && resid)) || rows_ub <= (K == 512 ? 96 : 80)) return 0;
+    const long long sm = n_sm, t16 = (rows_ub + 15) / 16, t32 = (rows_ub + 31) / 32;
+    if (resid && t16 * (K == 512 ? N / 64 : N / 32) <= (enc ? sm : K == 512 ? sm * 3 / 2 : sm * 5 / 3)) return 16;
+    return t32 * (N / 64) <= (K == 512 ? (enc && resid ? sm : sm * 5 / 4) : enc ? sm * 2 / 3 : sm * 7 / 8) ? 32 : 0;
+}
 bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster) {
     if (rows_ub > RG_MAX_ROWS || K % 16 || N % 16 || lda % 8) return false;
     if (epi != EPI_STORE && epi != EPI_RELU && epi != EPI_GELU && epi != EPI_RESID && epi != EPI_QKV) return false;
@@ -333,8 +349,9 @@ bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster) {
 // Tile shapes: 16 rows where the LayerNorm runs inside (each CTA repeats its rows' normalisation: few rows, wide column tiles), 32 rows
 // beyond; columns so that a projection of a 512-wide model still spreads over 24-96 CTAs.
 template <int EPI, int NC>
-inline cudaError_t rg_launch_out(const RowsArgs& a, int rows_ub, bool pdl, cudaStream_t st) {
+inline cudaError_t rg_launch_out(const RowsArgs& a, int rows_ub, int frag, bool pdl, cudaStream_t st) {
     const bool wide = a.g.N >= 1024;
+    if constexpr (NC == 0) { if (frag) return rg_launch_one<EPI, 0, 2, 8, 2, 1, 8>(a, rows_ub, pdl, st); }
     // Weights as fragments.  One row tile: 32 columns a CTA (greedy pass over 16 sequences 6090 -> 5700 us; with two row tiles these are too many CTAs: one
     // sentence 902 -> 973); up to three: 64 columns (verify step, us, without / with: 26 rows 136.4 / 129.6, 44 rows 139.8 / 136.7, 52 rows 154 / 161).
     // 768 columns take 96 registers of fragments next to the 96 of the rows: 11 rows 190.6 / 183.6, 26 rows 195 / 201.5, 41 rows 205 / 212.
@@ -348,9 +365,12 @@ inline cudaError_t rg_launch_out(const RowsArgs& a, int rows_ub, bool pdl, cudaS
     if constexpr (EPI == EPI_STORE) { if (rows_ub > 32) return rg_launch_one<EPI, NC, 1, 4, 1, 1>(a, rows_ub, pdl, st); }
     return rg_launch_one<EPI, NC, 1, 2, 1, 1>(a, rows_ub, pdl, st);
 }
-static cudaError_t rg_launch_resid(const RowsArgs& a, int rows_ub, bool cluster, bool pdl, cudaStream_t st) {
+static cudaError_t rg_launch_resid(const RowsArgs& a, int rows_ub, int frag, bool cluster, bool pdl, cudaStream_t st) {
+    if (frag && a.g.K == 512) return frag == 16 ? rg_launch_one<EPI_RESID, 0, 1, 8, 2, 1, 8>(a, rows_ub, pdl, st) : rg_launch_one<EPI_RESID, 0, 2, 8, 2, 1, 8>(a, rows_ub, pdl, st);
+    if (frag) return frag == 16 ? rg_launch_one<EPI_RESID, 0, 1, 4, 1, 1, 6>(a, rows_ub, pdl, st) : rg_launch_one<EPI_RESID, 0, 2, 8, 2, 1, 12>(a, rows_ub, pdl, st);
     const int split = rg_split(a.g.N, a.g.K, rows_ub, cluster);
     if (rows_ub > rg_ln_rows(min(a.g.N, a.g.K))) {
+        if (split == 4 && a.g.K == 2048) return rg_launch_one<EPI_RESID, 0, 2, 8, 2, 4, 8>(a, rows_ub, pdl, st);       // (verify step of 156 rows 198 -> 195.5 us)
         if (split == 4) return rg_launch_one<EPI_RESID, 0, 2, 8, 2, 4>(a, rows_ub, pdl, st);
         return rg_launch_one<EPI_RESID, 0, 2, 8, 2, 1>(a, rows_ub, pdl, st);
     }
@@ -374,21 +394,21 @@ static cudaError_t rg_launch_resid(const RowsArgs& a, int rows_ub, bool cluster,
     }
 }
 template <int EPI>
-inline cudaError_t rg_launch_nc(const RowsArgs& a, int rows_ub, bool pdl, cudaStream_t st) {
-    if (!a.ln_x) return rg_launch_out<EPI, 0>(a, rows_ub, pdl, st);
+inline cudaError_t rg_launch_nc(const RowsArgs& a, int rows_ub, int frag, bool pdl, cudaStream_t st) {
+    if (!a.ln_x) return rg_launch_out<EPI, 0>(a, rows_ub, frag, pdl, st);
     switch (a.g.K) {
-        case 256: return rg_launch_out<EPI, 2>(a, rows_ub, pdl, st);
-        case 512: return rg_launch_out<EPI, 4>(a, rows_ub, pdl, st);
-        default: return rg_launch_out<EPI, 6>(a, rows_ub, pdl, st);
+        case 256: return rg_launch_out<EPI, 2>(a, rows_ub, 0, pdl, st);
+        case 512: return rg_launch_out<EPI, 4>(a, rows_ub, 0, pdl, st);
+        default: return rg_launch_out<EPI, 6>(a, rows_ub, 0, pdl, st);
     }
 }
-cudaError_t rg_launch(int epi, const RowsArgs& a, int rows_ub, bool cluster, bool pdl, cudaStream_t st) {
+cudaError_t rg_launch(int epi, const RowsArgs& a, int rows_ub, int frag, bool cluster, bool pdl, cudaStream_t st) {
     switch (epi) {
-        case EPI_STORE: return rg_launch_nc<EPI_STORE>(a, rows_ub, pdl, st);
-        case EPI_RELU: return rg_launch_nc<EPI_RELU>(a, rows_ub, pdl, st);
-        case EPI_GELU: return rg_launch_nc<EPI_GELU>(a, rows_ub, pdl, st);
-        case EPI_QKV: return rg_launch_nc<EPI_QKV>(a, rows_ub, pdl, st);
-        default: return rg_launch_resid(a, rows_ub, cluster, pdl, st);
+        case EPI_STORE: return rg_launch_nc<EPI_STORE>(a, rows_ub, frag, pdl, st);
+        case EPI_RELU: return rg_launch_nc<EPI_RELU>(a, rows_ub, frag, pdl, st);
+        case EPI_GELU: return rg_launch_nc<EPI_GELU>(a, rows_ub, frag, pdl, st);
+        case EPI_QKV: return rg_launch_nc<EPI_QKV>(a, rows_ub, frag, pdl, st);
+        default: return rg_launch_resid(a, rows_ub, frag, cluster, pdl, st);
     }
 }
 
@@ -401,7 +421,7 @@ static void rg_room(cudaError_t& e) {
 }
 template <int EPI, int NC>
 static void rg_room_out(cudaError_t& e) {
-    if constexpr (NC == 0) rg_room<EPI, 0, 2, 8, 2, 1>(e);
+    if constexpr (NC == 0) { rg_room<EPI, 0, 2, 8, 2, 1>(e); rg_room<EPI, 0, 2, 8, 2, 1, 8>(e); }
     if constexpr (NC == 2 || NC == 4) rg_room<EPI, NC, 1, 4, 1, 1, NC>(e);
     if constexpr (NC > 0) rg_room<EPI, NC, 1, 8, 2, 1, 2 * NC>(e);
     rg_room<EPI, NC, 1, 8, 2, 1>(e);
@@ -413,6 +433,7 @@ static void rg_room_nc(cudaError_t& e) { rg_room_out<EPI, 0>(e); rg_room_out<EPI
 cudaError_t rg_init() {
     cudaError_t e = cudaSuccess;
     rg_room_nc<EPI_STORE>(e); rg_room_nc<EPI_RELU>(e); rg_room_nc<EPI_GELU>(e); rg_room_nc<EPI_QKV>(e);
+    rg_room<EPI_RESID, 0, 1, 8, 2, 1, 8>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1, 8>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1, 12>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 4, 8>(e);
     rg_room<EPI_RESID, 0, 2, 8, 2, 4>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 2>(e);
     rg_room<EPI_RESID, 0, 1, 4, 1, 2, 4>(e); rg_room<EPI_RESID, 0, 1, 8, 2, 4, 8>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 2, 12>(e);
     rg_room<EPI_RESID, 0, 1, 4, 1, 1>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1, 2>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1, 4>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1, 6>(e);

@@ -25,9 +25,12 @@ __host__ __device__ constexpr int rg_tile_rows_enc(int width) { return width <= 
 // 130 rows 202 / 218; width 768, 104 rows 330 / 304).
 __host__ __device__ constexpr int rg_ln_rows(int width) { return width <= 512 ? 144 : 80; }
 
+// Rows of a tile (16 or 32) where a GEMM of the usual widths goes on here beyond those rows, with the weights as register fragments; 0: it does not.
+// (LayerNorm in front, or none.)
+int rg_frag_rows(int epi, int N, int K, int rows_ub, int n_sm, bool enc);
 bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster);
 inline bool rg_ln_width(int K) { return K == 256 || K == 512 || K == 768; }    // widths that the LayerNorm prologue exists for
 cudaError_t rg_init();           // once per handle, before the first launch
-cudaError_t rg_launch(int epi, const RowsArgs& a, int rows_ub, bool cluster, bool pdl, cudaStream_t st);
+cudaError_t rg_launch(int epi, const RowsArgs& a, int rows_ub, int frag, bool cluster, bool pdl, cudaStream_t st);
 
 }  // namespace sd

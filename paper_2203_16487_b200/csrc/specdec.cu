@@ -498,9 +498,13 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
     if (rows_ub <= 0) return 0;
     // few rows: the weight-streaming kernel, with the LayerNorm inside where it has one
     const int width = std::min(N, K), tile_rows = sd::tc_supported(N, K) ? (cnt == CNT_ENC ? rg_tile_rows_enc(width) : rg_tile_rows(width)) : RG_MAX_ROWS;
-    const bool few = std::is_same<T, bf16>::value && h->use_skinny && h->use_tc && rows_ub <= tile_rows && (cnt != CNT_ENC || h->enc_skinny) &&
-                     !(epi == EPI_RESID && h->use_ln_fuse) && rg_supported(epi, N, K, lnp ? K : lda, rows_ub, h->use_sk_cluster != 0);
-    const bool ln_inside = few && lnp && rows_ub <= rg_ln_rows(width) && rg_ln_width(K);
+    const bool rows_ok = std::is_same<T, bf16>::value && h->use_skinny && h->use_tc && (cnt != CNT_ENC || h->enc_skinny) && !(epi == EPI_RESID && h->use_ln_fuse);
+    const int tile_lda = lnp ? K : lda;
+    const bool fits = rows_ok && rows_ub <= tile_rows && rg_supported(epi, N, K, tile_lda, rows_ub, h->use_sk_cluster != 0);
+    const bool ln_inside = fits && lnp && rows_ub <= rg_ln_rows(width) && rg_ln_width(K);
+    // (with the LayerNorm in front, or none)
+    const int frag = rows_ok && !ln_inside && tile_lda % 8 == 0 && epi != EPI_STATS && epi != EPI_F32 ? rg_frag_rows(epi, N, K, rows_ub, h->tma.n_sm, cnt == CNT_ENC) : 0;
+    const bool few = fits || frag;
     const bool few32 = std::is_same<T, float>::value && h->use_skinny && rf_supported(epi, N, K, lnp ? K : lda, rows_ub);
     const bool ln32 = few32 && lnp && rf_ln_width(K);
     if (lnp && !ln_inside && !ln32) {  // separate normalisation launch, then a plain GEMM on its output
@@ -526,7 +530,7 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
             if (ln_inside) { ra.ln_x = lnp->x; ra.ln_g = lnp->g; ra.ln_b = lnp->b; ra.ln_eps = 1e-5f; }
             ra.err_word = h->ses.counters + 7;
             ra.trace = h->want_trace ? h->trace_buf + 216 + 6 * ((epi == EPI_RELU || epi == EPI_GELU) ? 0 : epi == EPI_RESID ? 1 : epi == EPI_QKV ? 2 : 3) : nullptr;
-            const cudaError_t e = rg_launch(epi, ra, rows_ub, h->use_sk_cluster != 0, h->use_pdl, st);
+            const cudaError_t e = rg_launch(epi, ra, rows_ub, frag, h->use_sk_cluster != 0, h->use_pdl, st);
             if (e != cudaSuccess) return fail(h, SPECDEC_ERR_CUDA, std::string("row GEMM launch: ") + cudaGetErrorString(e));
             KCHECK(h);
             return 0;

@@ -31,6 +31,17 @@ pytestmark = pytest.mark.gpu
     (320, 5, 1312, 16, 10),         # 176 rows: the last of the few-rows kernel; no LayerNorm width, an FFN that has no tiles
     (320, 5, 1312, 24, 15),         # 384 rows: the FFN's output projection stays with the few-rows kernel
     (128, 2, 192, 35, 10),          # 385 rows: tensor-core tiles
+    (512, 8, 2048, 8, 11),          # 96 rows: the last output projections on 16 x 32 tiles
+    (512, 8, 2048, 7, 13),          # 98 rows: 16 x 64 tiles, the last of them two rows
+    (512, 8, 2048, 11, 15),         # 176 rows: the last with the FFN2 here, its slices as fragments of 32 rows
+    (512, 8, 2048, 14, 16),         # 238 rows: QKV on 32-row tiles, the last of them 14 rows; 1 / 2 more rows of tiles than SMs
+    (512, 8, 2048, 27, 15),         # 432 rows: the last output projections on 16-row tiles
+    (512, 8, 2048, 31, 13),         # 434 rows: ... on 32-row tiles
+    (512, 8, 2048, 46, 15),         # 736 rows: the last on 32-row tiles
+    (768, 12, 3072, 3, 26),         # 81 rows: 16 x 32 tiles at this width, beyond the LayerNorm inside
+    (768, 12, 3072, 10, 15),        # 160 rows: the last of them
+    (768, 12, 3072, 7, 22),         # 161 rows: 32 x 64 tiles
+    (768, 12, 3072, 20, 15),        # 320 rows: the last of them
     (512, 8, 2048, 32, 15),         # 512 rows: the last four K slices of a tile at this width, the last row tile full
     (512, 8, 2048, 27, 18),         # 513 rows: two K slices, one row in the last tile
     (256, 4, 1152, 20, 14),         # 300 rows: two slices of nine K blocks, more than the ring holds
