@@ -744,17 +744,19 @@ void prof_collect(specdec_handle* h) {
 }
 
 // Whether the attention kernel goes on to the output projection and the residual sum: for the two head counts that are one cluster, and few CTAs, since each
-// wants an SM of its own next to the GEMMs before and after it.  With the queries projected too (200 KB a CTA): 32 CTAs and 48 rows, the GEMMs in turn being
-// 128 CTAs beyond (verify step, us, without / with: 26 rows 151 / 147, 44 rows 156 / 151, 52 rows 162 / 164, 88 rows 183 / 188).  Otherwise 64 CTAs
-// (10 rows 149 / 146, 26 rows 157 / 151, 52 rows 163 / 162; 80 CTAs 203 / 205, 128 CTAs 158 / 196), or 96 where a gathering launch goes with it (drafts
-// of 6 x 25 rows 108 / 103).  Blocks of a few rows leave nothing to gain (greedy steps 2 % slower).
+// takes an SM from the GEMMs before and after it.  Eight heads: those GEMMs are quicker themselves since their weights are fragments, so only
+// self-attention of one tile of rows goes on (verify step, us, without / with: 6 rows 106.4 / 104.4, 16 rows 111.7 / 108.8, 26 rows 115.1 / 116.4, 44 rows 136.8 / 140.9, 8 x 6 rows
+// 132.5 / 148, 104 rows 161 / 167), of two with the queries projected too (200 KB a CTA; 16 rows 116.9 / 111.7, 26 rows 119.2 / 115.1, 33 rows 127.8 / 137, 44 rows
+// 128.4 / 136.8).  Four heads leave a CTA's SM room for others: 64 CTAs (52 rows 119.2 / 115.7, 104 rows 130.6 / 126.6, 208 rows 197 / 181) and 32, 48 rows (26 rows
+// 105.0 / 99.1, 48 rows 110.8 / 106.5).  Where a gathering launch goes with it 96 (drafts of 6 x 25 rows 95.1 / 91.2, 8 x 25 rows 95.5 / 97).  Blocks of a few rows leave nothing to gain
+// (greedy steps 2 % slower).
 enum OutUse { OUT_SELF, OUT_GATHERS, OUT_QUERIES };
 bool out_inside(const specdec_handle* h, int d_head, int q_ub, int n_heads, int cnt, int rows_ub, int max_keys, OutUse use) {
     if (!h->use_tc || !h->use_skinny || !h->use_tc_attn || !h->use_sk_cluster || h->use_ln_fuse) return false;
     if ((h->diag_repeat & 1) && 2 * n_heads * d_head > std::min(h->cfg.verifier.d_ffn, h->cfg.drafter.d_ffn)) return false;    // (no room for the extra launch's rows)
     if (d_head != 64 || (n_heads != 4 && n_heads != 8) || q_ub <= 4) return false;
     const long long ctas = (long long)cdiv(q_ub, 16) * n_heads * (cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub));
-    if (ctas > (use == OUT_QUERIES ? 32 : use == OUT_GATHERS ? 96 : 64) || (use == OUT_QUERIES && rows_ub > 48)) return false;
+    if (ctas > (use == OUT_GATHERS ? 96 : n_heads == 8 ? (use == OUT_QUERIES ? 16 : 8) : use == OUT_QUERIES ? 32 : 64) || (use == OUT_QUERIES && rows_ub > 48)) return false;
     const int ops = use == OUT_QUERIES ? ProjCfg<4, 8>::OPS : ProjCfg<0, 8>::OPS;
     return AttnCfg<1, 8, 16>::smem(max_keys, 3, use != OUT_QUERIES, ops) <= 227 * 1024 - 2048;      // (with the queries: up to 128 keys)
 }
@@ -802,11 +804,13 @@ int block_self(specdec_handle* h, const ModelW& m, const LayerW& w, float* x, co
     return 0;
 }
 
-// Whether the cross-attention kernel projects its queries itself: while its CTAs (16 queries of a head with the head's 64 rows of Wq, over 100 KB
-// of shared memory) fill the SMs once, or twice over at most 128 keys (verify step of 208 rows 262 / 241 us, 416 rows 364 / 358; 832 rows 396 / 453).
+// Whether the cross-attention kernel projects its queries itself: while its CTAs (16 queries of a head with the head's 64 rows of Wq) fill the SMs once (512 wide,
+// over 100 KB of shared memory; verify step, us, in a launch of its own / inside: 208 rows 216 / 201, 260 rows 229 / 232, 364 rows 236 / 253, 416 rows 256 / 270).  Over
+// at most 128 keys 768 wide a third more (208 rows 298 / 294, 312 rows 329 / 348), 256 wide, with several CTAs to an SM, twice (416 rows 216 / 198, 936 rows 246 / 230).
 bool query_inside(const specdec_handle* h, int d, int d_head, int q_ub, int n_heads, int max_keys) {
+    const long long ctas = (long long)cdiv(q_ub, 16) * n_heads * std::min(h->B, h->act_ub), sm = h->tma.n_sm;
     return h->use_tc && h->use_skinny && h->use_tc_attn && !h->use_ln_fuse && d_head == 64 && rg_ln_width(d) &&
-           (long long)cdiv(q_ub, 16) * n_heads * std::min(h->B, h->act_ub) <= (max_keys <= 128 ? 2 : 1) * h->tma.n_sm;
+           ctas <= (max_keys > 128 || d == 512 ? sm : d < 512 ? 2 * sm : sm * 4 / 3);
 }
 
 template <typename T>
