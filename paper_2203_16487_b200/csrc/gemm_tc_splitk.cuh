@@ -14,28 +14,39 @@
 namespace sd {
 
 constexpr int SPK_BN = 64;
-constexpr int SPK_STAGES = 7;                                  // ring depth: the receive buffer takes the rest of shared memory
-constexpr int SPK_A_KB = TC_BM * TC_BK * 2, SPK_STAGE = SPK_A_KB + SPK_BN * TC_BK * 2;
-constexpr int SPK_RECV = TC_BM * SPK_BN * 4;                   // SPLIT slices of 128 / SPLIT rows
-constexpr int SPK_SMEM = SPK_STAGES * SPK_STAGE + SPK_RECV + 1024;
-static_assert(SPK_STAGES * SPK_STAGE >= TC_EPI_WARPS * 4096, "the outgoing blocks reuse the ring");
+// AR = rows of a tile.  Of a 64-row box the MMA reads 64 rows more, which are the stage's weights, into accumulator lanes that nobody reads.
+template <int AR> struct SpkCfg {
+    static constexpr int STAGES = AR == 128 ? 7 : 8;           // ring depth: the receive buffer takes the rest of shared memory
+    static constexpr int A_KB = AR * TC_BK * 2, STAGE = A_KB + SPK_BN * TC_BK * 2;
+    static constexpr int RECV = AR * SPK_BN * 4;               // SPLIT slices of AR / SPLIT rows
+    static constexpr int SMEM = STAGES * STAGE + RECV + 1024;
+    static_assert(STAGES * STAGE >= TC_EPI_WARPS * 4096, "the outgoing blocks reuse the ring");
+    static_assert(AR == 128 || AR + SPK_BN >= 128, "the 128-row MMA read stays inside the stage");
+};
 
 // CTAs per tile: 4 while all clusters run at once, else 2, else none (0).  Shorter reductions gain less than the exchange costs (verify step, us, unsplit / split:
 // K = 768 in four 208 rows 318 / 310, in two 520 rows 399 / 403; K = 512 416 rows 279 / 286).  (Clusters of 4 do not use every SM: 36 of them on 148 SMs took two waves,
 // 392 us a verify
 // step of 312 rows at 768 columns where clusters of 2 take 361.)
-inline int spk_split(const TmaEncoder& enc, int N, int K, int rows_ub) {
-    if (N % SPK_BN || K < 768) return 0;
-    const long long tiles = (long long)((rows_ub + TC_BM - 1) / TC_BM) * (N / SPK_BN);
-    if (K % (4 * TC_BK) == 0 && tiles <= enc.spk_clusters4) return 4;
-    return K % (2 * TC_BK) == 0 && K >= 1024 && tiles <= enc.spk_clusters2 ? 2 : 0;
+// 64-row tiles while their clusters run at once, too: half of the activations to fetch behind the wait (182 rows 197 -> 194.5, 234 rows 208.8 -> 204.5, 104 rows at 768 columns
+// 258 -> 250), unless another stream's kernels share the SMs (two encoders over 144 rows 307 -> 315).
+struct SpkPlan { int split, rows; };
+inline SpkPlan spk_plan(const TmaEncoder& enc, int N, int K, int rows_ub, bool shared) {
+    if (N % SPK_BN || K < 768) return {0, 0};
+    const long long n = N / SPK_BN, tiles = (rows_ub + TC_BM - 1) / TC_BM * n;
+    if (K % (4 * TC_BK) == 0 && !shared && (rows_ub + 63) / 64 * n <= enc.spk_clusters4_64) return {4, 64};
+    if (K % (4 * TC_BK) == 0 && tiles <= enc.spk_clusters4) return {4, TC_BM};
+    return {K % (2 * TC_BK) == 0 && K >= 1024 && tiles <= enc.spk_clusters2 ? 2 : 0, TC_BM};
 }
 
-template <int SPLIT>
+template <int SPLIT, int AR>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, GemmArgs<bf16> g, int* err_word) {
-    constexpr int OWN = TC_BM / SPLIT;                         // rows that a CTA finishes
-    const int m0 = blockIdx.y * TC_BM, R = g.rows_static >= 0 ? g.rows_static : *g.n_rows;     // (a device-side count predates the step's chain)
+    using C = SpkCfg<AR>;
+    constexpr int SPK_STAGES = C::STAGES, SPK_A_KB = C::A_KB, SPK_STAGE = C::STAGE, SPK_RECV = C::RECV;
+    constexpr int OWN = AR / SPLIT, RB = OWN < 32 ? OWN : 32;  // rows that a CTA finishes; rows that a warp sends to one owner
+    static_assert(OWN % 16 == 0, "rows of 16 threads");
+    const int m0 = blockIdx.y * AR, R = g.rows_static >= 0 ? g.rows_static : *g.n_rows;     // (a device-side count predates the step's chain)
     if (m0 >= R && m0 > 0) return;                             // the whole cluster leaves; the first row tile always waits for the predecessor
     const int nkb = g.K / TC_BK / SPLIT;
     extern __shared__ uint8_t smem_raw[];
@@ -119,7 +130,7 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             x[i] = row0 + 16 * i < R ? *reinterpret_cast<const float4*>(g.resid + (size_t)(row0 + 16 * i) * g.N + n0 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_acc), 0, abort_flag, err_word, 3));      // the MMAs are done: the ring is free
         tc_fence_after();
-        if (ok) {
+        if (ok && q * 32 < AR) {
             float v[32];
             tmem_ld32(tmem_d + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32), v);
             // a row per lane, its 16-byte chunks XOR-swizzled by the row
@@ -129,27 +140,27 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 *reinterpret_cast<float4*>(blk + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
-            if (lane == 0) {
-                const uint32_t owner = q * 32 / OWN, dst = recv + (((rank * (OWN / 32) + q % (OWN / 32)) * 2 + half) << 12);
+            if (lane < 32 / RB) {
+                const uint32_t row = q * 32 + lane * RB, owner = row / OWN, dst = recv + ((rank * (OWN / RB) + row % OWN / RB) * 2 + half) * (RB * 128);
                 uint32_t ra, rb;
                 asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(dst), "r"(owner));
                 asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_u32(&bar_part)), "r"(owner));
                 asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             ::"r"(ra), "r"(ring + (warp - 2) * 4096), "r"(4096), "r"(rb) : "memory");
+                             ::"r"(ra), "r"(ring + (warp - 2) * 4096 + lane * (RB * 128)), "r"(RB * 128), "r"(rb) : "memory");
             }
             __syncwarp();
-            ok = mbar_wait(smem_u32(&bar_part), 0, abort_flag, err_word, 10);            // all slices of this CTA's rows have landed
         }
+        ok = ok && mbar_wait(smem_u32(&bar_part), 0, abort_flag, err_word, 10);          // all slices of this CTA's rows have landed
         if (ok) {
-            const uint8_t* src = ring_p + SPK_STAGES * SPK_STAGE + ((e & 15) >> 3) * 4096;
+            const uint8_t* src = ring_p + SPK_STAGES * SPK_STAGE + ((e & 15) >> 3) * (RB * 128);
 #pragma unroll
             for (int i = 0; i < OWN / 16; ++i) {
                 const int row = (e >> 4) + 16 * i;
-                const uint8_t* p = src + (row >> 5) * 8192 + (row & 31) * 128 + (((e & 7) ^ (row & 7)) << 4);
+                const uint8_t* p = src + row / RB * (RB * 256) + row % RB * 128 + (((e & 7) ^ (row & 7)) << 4);
                 float4 a = *reinterpret_cast<const float4*>(p);
 #pragma unroll
                 for (int s = 1; s < SPLIT; ++s) {                                        // rank order: fixed summation order
-                    const float4 t = *reinterpret_cast<const float4*>(p + s * (OWN / 32) * 8192);
+                    const float4 t = *reinterpret_cast<const float4*>(p + s * (OWN * 256));
                     a.x += t.x; a.y += t.y; a.z += t.z; a.w += t.w;
                 }
                 a.x += bz.x; a.y += bz.y; a.z += bz.z; a.w += bz.w;
@@ -164,10 +175,10 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     if (warp == 1) tmem_dealloc(tmem_d, 64);
 }
 
-template <int SPLIT>
+template <int SPLIT, int AR>
 inline cudaLaunchConfig_t spk_config(cudaLaunchAttribute* attr, dim3 grid, bool pdl, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = SPK_SMEM; cfg.stream = st;
+    cfg.gridDim = grid; cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = SpkCfg<AR>::SMEM; cfg.stream = st;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = SPLIT; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -175,34 +186,36 @@ inline cudaLaunchConfig_t spk_config(cudaLaunchAttribute* attr, dim3 grid, bool 
     cfg.attrs = attr; cfg.numAttrs = pdl ? 2 : 1;
     return cfg;
 }
-template <int SPLIT>
+template <int SPLIT, int AR>
 inline cudaError_t spk_init_one(int* clusters) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_tc_splitk<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SPK_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_gemm_tc_splitk<SPLIT, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, SpkCfg<AR>::SMEM);
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = spk_config<SPLIT>(attr, dim3(SPLIT), false, nullptr);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(clusters, k_gemm_tc_splitk<SPLIT>, &cfg);
+    const cudaLaunchConfig_t cfg = spk_config<SPLIT, AR>(attr, dim3(SPLIT), false, nullptr);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(clusters, k_gemm_tc_splitk<SPLIT, AR>, &cfg);
     return e;
 }
 inline cudaError_t spk_init(TmaEncoder& enc) {
-    const cudaError_t e = spk_init_one<4>(&enc.spk_clusters4);
-    return e == cudaSuccess ? spk_init_one<2>(&enc.spk_clusters2) : e;
+    cudaError_t e = spk_init_one<4, TC_BM>(&enc.spk_clusters4);
+    if (e == cudaSuccess) e = spk_init_one<4, 64>(&enc.spk_clusters4_64);
+    return e == cudaSuccess ? spk_init_one<2, TC_BM>(&enc.spk_clusters2) : e;
 }
 
-template <int SPLIT>
+template <int SPLIT, int AR>
 inline int spk_launch_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
-    const CUtensorMap* ta = enc.get(g.A, rows_ub, g.K, g.lda, TC_BM);
+    const CUtensorMap* ta = enc.get(g.A, rows_ub, g.K, g.lda, AR);
     const CUtensorMap* tw = enc.get(g.W, g.N, g.K, g.K, SPK_BN);
     if (!ta || !tw) return -1;
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = spk_config<SPLIT>(attr, dim3(g.N / SPK_BN * SPLIT, (rows_ub + TC_BM - 1) / TC_BM), enc.pdl, st);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc_splitk<SPLIT>, *ta, *tw, g, enc.err_word);
+    const cudaLaunchConfig_t cfg = spk_config<SPLIT, AR>(attr, dim3(g.N / SPK_BN * SPLIT, (rows_ub + AR - 1) / AR), enc.pdl, st);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc_splitk<SPLIT, AR>, *ta, *tw, g, enc.err_word);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { enc.err = std::string("launch (split-K): ") + cudaGetErrorString(e); return -1; }
     return 0;
 }
-inline int spk_launch(TmaEncoder& enc, int split, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
+inline int spk_launch(TmaEncoder& enc, SpkPlan plan, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
     if (!enc.ready) return -1;
-    return split == 4 ? spk_launch_one<4>(enc, g, rows_ub, st) : spk_launch_one<2>(enc, g, rows_ub, st);
+    if (plan.rows == 64) return spk_launch_one<4, 64>(enc, g, rows_ub, st);
+    return plan.split == 4 ? spk_launch_one<4, TC_BM>(enc, g, rows_ub, st) : spk_launch_one<2, TC_BM>(enc, g, rows_ub, st);
 }
 
 }  // namespace sd

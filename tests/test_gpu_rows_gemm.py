@@ -42,6 +42,9 @@ pytestmark = pytest.mark.gpu
     (768, 12, 3072, 10, 15),        # 160 rows: the last of them
     (768, 12, 3072, 7, 22),         # 161 rows: 32 x 64 tiles
     (768, 12, 3072, 20, 15),        # 320 rows: the last of them
+    (512, 8, 2048, 16, 11),         # 192 rows: four slices of three whole 64-row tiles
+    (512, 8, 2048, 16, 15),         # 256 rows: the last of them
+    (768, 12, 3072, 13, 9),         # 130 rows: 128-row tiles again at this width, the last of two rows
     (512, 8, 2048, 32, 15),         # 512 rows: the last four K slices of a tile at this width, the last row tile full
     (512, 8, 2048, 27, 18),         # 513 rows: two K slices, one row in the last tile
     (256, 4, 1152, 20, 14),         # 300 rows: two slices of nine K blocks, more than the ring holds
