@@ -33,6 +33,9 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm,
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
         ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
+// A tensor map's first use fetches it from memory.  The activations' map, which nothing uses ahead of the dependency wait, is asked for there (verify step
+// of 208 rows 200.5 -> 199.3 us, 416 rows 252 -> 250.7, 1664 rows 386.7 -> 384.6; encoders over 400 rows 386.7 -> 383.6).
+__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap* tm) { asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory"); }
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -502,6 +505,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             }
     }
     pdl_launch_dependents();
+    if (threadIdx.x == 0) tma_prefetch_map(&tmA);
     pdl_wait();                                        // activations, residual and outputs belong to the predecessors until here
     if (threadIdx.x == 0) tc_stamp(g.trace, 2);
 

@@ -85,6 +85,7 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             }
     }
     pdl_launch_dependents();
+    if (threadIdx.x == 0) tma_prefetch_map(&tmA);
     pdl_wait();
     if (warp == 0) {
         int s = 0; uint32_t par = 1;                           // (a fresh barrier counts as past the phase before its first)
