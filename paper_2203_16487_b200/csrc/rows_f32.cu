@@ -53,7 +53,16 @@ __global__ void __launch_bounds__(RF_THREADS) k_rows_f32(RowsF32Args a) {
         bt[i] = lane + 32 * i < K ? ldg_pinned(a.ln_b + lane + 32 * i) : 0.f;
     }
     if (EPI == EPI_QKV && tid < RF_BM) s_kv[tid] = tid < R ? (int)g.pg.row(g.seq[m0 + tid], g.pos[m0 + tid]) : 0;
+    // this thread's outputs: columns co + 16 i of row ro.  Their bias is a weight; fetched where it is added, it was a round trip at the end of every launch
+    constexpr int PO = BN / 16;
+    const int ro = tid >> 4, co = tid & 15;
+    float bz[PO];
+#pragma unroll
+    for (int i = 0; i < PO; ++i) bz[i] = EPI != EPI_STATS && g.bias && n0 + co + 16 * i < N ? ldg_pinned(g.bias + n0 + co + 16 * i) : 0.f;
     pdl_wait();
+    float ld = CUDART_INF_F;                           // EPI_STATS: the row's draft and its logit, requested with the rows
+    int id = -1;
+    if (EPI == EPI_STATS && ro < R) { if (g.ld) ld = g.ld[m0 + ro]; if (g.ld_id) id = g.ld_id[m0 + ro]; }
     if constexpr (LN > 0) {
         float x[2][LN], sum[2] = {0.f, 0.f}, mu[2], rs[2];
 #pragma unroll
@@ -100,10 +109,7 @@ __global__ void __launch_bounds__(RF_THREADS) k_rows_f32(RowsF32Args a) {
                 else *reinterpret_cast<float4*>(As + r * AP + c * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
             }
     }
-    // residual values of this thread's outputs: columns co + 16 i of row ro
-    constexpr int PO = BN / 16;
-    const int ro = tid >> 4, co = tid & 15;
-    float xo[PO];
+    float xo[PO];                                      // residual values
     if (EPI == EPI_RESID) {
 #pragma unroll
         for (int i = 0; i < PO; ++i) xo[i] = (ro < R && n0 + co + 16 * i < N) ? g.resid[(size_t)(m0 + ro) * N + n0 + co + 16 * i] : 0.f;
@@ -161,8 +167,6 @@ __global__ void __launch_bounds__(RF_THREADS) k_rows_f32(RowsF32Args a) {
     const int r = m0 + ro;
     if constexpr (EPI == EPI_STATS) {                  // the 16 threads of a row are half a warp
         const bool live = ro < R;
-        const float ld = (live && g.ld) ? g.ld[r] : CUDART_INF_F;
-        const int id = (live && g.ld_id) ? g.ld_id[r] : -1;
         RowPart p; p.mx = -CUDART_INF_F; p.arg = 0x7fffffff; p.sum = 0.f; p.cnt = 0;
 #pragma unroll
         for (int i = 0; i < PO; ++i) {
@@ -195,7 +199,7 @@ __global__ void __launch_bounds__(RF_THREADS) k_rows_f32(RowsF32Args a) {
         for (int i = 0; i < PO; ++i) {
             const int n = n0 + co + 16 * i;
             if (n >= N) continue;
-            float y = v[i] + (g.bias ? __ldg(g.bias + n) : 0.f);
+            float y = v[i] + bz[i];
             if (EPI == EPI_RESID) { g.resid[(size_t)r * N + n] = xo[i] + y; continue; }
             if (EPI == EPI_RELU) y = ffn_act(y, g.act);
             float* o = g.out + (size_t)r * g.ldo + n;
@@ -286,13 +290,22 @@ __global__ void __launch_bounds__(AF_WARPS * 32) k_attn_f32(AttnF32Args a) {
     for (int r = lane; r < nq; r += 32) nkmax = max(nkmax, min(a.nkeys[r0 + r], a.max_keys));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nkmax = max(nkmax, __shfl_xor_sync(0xffffffffu, nkmax, o));
+    // where this thread's first piece of the keys behind the wait lies: the page table predates the step, its round trip does not belong there
+    const int first = min(pre, nkmax), i0 = (first << sh) + tid;
+    const bool has = i0 < nkmax << sh;
+    const size_t off0 = has ? (PAGED ? a.pg.row(b, i0 >> sh) : (size_t)(kv0 + (i0 >> sh))) * a.kv_stride + h * dh + (i0 & (q4 - 1)) * 4 : 0;
     pdl_wait();
     for (int i = tid; i < nq << sh; i += AF_WARPS * 32) {
         const int r = i >> sh, c = (i & (q4 - 1)) * 4;
         const size_t qr = a.q_index ? (size_t)a.q_index[r0 + r] : (size_t)(r0 + r);
         cp_async16(smem_u32(Qs + r * dh + c), a.q + qr * a.q_stride + h * dh + c);
     }
-    load_keys(min(pre, nkmax), nkmax);
+    if (has) {
+        const uint32_t at = ((i0 >> sh) * KP + (i0 & (q4 - 1)) * 4) * 4;
+        cp_async16(smem_u32(Ks) + at, a.k + off0);
+        cp_async16(smem_u32(Vs) + at, a.v + off0);
+    }
+    load_keys(first + ((AF_WARPS * 32) >> sh), nkmax);  // (the others')
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     if (warp >= nq) return;
