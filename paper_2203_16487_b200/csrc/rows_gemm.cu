@@ -370,7 +370,6 @@ static cudaError_t rg_launch_resid(const RowsArgs& a, int rows_ub, int frag, boo
     if (frag) return frag == 16 ? rg_launch_one<EPI_RESID, 0, 1, 4, 1, 1, 6>(a, rows_ub, pdl, st) : rg_launch_one<EPI_RESID, 0, 2, 8, 2, 1, 12>(a, rows_ub, pdl, st);
     const int split = rg_split(a.g.N, a.g.K, rows_ub, cluster);
     if (rows_ub > rg_ln_rows(min(a.g.N, a.g.K))) {
-        if (split == 4 && a.g.K == 2048) return rg_launch_one<EPI_RESID, 0, 2, 8, 2, 4, 8>(a, rows_ub, pdl, st);       // (verify step of 156 rows 198 -> 195.5 us)
         if (split == 4) return rg_launch_one<EPI_RESID, 0, 2, 8, 2, 4>(a, rows_ub, pdl, st);
         return rg_launch_one<EPI_RESID, 0, 2, 8, 2, 1>(a, rows_ub, pdl, st);
     }
@@ -433,7 +432,7 @@ static void rg_room_nc(cudaError_t& e) { rg_room_out<EPI, 0>(e); rg_room_out<EPI
 cudaError_t rg_init() {
     cudaError_t e = cudaSuccess;
     rg_room_nc<EPI_STORE>(e); rg_room_nc<EPI_RELU>(e); rg_room_nc<EPI_GELU>(e); rg_room_nc<EPI_QKV>(e);
-    rg_room<EPI_RESID, 0, 1, 8, 2, 1, 8>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1, 8>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1, 12>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 4, 8>(e);
+    rg_room<EPI_RESID, 0, 1, 8, 2, 1, 8>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1, 8>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1, 12>(e);
     rg_room<EPI_RESID, 0, 2, 8, 2, 4>(e); rg_room<EPI_RESID, 0, 2, 8, 2, 1>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 2>(e);
     rg_room<EPI_RESID, 0, 1, 4, 1, 2, 4>(e); rg_room<EPI_RESID, 0, 1, 8, 2, 4, 8>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 2, 12>(e);
     rg_room<EPI_RESID, 0, 1, 4, 1, 1>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1, 2>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1, 4>(e); rg_room<EPI_RESID, 0, 1, 4, 1, 1, 6>(e);

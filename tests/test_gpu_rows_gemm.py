@@ -33,7 +33,8 @@ pytestmark = pytest.mark.gpu
     (128, 2, 192, 35, 10),          # 385 rows: tensor-core tiles
     (512, 8, 2048, 8, 11),          # 96 rows: the last output projections on 16 x 32 tiles
     (512, 8, 2048, 7, 13),          # 98 rows: 16 x 64 tiles, the last of them two rows
-    (512, 8, 2048, 11, 15),         # 176 rows: the last with the FFN2 here, its slices as fragments of 32 rows
+    (512, 8, 2048, 8, 15),          # 128 rows: the last with the FFN2 here
+    (512, 8, 2048, 10, 12),         # 130 rows: its split-K tiles
     (512, 8, 2048, 14, 16),         # 238 rows: QKV on 32-row tiles, the last of them 14 rows; 1 / 2 more rows of tiles than SMs
     (512, 8, 2048, 27, 15),         # 432 rows: the last output projections on 16-row tiles
     (512, 8, 2048, 31, 13),         # 434 rows: ... on 32-row tiles
