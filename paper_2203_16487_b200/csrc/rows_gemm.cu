@@ -24,11 +24,11 @@ struct RgCfg {
 
 // One CTA = 16 MT rows x 8 NT columns, K walked by the warps side by side (WN warps across the columns, 8 / WN K slices).
 //
-// Bound: latency.  A decoding step is a chain of 34 launches, 18 of them these, each over 0.5-2 MB of weights, so what counts is the
+// Bound: latency.  A decoding step of few rows is a chain of 39 launches, 24 of them these, each over 0.5-2 MB of weights, so what counts is the
 // time from the predecessor's last store to this kernel's.  Hence:
 //   * everything that does not depend on the predecessor -- the CTA's whole weight tile into shared memory, LayerNorm
 //     parameters, cache rows -- is requested before the dependency wait;
-//   * 256 threads of at most 80 registers (118 where a LayerNorm of 768 columns runs inside) and 20-100 KB of shared memory, so that the next two kernels of the chain are resident
+//   * 256 threads of at most 80 registers (118 where a LayerNorm of 768 columns runs inside; with fragments see below) and 20-100 KB of shared memory, so that the next two kernels of the chain are resident
 //     (their weights landed) while this one runs.  A 512-thread version with the weights in registers had shorter phases and a
 //     longer step (240 against 218 us), because its successors could not start early;
 //   * after the wait one round trip brings the rows; with NC > 0 they are normalised on the way (K = 128 NC, two rows per
@@ -39,8 +39,8 @@ struct RgCfg {
 //   * K is split over the warps (and, for long reductions, over a cluster of CS CTAs whose partial tiles meet in the owner's
 //     shared memory), the slices are added in a fixed order: results do not depend on timing.
 // Measured inside a verify step at 26 rows: 2.8 us for QKV and FFN1 with their LayerNorm (3.5 with the weights read from shared memory behind the
-// rows), 2.6 us for FFN2 (3.5); the step 145.1 -> 131, a greedy pass over 16 sequences 6262 -> 5680 us.  The fragments cost registers (up to 165 a
-// thread): beyond three row tiles with a LayerNorm inside too few of the successors' CTAs are resident (52 rows: 154 / 161 us a step), those keep the variant without.
+// rows), 2.6 us for FFN2 (3.5); the step 145.1 -> 131, a greedy pass over 16 sequences 6262 -> 5680 us.  The fragments cost registers (up to 158 a
+// thread, 768 columns 221): beyond three row tiles with a LayerNorm inside too few of the successors' CTAs are resident (52 rows: 154 / 161 us a step), those keep the variant without.
 template <int EPI, int NC, int MT, int NT, int WN, int CS, int ST>
 __global__ void __launch_bounds__(RG_THREADS, (NC > 0 && ST >= 8) || MT * ST > 16 ? 1 : NC > 4 || ST > 0 ? 2 : 3) k_rows(RowsArgs a) {
     using C = RgCfg<MT, NT, WN, CS>;

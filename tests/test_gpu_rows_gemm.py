@@ -35,7 +35,8 @@ pytestmark = pytest.mark.gpu
     (512, 8, 2048, 7, 13),          # 98 rows: 16 x 64 tiles, the last of them two rows
     (512, 8, 2048, 8, 15),          # 128 rows: the last with the FFN2 here
     (512, 8, 2048, 10, 12),         # 130 rows: its split-K tiles
-    (512, 8, 2048, 14, 16),         # 238 rows: QKV on 32-row tiles, the last of them 14 rows; 1 / 2 more rows of tiles than SMs
+    (512, 8, 2048, 14, 15),         # 224 rows: the last QKV projections on 32-row tiles
+    (512, 8, 2048, 14, 16),         # 238 rows: QKV on tensor-core tiles again, output projections on 16-row tiles, the last of them 14 rows
     (512, 8, 2048, 27, 15),         # 432 rows: the last output projections on 16-row tiles
     (512, 8, 2048, 31, 13),         # 434 rows: ... on 32-row tiles
     (512, 8, 2048, 46, 15),         # 736 rows: the last on 32-row tiles
