@@ -628,7 +628,7 @@ struct TmaEncoder {
     PFN_encodeTiled encode = nullptr;
     int* err_word = nullptr;            // device word the kernels raise on a wait timeout
     int n_sm = 148;
-    int spk_clusters4 = 0, spk_clusters4_64 = 0, spk_clusters2 = 0;   // split-K clusters that run at once
+    int spk_clusters4 = 0, spk_clusters4_64 = 0, spk_clusters2 = 0, spk_clusters2_128 = 0;   // split-K clusters that run at once
     int force_bn = 0;                   // experiments: 0 = choose, else 32 / 64 / 128 / 256
     bool pdl = true;                    // launch with programmatic stream serialization
     std::map<std::tuple<const void*, long long, int, int, int>, CUtensorMap> cache;

@@ -1,6 +1,6 @@
 // Residual GEMM over a few 128-row tiles with a long reduction (FFN2: K = 4 d), split along K inside a cluster:
 //     resid[r, n] += x[r, :] . W[n, :] + bias[n],   x bf16 [R, K], W bf16 [N, K], resid fp32 [R, N],
-// for row counts whose tiles x N / 64 x SPLIT CTAs still fit one wave.
+// for row counts whose tiles x N / 64 (or N / 128) x SPLIT CTAs still fit one wave.
 //
 // Bound by the serial walk over K: with 64-wide column tiles there are N / 64 CTAs per row tile (8 for d = 512), and 32 k-blocks at 0.2 us are two thirds
 // of the launch (9.4 us).  Here SPLIT CTAs of a cluster take a K slice of one tile each and then an equal share of its rows: every epilogue warp copies its
@@ -13,15 +13,14 @@
 
 namespace sd {
 
-constexpr int SPK_BN = 64;
 // AR = rows of a tile.  Of a 64-row box the MMA reads 64 rows more, which are the stage's weights, into accumulator lanes that nobody reads.
-template <int AR> struct SpkCfg {
-    static constexpr int STAGES = AR == 128 ? 7 : 8;           // ring depth: the receive buffer takes the rest of shared memory
-    static constexpr int A_KB = AR * TC_BK * 2, STAGE = A_KB + SPK_BN * TC_BK * 2;
-    static constexpr int RECV = AR * SPK_BN * 4;               // SPLIT slices of AR / SPLIT rows
+template <int AR, int BN> struct SpkCfg {
+    static constexpr int STAGES = BN == 128 ? 5 : AR == 128 ? 7 : 8;           // ring depth: the receive buffer takes the rest of shared memory
+    static constexpr int A_KB = AR * TC_BK * 2, STAGE = A_KB + BN * TC_BK * 2;
+    static constexpr int RECV = AR * BN * 4;               // SPLIT slices of AR / SPLIT rows
     static constexpr int SMEM = STAGES * STAGE + RECV + 1024;
-    static_assert(STAGES * STAGE >= TC_EPI_WARPS * 4096, "the outgoing blocks reuse the ring");
-    static_assert(AR == 128 || AR + SPK_BN >= 128, "the 128-row MMA read stays inside the stage");
+    static_assert(STAGES * STAGE >= TC_EPI_WARPS * (BN / 64) * 4096, "the outgoing blocks reuse the ring");
+    static_assert(AR == 128 || AR + BN >= 128, "the 128-row MMA read stays inside the stage");
 };
 
 // CTAs per tile: 4 while all clusters run at once, else 2, else none (0).  Shorter reductions gain less than the exchange costs (verify step, us, unsplit / split:
@@ -30,19 +29,25 @@ template <int AR> struct SpkCfg {
 // step of 312 rows at 768 columns where clusters of 2 take 361.)
 // 64-row tiles while their clusters run at once, too: half of the activations to fetch behind the wait (182 rows 197 -> 194.5, 234 rows 208.8 -> 204.5, 104 rows at 768 columns
 // 258 -> 250), unless another stream's kernels share the SMs (two encoders over 144 rows 307 -> 315).
-struct SpkPlan { int split, rows; };
+// Where two slices of 64-column tiles are more clusters than run at once, two of 128 columns, up to twice the rows: unsplit these are at most 72 CTAs that walk the whole K
+// (verify step of 1248 rows, us, unsplit / split: 354.4 / 348.2, 1408 rows 387 / 379, 1664 rows 385 / 379, 2048 rows 426 / 420; drafts over 2160 rows 137.4 / 134.5).  Beside
+// another stream's kernels (encoders) the unsplit ones stay.
+struct SpkPlan { int split, rows, cols; };
 inline SpkPlan spk_plan(const TmaEncoder& enc, int N, int K, int rows_ub, bool shared) {
-    if (N % SPK_BN || K < 768) return {0, 0};
-    const long long n = N / SPK_BN, tiles = (rows_ub + TC_BM - 1) / TC_BM * n;
-    if (K % (4 * TC_BK) == 0 && !shared && (rows_ub + 63) / 64 * n <= enc.spk_clusters4_64) return {4, 64};
-    if (K % (4 * TC_BK) == 0 && tiles <= enc.spk_clusters4) return {4, TC_BM};
-    return {K % (2 * TC_BK) == 0 && K >= 1024 && tiles <= enc.spk_clusters2 ? 2 : 0, TC_BM};
+    if (N % 64 || K < 768) return {0, 0, 0};
+    const long long n = N / 64, m = (rows_ub + TC_BM - 1) / TC_BM;
+    if (K % (4 * TC_BK) == 0 && !shared && (rows_ub + 63) / 64 * n <= enc.spk_clusters4_64) return {4, 64, 64};
+    if (K % (4 * TC_BK) == 0 && m * n <= enc.spk_clusters4) return {4, TC_BM, 64};
+    if (K % (2 * TC_BK) || K < 1024) return {0, 0, 0};
+    if (m * n <= enc.spk_clusters2) return {2, TC_BM, 64};
+    return {!shared && N % 128 == 0 && m * (N / 128) <= enc.spk_clusters2_128 ? 2 : 0, TC_BM, 128};
 }
 
-template <int SPLIT, int AR>
+template <int SPLIT, int AR, int BN>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, GemmArgs<bf16> g, int* err_word) {
-    using C = SpkCfg<AR>;
+    using C = SpkCfg<AR, BN>;
+    constexpr int NB = BN / 64;                                // 64-column blocks, one after the other in the outgoing and the receive buffer
     constexpr int SPK_STAGES = C::STAGES, SPK_A_KB = C::A_KB, SPK_STAGE = C::STAGE, SPK_RECV = C::RECV;
     constexpr int OWN = AR / SPLIT, RB = OWN < 32 ? OWN : 32;  // rows that a CTA finishes; rows that a warp sends to one owner
     static_assert(OWN % 16 == 0, "rows of 16 threads");
@@ -58,7 +63,7 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     uint32_t rank;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    const int n0 = (int)(blockIdx.x / SPLIT) * SPK_BN, kb0 = (int)rank * nkb;
+    const int n0 = (int)(blockIdx.x / SPLIT) * BN, kb0 = (int)rank * nkb;
 
     if (threadIdx.x == 0) {
         abort_s = 0;
@@ -69,7 +74,7 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_expect_tx(smem_u32(&bar_part), SPK_RECV);
     }
-    if (warp == 1) tmem_alloc(smem_u32(&tmem_base_s), 64);
+    if (warp == 1) tmem_alloc(smem_u32(&tmem_base_s), BN);
     tc_fence_before();
     tc_cluster_sync();                                         // every CTA's barriers exist before anybody sends
     tc_fence_after();
@@ -102,7 +107,7 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if (++s == SPK_STAGES) { s = 0; par ^= 1u; }
         }
     } else if (warp == 1) {
-        constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, SPK_BN);
+        constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, BN);
         int s = 0; uint32_t par = 0; bool ok = true;
         for (int kb = 0; kb < nkb; ++kb) {
             ok = mbar_wait_warp(full0 + 8 * s, par, abort_flag, err_word, 2);
@@ -122,64 +127,73 @@ k_gemm_tc_splitk(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (ok && elect_one()) umma_commit(smem_u32(&bar_acc));
     } else {
         const int q = warp & 3, half = (warp - 2) >> 2, e = (int)threadIdx.x - 64;
-        // the residual and bias of the outputs that this thread will finish: rows e / 16 + 16 i of the CTA's share, four columns
+        // the residual and bias of the outputs that this thread will finish: rows e / 16 + 16 i of the CTA's share, four columns of each block
         const int c = (e & 15) * 4, row0 = m0 + (int)rank * OWN + (e >> 4);
-        float4 x[OWN / 16], bz = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (g.bias) bz = __ldg(reinterpret_cast<const float4*>(g.bias + n0 + c));
+        float4 x[NB][OWN / 16], bz[NB];
 #pragma unroll
-        for (int i = 0; i < OWN / 16; ++i)
-            x[i] = row0 + 16 * i < R ? *reinterpret_cast<const float4*>(g.resid + (size_t)(row0 + 16 * i) * g.N + n0 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int n = 0; n < NB; ++n) {
+            bz[n] = g.bias ? __ldg(reinterpret_cast<const float4*>(g.bias + n0 + n * 64 + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < OWN / 16; ++i)
+                x[n][i] = row0 + 16 * i < R ? *reinterpret_cast<const float4*>(g.resid + (size_t)(row0 + 16 * i) * g.N + n0 + n * 64 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
         bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_acc), 0, abort_flag, err_word, 3));      // the MMAs are done: the ring is free
         tc_fence_after();
         if (ok && q * 32 < AR) {
-            float v[32];
-            tmem_ld32(tmem_d + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32), v);
-            // a row per lane, its 16-byte chunks XOR-swizzled by the row
-            uint8_t* blk = ring_p + (warp - 2) * 4096;
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                *reinterpret_cast<float4*>(blk + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane < 32 / RB) {
-                const uint32_t row = q * 32 + lane * RB, owner = row / OWN, dst = recv + ((rank * (OWN / RB) + row % OWN / RB) * 2 + half) * (RB * 128);
-                uint32_t ra, rb;
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(dst), "r"(owner));
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_u32(&bar_part)), "r"(owner));
-                asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             ::"r"(ra), "r"(ring + (warp - 2) * 4096 + lane * (RB * 128)), "r"(RB * 128), "r"(rb) : "memory");
+            for (int n = 0; n < NB; ++n) {
+                float v[32];
+                tmem_ld32(tmem_d + ((uint32_t)(q * 32) << 16) + (uint32_t)(n * 64 + half * 32), v);
+                // a row per lane, its 16-byte chunks XOR-swizzled by the row
+                const int out = (n * TC_EPI_WARPS + warp - 2) * 4096;
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    *reinterpret_cast<float4*>(ring_p + out + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane < 32 / RB) {
+                    const uint32_t row = q * 32 + lane * RB, owner = row / OWN,
+                                   dst = recv + n * (AR * 256) + ((rank * (OWN / RB) + row % OWN / RB) * 2 + half) * (RB * 128);
+                    uint32_t ra, rb;
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(dst), "r"(owner));
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_u32(&bar_part)), "r"(owner));
+                    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(ra), "r"(ring + out + lane * (RB * 128)), "r"(RB * 128), "r"(rb) : "memory");
+                }
+                __syncwarp();
             }
-            __syncwarp();
         }
         ok = ok && mbar_wait(smem_u32(&bar_part), 0, abort_flag, err_word, 10);          // all slices of this CTA's rows have landed
         if (ok) {
             const uint8_t* src = ring_p + SPK_STAGES * SPK_STAGE + ((e & 15) >> 3) * (RB * 128);
 #pragma unroll
-            for (int i = 0; i < OWN / 16; ++i) {
-                const int row = (e >> 4) + 16 * i;
-                const uint8_t* p = src + row / RB * (RB * 256) + row % RB * 128 + (((e & 7) ^ (row & 7)) << 4);
-                float4 a = *reinterpret_cast<const float4*>(p);
+            for (int n = 0; n < NB; ++n)
 #pragma unroll
-                for (int s = 1; s < SPLIT; ++s) {                                        // rank order: fixed summation order
-                    const float4 t = *reinterpret_cast<const float4*>(p + s * (OWN * 256));
-                    a.x += t.x; a.y += t.y; a.z += t.z; a.w += t.w;
+                for (int i = 0; i < OWN / 16; ++i) {
+                    const int row = (e >> 4) + 16 * i;
+                    const uint8_t* p = src + n * (AR * 256) + row / RB * (RB * 256) + row % RB * 128 + (((e & 7) ^ (row & 7)) << 4);
+                    float4 a = *reinterpret_cast<const float4*>(p);
+#pragma unroll
+                    for (int s = 1; s < SPLIT; ++s) {                                    // rank order: fixed summation order
+                        const float4 t = *reinterpret_cast<const float4*>(p + s * (OWN * 256));
+                        a.x += t.x; a.y += t.y; a.z += t.z; a.w += t.w;
+                    }
+                    a.x += bz[n].x; a.y += bz[n].y; a.z += bz[n].z; a.w += bz[n].w;
+                    a.x += x[n][i].x; a.y += x[n][i].y; a.z += x[n][i].z; a.w += x[n][i].w;
+                    if (row0 + 16 * i < R) *reinterpret_cast<float4*>(g.resid + (size_t)(row0 + 16 * i) * g.N + n0 + n * 64 + c) = a;
                 }
-                a.x += bz.x; a.y += bz.y; a.z += bz.z; a.w += bz.w;
-                a.x += x[i].x; a.y += x[i].y; a.z += x[i].z; a.w += x[i].w;
-                if (row0 + 16 * i < R) *reinterpret_cast<float4*>(g.resid + (size_t)(row0 + 16 * i) * g.N + n0 + c) = a;
-            }
         }
     }
     tc_fence_before();
     __syncwarp();
     tc_cluster_sync();                                         // nobody leaves while a copy from its shared memory may be under way
-    if (warp == 1) tmem_dealloc(tmem_d, 64);
+    if (warp == 1) tmem_dealloc(tmem_d, BN);
 }
 
-template <int SPLIT, int AR>
+template <int SPLIT, int AR, int BN>
 inline cudaLaunchConfig_t spk_config(cudaLaunchAttribute* attr, dim3 grid, bool pdl, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = SpkCfg<AR>::SMEM; cfg.stream = st;
+    cfg.gridDim = grid; cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = SpkCfg<AR, BN>::SMEM; cfg.stream = st;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = SPLIT; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -187,36 +201,38 @@ inline cudaLaunchConfig_t spk_config(cudaLaunchAttribute* attr, dim3 grid, bool 
     cfg.attrs = attr; cfg.numAttrs = pdl ? 2 : 1;
     return cfg;
 }
-template <int SPLIT, int AR>
+template <int SPLIT, int AR, int BN>
 inline cudaError_t spk_init_one(int* clusters) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_tc_splitk<SPLIT, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, SpkCfg<AR>::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_gemm_tc_splitk<SPLIT, AR, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SpkCfg<AR, BN>::SMEM);
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = spk_config<SPLIT, AR>(attr, dim3(SPLIT), false, nullptr);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(clusters, k_gemm_tc_splitk<SPLIT, AR>, &cfg);
+    const cudaLaunchConfig_t cfg = spk_config<SPLIT, AR, BN>(attr, dim3(SPLIT), false, nullptr);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(clusters, k_gemm_tc_splitk<SPLIT, AR, BN>, &cfg);
     return e;
 }
 inline cudaError_t spk_init(TmaEncoder& enc) {
-    cudaError_t e = spk_init_one<4, TC_BM>(&enc.spk_clusters4);
-    if (e == cudaSuccess) e = spk_init_one<4, 64>(&enc.spk_clusters4_64);
-    return e == cudaSuccess ? spk_init_one<2, TC_BM>(&enc.spk_clusters2) : e;
+    cudaError_t e = spk_init_one<4, TC_BM, 64>(&enc.spk_clusters4);
+    if (e == cudaSuccess) e = spk_init_one<4, 64, 64>(&enc.spk_clusters4_64);
+    if (e == cudaSuccess) e = spk_init_one<2, TC_BM, 64>(&enc.spk_clusters2);
+    return e == cudaSuccess ? spk_init_one<2, TC_BM, 128>(&enc.spk_clusters2_128) : e;
 }
 
-template <int SPLIT, int AR>
+template <int SPLIT, int AR, int BN>
 inline int spk_launch_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
     const CUtensorMap* ta = enc.get(g.A, rows_ub, g.K, g.lda, AR);
-    const CUtensorMap* tw = enc.get(g.W, g.N, g.K, g.K, SPK_BN);
+    const CUtensorMap* tw = enc.get(g.W, g.N, g.K, g.K, BN);
     if (!ta || !tw) return -1;
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = spk_config<SPLIT, AR>(attr, dim3(g.N / SPK_BN * SPLIT, (rows_ub + AR - 1) / AR), enc.pdl, st);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc_splitk<SPLIT, AR>, *ta, *tw, g, enc.err_word);
+    const cudaLaunchConfig_t cfg = spk_config<SPLIT, AR, BN>(attr, dim3(g.N / BN * SPLIT, (rows_ub + AR - 1) / AR), enc.pdl, st);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc_splitk<SPLIT, AR, BN>, *ta, *tw, g, enc.err_word);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { enc.err = std::string("launch (split-K): ") + cudaGetErrorString(e); return -1; }
     return 0;
 }
 inline int spk_launch(TmaEncoder& enc, SpkPlan plan, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
     if (!enc.ready) return -1;
-    if (plan.rows == 64) return spk_launch_one<4, 64>(enc, g, rows_ub, st);
-    return plan.split == 4 ? spk_launch_one<4, TC_BM>(enc, g, rows_ub, st) : spk_launch_one<2, TC_BM>(enc, g, rows_ub, st);
+    if (plan.rows == 64) return spk_launch_one<4, 64, 64>(enc, g, rows_ub, st);
+    if (plan.cols == 128) return spk_launch_one<2, TC_BM, 128>(enc, g, rows_ub, st);
+    return plan.split == 4 ? spk_launch_one<4, TC_BM, 64>(enc, g, rows_ub, st) : spk_launch_one<2, TC_BM, 64>(enc, g, rows_ub, st);
 }
 
 }  // namespace sd

@@ -547,7 +547,7 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
                 ++h->launches;
                 return 0;
             }
-            const sd::SpkPlan plan = epi == EPI_RESID && h->use_splitk && h->splitk_ready ? sd::spk_plan(h->tma, N, K, rows_ub, cnt == CNT_ENC) : sd::SpkPlan{0, 0};
+            const sd::SpkPlan plan = epi == EPI_RESID && h->use_splitk && h->splitk_ready ? sd::spk_plan(h->tma, N, K, rows_ub, cnt == CNT_ENC) : sd::SpkPlan{0, 0, 0};
             if (plan.split) {
                 if (sd::spk_launch(h->tma, plan, g, rows_ub, st) != 0)
                     return fail(h, SPECDEC_ERR_CUDA, "tensor-core GEMM launch failed: " + h->tma.err);

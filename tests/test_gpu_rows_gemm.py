@@ -49,6 +49,9 @@ pytestmark = pytest.mark.gpu
     (768, 12, 3072, 13, 9),         # 130 rows: 128-row tiles again at this width, the last of two rows
     (512, 8, 2048, 32, 15),         # 512 rows: the last four K slices of a tile at this width, the last row tile full
     (512, 8, 2048, 27, 18),         # 513 rows: two K slices, one row in the last tile
+    (512, 8, 2048, 61, 18),         # 1159 rows: two K slices of 128-column tiles, seven rows in the last of them
+    (512, 8, 2048, 96, 23),         # 2304 rows: the last of them, every tile full
+    (768, 12, 3072, 40, 21),        # 880 rows: at this width
     (256, 4, 1152, 20, 14),         # 300 rows: two slices of nine K blocks, more than the ring holds
 ])
 def test_rows_gemm_edges(d, H, f, B, k):
