@@ -507,6 +507,7 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
             // this warp's eight columns of the 16 rows, 256 bytes in place of the queries, go to every CTA of the cluster as one copy
             *reinterpret_cast<uint2*>(sm + kg * 256 + lane * 8) = make_uint2(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1));
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();                            // all 32 lanes' bytes are there before a lane copies them (the cluster barrier below was arrived at long before)
             cluster_wait();                          // every CTA of the cluster has begun and its barrier exists
             if (lane < ON) {
                 uint32_t ra, rb;
