@@ -633,12 +633,12 @@ struct TmaEncoder {
     bool pdl = true;                    // launch with programmatic stream serialization
     std::map<std::tuple<const void*, long long, int, int, int>, CUtensorMap> cache;
 
-    // 2-D bf16 tensor [rows, K] with row pitch ld elements; box = 64 x box_rows, 128-byte swizzle.
-    const CUtensorMap* get(const void* base, long long rows, int K, int ld, int box_rows) {
+    // 2-D bf16 tensor [rows, K] with row pitch ld elements; box = 64 x box_rows, 128-byte swizzle.  By value: a launch holds two maps, and the second
+    // may be the one for which the cache is emptied.
+    bool get(CUtensorMap& tm, const void* base, long long rows, int K, int ld, int box_rows) {
         auto key = std::make_tuple(base, rows, K, ld, box_rows);
         auto it = cache.find(key);
-        if (it != cache.end()) return &it->second;
-        CUtensorMap tm;
+        if (it != cache.end()) { tm = it->second; return true; }
         cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
         cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
         cuuint32_t box[2] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows};
@@ -646,9 +646,10 @@ struct TmaEncoder {
         CUresult rc = encode(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (rc != CUDA_SUCCESS) { err = "cuTensorMapEncodeTiled failed with code " + std::to_string((int)rc); return nullptr; }
+        if (rc != CUDA_SUCCESS) { err = "cuTensorMapEncodeTiled failed with code " + std::to_string((int)rc); return false; }
         if (cache.size() > 4096) cache.clear();
-        return &(cache[key] = tm);
+        cache[key] = tm;
+        return true;
     }
 };
 
@@ -703,9 +704,8 @@ inline int tc_init(TmaEncoder& enc, int* err_word) {
 
 template <int EPI, int BN, int AR = 128>
 inline int tc_launch_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
-    const CUtensorMap* ta = enc.get(g.A, rows_ub, g.K, g.lda, AR);
-    const CUtensorMap* tw = enc.get(g.W, g.N, g.K, g.K, BN);
-    if (!ta || !tw) return -1;
+    CUtensorMap ta, tw;
+    if (!enc.get(ta, g.A, rows_ub, g.K, g.lda, AR) || !enc.get(tw, g.W, g.N, g.K, g.K, BN)) return -1;
     const long long tiles_ub = (long long)((g.N + BN - 1) / BN) * ((rows_ub + TC_BM - 1) / TC_BM);
     const int grid = (int)std::min<long long>(tiles_ub, enc.n_sm);
     cudaLaunchConfig_t cfg = {};
@@ -714,7 +714,7 @@ inline int tc_launch_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cudaSt
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = enc.pdl ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc<EPI, BN, AR>, *ta, *tw, g, enc.err_word);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc<EPI, BN, AR>, ta, tw, g, enc.err_word);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { enc.err = std::string("launch: ") + cudaGetErrorString(e); return -1; }
     return 0;
@@ -724,9 +724,8 @@ inline int tc_launch_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cudaSt
 inline bool tc_ln_fusable(int N, int K) { return N % 128 == 0 && N <= 1024 && K % TC_BK == 0 && K >= TC_BK; }
 template <int BN>
 inline int tc_launch_ln_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
-    const CUtensorMap* ta = enc.get(g.A, rows_ub, g.K, g.lda, TC_BM);
-    const CUtensorMap* tw = enc.get(g.W, g.N, g.K, g.K, BN);
-    if (!ta || !tw) return -1;
+    CUtensorMap ta, tw;
+    if (!enc.get(ta, g.A, rows_ub, g.K, g.lda, TC_BM) || !enc.get(tw, g.W, g.N, g.K, g.K, BN)) return -1;
     const int n_tiles = g.N / BN, m_tiles = (rows_ub + TC_BM - 1) / TC_BM;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_tiles * m_tiles); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = TcCfg<BN, 128, true, true>::SMEM; cfg.stream = st;
@@ -736,7 +735,7 @@ inline int tc_launch_ln_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cud
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = enc.pdl ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc<EPI_RESID, BN, 128, true>, *ta, *tw, g, enc.err_word);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc<EPI_RESID, BN, 128, true>, ta, tw, g, enc.err_word);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { enc.err = std::string("launch (fused LayerNorm): ") + cudaGetErrorString(e); return -1; }
     return 0;

@@ -395,9 +395,8 @@ inline bool tc_pair_wanted(int epi, int N, int K, int rows_ub) {
 
 template <int EPI, int BN>
 inline int tc_pair_launch_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
-    const CUtensorMap* ta = enc.get(g.A, rows_ub, g.K, g.lda, TC_BM);
-    const CUtensorMap* tw = enc.get(g.W, g.N, g.K, g.K, BN / 2);
-    if (!ta || !tw) return -1;
+    CUtensorMap ta, tw;
+    if (!enc.get(ta, g.A, rows_ub, g.K, g.lda, TC_BM) || !enc.get(tw, g.W, g.N, g.K, g.K, BN / 2)) return -1;
     const long long tiles_ub = (long long)((g.N + BN - 1) / BN) * ((rows_ub + 2 * TC_BM - 1) / (2 * TC_BM));
     const int grid = 2 * (int)std::min<long long>(tiles_ub, enc.n_sm / 2);
     cudaLaunchConfig_t cfg = {};
@@ -407,16 +406,15 @@ inline int tc_pair_launch_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, c
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = enc.pdl ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc_pair<EPI, BN>, *ta, *tw, g, enc.err_word);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc_pair<EPI, BN>, ta, tw, g, enc.err_word);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { enc.err = std::string("pair launch: ") + cudaGetErrorString(e); return -1; }
     return 0;
 }
 
 inline int vocab_pair_launch(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
-    const CUtensorMap* ta = enc.get(g.A, rows_ub, g.K, g.lda, TC_BM);
-    const CUtensorMap* tw = enc.get(g.W, g.N, g.K, g.K, VP_BNH);
-    if (!ta || !tw) return -1;
+    CUtensorMap ta, tw;
+    if (!enc.get(ta, g.A, rows_ub, g.K, g.lda, TC_BM) || !enc.get(tw, g.W, g.N, g.K, g.K, VP_BNH)) return -1;
     const long long tiles_ub = (long long)((g.N + VP_BN - 1) / VP_BN) * ((rows_ub + 2 * TC_BM - 1) / (2 * TC_BM));
     const int grid = 2 * (int)std::min<long long>(tiles_ub, enc.n_sm / 2);
     cudaLaunchConfig_t cfg = {};
@@ -425,7 +423,7 @@ inline int vocab_pair_launch(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cu
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = enc.pdl ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_vocab_pair, *ta, *tw, g, enc.err_word, vp_stages(g.K));
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_vocab_pair, ta, tw, g, enc.err_word, vp_stages(g.K));
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { enc.err = std::string("vocabulary pair launch: ") + cudaGetErrorString(e); return -1; }
     return 0;

@@ -218,12 +218,11 @@ inline cudaError_t spk_init(TmaEncoder& enc) {
 
 template <int SPLIT, int AR, int BN>
 inline int spk_launch_one(TmaEncoder& enc, GemmArgs<bf16>& g, int rows_ub, cudaStream_t st) {
-    const CUtensorMap* ta = enc.get(g.A, rows_ub, g.K, g.lda, AR);
-    const CUtensorMap* tw = enc.get(g.W, g.N, g.K, g.K, BN);
-    if (!ta || !tw) return -1;
+    CUtensorMap ta, tw;
+    if (!enc.get(ta, g.A, rows_ub, g.K, g.lda, AR) || !enc.get(tw, g.W, g.N, g.K, g.K, BN)) return -1;
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = spk_config<SPLIT, AR, BN>(attr, dim3(g.N / BN * SPLIT, (rows_ub + AR - 1) / AR), enc.pdl, st);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc_splitk<SPLIT, AR, BN>, *ta, *tw, g, enc.err_word);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc_splitk<SPLIT, AR, BN>, ta, tw, g, enc.err_word);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { enc.err = std::string("launch (split-K): ") + cudaGetErrorString(e); return -1; }
     return 0;

@@ -293,8 +293,8 @@ inline cudaError_t vr_init() {
     return e != cudaSuccess ? e : cudaFuncSetAttribute(k_vocab_rows<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, VrCfg<32>::SMEM);
 }
 inline int vr_launch(TmaEncoder& enc, const VocabRowsArgs& a, int rows_ub, cudaStream_t st) {
-    const CUtensorMap* tw = enc.get(a.E, a.N, VR_K, VR_K, VR_BN);
-    if (!tw) return -1;
+    CUtensorMap tw;
+    if (!enc.get(tw, a.E, a.N, VR_K, VR_K, VR_BN)) return -1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((a.N + VR_BN - 1) / VR_BN); cfg.blockDim = dim3(TC_THREADS); cfg.stream = st;
     cfg.dynamicSmemBytes = rows_ub <= 16 ? VrCfg<16>::SMEM : VrCfg<32>::SMEM;
@@ -302,7 +302,7 @@ inline int vr_launch(TmaEncoder& enc, const VocabRowsArgs& a, int rows_ub, cudaS
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = enc.pdl ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, rows_ub <= 16 ? k_vocab_rows<16> : k_vocab_rows<32>, *tw, a, enc.err_word);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, rows_ub <= 16 ? k_vocab_rows<16> : k_vocab_rows<32>, tw, a, enc.err_word);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { enc.err = std::string("launch (vocabulary projection of few rows): ") + cudaGetErrorString(e); return -1; }
     return 0;

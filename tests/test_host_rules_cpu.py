@@ -1,0 +1,65 @@
+"""Host-side rules of the launchers that no launch on one device can reach, compiled from the headers into a small program (no device call is made)."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2203_16487_b200 import build
+
+PROGRAM = r"""
+#include <algorithm>
+#include <cstdio>
+#include <cstring>
+#include <map>
+#include <string>
+#include <tuple>
+#include "vocab_rows.cuh"
+
+// a map that carries its base address: what encoding leaves in it is this test's own
+static CUresult fake_encode(CUtensorMap* m, CUtensorMapDataType, cuuint32_t, void* base, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
+                            CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill) {
+    memset(m, 0, sizeof *m);
+    memcpy(m, &base, sizeof base);
+    return CUDA_SUCCESS;
+}
+static bool is_of(const CUtensorMap& m, const void* base) { return !memcmp(&m, &base, sizeof base); }
+
+// A launch's two maps, asked for while the cache is at its limit: both are what was asked for.
+static int maps_of_one_launch() {
+    sd::TmaEncoder enc;
+    enc.encode = fake_encode;
+    int wrong = 0;
+    for (long long i = 1; i < 20000; ++i) {
+        CUtensorMap a, w;
+        const void *pa = (const void*)(i << 20), *pw = (const void*)((i << 20) + 4096);
+        wrong += !enc.get(a, pa, i, 512, 512, 128) || !enc.get(w, pw, 512, 512, 512, 64) || !is_of(a, pa) || !is_of(w, pw);
+        CUtensorMap again;                               // ... from the cache, or encoded once more
+        wrong += !enc.get(again, pa, i, 512, 512, 128) || !is_of(again, pa);
+        if (enc.cache.size() > 5000) ++wrong;
+    }
+    return wrong;
+}
+
+int main() {
+    printf("maps_of_one_launch %d\n", maps_of_one_launch());
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def wrong(tmp_path_factory):
+    d = tmp_path_factory.mktemp("host_rules")
+    src, exe = d / "rules.cu", d / "rules"
+    src.write_text(PROGRAM)
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    r = subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=compute_100a", "-std=c++17", "-I", build.CSRC, "-o", str(exe), str(src)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    env = dict(os.environ, MALLOC_PERTURB_="165")        # what is freed does not keep its contents
+    out = subprocess.run([str(exe)], capture_output=True, text=True, check=True, timeout=60, env=env).stdout
+    return dict((name, int(n)) for name, n in (line.split() for line in out.splitlines()))
+
+
+def test_the_maps_of_a_launch_survive_the_eviction_between_them(wrong):
+    assert wrong["maps_of_one_launch"] == 0
