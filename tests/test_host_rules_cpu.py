@@ -56,7 +56,7 @@ def wrong(tmp_path_factory):
     r = subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=compute_100a", "-std=c++17", "-I", build.CSRC, "-o", str(exe), str(src)],
                        capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
-    env = dict(os.environ, MALLOC_PERTURB_="165")        # what is freed does not keep its contents
+    env = dict(os.environ, MALLOC_PERTURB_="165", GLIBC_TUNABLES="glibc.malloc.tcache_count=0")        # what is freed does not keep its contents
     out = subprocess.run([str(exe)], capture_output=True, text=True, check=True, timeout=60, env=env).stdout
     return dict((name, int(n)) for name, n in (line.split() for line in out.splitlines()))
 
