@@ -853,7 +853,7 @@ bool vocab_rows_inside(const specdec_handle* h, const ModelW& m, int rows_ub) {
 }
 int vocab_rows(specdec_handle* h, const ModelW& m, const float* x, int cnt, int rows_ub, const int* draft, int k, int* n_tiles, cudaStream_t st) {
     VocabRowsArgs a{x, m.dec_lnf_g, m.dec_lnf_b, 1e-5f, (const bf16*)m.embed, m.dm.vocab, h->ses.counters + cnt, static_rows(h, cnt, rows_ub),
-                    draft, h->rows.slot_seq, k, h->ld, h->ld_id, (bf16*)h->y, h->part, h->want_lse};
+                    draft, h->rows.slot_seq, k, cnt == CNT_VERIFY ? h->ld : nullptr, cnt == CNT_VERIFY ? h->ld_id : nullptr, (bf16*)h->y, h->part, h->want_lse};
     *n_tiles = cdiv(m.dm.vocab, VR_BN);
     for (int i = 0; i < (h->diag_repeat & 8 ? 2 : 1); ++i) {
         if (vr_launch(h->tma, a, rows_ub, st) != 0) return fail(h, SPECDEC_ERR_CUDA, "tensor-core GEMM launch failed: " + h->tma.err);

@@ -29,8 +29,8 @@ struct VocabRowsArgs {
     const float* x; const float* ln_g; const float* ln_b; float eps;
     const bf16* E; int N;
     const int* n_rows; int rows_static;
-    const int* draft; const int* slot_seq; int k;                      // verify: row slot (k + 1) + c checks draft c of the slot's sequence; draft null: no drafts
-    float* ld; int* ld_id;                                             // ... and its logit and id go here
+    const int* draft; const int* slot_seq; int k;                      // verify: row slot (k + 1) + c checks draft c of the slot's sequence; draft null (or k = 0): no drafts
+    float* ld; int* ld_id;                                             // the logit and id of every row's draft (+inf, -1: none) go here; null: the drafter's pass
     bf16* y;                                                           // the normalised rows, for whoever replays the projection
     RowPart* part;                                                     // [rows, tiles]
     int want_sum;                                                      // also accumulate sum exp(l - max)
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_vocab_rows(const __grid_const
                 const float l = !checks ? CUDART_INF_F : ok ? dot[i] : -CUDART_INF_F;
                 const int id = !checks ? -1 : ok ? tok[i] : -2;
                 s_ld[r] = l; s_id[r] = id;
-                if (a.draft && r == (int)blockIdx.x && r < R) { a.ld[r] = l; a.ld_id[r] = id; }
+                if (a.ld && r == (int)blockIdx.x && r < R) { a.ld[r] = l; a.ld_id[r] = id; }
             }
         }
         // ---- the accumulators: rows 0..31 are the lanes of quadrant 0, which two of the eight warps can read

@@ -41,3 +41,20 @@ def test_vocab_rows_edges(V, B, k):
     acc, bif = sd.verify(drafts, V, 1e9)
     assert acc.cpu().tolist() == [0] * B
     sd.close()
+
+
+def test_a_block_without_drafts_has_no_draft_logits():
+    """verify with k = 0 (no drafts: a null pointer) behind a block that had some: every row reports (+inf, -1), not what the earlier block left."""
+    from paper_2203_16487_b200 import binding
+    V, B = 20001, 2
+    dims = W.ModelDims(512, 8, 128, V, 1, 1, 64)
+    sd = binding.SpecDec(dims, W.make_weights(dims, 61, True), dims, W.make_weights(dims, 62, True), k_max=4, max_batch=B, max_src=12, max_tgt=24, bf16=True)
+    rng = np.random.default_rng(2)
+    sd.encode(*W.pad_batch([W.zipf_ids(rng, 9, V) for _ in range(B)]), None)
+    drafts = rng.integers(4, V, size=(B, 4)).astype(np.int32)
+    sd.verify(drafts, 3, 1.0)
+    assert sd.debug_row_stats(4)[:, :4, 5].cpu().numpy().astype(int).tolist() == drafts.tolist()
+    sd.verify(np.zeros((B, 0), np.int32), 3, 1.0)
+    stats = sd.debug_row_stats(0).cpu().numpy()
+    assert np.isposinf(stats[:, 0, 4]).all() and (stats[:, 0, 5] == -1).all(), stats
+    sd.close()
