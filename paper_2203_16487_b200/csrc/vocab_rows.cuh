@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_vocab_rows(const __grid_const
         int c4[4] = {0, 0, 0, 0}, a4[4];
 #pragma unroll
         for (int j = 4; j < CW; ++j) m4[j & 3] = fmaxf(m4[j & 3], x[j]);
-        p.mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+        p.mx = fmaxf(fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])), -CUDART_INF_F);      // (28 NaN columns lose every comparison of the merge)
 #pragma unroll
         for (int u = 0; u < 4; ++u) a4[u] = CW;
 #pragma unroll

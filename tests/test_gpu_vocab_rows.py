@@ -58,3 +58,30 @@ def test_a_block_without_drafts_has_no_draft_logits():
     stats = sd.debug_row_stats(0).cpu().numpy()
     assert np.isposinf(stats[:, 0, 4]).all() and (stats[:, 0, 5] == -1).all(), stats
     sd.close()
+
+
+@pytest.mark.parametrize("lse", [0, 1])
+def test_columns_that_are_nan_hide_no_others(lse):
+    """28 columns of a tile, all that one warp sees, are NaN (broken weights): the rest of the tile counts as in the launches that serve any number of rows."""
+    from paper_2203_16487_b200 import binding
+    V, k = 20001, 3
+    dims = W.ModelDims(512, 8, 128, V, 1, 1, 64)
+    wv = W.make_weights(dims, 61, True)
+    drafts = np.array([[224 * 40 + 100, 224 * 41 + 30, 224 * 42 + 200]], np.int32)     # (a row's largest logit is the token it was fed)
+    for first in (224 * 40, 224 * 41, 224 * 41 + 56, 224 * 42 + 84):
+        wv["embed"][first:first + 28] = np.nan
+    rng = np.random.default_rng(3)
+    src = W.zipf_ids(rng, 9, 5000)
+    got = {}
+    for skinny in (1, 0):
+        sd = binding.SpecDec(dims, wv, dims, wv, k_max=k, max_batch=1, max_src=12, max_tgt=24, bf16=True)
+        sd.set_option("skinny", skinny)
+        sd.set_option("row_lse", lse)
+        sd.encode(*W.pad_batch([src]), None)
+        acc, bif = sd.verify(drafts, 3, 1.0)
+        got[skinny] = sd.debug_row_stats(k).cpu().numpy()[0], acc.item(), bif.item()
+        sd.close()
+    assert got[1][0][:, 1].astype(int).tolist() == got[0][0][:, 1].astype(int).tolist() == [W.BOS_ID] + drafts[0].tolist()
+    assert got[1][1:] == got[0][1:]
+    assert np.abs(got[1][0][:, [0, 4]][:k] - got[0][0][:, [0, 4]][:k]).max() < 2e-2    # (bf16 operands: two orders of the same sums)
+    assert (got[1][0][:, 3] == got[0][0][:, 3])[:k].all()
