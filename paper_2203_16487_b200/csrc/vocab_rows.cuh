@@ -283,10 +283,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_vocab_rows(const __grid_const
     if (warp == 1) tmem_dealloc(tmem_d, 256);
 }
 
-// Where this kernel is used: widths and vocabularies whose 224-column tiles are one wave, and few enough rows that every CTA can normalise them all.
+// Where this kernel is used: widths and vocabularies whose 224-column tiles are one wave, and few enough rows that every CTA can normalise them all and
+// each row has a CTA that stores it (a device of a few SMs would have fewer tiles than rows).
 constexpr int VR_MAX_ROWS = 32;
 inline bool vr_supported(const TmaEncoder& enc, int N, int K, int rows_ub) {
-    return enc.ready && K == VR_K && rows_ub <= VR_MAX_ROWS && (N + 127) / 128 > enc.n_sm && (N + VR_BN - 1) / VR_BN <= enc.n_sm;
+    const int tiles = (N + VR_BN - 1) / VR_BN;
+    return enc.ready && K == VR_K && rows_ub <= VR_MAX_ROWS && (N + 127) / 128 > enc.n_sm && tiles <= enc.n_sm && tiles >= rows_ub;
 }
 inline cudaError_t vr_init() {
     const cudaError_t e = cudaFuncSetAttribute(k_vocab_rows<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, VrCfg<16>::SMEM);

@@ -40,7 +40,23 @@ static int maps_of_one_launch() {
     return wrong;
 }
 
+// The few-rows vocabulary kernel: CTA r of the grid stores row r, so there are as many tiles as rows wherever it is used; on 148 SMs every count up to 32 is.
+static int rows_without_a_cta() {
+    int wrong = 0;
+    sd::TmaEncoder enc;
+    enc.ready = true;
+    for (enc.n_sm = 1; enc.n_sm <= 200; ++enc.n_sm)
+        for (int N = 128; N <= 50000; N += 97)
+            for (int rows = 1; rows <= 33; ++rows)
+                wrong += sd::vr_supported(enc, N, 512, rows) && (N + sd::VR_BN - 1) / sd::VR_BN < rows;
+    enc.n_sm = 148;
+    for (int N = 18000; N <= 34000; ++N)
+        for (int rows = 1; rows <= 33; ++rows) wrong += sd::vr_supported(enc, N, 512, rows) != (N > 148 * 128 && N <= 148 * 224 && rows <= 32);
+    return wrong;
+}
+
 int main() {
+    printf("rows_without_a_cta %d\n", rows_without_a_cta());
     printf("maps_of_one_launch %d\n", maps_of_one_launch());
     return 0;
 }
@@ -63,3 +79,7 @@ def wrong(tmp_path_factory):
 
 def test_the_maps_of_a_launch_survive_the_eviction_between_them(wrong):
     assert wrong["maps_of_one_launch"] == 0
+
+
+def test_every_row_of_the_few_rows_vocabulary_kernel_has_a_cta(wrong):
+    assert wrong["rows_without_a_cta"] == 0
