@@ -18,8 +18,8 @@ constexpr int RG_MAX_ROWS = 384;                             // in general; shap
 // (verify step, us, this kernel / tiles: width 512: 130 rows 200 / 221, 160 rows 217 / 224, 182 rows 229 / 227, 208 rows 237 / 228;
 // width 768: 78 rows 262 / 294, 96 rows 285 / 294, 104 rows 309 / 291)
 __host__ __device__ constexpr int rg_tile_rows(int width) { return width <= 512 ? 176 : 96; }
-// ... reductions of 2048 and more sooner, to the split-K tiles (512 wide 121 rows 174.3 / 174.7, 130 rows 181.3 / 178.4, 156 rows 191.5 / 190; 768 wide 78 rows 254 / 254, 88 rows
-// 262 / 227) ...
+// ... reductions of 2048 and more sooner, to the split-K tiles, where these exist (512 wide 121 rows 174.3 / 174.7, 130 rows 181.3 / 178.4, 156 rows 191.5 / 190; 768 wide 78 rows
+// 254 / 254, 88 rows 262 / 227; a reduction of 2112, which has none, two layers: 130 rows 180.3 / 195.3 on whole tiles, 144 rows 193.6 / 209.3) ...
 __host__ __device__ constexpr int rg_tile_rows_long(int width) { return width <= 512 ? 128 : 80; }
 // ... and in the encoders, two of which run side by side on two streams and fill the SMs sooner (first tokens: width 512: 60 rows
 // 497 / 560, 80 rows 531 / 526, 120 rows 651 / 582; width 768: 40 rows 527 / 527, 60 rows 561 / 524).

@@ -497,8 +497,10 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
               int* n_tiles_out, const KvDest* kv, const LnSpec* lnp, bool again) {
     if (rows_ub <= 0) return 0;
     // few rows: the weight-streaming kernel, with the LayerNorm inside where it has one
+    const sd::SpkPlan plan = std::is_same<T, bf16>::value && epi == EPI_RESID && h->use_tc && h->use_splitk && h->splitk_ready && sd::tc_supported(N, K)
+                                 ? sd::spk_plan(h->tma, N, K, rows_ub, cnt == CNT_ENC) : sd::SpkPlan{0, 0, 0};
     const int width = std::min(N, K), tile_rows = !sd::tc_supported(N, K) ? RG_MAX_ROWS : cnt == CNT_ENC ? rg_tile_rows_enc(width) :
-                                                             epi == EPI_RESID && K >= 2048 && h->use_splitk && h->splitk_ready ? rg_tile_rows_long(width) : rg_tile_rows(width);
+                                                             K >= 2048 && plan.split ? rg_tile_rows_long(width) : rg_tile_rows(width);
     const bool rows_ok = std::is_same<T, bf16>::value && h->use_skinny && h->use_tc && (cnt != CNT_ENC || h->enc_skinny) && !(epi == EPI_RESID && h->use_ln_fuse);
     const int tile_lda = lnp ? K : lda;
     const bool fits = rows_ok && rows_ub <= tile_rows && rg_supported(epi, N, K, tile_lda, rows_ub, h->use_sk_cluster != 0);
@@ -547,7 +549,6 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
                 ++h->launches;
                 return 0;
             }
-            const sd::SpkPlan plan = epi == EPI_RESID && h->use_splitk && h->splitk_ready ? sd::spk_plan(h->tma, N, K, rows_ub, cnt == CNT_ENC) : sd::SpkPlan{0, 0, 0};
             if (plan.split) {
                 if (sd::spk_launch(h->tma, plan, g, rows_ub, st) != 0)
                     return fail(h, SPECDEC_ERR_CUDA, "tensor-core GEMM launch failed: " + h->tma.err);

@@ -1,0 +1,90 @@
+"""Which kernel serves a launch, read off the kernel nodes of a captured step: the rules that were set by measuring both sides, at their edges."""
+import ctypes as C
+import re
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2203_16487_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+CU_GRAPH_NODE_TYPE_KERNEL = 0
+RESID = "2"                                           # (the epilogue that adds to the residual stream)
+
+
+class KernelNode(C.Structure):                        # CUDA_KERNEL_NODE_PARAMS_v2
+    _fields_ = [("func", C.c_void_p)] + [(n, C.c_uint) for n in ("gx", "gy", "gz", "bx", "by", "bz", "smem")] + \
+               [(n, C.c_void_p) for n in ("params", "extra", "kern", "ctx")]
+
+
+def _kernels(graph):
+    """Names with template arguments, as k_rows<2,0,1,8,2,1,8>, of the graph's kernel nodes."""
+    cu, g, n = C.CDLL("libcuda.so.1"), C.c_void_p(graph.raw_cuda_graph()), C.c_size_t()
+    assert cu.cuGraphGetNodes(g, None, C.byref(n)) == 0
+    nodes = (C.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(g, nodes, C.byref(n)) == 0
+    names = []
+    for node in nodes:
+        t, p, name = C.c_int(), KernelNode(), C.c_char_p()
+        assert cu.cuGraphNodeGetType(C.c_void_p(node), C.byref(t)) == 0
+        if t.value != CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        assert cu.cuGraphKernelNodeGetParams_v2(C.c_void_p(node), C.byref(p)) == 0
+        assert (cu.cuFuncGetName(C.byref(name), C.c_void_p(p.func)) if p.func else cu.cuKernelGetName(C.byref(name), C.c_void_p(p.kern))) == 0
+        m = re.match(r"_ZN?(?:2sd)?\d+(k_[a-z0-9_]+?)(?:I(.*?)E+v.*|E?P.*|$)", name.value.decode())
+        args = re.findall(r"L[ib](\d+)E", m.group(2) + "E") if m and m.group(2) else []
+        names.append(f"{m.group(1)}<{','.join(args)}>" if m else name.value.decode())
+    return names
+
+
+def _step(dims, step, B, k, S):
+    from paper_2203_16487_b200 import binding
+    wv, wd = W.make_weights(dims, 5, True), W.make_weights(dims, 6, True)
+    sd = binding.SpecDec(dims, wv, dims, wd, k_max=max(k, 1), max_batch=B, max_src=S, max_tgt=40, bf16=True)
+    sd.set_option("graphs", 0)                        # the step calls launch into the capture themselves
+    rng = np.random.default_rng(1)
+    src = torch.from_numpy(np.stack([W.zipf_ids(rng, S, dims.vocab) for _ in range(B)])).cuda()
+    i32 = dict(dtype=torch.int32, device="cuda")
+    lens, draft, acc, bif = torch.full((B,), S, **i32), torch.zeros((B, max(k, 1)), **i32), torch.zeros(B, **i32), torch.zeros(B, **i32)
+    lib, ptr = sd._lib, binding._ptr
+    calls = {
+        "encode": lambda s: lib.specdec_encode(sd._h, ptr(src), ptr(lens), None, B, S, s),
+        "verify": lambda s: lib.specdec_verify(sd._h, ptr(draft), k, 3, 1.0, ptr(acc), ptr(bif), s),
+    }
+    sd.B = B
+    for name in dict.fromkeys(("encode", step)):      # an ordinary pass first: the session exists
+        assert calls[name](binding._stream()) == 0, sd.last_error()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        assert calls[step](binding._stream()) == 0, sd.last_error()
+    names = _kernels(g)
+    del g
+    sd.close()
+    return names
+
+
+def _resid(names):
+    """The launches that add to the residual stream, in order."""
+    return [n for n in names if n.startswith("k_gemm_tc_splitk") or re.match(rf"k_(rows|gemm_tc)<{RESID},", n)]
+
+
+# One decoder layer: output projections of both attentions, then FFN2.
+@pytest.mark.parametrize("d,f,B,k,ffn2", [
+    (512, 2112, 8, 15, "k_rows"),           # 128 rows.  K = 2112 is 33 K blocks, which no two or four slices share equally:
+    (512, 2112, 10, 12, "k_rows"),          # 130 rows: the few-rows kernel goes on to its own limit
+    (512, 2112, 11, 15, "k_rows"),          # 176 rows: the last
+    (512, 2112, 12, 15, "k_gemm_tc<"),      # 192 rows: whole tiles
+    (512, 2048, 8, 15, "k_rows"),           # 128 rows
+    (512, 2048, 10, 12, "k_gemm_tc_splitk"),
+    (512, 2176, 10, 12, "k_gemm_tc_splitk"),
+    (768, 2112, 8, 9, "k_rows"),            # 80 rows
+    (768, 2112, 8, 11, "k_rows"),           # 96 rows
+    (768, 2112, 7, 13, "k_gemm_tc<"),       # 98 rows
+    (768, 3072, 8, 10, "k_gemm_tc_splitk"),  # 88 rows
+])
+def test_ffn2_leaves_the_few_rows_kernel_for_split_tiles_only(d, f, B, k, ffn2):
+    names = _step(W.ModelDims(d, d // 64, f, 515, 1, 1, 64), "verify", B, k, 12)
+    assert _resid(names)[-1].startswith(ffn2), names

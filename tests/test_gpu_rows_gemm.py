@@ -35,6 +35,8 @@ pytestmark = pytest.mark.gpu
     (512, 8, 2048, 7, 13),          # 98 rows: 16 x 64 tiles, the last of them two rows
     (512, 8, 2048, 8, 15),          # 128 rows: the last with the FFN2 here
     (512, 8, 2048, 10, 12),         # 130 rows: its split-K tiles
+    (512, 8, 2112, 10, 12),         # 130 rows: a reduction that has no split-K tiles stays, two slices of 66 MMA steps
+    (512, 8, 2112, 11, 15),         # 176 rows: the last of them, four slices
     (512, 8, 2048, 14, 15),         # 224 rows: the last QKV projections on 32-row tiles
     (512, 8, 2048, 14, 16),         # 238 rows: QKV on tensor-core tiles again, output projections on 16-row tiles, the last of them 14 rows
     (512, 8, 2048, 27, 15),         # 432 rows: the last output projections on 16-row tiles
