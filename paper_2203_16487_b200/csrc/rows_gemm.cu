@@ -331,14 +331,16 @@ static int rg_split(int N, int K, int rows_ub, bool cluster) {
 // of the output projections: 208 rows 223 / 204 / 214, 312 rows 258 / 235 / 244, 416 rows 277 / 269 / 270, 520 rows 289 / 280 / 275, 624 rows 295 / 295 / 291.5, 832 rows
 // 312 / 333 / 312; the QKV projection: 182 rows 203 / - / 195, 208 rows 204 / - / 199.6, 312 rows 235 / - / 245.  Width 768 (50 KB, 32 columns; 149 KB, one to an SM): 130
 // rows 275 / 258 / 265, 156 rows 281 / 265 / 269, 208 rows 307 / 325 / 296, 312 rows 360 / 373 / 350, 364 rows 343 / - / 346.  The two encoders share the SMs (512: 144 rows
-// 316 / 273, 200 rows 324 / 299, 400 rows 380 / 392 on 16 rows, 496 rows 422 / 419, 640 rows 430 / 439; 768: 96 rows 203 / 193, 200 rows 270 / 260, 296 rows 303 / 314) and take these tiles
-// where they leave the few-rows ones, at 73 (768: 41) rows: beginning at 97 left whole tiles in between (512: 80 rows 165 / 145, 96 rows 167 / 148; 768: 60 rows 204 / 189).
+// 316 / 273, 200 rows 324 / 299; 768: 96 rows 203 / 193, 200 rows 270 / 260, 296 rows 303 / 314), so output projections with K = 512 stop sooner there: 16-row tiles at
+// 7/8 CTA per SM (256 rows at 512 columns), 32-row ones at 5/9 (320 rows): 6 + 12 layers, whole tiles / 16 rows / 32 rows: 256 rows 186.5 / 185 / -, 260 rows 225 / 229.5 / 221, 288 rows 226 /
+// 231 / 223, 320 rows 229 / - / 230, 360 rows 231 / - / 237.8, 512 rows 271.8 / - / 276, 560 rows 256.7 / - / 265.8.  They begin where the few-rows ones end, at 73 (768: 41) rows: from 97 on
+// left whole tiles in between (512: 80 rows 165 / 145, 96 rows 167 / 148; 768: 60 rows 204 / 189).
 int rg_frag_rows(int epi, int N, int K, int rows_ub, int n_sm, bool enc) {
     const bool resid = epi == EPI_RESID;
     if (N % 64 || !(K == 512 || (K == 768 && resid)) || rows_ub <= (enc ? rg_tile_rows_enc(min(N, K)) : K == 512 ? 96 : 80)) return 0;
     const long long sm = n_sm, t16 = (rows_ub + 15) / 16, t32 = (rows_ub + 31) / 32;
-    if (resid && t16 * (K == 512 ? N / 64 : N / 32) <= (enc ? sm : K == 512 ? sm * 3 / 2 : sm * 5 / 3)) return 16;
-    return t32 * (N / 64) <= (K == 512 ? (enc && resid ? sm : sm * 5 / 4) : enc ? sm * 2 / 3 : sm * 7 / 8) ? 32 : 0;
+    if (resid && t16 * (K == 512 ? N / 64 : N / 32) <= (!enc ? K == 512 ? sm * 3 / 2 : sm * 5 / 3 : K == 512 ? sm * 7 / 8 : sm)) return 16;
+    return t32 * (N / 64) <= (K == 512 ? (enc && resid ? sm * 5 / 9 : sm * 5 / 4) : enc ? sm * 2 / 3 : sm * 7 / 8) ? 32 : 0;
 }
 bool rg_supported(int epi, int N, int K, int lda, int rows_ub, bool cluster) {
     if (rows_ub > RG_MAX_ROWS || K % 16 || N % 16 || lda % 8) return false;

@@ -96,10 +96,15 @@ def test_ffn2_leaves_the_few_rows_kernel_for_split_tiles_only(d, f, B, k, ffn2):
     (512, 1, 73, "k_rows<2,0,1,8,2,1,8>"),      # 16-row tiles with the weights as fragments, from here on
     (512, 8, 12, "k_rows<2,0,1,8,2,1,8>"),      # 96 rows
     (512, 1, 97, "k_rows<2,0,1,8,2,1,8>"),
+    (512, 16, 16, "k_rows<2,0,1,8,2,1,8>"),     # 256 rows: the last
+    (512, 1, 257, "k_rows<2,0,2,8,2,1,8>"),     # 32-row tiles
+    (512, 20, 16, "k_rows<2,0,2,8,2,1,8>"),     # 320 rows: the last
+    (512, 3, 107, "k_gemm_tc<2,"),              # 321 rows
+    (512, 36, 16, "k_gemm_tc<2,"),              # 576 rows
     (768, 4, 10, "k_rows<2,0,1,"),              # 40 rows
     (768, 1, 41, "k_rows<2,0,1,4,1,1,6>"),      # 41 rows
     (768, 2, 48, "k_rows<2,0,1,4,1,1,6>"),      # 96 rows: the last at this width
 ])
 def test_output_projections_of_the_encoders(d, B, S, out):
-    names = _resid(_step(W.ModelDims(d, d // 64, 4 * d, 515, 1, 1, 128), "encode", B, 0, S))
+    names = _resid(_step(W.ModelDims(d, d // 64, 4 * d, 515, 1, 1, 320), "encode", B, 0, S))
     assert len(names) == 4 and names[0].startswith(out) and names[2].startswith(out), names
