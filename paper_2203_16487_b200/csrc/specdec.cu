@@ -473,6 +473,12 @@ template <typename T> bool kv_in_gemm(const specdec_handle* h, int d, int rows_u
 // LayerNorm fused in front of a GEMM: x fp32 rows, gain, bias.
 struct LnSpec { const float* x; const float* g; const float* b; };
 
+// Whether both encoders' attention is the tile kernel.
+inline bool enc_tile_attn(const specdec_handle* h) {
+    auto wide = [](const specdec_model_dims& m) { return m.d_model == 64 * m.n_heads; };
+    return h->use_tc_attn && wide(h->cfg.verifier) && wide(h->cfg.drafter);
+}
+
 // out = A W^T (+bias) with one of the epilogues; rows_ub bounds the grid, the live count is on the device.
 template <typename T>
 int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W, const float* bias, int N, int K, int cnt,
@@ -505,8 +511,10 @@ int gemm_once(specdec_handle* h, int epi, const void* A, int lda, const void* W,
     const int tile_lda = lnp ? K : lda;
     const bool fits = rows_ok && rows_ub <= tile_rows && rg_supported(epi, N, K, tile_lda, rows_ub, h->use_sk_cluster != 0);
     const bool ln_inside = fits && lnp && rows_ub <= rg_ln_rows(width) && rg_ln_width(K);
-    // (with the LayerNorm in front, or none)
-    const int frag = rows_ok && !ln_inside && tile_lda % 8 == 0 && epi != EPI_STATS && epi != EPI_F32 ? rg_frag_rows(epi, N, K, rows_ub, h->tma.n_sm, cnt == CNT_ENC) : 0;
+    // (with the LayerNorm in front, or none; no 32-row tiles beside an encoder whose attention is the warp-per-row kernel: these take registers and CTA slots that it
+    // would fill on the other stream, encoders of 160 / 192 / 200 rows with 32-wide heads 385 / 466 / 815 us without, 413 / 522 / 956 with)
+    int frag = rows_ok && !ln_inside && tile_lda % 8 == 0 && epi != EPI_STATS && epi != EPI_F32 ? rg_frag_rows(epi, N, K, rows_ub, h->tma.n_sm, cnt == CNT_ENC) : 0;
+    if (frag == 32 && cnt == CNT_ENC && !enc_tile_attn(h)) frag = 0;
     const bool few = fits || frag;
     const bool few32 = std::is_same<T, float>::value && h->use_skinny && rf_supported(epi, N, K, lnp ? K : lda, rows_ub);
     const bool ln32 = few32 && lnp && rf_ln_width(K);

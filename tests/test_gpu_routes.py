@@ -108,3 +108,11 @@ def test_ffn2_leaves_the_few_rows_kernel_for_split_tiles_only(d, f, B, k, ffn2):
 def test_output_projections_of_the_encoders(d, B, S, out):
     names = _resid(_step(W.ModelDims(d, d // 64, 4 * d, 515, 1, 1, 320), "encode", B, 0, S))
     assert len(names) == 4 and names[0].startswith(out) and names[2].startswith(out), names
+
+
+# The projections of 32-row tiles (QKV, FFN1, wider output projections) of encoders with 64- and with 32-wide heads.
+@pytest.mark.parametrize("d,B,S", [(512, 8, 12), (512, 10, 16), (512, 14, 16), (512, 20, 16), (768, 12, 16)])       # 96, 160, 224, 320, 192 rows
+def test_32_row_tiles_of_the_encoders_go_with_tile_attention(d, B, S):
+    wide, narrow = (sum(n.startswith("k_rows<") and ",0,2,8,2,1," in n for n in _step(W.ModelDims(d, d // dh, 4 * d, 515, 1, 1, 128), "encode", B, 0, S))
+                    for dh in (64, 32))
+    assert wide > 0 and narrow == 0
