@@ -31,7 +31,9 @@ template <int AR, int BN> struct SpkCfg {
 // 258 -> 250), unless another stream's kernels share the SMs (two encoders over 144 rows 307 -> 315).
 // Where two slices of 64-column tiles are more clusters than run at once, two of 128 columns, up to twice the rows: unsplit these are at most 72 CTAs that walk the whole K
 // (verify step of 1248 rows, us, unsplit / split: 354.4 / 348.2, 1408 rows 387 / 379, 1664 rows 385 / 379, 2048 rows 426 / 420; drafts over 2160 rows 137.4 / 134.5).  Beside
-// another stream's kernels (encoders) the unsplit ones stay.
+// another stream's kernels (encoders) the unsplit ones stay, and for reductions that gain less than the exchange costs (two layers, 512 columns, verify / draft step of 1248 and of 2080 rows:
+// K = 1024 287.2 / 295.3, 291 / 299 and 323 / 330, 325.5 / 334.4; 1536 300 / 300.5, 302 / 304.8 and 339 / 341, 341 / 346; 1664 302 / 302, 307 / 308 and 348 / 349.5, 351.4 / 352.5;
+// 1792 308 / 305, 309.6 / 310.8 and 352 / 350, 354 / 355.3; 1024-wide output projections of 1040 rows 402 / 415, 408.5 / 423).
 struct SpkPlan { int split, rows, cols; };
 inline SpkPlan spk_plan(const TmaEncoder& enc, int N, int K, int rows_ub, bool shared) {
     if (N % 64 || K < 768) return {0, 0, 0};
@@ -40,7 +42,7 @@ inline SpkPlan spk_plan(const TmaEncoder& enc, int N, int K, int rows_ub, bool s
     if (K % (4 * TC_BK) == 0 && m * n <= enc.spk_clusters4) return {4, TC_BM, 64};
     if (K % (2 * TC_BK) || K < 1024) return {0, 0, 0};
     if (m * n <= enc.spk_clusters2) return {2, TC_BM, 64};
-    return {!shared && N % 128 == 0 && m * (N / 128) <= enc.spk_clusters2_128 ? 2 : 0, TC_BM, 128};
+    return {!shared && K >= 1792 && N % 128 == 0 && m * (N / 128) <= enc.spk_clusters2_128 ? 2 : 0, TC_BM, 128};
 }
 
 template <int SPLIT, int AR, int BN>

@@ -116,3 +116,16 @@ def test_32_row_tiles_of_the_encoders_go_with_tile_attention(d, B, S):
     wide, narrow = (sum(n.startswith("k_rows<") and ",0,2,8,2,1," in n for n in _step(W.ModelDims(d, d // dh, 4 * d, 515, 1, 1, 128), "encode", B, 0, S))
                     for dh in (64, 32))
     assert wide > 0 and narrow == 0
+
+
+@pytest.mark.parametrize("d,f,split", [
+    (512, 1024, False),
+    (512, 1664, False),
+    (512, 1792, True),                      # 512 columns: the shortest reduction that gains
+    (512, 2048, True),
+    (1024, 2048, True),                     # (output projections: K = 1024)
+])
+def test_two_slices_of_128_columns_are_for_long_reductions(d, f, split):
+    B, k = (48, 25) if d == 512 else (40, 25)
+    names = _resid(_step(W.ModelDims(d, d // 64, f, 515, 1, 1, 128), "verify", B, k, 12))
+    assert [n.startswith("k_gemm_tc_splitk<2,128,128>") for n in names] == [False, False, split], names

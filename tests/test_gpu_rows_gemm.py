@@ -53,6 +53,7 @@ pytestmark = pytest.mark.gpu
     (512, 8, 2048, 27, 18),         # 513 rows: two K slices, one row in the last tile
     (512, 8, 2048, 61, 18),         # 1159 rows: two K slices of 128-column tiles, seven rows in the last of them
     (512, 8, 2048, 96, 23),         # 2304 rows: the last of them, every tile full
+    (512, 8, 1664, 48, 25),         # 1248 rows: a reduction too short for them
     (768, 12, 3072, 40, 21),        # 880 rows: at this width
     (256, 4, 1152, 20, 14),         # 300 rows: two slices of nine K blocks, more than the ring holds
 ])
