@@ -69,8 +69,12 @@ def test_queries_projected_inside_the_attention(d, f, B, k, S):
 
 @pytest.mark.parametrize("d,B,k,S,cached", [
     (256, 1, 4, 12, False),          # 5 rows of one tile: the fewest
-    (512, 2, 16, 128, False),        # a tile and one row; as many keys as fit beside the queries' projection
-    (512, 1, 47, 129, True),         # 48 rows; one key too many for it
+    (512, 1, 15, 128, False),        # 16 rows of eight heads, 8 CTAs: both attentions go on to their output projections; as many keys as fit beside the queries'
+    (512, 1, 15, 129, True),         # one key too many for that: the cross-attention projects its queries only
+    (512, 1, 16, 128, False),        # 17 rows, 16 CTAs: the cross-attention only, and the last
+    (512, 1, 32, 128, False),        # 33 rows, 24 CTAs: neither
+    (256, 2, 23, 128, False),        # four heads, 48 rows: the most with the queries projected too
+    (256, 1, 48, 128, True),         # 49 rows: the self-attention only
     (256, 3, 16, 300, True),         # three stages of keys
 ])
 def test_output_projected_inside_the_attention(d, B, k, S, cached):
@@ -91,7 +95,8 @@ def test_output_projected_inside_the_attention(d, B, k, S, cached):
     sd.close()
 
 
-@pytest.mark.parametrize("bf16,d,H,cached", [(True, 256, 4, False), (True, 256, 4, True), (False, 64, 16, False), (False, 64, 16, True)])
+@pytest.mark.parametrize("bf16,d,H,cached", [(True, 256, 4, False), (True, 256, 4, True), (True, 512, 8, False), (True, 512, 8, True),
+                                             (False, 64, 16, False), (False, 64, 16, True)])
 def test_slices_of_unfinished_sequences(bf16, d, H, cached):
     """A ragged batch whose sequences end one after another: the attention launches shrink to the unfinished ones (32, 16, ... of 33).
     Every draft is accepted, so what comes out is what the drafter's passes computed, and each (k + 1)-th token what the verifier's did."""
@@ -113,13 +118,29 @@ def test_slices_of_unfinished_sequences(bf16, d, H, cached):
     sd.set_option("drafter_prefix_causal", int(cached))
     out, n, _ = sd.generate(*W.pad_batch(srcs), np.array(tgt, np.int32), k, beta, tau)
     out, n = out.cpu().numpy(), n.cpu().numpy()
-    wrong, seen = 0, set()
+
+    def gap_at_the_first_difference(b, got, ref):
+        """By how much the oracle's logits of that position prefer its token to the other one, on the prefix that both share."""
+        p = next((i for i, (x, y) in enumerate(zip(got, ref)) if x != y), None)
+        assert p is not None, (b, got, ref)              # (one ends early: no margin explains that)
+        j = p // (k + 1) * (k + 1)                       # tokens committed before this block
+        if p - j < k:
+            row = O.decoder_rows(md, [W.BOS_ID] + ref[:j] + [W.MASK_ID] * k, O.encode(md, srcs[b]), causal=False, n_causal=j + 1 if cached else None)[j + 1 + p - j]
+        else:
+            row = O.decoder_rows(mv, [W.BOS_ID] + ref[:p], O.encode(mv, srcs[b]), causal=True)[-1]
+        assert row.argmax() == ref[p]
+        return row[ref[p]] - row[got[p]]
+
+    gaps, seen = [], set()
     for b in range(B):
         ref, _ = O.specdec_generate(mv, md, srcs[b], tgt[b], k, beta, tau, W.BOS_ID, W.EOS_ID, W.MASK_ID,
                                     drafter_reading="prefix_causal" if cached else "bidirectional")
-        wrong += out[b, :n[b]].tolist() != ref
+        got = out[b, :n[b]].tolist()
+        if got != ref:
+            gaps.append(gap_at_the_first_difference(b, got, ref))
         seen.update(ref)
-    assert len(seen) > 50                                # (the drafts do vary)
-    # fp32: exact.  bf16: about 1300 arguments of a maximum over 515 logits of spread ~1 that agree to 2e-3: a few near-ties are expected
-    assert wrong <= (4 if bf16 else 0), wrong
+    assert len(seen) > 40                                # (the drafts do vary)
+    # fp32: exact.  bf16: two logits that each agree with the oracle's to 2e-3 may change places where these are less than twice that apart (about 1300 arguments of
+    # a maximum over 515 logits of spread ~1: a few near-ties are expected).  A slice that is lost or swapped differs by the spread.
+    assert not gaps if not bf16 else all(g < 4e-3 for g in gaps), gaps
     sd.close()

@@ -129,3 +129,23 @@ def test_two_slices_of_128_columns_are_for_long_reductions(d, f, split):
     B, k = (48, 25) if d == 512 else (40, 25)
     names = _resid(_step(W.ModelDims(d, d // 64, f, 515, 1, 1, 128), "verify", B, k, 12))
     assert [n.startswith("k_gemm_tc_splitk<2,128,128>") for n in names] == [False, False, split], names
+
+
+# One decoder layer: whether the self-attention goes on to its output projection, the cross-attention projects its queries, and goes on to its output projection.
+@pytest.mark.parametrize("d,B,k,S,self_out,cross_q,cross_out", [
+    (512, 1, 3, 12, 0, 1, 0),               # 4 rows: too few to gain
+    (256, 1, 4, 12, 1, 1, 1),               # 5 rows
+    (512, 1, 15, 128, 1, 1, 1),             # eight heads, 8 CTAs; as many keys as fit beside the queries' projection
+    (512, 1, 15, 129, 1, 1, 0),             # a key more
+    (512, 1, 16, 128, 0, 1, 1),             # 16 CTAs
+    (512, 2, 15, 128, 0, 1, 1),
+    (512, 1, 32, 128, 0, 1, 0),             # 24 CTAs
+    (256, 2, 23, 128, 1, 1, 1),             # four heads, 48 rows
+    (256, 1, 48, 128, 1, 1, 0),             # 49 rows
+    (256, 8, 16, 12, 1, 1, 0),              # 64 CTAs
+    (256, 9, 16, 12, 0, 1, 0),              # 72 CTAs
+])
+def test_projections_inside_the_attention(d, B, k, S, self_out, cross_q, cross_out):
+    names = _step(W.ModelDims(d, d // 64, 2 * d, 515, 1, 1, 256), "verify", B, k, S)
+    (_, s_out), (c_q, c_out) = ([int(v) > 0 for v in n[:-1].split(",")[-2:]] for n in names if n.startswith("k_attn<"))
+    assert (s_out, c_q, c_out) == (self_out, cross_q, cross_out), names
