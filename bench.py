@@ -328,7 +328,7 @@ def tokens_leg(torch, binding, B: int, K_: int, W_: int, rank: int, world: int, 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of the verify microbenchmark, by batch: the
 # number of kernels of the step that was captured, one whole step, and the vocabulary kernel alone.  ncu measures every kernel with cold
 # caches, so at batch 128 the step figure counts activations that normally stay in L2 (an upper bound).
-NCU_TRAFFIC = {1: {"launches": 34, "step": 83054336, "vocabulary": 33642752}, 128: {"launches": 70, "step": 817090048, "vocabulary": 37050112}}
+NCU_TRAFFIC = {1: {"launches": 39, "step": 83115008, "vocabulary": 33659392}, 128: {"launches": 70, "step": 817090048, "vocabulary": 37050112}}
 
 
 def ncu_traffic(B: int, launches_per_step: int, what: str):
