@@ -265,13 +265,14 @@ int specdec_profile_read(specdec_handle* h, double* h_ms, long long* h_launches)
  * "gemm"         0 SIMT reference GEMM / 1 tcgen05 tensor-core GEMM (bf16 handles; default 1)
  * "attn"         0 warp-per-row reference attention / 1 tile attention (bf16: 64-wide heads on tensor cores; fp32: head sizes 4 .. 128, powers
  *                of two; default 1)
- * "skinny"       0/1 weight-streaming GEMM for passes of few rows (at most 176, wider than 512 at most 96; default 1), up
- *                to 144 or 80 rows with the LayerNorm in front fused; fp32 handles: the fp32 GEMM of passes of at most 768 rows, LayerNorm fused up to 512 wide
+ * "skinny"       0/1 weight-streaming GEMM for passes of few rows (at most 176, wider than 512 at most 96, of these up
+ *                to 144 or 80 rows with the LayerNorm in front fused; reductions of 512 and, for output projections, 768 beyond that while their CTAs are
+ *                resident: 512 wide QKV at most 224 rows, output projections 736, 768 wide 320; default 1); fp32 handles: the fp32 GEMM of passes of at most 768 rows, LayerNorm fused up to 512 wide
  * "sk_cluster"   0/1 (default 1): that GEMM splits reductions of 1024 and more across a cluster of 2 or 4 CTAs, and attention over few
  *                rows of 4 or 8 64-wide heads runs on to the output projection, a cluster per 16 rows
  * "pair"         0/1 two-SM tensor-core tiles (cta_group::2) for GEMMs with >= 1024 rows and columns (default 0)
  * "enc_skinny"   0 / 1 (default) / 2: the weight-streaming GEMM does not / does / does serve the encoders (up to 72 rows, wider
- *                than 512 up to 40)
+ *                than 512 up to 40; those reductions beyond that, output projections up to 320 rows, 768 wide 256)
  * "ln_fuse"      0/1 the LayerNorm that reads the residual stream next runs inside the residual GEMM (default 0)
  * "splitk"       0/1 residual GEMMs with K >= 768 over few row tiles split K across a cluster (default 1)
  * "attn_stream"  0 / 1 by rule (default) / 2 / 3 / 4: attention CTAs of 16 queries with the keys spread over their warps, or of

@@ -15,7 +15,7 @@
 // kernel this one replaces, 161 with MT = 1, KG = 4).  Many CTAs: the fixed-latency chain inside a warp, so
 // warps per SM and whole waves count: 16 of them, in CTAs of 64 queries with a ring of two 64-key blocks (128 sequences x 51 queries x 307 keys, verify
 // step with 12 warps and a ring of three 1107 us, now 1055-1075) or of 32 queries with 32-key blocks (x 26 x 90: 555 with 8 warps and
-// 64-key blocks, now 514).  Both are cut to 128 registers; with 64 queries that leaves 8 bytes a thread in local memory, 20 with paged keys.  The tensor
+// 64-key blocks, now 514).  Both are cut to 128 registers; with 64 queries that leaves 16 bytes a thread in local memory.  The tensor
 // pipe is active 26 % of the time there, shared memory 41 %, and a warp waits 8.8 cycles for each instruction.  Below four CTAs an SM there is nothing to
 // fill the SMs with, and 64-key blocks have more independent work per barrier: 32 queries take those, at 174 registers and 8 warps an SM.
 #pragma once

@@ -28,7 +28,7 @@ struct RgCfg {
 // time from the predecessor's last store to this kernel's.  Hence:
 //   * everything that does not depend on the predecessor -- the CTA's whole weight tile into shared memory, LayerNorm
 //     parameters, cache rows -- is requested before the dependency wait;
-//   * 256 threads of at most 80 registers (118 where a LayerNorm of 768 columns runs inside; with fragments see below) and 20-100 KB of shared memory, so that the next two kernels of the chain are resident
+//   * 256 threads of at most 80 registers (118 to 120 where a LayerNorm of 768 columns runs inside; with fragments see below) and 20-100 KB of shared memory, so that the next two kernels of the chain are resident
 //     (their weights landed) while this one runs.  A 512-thread version with the weights in registers had shorter phases and a
 //     longer step (240 against 218 us), because its successors could not start early;
 //   * after the wait one round trip brings the rows; with NC > 0 they are normalised on the way (K = 128 NC, two rows per
