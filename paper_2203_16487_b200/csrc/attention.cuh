@@ -144,8 +144,9 @@ template <int MT, int KG, int KW>
 struct AttnCfg {
     static constexpr int KB = KG * KW;                                    // keys per block
     static constexpr int STAGE = KB * 256;                                // K and V of a block
-    static constexpr int MERGE = KG > 1 ? MT * KG * 16 * (68 + 2) * 4 : 0;     // partial outputs (padded rows) and (maximum, sum); reuses the stages
-    // queries, ring (or merge buffers), operands of the query projection, and for paged keys the table of their rows
+    static constexpr int PP = KW * 2 + 16;                                // bytes per row of a key group's probabilities: 16 rows, in place of the group's keys
+    static constexpr int MERGE = KG > 1 ? MT * KG * 16 * (72 + 2) * 4 : 0;     // partial outputs (padded rows) and (maximum, sum); reuses the stages
+    // queries, ring (or merge buffers), operands of the projections, and for paged keys the table of their rows
     static size_t smem(int max_keys, int ns, bool paged, int query_bytes = 0) {
         const int nb = (max_keys + KB - 1) / KB;
         const size_t ring = (size_t)(nb < ns ? (nb < 1 ? 1 : nb) : ns) * STAGE;
@@ -155,7 +156,7 @@ struct AttnCfg {
 
 // CTAs per SM that the registers are cut for; 0 leaves it to the compiler (told 1, it takes 148 registers for MT = 1, KG = 4 where 100 do, and the
 // verify step of 832 rows 334 us instead of 316; MT = 2 with 64-key blocks is better with its 174 than with 129: 1664 rows 388 / 400 us).
-constexpr int attn_ctas(int mt, int kg, int kw) { return kg > 1 ? 0 : mt == 4 ? 4 : kw == 32 ? 8 : 1; }
+constexpr int attn_ctas(int mt, int kg, int kw, bool share) { return kg > 1 ? (share && kg == 4 ? 5 : 0) : mt == 4 ? 4 : kw == 32 ? 8 : 1; }
 
 // QNC > 0: the queries are projected here (QueryArgs; MT = 1, KG = 8).  The CTA's 64 rows of Wq are requested ahead of the wait, the
 // 16 rows normalised behind it; one launch and its round trip through memory less per layer (26 rows, K = 512: 5.5 -> 4.4 us).
@@ -165,21 +166,31 @@ constexpr int attn_ctas(int mt, int kg, int kw) { return kg > 1 ? 0 : mt == 4 ? 
 // of Wo and adds the residual.  A launch and its round trip less (verify step of 26 rows, both attentions of six layers: 156.5 -> 147.2 us).
 //   * Wo, and Wq with QNC, are requested ahead of the wait and are register fragments by the time it returns (fetched behind it 155.2 us; turned into fragments
 //     behind it, while the rows arrive, their 128 KB from shared memory delayed the LayerNorm: rows and LayerNorm 1.5 us, now 1.0);
-//   * every warp sends its eight columns as one bulk copy of 256 bytes to each CTA, counted on the receiver's mbarrier: 0.45 us from the combined rows to the
-//     first MMA, 0.85 with 16-byte asynchronous remote stores, more with plain ones behind a cluster barrier (the step: 147.3, 145.1; both changes, beside
-//     others by then, 125.8 -> 120.4).
-template <bool PAGED, int MT, int KG, int KW, int NS, int QNC = 0, int ON = 0>
-__global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {
+//   * the head's 16 rows, 2 KB, go to each CTA as one bulk copy, every copy issued by another warp and counted on the receiver's mbarrier.  (As eight copies of 256
+//     bytes from the lanes of every warp their issue alone took 790 clocks, one lane after the other; 16-byte asynchronous remote stores 0.85 us, plain ones behind a
+//     cluster barrier more.)
+//
+// SHARE: the keys are one block (at most KG KW), and the groups do not add up partial outputs of all 64 columns through shared memory (35 KB written and read for
+// eight groups: 990 + 910 clocks, half of it bank conflicts) but leave their probabilities there, where their keys were (6 KB); every warp then multiplies those of all groups by its own
+// 64 / KG columns of the values.  The groups' shares are scaled and added in the same order with the same roundings: results are the same to the bit.  With the
+// copies above, verify step, us, before / after: 5 rows 104.7 / 98.8, 16 rows 108.1 / 103.3, 136 rows 187.6 / 183.2, 416 rows 248 / 236.6; 768 columns, 26 rows 179.4 / 175.2; drafts of 136 rows
+// 83.6 / 81.8; encoders of 480 rows 419.6 / 410.3.  Over several blocks every warp would read the probabilities of eight groups once a block (2 sequences, 512 keys: 691 / 714 us an encode
+// pass), and tiles of up to four queries over four groups have too little to share (64 sequences, one query each: 161.6 / 166.2): those add partial outputs, in rows of 72 floats
+// that keep stores and loads out of each other's banks (68 before; 2 sequences, 512 keys: 693 / 686).
+template <bool PAGED, int MT, int KG, int KW, int NS, int QNC = 0, int ON = 0, bool SHARE = false>
+__global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW, SHARE)) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {
     using C = AttnCfg<MT, KG, KW>;
     static_assert((QNC == 0 && ON == 0) || (MT == 1 && KG == 8), "the projections are laid out for eight warps and 16 rows");
     static_assert(QNC == 0 || ON == 0 || ON == 2 * QNC, "one width");
     static_assert(NS >= 1 && NS <= 4 && KW % 16 == 0, "ring depth, keys per warp");
+    static_assert(!SHARE || (KG > 1 && MT == 1 && 16 * C::PP <= KW * 128), "key groups: one row tile, probabilities where the keys were");
     constexpr int THREADS = MT * KG * 32, KB = C::KB, NT = KW / 8, BM = MT * 16;
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ int s_nk[BM];
     __shared__ int s_nkmax;
     __shared__ __align__(8) uint64_t heads_bar;               // ON: counts the heads' rows as they arrive
     __shared__ int abort_s;
+    __shared__ float2 s_ml[SHARE ? KG : 1][16];                // (maximum, sum) of every key group and row
     const int b = a.seq_of ? a.seq_of[blockIdx.z] : (int)blockIdx.z, h = blockIdx.y, qt = blockIdx.x;
     if (b < 0) return;
     // Row metadata, page table and sequence lengths are written at the start of the step, before the first
@@ -358,7 +369,8 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
     const int nk0 = s_nk[mt * 16 + g], nk1 = s_nk[mt * 16 + g + 8];
     uint32_t qf[4][4];
     float m_run[2] = {-CUDART_INF_F, -CUDART_INF_F}, l_run[2] = {0.f, 0.f};   // rows g, g + 8 (sums: this lane's share)
-    float acc[8][4];
+    constexpr int NJ = SHARE ? 8 / KG : 8;       // 8-column tiles of a warp: all of them, or its share for every key group
+    float acc[8][4];                             // [column tile], [key group * NJ + column tile]
 #pragma unroll
     for (int j = 0; j < 8; ++j)
 #pragma unroll
@@ -371,7 +383,7 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
     for (int o = 4; o < 32; o <<= 1) nkall = min(nkall, __shfl_xor_sync(0xffffffffu, nkall, o));
 
     while (issued < min(ring, nblk)) issue();
-    for (int blk = 0; blk < nblk; ++blk) {
+    for (int blk = 0; blk < (SHARE ? 1 : nblk); ++blk) {
         cp_wait_pending(issued - blk - 1);
         __syncthreads();
         if (blk == 0) {
@@ -418,7 +430,7 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
             const float mn0 = fmaxf(m_run[0], bm0), mn1 = fmaxf(m_run[1], bm1);
             // a row with no visible key so far keeps maximum -inf: its terms are 0 against a base of 0
             const float mb0 = (mn0 == -CUDART_INF_F) ? 0.f : mn0 * sl, mb1 = (mn1 == -CUDART_INF_F) ? 0.f : mn1 * sl;
-            if (blk > 0) {
+            if (!SHARE && blk > 0) {
                 const float al0 = ex2(fmaf(m_run[0], sl, -mb0)), al1 = ex2(fmaf(m_run[1], sl, -mb1));      // (maximum -inf: 0, on sums that are 0)
                 l_run[0] *= al0; l_run[1] *= al1;
 #pragma unroll
@@ -439,6 +451,13 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
                     pf[hf * 2] = *reinterpret_cast<uint32_t*>(&p01);
                     pf[hf * 2 + 1] = *reinterpret_cast<uint32_t*>(&p23);
                 }
+                if constexpr (SHARE) {
+                    unsigned char* pr = sm + (Ks - Qs) + g * C::PP + kt * 32 + t4 * 4;
+                    if (kt == 0) __syncwarp();       // (all lanes' keys have been read)
+                    *reinterpret_cast<uint32_t*>(pr) = pf[0]; *reinterpret_cast<uint32_t*>(pr + 8 * C::PP) = pf[1];
+                    *reinterpret_cast<uint32_t*>(pr + 16) = pf[2]; *reinterpret_cast<uint32_t*>(pr + 8 * C::PP + 16) = pf[3];
+                    continue;
+                }
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     uint32_t vf[4];
@@ -448,7 +467,7 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
                 }
             }
         }
-        if (issued < nblk || (KG > 1 && blk + 1 == nblk)) __syncthreads();       // the stage is about to be overwritten (by a later block, or by the merge)
+        if (!SHARE && (issued < nblk || (KG > 1 && blk + 1 == nblk))) __syncthreads();       // the stage is about to be overwritten (by a later block, or by the merge)
         if (issued < nblk) issue();
     }
 
@@ -467,58 +486,122 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
             }
         }
     } else {
-        // ---- the key groups of a row tile meet in shared memory; each of its warps combines 64 / KG columns, in group order
-        float* mO = reinterpret_cast<float*>(Sp);                        // [MT][KG][16 rows][68]
-        float* mML = mO + MT * KG * 16 * 68;                             // [MT][KG][16 rows][maximum, sum]
-        float* po = mO + (mt * KG + kg) * 16 * 68;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            *reinterpret_cast<float2*>(po + g * 68 + j * 8 + t4 * 2) = make_float2(acc[j][0], acc[j][1]);
-            *reinterpret_cast<float2*>(po + (g + 8) * 68 + j * 8 + t4 * 2) = make_float2(acc[j][2], acc[j][3]);
-        }
-        if (t4 == 0) {
-            float* ml = mML + (mt * KG + kg) * 32;
-            ml[g * 2] = m_run[0]; ml[g * 2 + 1] = l_run[0];
-            ml[(g + 8) * 2] = m_run[1]; ml[(g + 8) * 2 + 1] = l_run[1];
-        }
-        __syncthreads();
-        constexpr int CW = 64 / KG, PER = CW / 2;                        // columns per warp; two lanes per row
-        const int rr = lane >> 1, c0 = kg * CW + (lane & 1) * PER, r = mt * 16 + rr;
-        float m = -CUDART_INF_F;
-        float f[KG];
-#pragma unroll
-        for (int q = 0; q < KG; ++q) { f[q] = mML[(mt * KG + q) * 32 + rr * 2]; m = fmaxf(m, f[q]); }
-        float den = 0.f;
-#pragma unroll
-        for (int q = 0; q < KG; ++q) {
-            f[q] = (f[q] == -CUDART_INF_F) ? 0.f : ex2((f[q] - m) * sl);
-            den = fmaf(mML[(mt * KG + q) * 32 + rr * 2 + 1], f[q], den);
-        }
-        const float inv = den > 0.f ? 1.0f / den : 0.f;
-        if constexpr (ON > 0) {
-            static_assert(PER == 4, "eight key groups");
-            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        [[maybe_unused]] float* mO = reinterpret_cast<float*>(Sp);       // [MT][KG][16 rows][72]
+        if constexpr (SHARE) {
+            // ---- every warp takes the probabilities of all groups, and of the values its own 64 / KG columns; the groups' shares are added in group order
+            if (t4 == 0) { s_ml[kg][g] = make_float2(m_run[0], l_run[0]); s_ml[kg][g + 8] = make_float2(m_run[1], l_run[1]); }
+            __syncthreads();
+            const uint32_t Vb = St + KB * 128;
 #pragma unroll
             for (int q = 0; q < KG; ++q) {
-                const float4 t = *reinterpret_cast<const float4*>(mO + ((mt * KG + q) * 16 + rr) * 68 + c0);
-                x.x = fmaf(t.x, f[q], x.x); x.y = fmaf(t.y, f[q], x.y); x.z = fmaf(t.z, f[q], x.z); x.w = fmaf(t.w, f[q], x.w);
+                if (q * KW >= nkmax) break;
+#pragma unroll
+                for (int kt = 0; kt < KW / 16; ++kt) {
+                    uint32_t pf[4], vf[4];
+                    ldsm_x4(St + q * KW * 128 + (lane & 15) * C::PP + kt * 32 + (lane >> 4) * 16, pf[0], pf[1], pf[2], pf[3]);
+                    const int t = q * KW + kt * 16 + (lane & 15);
+                    if constexpr (NJ == 1) {
+                        asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(vf[0]), "=r"(vf[1]) : "r"(Vb + swz(t, kg)));
+                        mma_bf16(acc[q], pf, vf[0], vf[1]);
+                    } else {
+                        ldsm_x4_t(Vb + swz(t, kg * 2 + (lane >> 4)), vf[0], vf[1], vf[2], vf[3]);
+                        mma_bf16(acc[q * NJ], pf, vf[0], vf[1]);
+                        mma_bf16(acc[q * NJ + 1], pf, vf[2], vf[3]);
+                    }
+                }
             }
-            __nv_bfloat162 p0 = __floats2bfloat162_rn(x.x * inv, x.y * inv), p1 = __floats2bfloat162_rn(x.z * inv, x.w * inv);
-            // this warp's eight columns of the 16 rows, 256 bytes in place of the queries, go to every CTA of the cluster as one copy
-            *reinterpret_cast<uint2*>(sm + kg * 256 + lane * 8) = make_uint2(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1));
+            float2 ma[KG], mb[KG];
+            float m0 = -CUDART_INF_F, m1 = -CUDART_INF_F, den0 = 0.f, den1 = 0.f;
+#pragma unroll
+            for (int q = 0; q < KG; ++q) { ma[q] = s_ml[q][g]; mb[q] = s_ml[q][g + 8]; m0 = fmaxf(m0, ma[q].x); m1 = fmaxf(m1, mb[q].x); }
+            float x[NJ][4];
+#pragma unroll
+            for (int j = 0; j < NJ; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) x[j][e] = 0.f;
+#pragma unroll
+            for (int q = 0; q < KG; ++q) {
+                const float f0 = ma[q].x == -CUDART_INF_F ? 0.f : ex2((ma[q].x - m0) * sl), f1 = mb[q].x == -CUDART_INF_F ? 0.f : ex2((mb[q].x - m1) * sl);
+                den0 = fmaf(ma[q].y, f0, den0); den1 = fmaf(mb[q].y, f1, den1);
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) {
+                    const float* t = acc[q * NJ + j];
+                    x[j][0] = fmaf(t[0], f0, x[j][0]); x[j][1] = fmaf(t[1], f0, x[j][1]); x[j][2] = fmaf(t[2], f1, x[j][2]); x[j][3] = fmaf(t[3], f1, x[j][3]);
+                }
+            }
+            const float inv0 = den0 > 0.f ? 1.0f / den0 : 0.f, inv1 = den1 > 0.f ? 1.0f / den1 : 0.f;
+            bf16* o = a.out + (size_t)(r0 + g) * a.out_stride + h * 64 + kg * 8 * NJ + t4 * 2;
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                const __nv_bfloat162 p0 = __floats2bfloat162_rn(x[j][0] * inv0, x[j][1] * inv0), p1 = __floats2bfloat162_rn(x[j][2] * inv1, x[j][3] * inv1);
+                if constexpr (ON > 0) {              // eight columns of the 16 rows, in place of the queries
+                    *reinterpret_cast<__nv_bfloat162*>(sm + kg * 256 + g * 16 + t4 * 4) = p0;
+                    *reinterpret_cast<__nv_bfloat162*>(sm + kg * 256 + (g + 8) * 16 + t4 * 4) = p1;
+                } else {
+                    if (g < nq) *reinterpret_cast<__nv_bfloat162*>(o + j * 8) = p0;
+                    if (g + 8 < nq) *reinterpret_cast<__nv_bfloat162*>(o + (size_t)8 * a.out_stride + j * 8) = p1;
+                }
+            }
+        } else {
+            // ---- the key groups of a row tile meet in shared memory; each of its warps combines 64 / KG columns, in group order.  (Rows 72 floats apart: neither
+            // the stores of the groups nor the loads across them meet in a bank.)
+            float* mML = mO + MT * KG * 16 * 72;                         // [MT][KG][16 rows][maximum, sum]
+            float* po = mO + (mt * KG + kg) * 16 * 72;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                *reinterpret_cast<float2*>(po + g * 72 + j * 8 + t4 * 2) = make_float2(acc[j][0], acc[j][1]);
+                *reinterpret_cast<float2*>(po + (g + 8) * 72 + j * 8 + t4 * 2) = make_float2(acc[j][2], acc[j][3]);
+            }
+            if (t4 == 0) {
+                float* ml = mML + (mt * KG + kg) * 32;
+                ml[g * 2] = m_run[0]; ml[g * 2 + 1] = l_run[0];
+                ml[(g + 8) * 2] = m_run[1]; ml[(g + 8) * 2 + 1] = l_run[1];
+            }
+            __syncthreads();
+            constexpr int CW = 64 / KG;                                  // columns per warp; two lanes per row take four of every eight
+            const int rr = lane >> 1, c0 = kg * CW + (lane & 1) * 4, r = mt * 16 + rr;
+            float m = -CUDART_INF_F;
+            float f[KG];
+#pragma unroll
+            for (int q = 0; q < KG; ++q) { f[q] = mML[(mt * KG + q) * 32 + rr * 2]; m = fmaxf(m, f[q]); }
+            float den = 0.f;
+#pragma unroll
+            for (int q = 0; q < KG; ++q) {
+                f[q] = (f[q] == -CUDART_INF_F) ? 0.f : ex2((f[q] - m) * sl);
+                den = fmaf(mML[(mt * KG + q) * 32 + rr * 2 + 1], f[q], den);
+            }
+            const float inv = den > 0.f ? 1.0f / den : 0.f;
+#pragma unroll
+            for (int c = 0; c < CW; c += 8) {
+                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int q = 0; q < KG; ++q) {
+                    const float4 t = *reinterpret_cast<const float4*>(mO + ((mt * KG + q) * 16 + rr) * 72 + c0 + c);
+                    x.x = fmaf(t.x, f[q], x.x); x.y = fmaf(t.y, f[q], x.y); x.z = fmaf(t.z, f[q], x.z); x.w = fmaf(t.w, f[q], x.w);
+                }
+                __nv_bfloat162 p0 = __floats2bfloat162_rn(x.x * inv, x.y * inv), p1 = __floats2bfloat162_rn(x.z * inv, x.w * inv);
+                const uint2 pk = make_uint2(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1));
+                if constexpr (ON > 0) *reinterpret_cast<uint2*>(sm + kg * 256 + lane * 8) = pk;          // eight columns of the 16 rows, in place of the queries
+                else if (r < nq) *reinterpret_cast<uint2*>(a.out + (size_t)(r0 + r) * a.out_stride + h * 64 + c0 + c) = pk;
+            }
+        }
+        if constexpr (ON > 0) {
+            static_assert(KG == 8, "eight key groups: eight columns a warp");
+            // the head's 64 columns, 2 KB, go to every CTA of the cluster as one copy, each issued by a warp of its own
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();                            // all 32 lanes' bytes are there before a lane copies them (the cluster barrier below was arrived at long before)
             cluster_wait();                          // every CTA of the cluster has begun and its barrier exists
-            if (lane < ON) {
+            __syncthreads();                         // (all warps' columns are there; what the stages held is dead)
+            if (warp < ON && lane == 0) {
                 uint32_t ra, rb;
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(oops + (h * 8 + kg) * 256), "r"(lane));
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_u32(&heads_bar)), "r"(lane));
-                asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], 256, [%2];"
-                             ::"r"(ra), "r"(Qs + kg * 256), "r"(rb) : "memory");
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(oops + h * 2048), "r"(warp));
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_u32(&heads_bar)), "r"(warp));
+                asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], 2048, [%2];"
+                             ::"r"(ra), "r"(Qs), "r"(rb) : "memory");
             }
+            __syncwarp();
             mbar_wait(smem_u32(&heads_bar), 0, &abort_s, oa.err_word, 12);
-            __syncthreads();                         // (the partial outputs of the key groups are dead)
-            cluster_arrive_relaxed();                // this CTA has what was sent to it
+            __syncwarp();
+            cluster_arrive_relaxed();                // this thread has seen what was sent to its CTA
             wo.template multiply<true>(oops, mO, warp, lane);
             __syncthreads();
             const float4 t = Proj64<OC::K>::sum(mO, tid);
@@ -526,19 +609,6 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW)) k_attn(At
                 *reinterpret_cast<float4*>(oa.x_out + (size_t)(r0 + (tid >> 4)) * OC::K + h * 64 + (tid & 15) * 4) =
                     make_float4(t.x + ob.x + res.x, t.y + ob.y + res.y, t.z + ob.z + res.z, t.w + ob.w + res.w);
             cluster_wait();                          // nobody leaves while a copy from its shared memory may be under way
-        } else if (r < nq) {
-            bf16* o = a.out + (size_t)(r0 + r) * a.out_stride + h * 64 + c0;
-#pragma unroll
-            for (int c = 0; c < PER; c += 4) {
-                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int q = 0; q < KG; ++q) {
-                    const float4 t = *reinterpret_cast<const float4*>(mO + ((mt * KG + q) * 16 + rr) * 68 + c0 + c);
-                    x.x = fmaf(t.x, f[q], x.x); x.y = fmaf(t.y, f[q], x.y); x.z = fmaf(t.z, f[q], x.z); x.w = fmaf(t.w, f[q], x.w);
-                }
-                __nv_bfloat162 p0 = __floats2bfloat162_rn(x.x * inv, x.y * inv), p1 = __floats2bfloat162_rn(x.z * inv, x.w * inv);
-                *reinterpret_cast<uint2*>(o + c) = make_uint2(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1));
-            }
         }
     }
 }

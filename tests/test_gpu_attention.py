@@ -67,6 +67,24 @@ def test_queries_projected_inside_the_attention(d, f, B, k, S):
     sd.close()
 
 
+@pytest.mark.parametrize("S,k", [(128, 4), (129, 4), (128, 3), (5, 5), (4, 2), (33, 20)])
+def test_key_groups_share_their_probabilities(S, k):
+    """Encoder self-attention and cross-attention of four key groups over one block of keys and over one key more, with as few queries as share and one less; groups without keys."""
+    from paper_2203_16487_b200 import binding
+    V = 515
+    dims = W.ModelDims(128, 2, 128, V, 2, 1, 512)
+    wv, wd = W.make_weights(dims, 85, True), W.make_weights(dims, 86, True)
+    mv, md = O.model_from(dims, wv, mode="bf16"), O.model_from(dims, wd, mode="bf16")
+    rng = np.random.default_rng(S + k)
+    srcs = [W.zipf_ids(rng, n, V) for n in (S, max(S // 3, 1), 1)]
+    sd = binding.SpecDec(dims, wv, dims, wd, k_max=k, max_batch=3, max_src=S, max_tgt=40, bf16=True)
+    sd.set_option("debug_checks", 1)
+    rep = lockstep.run(sd, mv, md, srcs, [40] * 3, k, 3, 1.0, margin=1e-3, check_logits_every=1, max_iters=3)
+    assert rep.ok, rep.notes
+    assert rep.max_logit_err < 2e-2 and rep.max_stat_err < 2e-2
+    sd.close()
+
+
 @pytest.mark.parametrize("d,B,k,S,cached", [
     (256, 1, 4, 12, False),          # 5 rows of one tile: the fewest
     (512, 1, 15, 128, False),        # 16 rows of eight heads, 8 CTAs: both attentions go on to their output projections; as many keys as fit beside the queries'
