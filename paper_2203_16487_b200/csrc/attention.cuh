@@ -177,7 +177,8 @@ constexpr int attn_ctas(int mt, int kg, int kw, bool share) { return kg > 1 ? (s
 // 83.6 / 81.8; encoders of 480 rows 419.6 / 410.3.  Over several blocks every warp would read the probabilities of eight groups once a block (2 sequences, 512 keys: 691 / 714 us an encode
 // pass), and tiles of up to four queries over four groups have too little to share (64 sequences, one query each: 161.6 / 166.2): those add partial outputs, in rows of 72 floats
 // that keep stores and loads out of each other's banks (68 before; 2 sequences, 512 keys: 693 / 686).
-template <bool PAGED, int MT, int KG, int KW, int NS, int QNC = 0, int ON = 0, bool SHARE = false>
+// (QNC and ON stay the last two: the test of the routes reads them off the kernel's name.)
+template <bool PAGED, int MT, int KG, int KW, int NS, bool SHARE = false, int QNC = 0, int ON = 0>
 __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW, SHARE)) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {
     using C = AttnCfg<MT, KG, KW>;
     static_assert((QNC == 0 && ON == 0) || (MT == 1 && KG == 8), "the projections are laid out for eight warps and 16 rows");

@@ -639,8 +639,8 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
                     KCHECK(h);
                     return 0;
                 };
-#define OUT_GO(SH) (n_heads == 4 ? goo(qp ? k_attn<false, 1, 8, 16, 3, 2, 4, SH> : paged ? k_attn<true, 1, 8, 16, 3, 0, 4, SH> : k_attn<false, 1, 8, 16, 3, 0, 4, SH>, qp ? ProjCfg<2, 4>::OPS : ProjCfg<0, 4>::OPS) \
-                                 : goo(qp ? k_attn<false, 1, 8, 16, 3, 4, 8, SH> : paged ? k_attn<true, 1, 8, 16, 3, 0, 8, SH> : k_attn<false, 1, 8, 16, 3, 0, 8, SH>, qp ? ProjCfg<4, 8>::OPS : ProjCfg<0, 8>::OPS))
+#define OUT_GO(SH) (n_heads == 4 ? goo(qp ? k_attn<false, 1, 8, 16, 3, SH, 2, 4> : paged ? k_attn<true, 1, 8, 16, 3, SH, 0, 4> : k_attn<false, 1, 8, 16, 3, SH, 0, 4>, qp ? ProjCfg<2, 4>::OPS : ProjCfg<0, 4>::OPS) \
+                                 : goo(qp ? k_attn<false, 1, 8, 16, 3, SH, 4, 8> : paged ? k_attn<true, 1, 8, 16, 3, SH, 0, 8> : k_attn<false, 1, 8, 16, 3, SH, 0, 8>, qp ? ProjCfg<4, 8>::OPS : ProjCfg<0, 8>::OPS))
                 return share ? OUT_GO(true) : OUT_GO(false);
 #undef OUT_GO
             }
@@ -654,7 +654,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
                 // (64-wide heads: the width is 64 n_heads.)  More than 128 keys in blocks of 256 where shared memory has room for two: sources of 512 tokens, 8
                 // sequences decoded 7834 -> 7757 us, 2 sequences 5660 -> 5528; verify step over 233 keys 236 -> 234.
                 switch (n_heads) {
-#define QUERY_GO(KW, NS, QNC, SH) goq(k_attn<false, 1, 8, KW, NS, QNC, 0, SH>, AttnCfg<1, 8, KW>::smem(max_keys, NS, false, QueryCfg<QNC>::OPS))
+#define QUERY_GO(KW, NS, QNC, SH) goq(k_attn<false, 1, 8, KW, NS, SH, QNC>, AttnCfg<1, 8, KW>::smem(max_keys, NS, false, QueryCfg<QNC>::OPS))
                     case 4: return share ? QUERY_GO(16, 3, 2, true) : QUERY_GO(32, 2, 2, false);
                     case 8: return share ? QUERY_GO(16, 3, 4, true) : QUERY_GO(32, 2, 4, false);
                     default: return share ? QUERY_GO(16, 3, 6, true) : QUERY_GO(16, 3, 6, false);
@@ -676,7 +676,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             if (spread) {
                 const bool eight = h->attn_warps ? h->attn_warps == 8 : (max_keys > 256 && tiles16 <= h->tma.n_sm);
                 if (!eight && share && q_ub > 4)
-                    return paged ? go(k_attn<true, 1, 4, 32, 3, 0, 0, true>, 16, 4, AttnCfg<1, 4, 32>::smem(max_keys, 3, true)) : go(k_attn<false, 1, 4, 32, 3, 0, 0, true>, 16, 4, AttnCfg<1, 4, 32>::smem(max_keys, 3, false));
+                    return paged ? go(k_attn<true, 1, 4, 32, 3, true>, 16, 4, AttnCfg<1, 4, 32>::smem(max_keys, 3, true)) : go(k_attn<false, 1, 4, 32, 3, true>, 16, 4, AttnCfg<1, 4, 32>::smem(max_keys, 3, false));
                 return eight ? ATTN_GO(1, 8, 32, 2) : ATTN_GO(1, 4, 32, 3);
             }
             // Otherwise 64 or 32 queries per CTA, a warp for every 16: 64 share one pass over the keys (51 queries x 307 keys, 128
@@ -1640,13 +1640,13 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
             else if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048);
         };
 #define ATTN_ROOM(MT, KG, KW, NS) room(k_attn<true, MT, KG, KW, NS>, AttnCfg<MT, KG, KW>::smem(max_keys, NS, true)); room(k_attn<false, MT, KG, KW, NS>, 0)
-        room(k_attn<false, 1, 8, 16, 3, 2, 0, true>, 0); room(k_attn<false, 1, 8, 16, 3, 4, 0, true>, 0); room(k_attn<false, 1, 8, 16, 3, 6, 0, true>, 0); room(k_attn<false, 1, 8, 16, 3, 6>, 0);   // (at most 222 KB: no table of rows)
-        room(k_attn<false, 1, 8, 32, 2, 2>, 0); room(k_attn<false, 1, 8, 32, 2, 4>, 0);
-        room(k_attn<false, 1, 8, 16, 3, 2, 4>, 0); room(k_attn<true, 1, 8, 16, 3, 0, 4>, 0); room(k_attn<false, 1, 8, 16, 3, 0, 4>, 0);
-        room(k_attn<false, 1, 8, 16, 3, 2, 4, true>, 0); room(k_attn<true, 1, 8, 16, 3, 0, 4, true>, 0); room(k_attn<false, 1, 8, 16, 3, 0, 4, true>, 0);
-        room(k_attn<false, 1, 8, 16, 3, 4, 8>, 0); room(k_attn<true, 1, 8, 16, 3, 0, 8>, 0); room(k_attn<false, 1, 8, 16, 3, 0, 8>, 0);
-        room(k_attn<false, 1, 8, 16, 3, 4, 8, true>, 0); room(k_attn<true, 1, 8, 16, 3, 0, 8, true>, 0); room(k_attn<false, 1, 8, 16, 3, 0, 8, true>, 0);
-        room(k_attn<true, 1, 4, 32, 3, 0, 0, true>, 0); room(k_attn<false, 1, 4, 32, 3, 0, 0, true>, 0);
+        room(k_attn<false, 1, 8, 16, 3, true, 2>, 0); room(k_attn<false, 1, 8, 16, 3, true, 4>, 0); room(k_attn<false, 1, 8, 16, 3, true, 6>, 0); room(k_attn<false, 1, 8, 16, 3, false, 6>, 0);   // (at most 222 KB: no table of rows)
+        room(k_attn<false, 1, 8, 32, 2, false, 2>, 0); room(k_attn<false, 1, 8, 32, 2, false, 4>, 0);
+        room(k_attn<false, 1, 8, 16, 3, false, 2, 4>, 0); room(k_attn<true, 1, 8, 16, 3, false, 0, 4>, 0); room(k_attn<false, 1, 8, 16, 3, false, 0, 4>, 0);
+        room(k_attn<false, 1, 8, 16, 3, true, 2, 4>, 0); room(k_attn<true, 1, 8, 16, 3, true, 0, 4>, 0); room(k_attn<false, 1, 8, 16, 3, true, 0, 4>, 0);
+        room(k_attn<false, 1, 8, 16, 3, false, 4, 8>, 0); room(k_attn<true, 1, 8, 16, 3, false, 0, 8>, 0); room(k_attn<false, 1, 8, 16, 3, false, 0, 8>, 0);
+        room(k_attn<false, 1, 8, 16, 3, true, 4, 8>, 0); room(k_attn<true, 1, 8, 16, 3, true, 0, 8>, 0); room(k_attn<false, 1, 8, 16, 3, true, 0, 8>, 0);
+        room(k_attn<true, 1, 4, 32, 3, true>, 0); room(k_attn<false, 1, 4, 32, 3, true>, 0);
         ATTN_ROOM(1, 4, 32, 3); ATTN_ROOM(1, 8, 32, 2); ATTN_ROOM(4, 1, 64, 2); ATTN_ROOM(2, 1, 64, 3); ATTN_ROOM(2, 1, 32, 3);
         if (e != cudaSuccess) { cudaGetLastError(); h->use_tc_attn = 0; }
         if (sd::tc_init(h->tma, h->ses.counters + 7) != 0) h->use_tc = 0;     // reported through specdec_last_error; SIMT GEMM still runs on the GPU
