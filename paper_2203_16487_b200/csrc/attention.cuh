@@ -139,6 +139,8 @@ struct Proj64 {
     }
 };
 
+constexpr int ATTN_SMEM = 227 * 1024 - 2048;              // dynamic shared memory of a CTA; the rest is for what the kernel declares
+
 // MT row tiles of 16 queries x KG key groups = MT KG warps; a key block holds KW keys for each group; NS stages.
 template <int MT, int KG, int KW>
 struct AttnCfg {
@@ -147,7 +149,7 @@ struct AttnCfg {
     static constexpr int PP = KW * 2 + 16;                                // bytes per row of a key group's probabilities: 16 rows, in place of the group's keys
     static constexpr int MERGE = KG > 1 ? MT * KG * 16 * (72 + 2) * 4 : 0;     // partial outputs (padded rows) and (maximum, sum); reuses the stages
     // queries, ring (or merge buffers), operands of the projections, and for paged keys the table of their rows
-    static size_t smem(int max_keys, int ns, bool paged, int query_bytes = 0) {
+    static constexpr size_t smem(int max_keys, int ns, bool paged, int query_bytes = 0) {
         const int nb = (max_keys + KB - 1) / KB;
         const size_t ring = (size_t)(nb < ns ? (nb < 1 ? 1 : nb) : ns) * STAGE;
         return (size_t)MT * 2048 + (ring > MERGE ? ring : MERGE) + query_bytes + (paged ? (size_t)((max_keys + 3) & ~3) * 4 : 0);

@@ -639,8 +639,9 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
                     KCHECK(h);
                     return 0;
                 };
-#define OUT_GO(SH) (n_heads == 4 ? goo(qp ? k_attn<false, 1, 8, 16, 3, SH, 2, 4> : paged ? k_attn<true, 1, 8, 16, 3, SH, 0, 4> : k_attn<false, 1, 8, 16, 3, SH, 0, 4>, qp ? ProjCfg<2, 4>::OPS : ProjCfg<0, 4>::OPS) \
-                                 : goo(qp ? k_attn<false, 1, 8, 16, 3, SH, 4, 8> : paged ? k_attn<true, 1, 8, 16, 3, SH, 0, 8> : k_attn<false, 1, 8, 16, 3, SH, 0, 8>, qp ? ProjCfg<4, 8>::OPS : ProjCfg<0, 8>::OPS))
+                if (qp) return n_heads == 4 ? goo(k_attn<false, 1, 8, 16, 3, true, 2, 4>, ProjCfg<2, 4>::OPS) : goo(k_attn<false, 1, 8, 16, 3, true, 4, 8>, ProjCfg<4, 8>::OPS);     // (one block of keys: see out_inside)
+#define OUT_GO(SH) (n_heads == 4 ? goo(paged ? k_attn<true, 1, 8, 16, 3, SH, 0, 4> : k_attn<false, 1, 8, 16, 3, SH, 0, 4>, ProjCfg<0, 4>::OPS) \
+                                 : goo(paged ? k_attn<true, 1, 8, 16, 3, SH, 0, 8> : k_attn<false, 1, 8, 16, 3, SH, 0, 8>, ProjCfg<0, 8>::OPS))
                 return share ? OUT_GO(true) : OUT_GO(false);
 #undef OUT_GO
             }
@@ -773,7 +774,9 @@ bool out_inside(const specdec_handle* h, int d_head, int q_ub, int n_heads, int 
     const long long ctas = (long long)cdiv(q_ub, 16) * n_heads * (cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub));
     if (ctas > (use == OUT_GATHERS ? 96 : n_heads == 8 ? (use == OUT_QUERIES ? 16 : 8) : use == OUT_QUERIES ? 32 : 64) || (use == OUT_QUERIES && rows_ub > 48)) return false;
     const int ops = use == OUT_QUERIES ? ProjCfg<4, 8>::OPS : ProjCfg<0, 8>::OPS;
-    return AttnCfg<1, 8, 16>::smem(max_keys, 3, use != OUT_QUERIES, ops) <= 227 * 1024 - 2048;      // (with the queries: up to 128 keys)
+    static_assert(AttnCfg<1, 8, 16>::smem(128, 3, false, ProjCfg<4, 8>::OPS) <= ATTN_SMEM && AttnCfg<1, 8, 16>::smem(129, 3, false, ProjCfg<4, 8>::OPS) > ATTN_SMEM,
+                  "both projections inside: one block of keys, so k_attn's groups share their probabilities");
+    return AttnCfg<1, 8, 16>::smem(max_keys, 3, use != OUT_QUERIES, ops) <= ATTN_SMEM;
 }
 
 // One pre-LN block on `rows_ub` rows of the residual stream x (encoder: no cross-attention).
@@ -1636,15 +1639,15 @@ int specdec_create(const specdec_config* cfg, const specdec_tensor* weights, int
         const int max_keys = std::max(h->S_cap, h->T_cap + h->k_cap + 1);
         cudaError_t e = cudaSuccess;
         auto room = [&](auto* kernel, size_t smem) {
-            if (smem > 227 * 1024 - 2048) h->use_tc_attn = 0;
-            else if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048);
+            if (smem > ATTN_SMEM) h->use_tc_attn = 0;
+            else if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ATTN_SMEM);
         };
 #define ATTN_ROOM(MT, KG, KW, NS) room(k_attn<true, MT, KG, KW, NS>, AttnCfg<MT, KG, KW>::smem(max_keys, NS, true)); room(k_attn<false, MT, KG, KW, NS>, 0)
         room(k_attn<false, 1, 8, 16, 3, true, 2>, 0); room(k_attn<false, 1, 8, 16, 3, true, 4>, 0); room(k_attn<false, 1, 8, 16, 3, true, 6>, 0); room(k_attn<false, 1, 8, 16, 3, false, 6>, 0);   // (at most 222 KB: no table of rows)
         room(k_attn<false, 1, 8, 32, 2, false, 2>, 0); room(k_attn<false, 1, 8, 32, 2, false, 4>, 0);
-        room(k_attn<false, 1, 8, 16, 3, false, 2, 4>, 0); room(k_attn<true, 1, 8, 16, 3, false, 0, 4>, 0); room(k_attn<false, 1, 8, 16, 3, false, 0, 4>, 0);
+        room(k_attn<true, 1, 8, 16, 3, false, 0, 4>, 0); room(k_attn<false, 1, 8, 16, 3, false, 0, 4>, 0);
         room(k_attn<false, 1, 8, 16, 3, true, 2, 4>, 0); room(k_attn<true, 1, 8, 16, 3, true, 0, 4>, 0); room(k_attn<false, 1, 8, 16, 3, true, 0, 4>, 0);
-        room(k_attn<false, 1, 8, 16, 3, false, 4, 8>, 0); room(k_attn<true, 1, 8, 16, 3, false, 0, 8>, 0); room(k_attn<false, 1, 8, 16, 3, false, 0, 8>, 0);
+        room(k_attn<true, 1, 8, 16, 3, false, 0, 8>, 0); room(k_attn<false, 1, 8, 16, 3, false, 0, 8>, 0);
         room(k_attn<false, 1, 8, 16, 3, true, 4, 8>, 0); room(k_attn<true, 1, 8, 16, 3, true, 0, 8>, 0); room(k_attn<false, 1, 8, 16, 3, true, 0, 8>, 0);
         room(k_attn<true, 1, 4, 32, 3, true>, 0); room(k_attn<false, 1, 4, 32, 3, true>, 0);
         ATTN_ROOM(1, 4, 32, 3); ATTN_ROOM(1, 8, 32, 2); ATTN_ROOM(4, 1, 64, 2); ATTN_ROOM(2, 1, 64, 3); ATTN_ROOM(2, 1, 32, 3);
