@@ -139,6 +139,7 @@ struct Proj64 {
     }
 };
 
+constexpr int SHARE_KEYS = 128;                           // up to so many keys the groups share probabilities: the one block of every SHARE kernel
 constexpr int ATTN_SMEM = 227 * 1024 - 2048;              // dynamic shared memory of a CTA; the rest is for what the kernel declares
 
 // MT row tiles of 16 queries x KG key groups = MT KG warps; a key block holds KW keys for each group; NS stages.
@@ -186,7 +187,8 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW, SHARE)) k_
     static_assert((QNC == 0 && ON == 0) || (MT == 1 && KG == 8), "the projections are laid out for eight warps and 16 rows");
     static_assert(QNC == 0 || ON == 0 || ON == 2 * QNC, "one width");
     static_assert(NS >= 1 && NS <= 4 && KW % 16 == 0, "ring depth, keys per warp");
-    static_assert(!SHARE || (KG > 1 && MT == 1 && 16 * C::PP <= KW * 128), "key groups: one row tile, probabilities where the keys were");
+    static_assert(!SHARE || C::KB >= SHARE_KEYS, "one block holds all keys: there is no second pass");
+    static_assert(!SHARE || ((KG == 4 || KG == 8) && MT == 1 && 16 * C::PP <= KW * 128), "a warp's one or two 8-column tiles, one row tile, probabilities where the keys were");
     constexpr int THREADS = MT * KG * 32, KB = C::KB, NT = KW / 8, BM = MT * 16;
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ int s_nk[BM];
@@ -459,14 +461,14 @@ __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW, SHARE)) k_
                     if (kt == 0) __syncwarp();       // (all lanes' keys have been read)
                     *reinterpret_cast<uint32_t*>(pr) = pf[0]; *reinterpret_cast<uint32_t*>(pr + 8 * C::PP) = pf[1];
                     *reinterpret_cast<uint32_t*>(pr + 16) = pf[2]; *reinterpret_cast<uint32_t*>(pr + 8 * C::PP + 16) = pf[3];
-                    continue;
-                }
+                } else {
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    uint32_t vf[4];
-                    ldsm_x4_t(Vs + swz(kt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, v * 2 + (lane >> 4)), vf[0], vf[1], vf[2], vf[3]);
-                    mma_bf16(acc[2 * v], pf, vf[0], vf[1]);
-                    mma_bf16(acc[2 * v + 1], pf, vf[2], vf[3]);
+                    for (int v = 0; v < 4; ++v) {
+                        uint32_t vf[4];
+                        ldsm_x4_t(Vs + swz(kt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, v * 2 + (lane >> 4)), vf[0], vf[1], vf[2], vf[3]);
+                        mma_bf16(acc[2 * v], pf, vf[0], vf[1]);
+                        mma_bf16(acc[2 * v + 1], pf, vf[2], vf[3]);
+                    }
                 }
             }
         }

@@ -627,7 +627,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             const AttnSlots slots = attn_slots(h, cnt, q_ub, n_heads);
             a.seq_of = slots.seq_of;
             const int n_seq = cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub);
-            const bool share = max_keys <= 128;              // one block of keys: the groups share their probabilities (see k_attn), with four groups from five queries on
+            const bool share = max_keys <= SHARE_KEYS;              // one block of keys: the groups share their probabilities (see k_attn), with four groups from five queries on
             QueryArgs qa{};
             OutArgs oa{};
             if (qp) qa = *qp;
@@ -774,7 +774,7 @@ bool out_inside(const specdec_handle* h, int d_head, int q_ub, int n_heads, int 
     const long long ctas = (long long)cdiv(q_ub, 16) * n_heads * (cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub));
     if (ctas > (use == OUT_GATHERS ? 96 : n_heads == 8 ? (use == OUT_QUERIES ? 16 : 8) : use == OUT_QUERIES ? 32 : 64) || (use == OUT_QUERIES && rows_ub > 48)) return false;
     const int ops = use == OUT_QUERIES ? ProjCfg<4, 8>::OPS : ProjCfg<0, 8>::OPS;
-    static_assert(AttnCfg<1, 8, 16>::smem(128, 3, false, ProjCfg<4, 8>::OPS) <= ATTN_SMEM && AttnCfg<1, 8, 16>::smem(129, 3, false, ProjCfg<4, 8>::OPS) > ATTN_SMEM,
+    static_assert(AttnCfg<1, 8, 16>::smem(SHARE_KEYS, 3, false, ProjCfg<4, 8>::OPS) <= ATTN_SMEM && AttnCfg<1, 8, 16>::smem(SHARE_KEYS + 1, 3, false, ProjCfg<4, 8>::OPS) > ATTN_SMEM,
                   "both projections inside: one block of keys, so k_attn's groups share their probabilities");
     return AttnCfg<1, 8, 16>::smem(max_keys, 3, use != OUT_QUERIES, ops) <= ATTN_SMEM;
 }

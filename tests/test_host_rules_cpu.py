@@ -83,3 +83,17 @@ def test_the_maps_of_a_launch_survive_the_eviction_between_them(wrong):
 
 def test_every_row_of_the_few_rows_vocabulary_kernel_has_a_cta(wrong):
     assert wrong["rows_without_a_cta"] == 0
+
+
+@pytest.mark.parametrize("kg,kw,message", [
+    (4, 32, None),
+    (2, 64, "8-column tiles"),                           # would leave half of the output's columns zero
+    (4, 16, "no second pass"),                           # would leave out the keys beyond its one block
+])
+def test_key_groups_share_probabilities_in_the_forms_the_kernel_handles(kg, kw, message, tmp_path):
+    src = tmp_path / "k.cu"
+    src.write_text('#include "attention.cuh"\n'
+                   f"template __global__ void sd::k_attn<false, 1, {kg}, {kw}, 3, true>(sd::AttnTcArgs, sd::QueryArgs, sd::OutArgs);\n")
+    r = subprocess.run([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-I" + build.CSRC, "-cubin",
+                        "-o", str(tmp_path / "k.out"), str(src)], capture_output=True, text=True)
+    assert (r.returncode == 0) == (message is None) and (message or "") in r.stderr, r.stderr
