@@ -3,10 +3,12 @@ over key counts at the edges of its key blocks (32 a warp, 64, 128, 256 a block)
 than one block, query counts at the edges of the query tiles, cached prefixes that end inside a block."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import specdec_oracle as O
 from paper_2203_16487_b200 import workloads as W
 from tests import lockstep
+from tests.test_gpu_routes import launched
 
 pytestmark = pytest.mark.gpu
 
@@ -93,7 +95,7 @@ def test_key_groups_share_their_probabilities(S, k):
     (512, 1, 32, 128, False),        # 33 rows, 24 CTAs: neither
     (256, 2, 23, 128, False),        # four heads, 48 rows: the most with the queries projected too
     (256, 1, 48, 128, True),         # 49 rows: the self-attention only
-    (256, 3, 16, 300, True),         # three stages of keys
+    (256, 3, 16, 300, True),         # 300 keys: the self-attention only; the cross-attention projects its queries (two blocks of 256)
 ])
 def test_output_projected_inside_the_attention(d, B, k, S, cached):
     """Attention of few rows that goes on to the output projection and the residual, self- and cross-attention, the drafter's [MASK] rows among them."""
@@ -111,6 +113,98 @@ def test_output_projected_inside_the_attention(d, B, k, S, cached):
     assert rep.ok, rep.notes
     assert rep.max_logit_err < 2e-2 and rep.max_stat_err < 2e-2
     sd.close()
+
+
+def _weights(d, seed, V, layers=2):
+    """A verifier or drafter whose self-attention counts: leaving out one of 130 keys moves the oracle's logits by 2e-2 (512 columns) and 8e-3 (256), a group of 16 keys by 0.2."""
+    dims = W.ModelDims(d, d // 64, 128, V, 1, layers, 512)
+    w = W.make_weights(dims, seed, True)
+    for name in w:
+        if name.endswith((".self.v.w", ".self.o.w")):
+            w[name] = w[name] * 4
+    return dims, w
+
+
+@pytest.mark.parametrize("d,B,k,S,blocks,cached", [
+    (512, 1, 15, 12, 8, False),      # a prefix of 112: 128 keys, one block; the draft over 144 (eight heads, its last layer)
+    (512, 1, 12, 12, 10, True),      # 130 keys: two in the second block
+    (512, 1, 15, 12, 17, False),     # 272 keys
+    (512, 1, 15, 12, 26, True),      # 416 keys: the ring of three blocks wraps
+    (256, 1, 42, 129, 3, False),     # 129 keys: one in the second block, of encoder and decoder; 43 rows, the drafter's other layer in 11 tiles
+    (256, 2, 23, 128, 12, True),     # 288 keys, four tiles; the encoder over one block in 64 CTAs
+    (256, 1, 15, 256, 17, False),    # an encoder of 256 keys in 64 CTAs, two whole blocks
+])
+def test_output_projected_inside_over_several_key_blocks(d, B, k, S, blocks, cached):
+    """Heads of a tile as one cluster behind a merge of partial outputs (more keys than one block holds): encoder, verifier over its paged prefix, the drafter's last layer."""
+    from paper_2203_16487_b200 import binding
+    V, T = 515, 430
+    (dims, wv), (_, wd) = _weights(d, 87, V), _weights(d, 88, V)
+    mv, md = O.model_from(dims, wv, mode="bf16"), O.model_from(dims, wd, mode="bf16")
+    rng = np.random.default_rng(d + blocks)
+    srcs = [W.zipf_ids(rng, n, V) for n in [S, max(S // 2, 1)][:B]]
+    sd = binding.SpecDec(dims, wv, dims, wd, k_max=k, max_batch=B, max_src=S, max_tgt=T, bf16=True)
+    sd.set_option("graphs", 0)                           # (the number of keys as it is, not rounded up)
+    sd.set_option("debug_checks", 1)
+    # every draft is accepted: the prefix is random tokens, k + 1 more a step
+    rep = lockstep.run(sd, mv, md, srcs, [T] * B, k, V, 1e9, margin=8e-3, check_logits_every=1, max_iters=blocks,
+                       draft_fn=lambda b, out, n: rng.integers(4, V, size=n).astype(np.int32), drafter_reading="prefix_causal" if cached else "bidirectional")
+    assert rep.ok, rep.notes
+    assert [len(o) for o in rep.outputs] == [blocks * (k + 1)] * B
+    # What rounding to bf16 moves the oracle's logits of these rows by; as far on the other side of the unrounded ones another correct order of the sums may be.
+    fv, fd = O.model_from(dims, wv, mode="pure"), O.model_from(dims, wd, mode="pure")
+
+    def rounding(m, f, tokens, b, **mask):
+        x, y = (O.decoder_rows(o, [W.BOS_ID] + tokens, O.encode(o, srcs[b]), **mask) for o in (m, f))
+        return x, 2 * np.abs(x - y).max()
+
+    tol = max(rounding(mv, fv, rep.outputs[b], b, causal=True)[1] for b in range(B))
+    assert tol < 2e-2 and rep.max_logit_err < tol and rep.max_stat_err < tol, (rep.max_logit_err, rep.max_stat_err, tol)
+    drafts = sd.draft(k).cpu().numpy()
+    for b in range(B):
+        out = rep.outputs[b]
+        logits, tol = rounding(md, fd, out + [W.MASK_ID] * k, b, causal=False, n_causal=len(out) + 1 if cached else None)
+        logits = logits[len(out) + 1:]
+        gap = logits.max(axis=1) - logits[np.arange(k), drafts[b]]
+        assert gap.max() < 2 * tol, (b, gap)             # (two logits)
+    # ... by the kernels that this is about: share, queries inside, output inside
+    sd.set_option("debug_checks", 0)
+    buf, acc = torch.zeros((B, k), dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda")
+    self_attn = [n for n in launched(lambda: sd.verify_raw(buf, 1, 0.0, acc, acc)) if n.startswith("k_attn<1")]
+    assert self_attn == [f"k_attn<1,1,8,16,3,0,0,{d // 64}>"] * 2, self_attn
+    last = [n for n in launched(lambda: sd.draft(k)) if n.startswith(f"k_attn<{int(cached)}")]
+    assert f"k_attn<{int(cached)},1,8,16,3,0,0,{d // 64}>" in last, last
+    if d == 256:
+        src = W.pad_batch(srcs)
+        src = [torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).cuda() for a in src]
+        assert [n for n in launched(lambda: sd.encode(*src)) if n.startswith("k_attn<")] == [f"k_attn<0,1,8,16,3,{int(S <= 128)},0,4>"] * 2
+    sd.close()
+
+
+@pytest.mark.parametrize("d", [128, 256, 512, 768])
+def test_shared_probabilities_give_the_same_bits(d):
+    """The same 16 rows over the same 127 keys, once in a session that could hold no more keys and once where the launch has to allow for a second block."""
+    from paper_2203_16487_b200 import binding
+    V, k = 515, 15
+    dims, w = _weights(d, 89, V)
+    rng = np.random.default_rng(d)
+    src, lens = W.pad_batch([W.zipf_ids(rng, 33, V)])
+    blocks = [rng.integers(4, V, size=(1, k)).astype(np.int32) for _ in range(9)]
+    got, kernels = [], []
+    for max_tgt in (112, 200):
+        sd = binding.SpecDec(dims, w, dims, w, k_max=k, max_batch=1, max_src=33, max_tgt=max_tgt, bf16=True)
+        sd.set_option("graphs", 0)
+        sd.encode(src, lens, np.array([max_tgt], np.int32))
+        for i in range(8):                               # 111 tokens: as far as the launches can know, min(8 * 16, max_tgt)
+            sd.verify(blocks[i], V, 1e9)
+            sd.commit(np.array([5 if i == 0 else 14], np.int32), np.array([9], np.int32))
+        sd.verify(blocks[8], V, 1e9)
+        got.append(sd.debug_logits(0, k + 1).cpu().numpy())
+        buf, acc = torch.zeros((1, k), dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+        kernels.append(launched(lambda: sd.verify_raw(buf, 1, 0.0, acc, acc)))
+        sd.close()
+    one, two = kernels
+    assert one != two and [n.replace(",3,1,", ",3,0,") if n.startswith("k_attn<1") else n for n in one] == two, kernels
+    assert np.abs(got[0]).max() > 0.1 and np.array_equal(got[0], got[1])
 
 
 @pytest.mark.parametrize("bf16,d,H,cached", [(True, 256, 4, False), (True, 256, 4, True), (True, 512, 8, False), (True, 512, 8, True),

@@ -39,6 +39,15 @@ def _kernels(graph):
     return names
 
 
+def launched(call):
+    """Names of the kernels that a step call launches (a handle without graphs: its launches go into the capture)."""
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        call()
+    return _kernels(g)
+
+
 def _step(dims, step, B, k, S):
     from paper_2203_16487_b200 import binding
     wv, wd = W.make_weights(dims, 5, True), W.make_weights(dims, 6, True)
@@ -149,3 +158,29 @@ def test_projections_inside_the_attention(d, B, k, S, self_out, cross_q, cross_o
     names = _step(W.ModelDims(d, d // 64, 2 * d, 515, 1, 1, 256), "verify", B, k, S)
     (_, s_out), (c_q, c_out) = ([int(v) > 0 for v in n[:-1].split(",")[-2:]] for n in names if n.startswith("k_attn<"))
     assert (s_out, c_q, c_out) == (self_out, cross_q, cross_out), names
+
+
+# One layer: the attention kernels of a verify step (self, cross) or of the two encoders.  Over at most 128 keys the key groups share their probabilities (the sixth argument), four
+# groups from five queries on.
+@pytest.mark.parametrize("step,d,k,S,kernels", [
+    ("verify", 128, 4, 128, "1,1,4,32,3,1,0,0 0,1,4,32,3,1,0,0"),       # 5 queries
+    ("verify", 128, 4, 129, "1,1,4,32,3,1,0,0 0,1,4,32,3,0,0,0"),       # a key more
+    ("verify", 128, 3, 128, "1,1,4,32,3,0,0,0 0,1,4,32,3,0,0,0"),       # 4 queries
+    ("verify", 512, 3, 128, "1,1,4,32,3,0,0,0 0,1,8,16,3,1,4,0"),       # eight groups share from one query on
+    ("verify", 512, 0, 128, "1,1,4,32,3,0,0,0 0,1,8,16,3,1,4,0"),
+    ("verify", 512, 3, 129, "1,1,4,32,3,0,0,0 0,1,8,32,2,0,4,0"),
+    ("verify", 256, 4, 128, "1,1,8,16,3,1,0,4 0,1,8,16,3,1,2,4"),
+    ("verify", 256, 4, 129, "1,1,8,16,3,1,0,4 0,1,8,32,2,0,2,0"),       # no room for both projections beside a second block
+    ("verify", 512, 15, 128, "1,1,8,16,3,1,0,8 0,1,8,16,3,1,4,8"),
+    ("verify", 768, 4, 128, "1,1,4,32,3,1,0,0 0,1,8,16,3,1,6,0"),
+    ("verify", 768, 4, 129, "1,1,4,32,3,1,0,0 0,1,8,16,3,0,6,0"),
+    ("encode", 128, 0, 128, "0,1,4,32,3,1,0,0 0,1,4,32,3,1,0,0"),
+    ("encode", 128, 0, 129, "0,1,4,32,3,0,0,0 0,1,4,32,3,0,0,0"),
+    ("encode", 128, 0, 5, "0,1,4,32,3,1,0,0 0,1,4,32,3,1,0,0"),
+    ("encode", 128, 0, 4, "0,1,4,32,3,0,0,0 0,1,4,32,3,0,0,0"),
+    ("encode", 256, 0, 128, "0,1,8,16,3,1,0,4 0,1,8,16,3,1,0,4"),
+    ("encode", 256, 0, 129, "0,1,8,16,3,0,0,4 0,1,8,16,3,0,0,4"),
+])
+def test_key_groups_share_probabilities_over_one_block(step, d, k, S, kernels):
+    names = _step(W.ModelDims(d, d // 64, 2 * d, 515, 1, 1, 256), step, 1, k, S)
+    assert [n for n in names if n.startswith("k_attn<")] == [f"k_attn<{a}>" for a in kernels.split()], names
