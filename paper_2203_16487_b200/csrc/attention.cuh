@@ -3,10 +3,11 @@
 //
 // K and V walk through a ring of NS cp.async stages (128-byte rows, XOR-swizzled 16-byte chunks).  Warp (row tile mt, key group
 // kg) takes KW keys of every block for 16 queries: S = Q K^T (mma.sync m16n8k16, fp32 accumulation), running row maximum and
-// sum in registers, P (bf16, relative to the running maximum) straight from the score registers into the second
-// contraction; the result is divided by the fp32 sum of the unrounded exponentials.  (A bf16 value keeps its relative precision whatever the
-// maximum it is taken relative to: against 64 bits the result is 1.0e-3 off with the running maximum where it is 1.2e-3 with the row's, 512 keys.)  With KG > 1 the key groups of a row tile
-// meet in shared memory at the end, added in group order.  Work per CTA is 64 keys x 64 x 16 MT x 4 flops a block: too little to
+// sum in registers, P (bf16, relative to the running maximum); the result is divided by the fp32 sum of the unrounded exponentials.  (A bf16 value keeps its relative precision whatever the
+// maximum it is taken relative to: against 64 bits the result is 1.0e-3 off with the running maximum where it is 1.2e-3 with the row's, 512 keys.)
+// P goes straight from the score registers into the second contraction, and with KG > 1 the partial outputs of a row tile's key groups meet in shared memory at the
+// end, added in group order; or, over one block of keys (SHARE), every group leaves its P in shared memory where its keys were, and each warp contracts all groups' P with its own
+// slice of V's columns.  Work per CTA is 64 keys x 64 x 16 MT x 4 flops a block: too little to
 // fill a 128-row tcgen05 tile, which is why this contraction uses warp-level MMA (8 clocks each per scheduler, measured).
 //
 // What bounds it.  Few CTAs: the chain of round trips of one CTA.  Everything that predates the step -- row counts, the page
@@ -158,7 +159,8 @@ struct AttnCfg {
 };
 
 // CTAs per SM that the registers are cut for; 0 leaves it to the compiler (told 1, it takes 148 registers for MT = 1, KG = 4 where 100 do, and the
-// verify step of 832 rows 334 us instead of 316; MT = 2 with 64-key blocks is better with its 174 than with 129: 1664 rows 388 / 400 us).
+// verify step of 832 rows 334 us instead of 316; MT = 2 with 64-key blocks is better with its 174 than with 129: 1664 rows 388 / 400 us).  Four groups that share are told 5
+// (86 registers; left to itself it takes 59: verify steps of 26 rows 112.9 / 115.0, 416 rows of 768 columns 364.4 / 367.5, encoder of 64 ids 215.8 / 219.7, others level to 1 %).
 constexpr int attn_ctas(int mt, int kg, int kw, bool share) { return kg > 1 ? (share && kg == 4 ? 5 : 0) : mt == 4 ? 4 : kw == 32 ? 8 : 1; }
 
 // QNC > 0: the queries are projected here (QueryArgs; MT = 1, KG = 8).  The CTA's 64 rows of Wq are requested ahead of the wait, the
@@ -173,13 +175,16 @@ constexpr int attn_ctas(int mt, int kg, int kw, bool share) { return kg > 1 ? (s
 //     bytes from the lanes of every warp their issue alone took 790 clocks, one lane after the other; 16-byte asynchronous remote stores 0.85 us, plain ones behind a
 //     cluster barrier more.)
 //
-// SHARE: the keys are one block (at most KG KW), and the groups do not add up partial outputs of all 64 columns through shared memory (35 KB written and read for
-// eight groups: 990 + 910 clocks, half of it bank conflicts) but leave their probabilities there, where their keys were (6 KB); every warp then multiplies those of all groups by its own
-// 64 / KG columns of the values.  The groups' shares are scaled and added in the same order with the same roundings: results are the same to the bit.  With the
-// copies above, verify step, us, before / after: 5 rows 104.7 / 98.8, 16 rows 108.1 / 103.3, 136 rows 187.6 / 183.2, 416 rows 248 / 236.6; 768 columns, 26 rows 179.4 / 175.2; drafts of 136 rows
-// 83.6 / 81.8; encoders of 480 rows 419.6 / 410.3.  Over several blocks every warp would read the probabilities of eight groups once a block (2 sequences, 512 keys: 691 / 714 us an encode
-// pass), and tiles of up to four queries over four groups have too little to share (64 sequences, one query each: 161.6 / 166.2): those add partial outputs, in rows of 72 floats
-// that keep stores and loads out of each other's banks (68 before; 2 sequences, 512 keys: 693 / 686).
+// SHARE: the keys are one block (at most SHARE_KEYS), and the groups do not add up partial outputs of all 64 columns through shared memory (35 KB written and read for
+// eight groups: 990 + 910 clocks) but leave their probabilities there, where their keys were (6 KB); every warp then multiplies those of all groups by its own
+// 64 / KG columns of the values.  The groups' shares are scaled and added in the same order with the same roundings: results are the same to the bit.
+// us a pass, in turn: before | with the 2 KB copies above and the pitch below | sharing as well.
+//   verify  5 rows 104.9 | 100.8 | 98.9    16 rows 107.9 | 104.9 | 103.6    26 rows 115.1 | 113.2 | 112.9    416 rows 249.1 | 245.2 | 234.0    624 rows 284.8 | 280.4 | 276.4
+//           832 rows 311.5 | 304.9 | 306.1 (sharing itself loses 0.4 % there)       768 columns, 416 rows 370.7 | 363.4 | 364.4
+//   drafts of 8 x (21 + 16) rows 83.9 | - | 81.4;  encoders of 64 ids 218.7 | 217.9 | 215.8, of 120 268.9 | 266.0 | 262.0, of 480 417.8 | 411.1 | 409.9
+// Over several blocks every warp would read the probabilities of eight groups once a block (2 sequences, 512 keys: 691 / 714 us an encode
+// pass): those add partial outputs, in rows of 72 floats, which keep stores and loads out of each other's banks (68 | 72: 26 rows over 276 keys 133.5 | 130.1, 4 x 26 rows
+// 175.1 | 172.0, encoders of 2 x 512 ids 693.4 | 685.7; no pass of 22 got slower).
 // (QNC and ON stay the last two: the test of the routes reads them off the kernel's name.)
 template <bool PAGED, int MT, int KG, int KW, int NS, bool SHARE = false, int QNC = 0, int ON = 0>
 __global__ void __launch_bounds__(MT * KG * 32, attn_ctas(MT, KG, KW, SHARE)) k_attn(AttnTcArgs a, QueryArgs qa, OutArgs oa) {

@@ -627,7 +627,7 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             const AttnSlots slots = attn_slots(h, cnt, q_ub, n_heads);
             a.seq_of = slots.seq_of;
             const int n_seq = cnt == CNT_ENC ? h->B : std::min(h->B, h->act_ub);
-            const bool share = max_keys <= SHARE_KEYS;              // one block of keys: the groups share their probabilities (see k_attn), with four groups from five queries on
+            const bool share = max_keys <= SHARE_KEYS;       // one block of keys: the groups share their probabilities (see k_attn)
             QueryArgs qa{};
             OutArgs oa{};
             if (qp) qa = *qp;
@@ -676,6 +676,9 @@ int attn_once(specdec_handle* h, bool paged, const void* q, int q_stride, const 
             const bool spread = h->attn_warps || h->attn_stream == 0 || (h->attn_stream == 1 && tiles16 <= 4LL * h->tma.n_sm);
             if (spread) {
                 const bool eight = h->attn_warps ? h->attn_warps == 8 : (max_keys > 256 && tiles16 <= h->tma.n_sm);
+                // Four groups share from five queries on.  With one query there is nothing to gain (64 sequences, partial outputs / shared: 164.5 / 165.4 us a greedy step, 32:
+                // 136.6 / 136.0).  With two to four most passes would be up to 5 % faster (40 sequences x 3 rows 191 / 181, 64 x 4 229.5 / 221.3), level from 96 sequences on,
+                // but 16 x 4 rows 2 to 3 % slower (150.4 / 154.6; 152.4 before anything was shared), 20 x 4 1 % (159.8 / 161.5): the line stays where no pass became slower than it was.
                 if (!eight && share && q_ub > 4)
                     return paged ? go(k_attn<true, 1, 4, 32, 3, true>, 16, 4, AttnCfg<1, 4, 32>::smem(max_keys, 3, true)) : go(k_attn<false, 1, 4, 32, 3, true>, 16, 4, AttnCfg<1, 4, 32>::smem(max_keys, 3, false));
                 return eight ? ATTN_GO(1, 8, 32, 2) : ATTN_GO(1, 4, 32, 3);
